@@ -21,7 +21,7 @@ inline size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 struct Layout {
   size_t status, kbar_hi, kbar_lo, vq, qpp, q_h, q_m, q_l, av, VT, p_h, p_m, p_l, vq3, av3, ukt, qbar_hi, qbar_lo, wts, NT, rA, rB, part, lse, s, anchors, z, m, invm, Y, logphi,
       qcat, wcat, Ut_hi, Ut_lo, S_hi, S_lo, best, kappa, kmap, perm, goff, cursor, LC, Phi, Gram, Linv, rhs, wsol, R, Z,
-      ck3, YT_hi, YT_lo, G64, L64, B64, Z64, X64, Sl, Sl2, eR, eC, ir_u, ir_sq, ir_lam, Sl3, eC2, cl_lam, total;
+      ck3, YT_hi, YT_lo, G64, L64, B64, Z64, X64, Sl, Sl2, eR, eC, ir_u, ir_sq, ir_lam, Sl3, eC2, cl_lam, ctrip, total;
 };
 
 Dims dims_of(const arckv_config& c) {
@@ -146,6 +146,7 @@ Layout plan(const arckv_config& c) {
   L.Sl3 = take(dual ? 5 * H * 128 * sliced_ld((int)n) * 2 : 0);
   L.eC2 = take(dual ? H * 128 * 4 : 0);
   L.cl_lam = take(dual ? H * 8 : 0);
+  L.ctrip = take(dual ? 0 : chol_trip_bytes(c.H_kv, (int)t));
   L.total = o;
   return L;
 }
@@ -380,7 +381,7 @@ arckv_status arckv_compact(const arckv_config* cfg, const void* K, const void* V
             (double*)(w + L.X64), (bf16*)(w + L.Ut_hi),   // Ut_hi [H][T][ldn] is free after the assignment
             (bf16*)(w + L.ck3), (bf16*)(w + L.Sl), (bf16*)(w + L.Sl2), I32(L.eR), I32(L.eC),
             (double*)(w + L.ir_u), (double*)(w + L.ir_sq), (double*)(w + L.ir_lam), (bf16*)(w + L.Sl3),
-            I32(L.eC2), (double*)(w + L.cl_lam)};
+            I32(L.eC2), (double*)(w + L.cl_lam), (uint8_t*)(w + L.ctrip)};
   const int nlf = launch_fits(D, scale, cfg->ridge_w, cfg->ridge_v, cfg->eps_w, cfg->b_min, cfg->b_max, Qb, C_k,
                               F(L.z), F(L.m), F(L.Y), B, beta, C_v, stt, st, ev);
   if (nlf < 0) return ARCKV_ERR_CUDA;

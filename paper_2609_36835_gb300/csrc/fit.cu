@@ -10,18 +10,17 @@
 // right-looking Cholesky factorisation (64 x 64 blocks; each diagonal block
 // is factored and inverted in shared memory) with the forward substitution
 // fused into the trailing updates, then blocked back substitution, all in one
-// cluster launch per system (chol_cluster_kernel).
+// cluster launch per system (chol.cu).
 #include <cooperative_groups.h>
 #include <map>
 #include <mutex>
 #include <type_traits>
 
+#include "chol.cuh"
 #include "kernels.h"
 #include "tc_gemm.cuh"
 
 namespace arckv {
-
-constexpr int NB = kCholNB;
 
 __global__ void phi_kernel(const float* LC, const float* z, float* Phi, int n, int t, long long count) {
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count;
@@ -63,7 +62,7 @@ __global__ void __launch_bounds__(1024) mass_rhs_kernel(const float* Phi, const 
 
 // ---------------------------------------------------------------------------
 // Cluster Cholesky solver: (Gram + lam I) X = B for every head in ONE launch.
-// One cluster of kCL CTAs (cluster_size) per head; the matrix, its factor and the right-hand
+// One cluster of kCL CTAs per head; the matrix, its factor and the right-hand
 // sides live in global memory (L2-resident at these sizes) and are read with
 // ld.global.cg so that no CTA sees a stale L1 line of another CTA's writes.
 // Phases of each 64-wide block step k are separated by hardware cluster
@@ -77,439 +76,8 @@ __global__ void __launch_bounds__(1024) mass_rhs_kernel(const float* Phi, const 
 // Z_i -= L_ki^T X_k (i < k).  lam = ridge * trace(Gram) / tdiv is added to the
 // diagonal as each diagonal block is factored (tdiv = t, or the primal size
 // when the dual system is solved).
-// fp32 systems run the trailing updates and (up to 128 right-hand sides) the
-// back substitution as tcgen05 units of bf16-triple products; with one
-// right-hand side rank 0 does the back substitution alone.  fp64 systems use
-// SIMT tile products throughout.
-// CTAs per cluster (one cluster per head): 4 up to 16 blocks (t <= 1024) --
-// half the SMs of 8 at nearly the same latency, which leaves room for the
-// concurrent layers -- and 8 for longer systems, whose tile work dominates.
-constexpr int cluster_size(int t) { return (t + NB - 1) / NB > 16 ? 8 : 4; }
-constexpr int kCT = 512;
-// Shared tiles are [NB][NBP] with rows padded to a 16-byte multiple, so that
-// mm64 can read them with vector loads.
-template <typename R>
-constexpr int NBP = NB + 16 / (int)sizeof(R);
-template <typename R>
-using Tile = R (*)[NBP<R>];
-template <typename R>
-constexpr int kTileF = NB * NBP<R>;
-
-__device__ __forceinline__ float fma_r(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fma_r(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float rcp_r(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double rcp_r(double x) { return __drcp_rn(x); }
-
-// Double-float arithmetic: a value hi + lo of two fp32 numbers (|lo| <= ulp(hi) / 2),
-// ~48 significant bits.  The GB300's fp64 pipe issues at a small fraction of its
-// fp32 rate, so the fp64 64 x 64 diagonal blocks of the dual Cholesky are
-// factored in this arithmetic (each operation a short chain of fp32 operations:
-// the error-free sum and product transformations of Dekker and Knuth, and one
-// Newton step for the reciprocal and the square root), with the block read
-// from and written back to fp64 storage.
-struct df64 {
-  float hi, lo;
-  df64() = default;
-  __device__ __forceinline__ df64(float h, float l) : hi(h), lo(l) {}
-  __device__ __forceinline__ explicit df64(int v) : hi((float)v), lo(0.f) {}
-};
-__device__ __forceinline__ df64 df_fast2(float a, float b) {   // |a| >= |b| (or a = 0)
-  const float s = a + b;
-  return df64(s, b - (s - a));
-}
-__device__ __forceinline__ df64 df_two(float a, float b) {
-  const float s = a + b, bb = s - a;
-  return df64(s, (a - (s - bb)) + (b - bb));
-}
-__device__ __forceinline__ df64 operator+(df64 x, df64 y) {
-  df64 s = df_two(x.hi, y.hi);
-  const df64 t = df_two(x.lo, y.lo);
-  s.lo += t.hi;
-  s = df_fast2(s.hi, s.lo);
-  s.lo += t.lo;
-  return df_fast2(s.hi, s.lo);
-}
-__device__ __forceinline__ df64 operator-(df64 x) { return df64(-x.hi, -x.lo); }
-__device__ __forceinline__ df64 operator-(df64 x, df64 y) { return x + (-y); }
-__device__ __forceinline__ df64 operator*(df64 x, df64 y) {
-  const float p = x.hi * y.hi;
-  float e = fmaf(x.hi, y.hi, -p);
-  e = fmaf(x.hi, y.lo, e);
-  e = fmaf(x.lo, y.hi, e);
-  return df_fast2(p, e);
-}
-__device__ __forceinline__ df64& operator*=(df64& x, df64 y) { return x = x * y; }
-__device__ __forceinline__ bool operator>(df64 x, df64 y) { return x.hi > y.hi || (x.hi == y.hi && x.lo > y.lo); }
-__device__ __forceinline__ bool finite_r(float x) { return isfinite(x); }
-__device__ __forceinline__ bool finite_r(double x) { return isfinite(x); }
-__device__ __forceinline__ bool finite_r(df64 x) { return isfinite(x.hi); }
-__device__ __forceinline__ df64 fma_r(df64 a, df64 b, df64 c) { return a * b + c; }
-__device__ __forceinline__ df64 rcp_r(df64 x) {   // r + r (1 - x r)
-  const df64 r(__frcp_rn(x.hi), 0.f);
-  return r + r * (df64(1) - x * r);
-}
-__device__ __forceinline__ float sqrt_r(float x) { return sqrtf(x); }
-__device__ __forceinline__ double sqrt_r(double x) { return ::sqrt(x); }
-__device__ __forceinline__ df64 sqrt_r(df64 x) {    // s + (x - s^2) / (2 s)
-  if (!(x.hi > 0.f)) return df64(sqrtf(x.hi), 0.f);
-  const float s = sqrtf(x.hi);
-  const df64 r = x - df64(s, 0.f) * df64(s, 0.f);
-  return df_fast2(s, r.hi * (0.5f / s));
-}
-// storage conversions (the block lives in fp64 in global memory)
-template <typename R, typename G>
-__device__ __forceinline__ R to_reg(G v) { return v; }
-template <>
-__device__ __forceinline__ df64 to_reg<df64, double>(double v) {
-  const float h = __double2float_rn(v);
-  return df64(h, __double2float_rn(v - (double)h));
-}
-template <typename G, typename R>
-__device__ __forceinline__ G to_mem(R v) { return v; }
-template <>
-__device__ __forceinline__ double to_mem<double, df64>(df64 v) { return (double)v.hi + (double)v.lo; }
-template <typename R>
-__device__ __forceinline__ R warp_sum_r(R v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ unsigned cluster_rank() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-
-// S[r][c] = G[(r0 + r) * ld + c0 + c] (or S[c][r] with `trans`), zero outside
-// rows < rmax, cols < cmax of the source block.  Split into a fetch (eight
-// loads per thread into registers) and a put (the shared stores), so that a
-// caller loading two tiles issues all sixteen loads before its first store and
-// pays the L2 latency once.  The transposed form maps a warp to 4 rows x 8
-// columns, so its shared stores hit 32 distinct banks.
-template <typename R>
-struct TileRegs {
-  static constexpr int NE = NB * NB / kCT;
-  R v[NE];
-  bool trans;
-};
-// element q of this thread: (row, col) of the source block
-__device__ __forceinline__ void tile_pos(int q, bool trans, int& r, int& c) {
-  const int e = threadIdx.x + q * kCT;
-  if (!trans) {
-    r = e / NB;
-    c = e % NB;
-  } else {
-    const int lane = e & 31, w = e >> 5;
-    c = (w & 7) * 8 + (lane & 7);
-    r = (w >> 3) * 4 + (lane >> 3);
-  }
-}
-template <typename R>
-__device__ __forceinline__ void tile_fetch(TileRegs<R>& f, const R* G, long long ld, int r0, int c0, int rmax,
-                                           int cmax, bool trans) {
-  f.trans = trans;
-#pragma unroll
-  for (int q = 0; q < TileRegs<R>::NE; ++q) {
-    int r, c;
-    tile_pos(q, trans, r, c);
-    f.v[q] = (r < rmax && c < cmax) ? __ldcg(G + (long long)(r0 + r) * ld + c0 + c) : R(0);
-  }
-}
-template <typename R>
-__device__ __forceinline__ void tile_put(Tile<R> S, const TileRegs<R>& f) {
-#pragma unroll
-  for (int q = 0; q < TileRegs<R>::NE; ++q) {
-    int r, c;
-    tile_pos(q, f.trans, r, c);
-    if (f.trans) S[c][r] = f.v[q];
-    else S[r][c] = f.v[q];
-  }
-}
-template <typename R>
-__device__ __forceinline__ void ld_tile(Tile<R> S, const R* G, long long ld, int r0, int c0, int rmax, int cmax,
-                                        bool trans) {
-  TileRegs<R> f;
-  tile_fetch(f, G, ld, r0, c0, rmax, cmax, trans);
-  tile_put(S, f);
-}
-// two tiles, one L2 round trip
-template <typename R>
-__device__ __forceinline__ void ld_tiles(Tile<R> S1, const R* G1, long long ld1, int r1, int c1, int rm1, int cm1,
-                                         bool tr1, Tile<R> S2, const R* G2, long long ld2, int r2, int c2, int rm2,
-                                         int cm2, bool tr2) {
-  TileRegs<R> f1, f2;
-  tile_fetch(f1, G1, ld1, r1, c1, rm1, cm1, tr1);
-  tile_fetch(f2, G2, ld2, r2, c2, rm2, cm2, tr2);
-  tile_put(S1, f1);
-  tile_put(S2, f2);
-}
-
-// Thread tile of the 64 x 64 products: kTP rows x kTQ columns at (tile_ry, tile_cx).
-// A warp covers 16 rows x 16 columns, so each k step of mm64 costs it one
-// 16-byte load of the transposed left operand (4 rows) and one 8-byte load of
-// the right one (2 columns): two shared wavefronts for 8 FMAs per thread.
-constexpr int kTP = 4, kTQ = 2;
-__device__ __forceinline__ int tile_ry() { return (threadIdx.x >> 7) * 16 + ((threadIdx.x >> 3) & 3) * 4; }
-__device__ __forceinline__ int tile_cx() { return ((threadIdx.x >> 5) & 3) * 16 + (threadIdx.x & 7) * 2; }
-
-// P[p*ld + q] -= acc[p][q] for p < pn, q < qn (all loads issued before the stores)
-template <typename R>
-__device__ __forceinline__ void rmw_sub(R* P, long long ld, int pn, int qn, const R (&acc)[kTP][kTQ]) {
-  R old[kTP][kTQ];
-#pragma unroll
-  for (int p = 0; p < kTP; ++p)
-#pragma unroll
-    for (int q = 0; q < kTQ; ++q) old[p][q] = (p < pn && q < qn) ? __ldcg(P + p * ld + q) : R(0);
-#pragma unroll
-  for (int p = 0; p < kTP; ++p)
-#pragma unroll
-    for (int q = 0; q < kTQ; ++q)
-      if (p < pn && q < qn) P[p * ld + q] = old[p][q] - acc[p][q];
-}
-
-__device__ __forceinline__ void lds2(float (&a)[2], const float* p) {
-  const float2 v = *(const float2*)p;
-  a[0] = v.x; a[1] = v.y;
-}
-__device__ __forceinline__ void lds4(float (&a)[4], const float* p) {
-  const float4 v = *(const float4*)p;
-  a[0] = v.x; a[1] = v.y; a[2] = v.z; a[3] = v.w;
-}
-__device__ __forceinline__ void lds2(double (&a)[2], const double* p) {
-  const double2 v = *(const double2*)p;
-  a[0] = v.x; a[1] = v.y;
-}
-__device__ __forceinline__ void lds4(double (&a)[4], const double* p) {
-  const double2 v = *(const double2*)p, u = *(const double2*)(p + 2);
-  a[0] = v.x; a[1] = v.y; a[2] = u.x; a[3] = u.y;
-}
-
-// acc[p][q] = sum_l XT[l][ry+p] Y[l][cx+q] (ry = tile_ry(), cx = tile_cx()): the left
-// operand is held transposed so that each l takes one 4-wide and one 2-wide
-// shared load.
-template <typename R>
-__device__ __forceinline__ void mm64(Tile<R> XT, Tile<R> Y, R (&acc)[kTP][kTQ]) {
-  const int ry = tile_ry(), cx = tile_cx();
-#pragma unroll
-  for (int p = 0; p < kTP; ++p)
-#pragma unroll
-    for (int q = 0; q < kTQ; ++q) acc[p][q] = R(0);
-#pragma unroll 8
-  for (int l = 0; l < NB; ++l) {
-    R a[4], c[2];
-    lds4(a, &XT[l][ry]);
-    lds2(c, &Y[l][cx]);
-#pragma unroll
-    for (int p = 0; p < kTP; ++p)
-#pragma unroll
-      for (int q = 0; q < kTQ; ++q) acc[p][q] = fma_r(a[p], c[q], acc[p][q]);
-  }
-}
-
-// Load the lower part of A_kk + lam I into the tile L (identity beyond the
-// matrix when kb < NB; zero above the diagonal).
-template <typename R, typename G>
-__device__ __forceinline__ void load_diag(Tile<R> L, const G* Ab, int t, int k0, int kb, G lam) {
-  constexpr int NE = NB * NB / kCT;
-  R v[NE];
-#pragma unroll
-  for (int q = 0; q < NE; ++q) {
-    const int e = threadIdx.x + q * kCT, r = e / NB, c = e % NB;
-    v[q] = (r < kb && c <= r) ? to_reg<R>(__ldcg(Ab + (long long)(k0 + r) * t + k0 + c) + (r == c ? lam : G(0)))
-                              : (r == c ? R(1) : R(0));
-  }
-#pragma unroll
-  for (int q = 0; q < NE; ++q) {
-    const int e = threadIdx.x + q * kCT;
-    L[e / NB][e % NB] = v[q];
-  }
-}
-
-// Write L_kk (lower part, rows < kb) into A and the full tile Li into Linv[k].
-template <typename R, typename G>
-__device__ __forceinline__ void store_diag(Tile<R> L, Tile<R> Li, G* Ab, G* Lb, int t, int k, int kb) {
-  G* Lo = Lb + (long long)k * NB * NB;
-  const int k0 = k * NB;
-  for (int e = threadIdx.x; e < NB * NB; e += kCT) {
-    const int rr = e / NB, cc = e % NB;
-    Lo[e] = cc <= rr ? to_mem<G>(Li[rr][cc]) : G(0);   // the inverse is lower triangular
-    if (rr < kb && cc <= rr) Ab[(long long)(k0 + rr) * t + k0 + cc] = to_mem<G>(L[rr][cc]);
-  }
-}
-
-// Factor diagonal block k (lower part of A_kk + lam I) in shared memory and
-// invert the factor: L_kk goes into A and L_kk^-1 into Linv[k].  Blocked in
-// four 16-wide panels, every phase on all warps:
-//   panel p: factor its 16 x 16 diagonal block (unscaled right-looking, one
-//            element per thread, one barrier per column; then the column
-//            scaling by sqrt(a_cc)) and invert it (forward substitution by
-//            columns, one barrier per row); L_panel = A_panel X_pp^T below it;
-//            trailing update A -= L_panel L_panel^T;
-//   inverse: off-diagonal 16 x 16 blocks X_ij = -X_ii sum_{m=j}^{i-1} L_im X_mj,
-//            level by level (i - j = 1, 2, 3).
-// Tiles: L (the block; pad column NB holds 1 / l_cc), Li (the inverse), T
-// (scratch).  Pad rows beyond the matrix (kb < NB) are the identity.
-template <typename R, typename G = R>
-__device__ void factor_diag(G* Ab, G* Lb, int t, int k, G lam, Tile<R> L, Tile<R> Li, Tile<R> T, int* bad) {
-  static_assert(kCT == 512 && NB == 64, "thread map of the 16-wide panels");
-  const int tid = threadIdx.x, k0 = k * NB, kb = min(NB, t - k0);
-  load_diag(L, Ab, t, k0, kb, lam);
-  for (int e = tid; e < NB * NB; e += kCT) Li[e / NB][e % NB] = R(0);
-  __syncthreads();
-  const bool blk = tid < 256;
-  const int er = (tid >> 4) & 15, ec = tid & 15;   // element of a 16 x 16 block (threads < 256)
-  for (int p = 0; p < 4; ++p) {
-    const int c0 = 16 * p;
-    for (int j = 0; j < 15; ++j) {   // factor the diagonal block
-      if (blk && ec > j && er >= ec) {
-        R piv = L[c0 + j][c0 + j];
-        if (!(piv > R(0)) || !finite_r(piv)) piv = R(1);
-        L[c0 + er][c0 + ec] = fma_r(-L[c0 + er][c0 + j] * rcp_r(piv), L[c0 + ec][c0 + j], L[c0 + er][c0 + ec]);
-      }
-      __syncthreads();
-    }
-    R v = R(0);
-    if (blk && er >= ec) {   // column scaling
-      R pc = L[c0 + ec][c0 + ec];
-      if (!(pc > R(0)) || !finite_r(pc)) {
-        if (er == ec && c0 + ec < kb) *bad = 1;
-        pc = R(1);
-      }
-      const R d = sqrt_r(pc);
-      v = (er == ec) ? d : L[c0 + er][c0 + ec] * rcp_r(d);
-    }
-    __syncthreads();
-    if (blk && er >= ec) {
-      L[c0 + er][c0 + ec] = v;
-      if (er == ec) {
-        L[c0 + er][NB] = rcp_r(v);
-        Li[c0 + er][c0 + er] = R(1);
-      }
-    }
-    __syncthreads();
-    for (int i = 0; i < 15; ++i) {   // Y = I; y_lj -= l_li y_ij / l_ii for l > i, j <= i
-      if (blk && er > i && ec <= i)
-        Li[c0 + er][c0 + ec] = fma_r(-L[c0 + er][c0 + i] * L[c0 + i][NB], Li[c0 + i][c0 + ec], Li[c0 + er][c0 + ec]);
-      __syncthreads();
-    }
-    if (blk && ec <= er) Li[c0 + er][c0 + ec] *= L[c0 + er][NB];   // X_pp = diag(1 / l_rr) Y
-    __syncthreads();
-    if (p == 3) break;
-    {  // panel below: L[r][c0 + c] = sum_m A[r][c0 + m] X_pp[c][m] (all reads before the writes)
-      const int rows = NB - c0 - 16;
-      R o[2];
-      int pr[2], pcol[2];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int e = tid + q * kCT;
-        pr[q] = -1;
-        if (e < rows * 16) {
-          const int r = c0 + 16 + e / 16, c = e % 16;
-          R a = R(0);
-          for (int m = 0; m <= c; ++m) a = fma_r(L[r][c0 + m], Li[c0 + c][c0 + m], a);
-          o[q] = a;
-          pr[q] = r;
-          pcol[q] = c;
-        }
-      }
-      __syncthreads();
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-        if (pr[q] >= 0) L[pr[q]][c0 + pcol[q]] = o[q];
-      __syncthreads();
-    }
-    {  // trailing update: L[r][c] -= sum_m L[r][c0 + m] L[c][c0 + m], c0 + 16 <= c <= r
-      const int c1 = c0 + 16, wdt = NB - c1, ntri = wdt * (wdt + 1) / 2;
-      for (int e = tid; e < ntri; e += kCT) {
-        int r = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
-        while (r * (r + 1) / 2 > e) --r;
-        while ((r + 1) * (r + 2) / 2 <= e) ++r;
-        const int c = e - r * (r + 1) / 2;
-        R a = L[c1 + r][c1 + c];
-#pragma unroll
-        for (int m = 0; m < 16; ++m) a = fma_r(-L[c1 + r][c0 + m], L[c1 + c][c0 + m], a);
-        L[c1 + r][c1 + c] = a;
-      }
-      __syncthreads();
-    }
-  }
-  for (int lv = 1; lv < 4; ++lv) {   // off-diagonal blocks of the inverse, level i - j = lv
-    const int nbk = 4 - lv;
-    for (int e = tid; e < nbk * 256; e += kCT) {
-      const int j = e >> 8, i = j + lv, r = (e >> 4) & 15, c = e & 15;
-      R a = R(0);
-      for (int m = j; m < i; ++m)
-#pragma unroll
-        for (int q = 0; q < 16; ++q) a = fma_r(L[16 * i + r][16 * m + q], Li[16 * m + q][16 * j + c], a);
-      T[16 * i + r][16 * j + c] = a;
-    }
-    __syncthreads();
-    for (int e = tid; e < nbk * 256; e += kCT) {
-      const int j = e >> 8, i = j + lv, r = (e >> 4) & 15, c = e & 15;
-      R a = R(0);
-      for (int q = 0; q <= r; ++q) a = fma_r(Li[16 * i + r][16 * i + q], T[16 * i + q][16 * j + c], a);
-      Li[16 * i + r][16 * j + c] = -a;
-    }
-    __syncthreads();
-  }
-  store_diag(L, Li, Ab, Lb, t, k, kb);
-  __syncthreads();
-}
-
-// S[r][c] = G1[(r0 + r) * ld + c0 + c] + G2[...] (zero outside rows < rmax, cols < cmax)
-template <typename R>
-__device__ __forceinline__ void ld_tile_sum(Tile<R> S, const R* G1, const R* G2, long long ld, int r0, int c0,
-                                            int rmax, int cmax) {
-  constexpr int NE = NB * NB / kCT;
-  R v[NE], u[NE];
-#pragma unroll
-  for (int q = 0; q < NE; ++q) {
-    const int e = threadIdx.x + q * kCT, r = e / NB, c = e % NB;
-    const bool ok = r < rmax && c < cmax;
-    const long long o = (long long)(r0 + r) * ld + c0 + c;
-    v[q] = ok ? __ldcg(G1 + o) : R(0);
-    u[q] = ok ? __ldcg(G2 + o) : R(0);
-  }
-#pragma unroll
-  for (int q = 0; q < NE; ++q) {
-    const int e = threadIdx.x + q * kCT;
-    S[e / NB][e % NB] = v[q] + u[q];
-  }
-}
-
-// P[p*ld + q] = acc[p][q] for p < pn, q < qn
-template <typename R>
-__device__ __forceinline__ void st_acc(R* P, long long ld, int pn, int qn, const R (&acc)[kTP][kTQ]) {
-#pragma unroll
-  for (int p = 0; p < kTP; ++p)
-#pragma unroll
-    for (int q = 0; q < kTQ; ++q)
-      if (p < pn && q < qn) P[p * ld + q] = acc[p][q];
-}
-
-// Eight fp32 values of operand row r, K elements 8 ch .. 8 ch + 7, as bf16
-// triples at their 128-byte-swizzled K-major positions (row r at r * 128
-// bytes, 16-byte chunk ch at ch ^ (r % 8)) of the three part tiles.
-__device__ __forceinline__ void put_split3_chunk(uint8_t* h, uint8_t* m, uint8_t* l, int r, int ch,
-                                                 const float (&x)[8]) {
-  __align__(16) bf16 hh[8], mm[8], ll[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) split3_bf16(x[e], hh[e], mm[e], ll[e]);
-  const int off = r * 128 + ((ch ^ (r & 7)) << 4);
-  *(uint4*)(h + off) = *(const uint4*)hh;
-  *(uint4*)(m + off) = *(const uint4*)mm;
-  *(uint4*)(l + off) = *(const uint4*)ll;
-}
-
-// Shared memory of the fp32 solver beyond its four tiles: the bf16 triples of
-// the tensor-core update operands (A: 128 x 64, B: 64 x 64), 1024-byte aligned.
-constexpr int kTcStageA = 128 * 128, kTcStageB = 64 * 128;
-constexpr int kTcStageBytes = 3 * (kTcStageA + kTcStageB) + 1024;
-
+// SIMT tile products throughout: the fp64 dual systems beyond kSlicedMaxK (the
+// fp32 systems run in chol.cu).
 template <typename R, int kCL>
 __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
     chol_cluster_kernel(R* A, R* Linv, R* B, R* Z, R* X, int t, int nrhs, int ldb, long long bbs, R ridge, R tdiv,
@@ -524,10 +92,6 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
   __shared__ R red[kCT / 32];
   __shared__ int bad, grab;
   __shared__ int ctr[2];   // rank 0's pair deals the tiles of alternate dynamic phases
-  constexpr bool kTc = std::is_same<R, float>::value;   // tensor-core trailing updates (fp32 systems)
-  __shared__ uint64_t mma_bar;
-  __shared__ uint32_t tmem_slot;
-  __shared__ int tc_abort;
   const int head = blockIdx.x / kCL;
   const int rank = (int)cluster_rank();
   const int tid = threadIdx.x;
@@ -540,33 +104,6 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
   const int ry = tile_ry(), cx = tile_cx();
   R acc[kTP][kTQ];
   int* ctr0 = cg::this_cluster().map_shared_rank(ctr, 0);
-  // tensor-core update state: operand triples, a 64-column TMEM accumulator, its mbarrier
-  uint8_t* stg = nullptr;
-  uint32_t tmem = 0, mma_ph = 0;
-  if constexpr (kTc) {
-    const uint32_t s0 = tc::smem_u32(smraw), e0 = s0 + 4u * kTileF<R> * (uint32_t)sizeof(R);
-    stg = smraw + (((e0 + 1023u) & ~1023u) - s0);
-    if (tid == 0) {
-      tc::mbar_init(&mma_bar, 1);
-      tc_abort = 0;
-      tc::mbar_fence_init();
-    }
-    if (tid < 32) tc::tmem_alloc(&tmem_slot, 64);
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    tmem = tmem_slot;
-  }
-  auto tc_release = [&]() {   // every exit of a CTA that allocated TMEM
-    if constexpr (kTc) {
-      tc::fence_before_sync();
-      __syncthreads();
-      if (tid < 32) {
-        tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, 64);
-      }
-    }
-  };
   int ep = 0;   // dynamic phase number; phase ep draws from ctr0[ep & 1]
   // next tile of the current dynamic phase (block-uniform)
   auto next_tile = [&]() -> int {
@@ -575,24 +112,6 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
     __syncthreads();
     return grab;
   };
-  // the same with the grab issued one draw ahead: next_tile_ahead() returns the
-  // index grabbed by the previous call and already issues the following grab,
-  // whose round trip to rank 0 then overlaps the caller's unit (thread 0 keeps
-  // it in a register); start_ahead() issues the first grab of a phase
-  int ahead = 0;
-  auto start_ahead = [&]() {
-    if (tid == 0) ahead = atomicAdd(ctr0 + (ep & 1), 1);
-  };
-  auto next_tile_ahead = [&]() -> int {
-    __syncthreads();
-    if (tid == 0) {
-      grab = ahead;
-      ahead = atomicAdd(ctr0 + (ep & 1), 1);
-    }
-    __syncthreads();
-    return grab;
-  };
-
   // lam = ridge * trace / t (every CTA forms it; the trace precedes all writes)
   R tr = R(0);
   for (int r = tid; r < t; r += kCT) tr += __ldcg(Ab + (long long)r * t + r);
@@ -689,238 +208,6 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
   };
 
 
-  // Tensor-core trailing update (fp32 systems).  Row i of step k holds the
-  // syrk tiles A_ij -= L_ik L_jk^T (j = k+1 .. i) and then the rhs tiles
-  // B_i -= L_ik Y_k; all share L_ik, so a unit takes two tiles of one row:
-  //   D [128 x 64] = [X_1; X_2] L_ik^T,  X = L_jk (syrk) or Y_k^T (rhs),
-  // D's rows m < 64 being tile 1 transposed and the rest tile 2.  Operands
-  // enter as bf16 triples (hh, hm, mh, hl, lh, mm per 16-wide K step:
-  // fp32-grade products); one thread issues the 24 MMAs into TMEM and every
-  // warp then subtracts a 32-row x 16-column slice of D from its tile.
-  // D [128 x 64] = A B^T from the staged triples (24 MMAs by one thread), then
-  // wait for it; false when the wait gave up
-  auto tc_mma = [&]() -> bool {
-    uint8_t *Ah = stg, *Am = stg + kTcStageA, *Al = stg + 2 * kTcStageA;
-    uint8_t *Bh = stg + 3 * kTcStageA, *Bm = Bh + kTcStageB, *Bl = Bh + 2 * kTcStageB;
-    tc::fence_proxy_async_smem();
-    __syncthreads();
-    if (tid == 0) {
-      tc::fence_after_sync();
-      constexpr uint32_t idesc = tc::idesc_bf16_f32(64);
-#pragma unroll
-      for (int ks = 0; ks < 4; ++ks) {
-        const uint32_t o = ks * 32;
-        const uint64_t ah = tc::sdesc_k128(tc::smem_u32(Ah) + o), am = tc::sdesc_k128(tc::smem_u32(Am) + o),
-                       al = tc::sdesc_k128(tc::smem_u32(Al) + o);
-        const uint64_t bh = tc::sdesc_k128(tc::smem_u32(Bh) + o), bm = tc::sdesc_k128(tc::smem_u32(Bm) + o),
-                       bl = tc::sdesc_k128(tc::smem_u32(Bl) + o);
-        tc::mma_f16(tmem, ah, bh, idesc, ks > 0 ? 1u : 0u);
-        tc::mma_f16(tmem, ah, bm, idesc, 1u);
-        tc::mma_f16(tmem, am, bh, idesc, 1u);
-        tc::mma_f16(tmem, ah, bl, idesc, 1u);
-        tc::mma_f16(tmem, al, bh, idesc, 1u);
-        tc::mma_f16(tmem, am, bm, idesc, 1u);
-      }
-      tc::mma_commit(&mma_bar);
-    }
-    volatile int* abp = &tc_abort;
-    const bool ok = tc::mbar_wait(&mma_bar, mma_ph, abp, stt);
-    mma_ph ^= 1u;
-    tc::fence_after_sync();
-    return ok;
-  };
-  // operand rows r < rows of a triple from a column-major source: element
-  // (r, l) = G[l * ld + r] (+ G2[...] when given) for r < rvalid, l < kvalid,
-  // zero elsewhere; consecutive threads take consecutive r (coalesced)
-  auto stage_cols = [&](uint8_t* h, uint8_t* mm, uint8_t* l, int rows, const R* G, const R* G2, long long ld,
-                        int rvalid, int kvalid) {
-    for (int task = tid; task < rows * 8; task += kCT) {
-      const int r = task % rows, ch = task / rows;
-      float xv[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int kk = 8 * ch + q;
-        float v = 0.f;
-        if (r < rvalid && kk < kvalid) {
-          v = (float)__ldcg(G + (long long)kk * ld + r);
-          if (G2) v += (float)__ldcg(G2 + (long long)kk * ld + r);
-        }
-        xv[q] = v;
-      }
-      put_split3_chunk(h, mm, l, r, ch, xv);
-    }
-  };
-  // D's slice of this warp: rows (TMEM lanes) 32 (w % 4) + lane, columns 16 (w / 4) ..
-  auto tc_slice = [&](float (&v)[16], int& mrow, int& ncol) {
-    const int warp = tid >> 5, lane = tid & 31, q = warp & 3, g = warp >> 2;
-    tc::tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * 16), v);
-    mrow = q * 32 + lane;
-    ncol = g * 16;
-  };
-  // back substitution on the tensor cores (nrhs <= 128): rows m of D are the
-  // right-hand-side columns, its columns n the rows of the block
-  //   Z_i -= L_ki^T X_k:     D = X_k^T L_ki,         Z_i[n][m] -= D[m][n]
-  //   X_k = Linv^T (Y + Z):  D = (Y_k + Z_k)^T Linv,  X_k[n][m] = D[m][n]
-  auto tc_z_unit = [&](int k, int i) {
-    const int k0 = k * NB, kb = min(NB, t - k0), i0 = i * NB;
-    uint8_t* Ah = stg;
-    uint8_t* Bh = stg + 3 * kTcStageA;
-    stage_cols(Ah, Ah + kTcStageA, Ah + 2 * kTcStageA, 128, Xb + (long long)k0 * ldb, nullptr, ldb, nrhs, kb);
-    stage_cols(Bh, Bh + kTcStageB, Bh + 2 * kTcStageB, 64, Ab + (long long)k0 * t + i0, nullptr, t, 64, kb);
-    const bool ok = tc_mma();
-    float v[16];
-    int mrow, ncol;
-    tc_slice(v, mrow, ncol);
-    if (ok && mrow < nrhs) {   // block i < k is full
-      R* dst = Zb + (long long)(i0 + ncol) * ldb + mrow;
-      R old[16];
-#pragma unroll
-      for (int c = 0; c < 16; ++c) old[c] = __ldcg(dst + (long long)c * ldb);
-#pragma unroll
-      for (int c = 0; c < 16; ++c) dst[(long long)c * ldb] = old[c] - (R)v[c];
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-  };
-  auto tc_x_unit = [&](int k) {
-    const int k0 = k * NB, kb = min(NB, t - k0);
-    uint8_t* Ah = stg;
-    uint8_t* Bh = stg + 3 * kTcStageA;
-    stage_cols(Ah, Ah + kTcStageA, Ah + 2 * kTcStageA, 128, Bb + (long long)k0 * ldb, Zb + (long long)k0 * ldb, ldb,
-               nrhs, kb);
-    stage_cols(Bh, Bh + kTcStageB, Bh + 2 * kTcStageB, 64, Lb + (long long)k * NB * NB, nullptr, NB, 64, NB);
-    const bool ok = tc_mma();
-    float v[16];
-    int mrow, ncol;
-    tc_slice(v, mrow, ncol);
-    if (ok && mrow < nrhs) {
-      R* dst = Xb + (long long)(k0 + ncol) * ldb + mrow;
-#pragma unroll
-      for (int c = 0; c < 16; ++c)
-        if (ncol + c < kb) dst[(long long)c * ldb] = (R)v[c];
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-  };
-  auto tc_units = [&](int m) {   // units of step k with m trailing blocks
-    int u = 0;
-    for (int ii = 0; ii < m; ++ii) u += (ii + 2 + nct) / 2;
-    return u;
-  };
-  auto tc_update_unit = [&](int k, int m, int x) {
-    const int k0 = k * NB;
-    int ii = 0, rem = x;
-    for (; ii < m; ++ii) {
-      const int u = (ii + 2 + nct) / 2;
-      if (rem < u) break;
-      rem -= u;
-    }
-    const int i0 = (k + 1 + ii) * NB, len = ii + 1 + nct, e0 = 2 * rem;
-    uint8_t *Ah = stg, *Am = stg + kTcStageA, *Al = stg + 2 * kTcStageA;
-    uint8_t *Bh = stg + 3 * kTcStageA, *Bm = Bh + kTcStageB, *Bl = Bh + 2 * kTcStageB;
-    // B operand: L_ik, rows i0 + n (zero past t), K = block k (full)
-    for (int task = tid; task < 64 * 8; task += kCT) {
-      const int n = task >> 3, ch = task & 7;
-      float xv[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        xv[e] = (i0 + n < t) ? (float)__ldcg(Ab + (long long)(i0 + n) * t + k0 + 8 * ch + e) : 0.f;
-      put_split3_chunk(Bh, Bm, Bl, n, ch, xv);
-    }
-    // A operand: rows 64 h + r from tile e0 + h
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int e = e0 + h;
-      if (e < ii + 1) {   // syrk: L_jk rows j0 + r
-        const int j0 = (k + 1 + e) * NB;
-        for (int task = tid; task < 64 * 8; task += kCT) {
-          const int r = task >> 3, ch = task & 7;
-          float xv[8];
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            xv[q] = (j0 + r < t) ? (float)__ldcg(Ab + (long long)(j0 + r) * t + k0 + 8 * ch + q) : 0.f;
-          put_split3_chunk(Ah, Am, Al, 64 * h + r, ch, xv);
-        }
-      } else if (e < len) {   // rhs: Y_k^T, row r = column c0 + r of Y_k (zero past nrhs)
-        const int c0 = (e - ii - 1) * NB;
-        for (int task = tid; task < 64 * 8; task += kCT) {
-          const int r = task & 63, ch = task >> 6;
-          float xv[8];
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            xv[q] = (c0 + r < nrhs) ? (float)__ldcg(Bb + (long long)(k0 + 8 * ch + q) * ldb + c0 + r) : 0.f;
-          put_split3_chunk(Ah, Am, Al, 64 * h + r, ch, xv);
-        }
-      } else {   // no second tile
-        for (int task = tid; task < 64 * 8; task += kCT) {
-          const float z[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-          put_split3_chunk(Ah, Am, Al, 64 * h + (task >> 3), task & 7, z);
-        }
-      }
-    }
-    tc::fence_proxy_async_smem();
-    __syncthreads();
-    if (tid == 0) {
-      tc::fence_after_sync();
-      constexpr uint32_t idesc = tc::idesc_bf16_f32(64);
-#pragma unroll
-      for (int ks = 0; ks < 4; ++ks) {
-        const uint32_t o = ks * 32;
-        const uint64_t ah = tc::sdesc_k128(tc::smem_u32(Ah) + o), am = tc::sdesc_k128(tc::smem_u32(Am) + o),
-                       al = tc::sdesc_k128(tc::smem_u32(Al) + o);
-        const uint64_t bh = tc::sdesc_k128(tc::smem_u32(Bh) + o), bm = tc::sdesc_k128(tc::smem_u32(Bm) + o),
-                       bl = tc::sdesc_k128(tc::smem_u32(Bl) + o);
-        tc::mma_f16(tmem, ah, bh, idesc, ks > 0 ? 1u : 0u);
-        tc::mma_f16(tmem, ah, bm, idesc, 1u);
-        tc::mma_f16(tmem, am, bh, idesc, 1u);
-        tc::mma_f16(tmem, ah, bl, idesc, 1u);
-        tc::mma_f16(tmem, al, bh, idesc, 1u);
-        tc::mma_f16(tmem, am, bm, idesc, 1u);
-      }
-      tc::mma_commit(&mma_bar);
-    }
-    volatile int* abp = &tc_abort;
-    const bool ok = tc::mbar_wait(&mma_bar, mma_ph, abp, stt);
-    mma_ph ^= 1u;
-    tc::fence_after_sync();
-    // warp w: TMEM lanes 32 (w % 4) .. (rows of D), columns 16 (w / 4) ..
-    const int warp = tid >> 5, lane = tid & 31, q = warp & 3, g = warp >> 2;
-    float v[16];
-    tc::tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * 16), v);
-    const int h = q >> 1, r = (q & 1) * 32 + lane, e = e0 + h;
-    if (ok && e < len) {
-      R* dst;
-      long long ld;
-      bool col_ok;
-      if (e < ii + 1) {   // A_ij[n][r] -= D[64 h + r][n]
-        const int j0 = (k + 1 + e) * NB;
-        dst = Ab + (long long)i0 * t + j0 + r;
-        ld = t;
-        col_ok = j0 + r < t;
-      } else {            // B_i[n][c0 + r] -= D[64 h + r][n]
-        const int c0 = (e - ii - 1) * NB;
-        dst = Bb + (long long)i0 * ldb + c0 + r;
-        ld = ldb;
-        col_ok = c0 + r < nrhs;
-      }
-      if (col_ok) {
-        R old[16];
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          const int n = 16 * g + c;
-          old[c] = (i0 + n < t) ? __ldcg(dst + (long long)n * ld) : R(0);
-        }
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          const int n = 16 * g + c;
-          if (i0 + n < t) dst[(long long)n * ld] = old[c] - (R)v[c];
-        }
-      }
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-  };
-
   // step k = -1 only factors the first diagonal block (one call site keeps the
   // register-resident factorisation inlined once)
   for (int k = -1; k < nblk; ++k) {
@@ -954,29 +241,15 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
     // updates); every CTA then draws the remaining tiles from the counter
     const int ntri = k >= 0 ? m * (m + 1) / 2 : 0, ntot = k >= 0 ? ntri + m * nct : 0;
     if (rank == 0 && tid == 0) ctr[(ep + 1) & 1] = 0;
-    if constexpr (kTc) {
-      // unit 0 holds the diagonal tile (k+1, k+1): its owner updates and factors it first
-      const int nu = k >= 0 ? tc_units(m) : 0;
-      if (rank == (k + 1) % kCL) {
-        if (k >= 0) tc_update_unit(k, m, 0);
-        factor_diag(Ab, Lb, t, k + 1, lam, S1, S2, S3, &bad);
-      }
-      start_ahead();
-      for (;;) {
-        const int x = 1 + next_tile_ahead();
-        if (x >= nu) break;
-        tc_update_unit(k, m, x);
-      }
-    } else {
-      if (rank == (k + 1) % kCL) {
-        if (k >= 0) update_tiles(k, 0, ntot, ntot, ntri);
-        factor_diag(Ab, Lb, t, k + 1, lam, S1, S2, S3, &bad);
-      }
-      for (;;) {   // tiles are drawn two at a time
-        const int x = 1 + 2 * next_tile();
-        if (x >= ntot) break;
-        update_tiles(k, x, x + 1, ntot, ntri);
-      }
+    if (rank == (k + 1) % kCL) {
+      if (k >= 0) update_tiles(k, 0, ntot, ntot, ntri);
+      load_diag(S1, Ab, t, (k + 1) * NB, min(NB, t - (k + 1) * NB), lam);
+      factor_diag<R>(Ab, Lb, t, k + 1, S1, S2, S3, &bad);
+    }
+    for (;;) {   // tiles are drawn two at a time
+      const int x = 1 + 2 * next_tile();
+      if (x >= ntot) break;
+      update_tiles(k, x, x + 1, ntot, ntri);
     }
     ++ep;
     cluster_sync_all();
@@ -1006,72 +279,6 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
     rmw_sub(Zb + (long long)(i0 + ry) * ldb + c0 + cx, ldb, NB - ry, nc - cx, acc);   // block i < k is full
     __syncthreads();
   };
-  if (nrhs == 1 && t <= 2 * kTileF<R>) {
-    // one right-hand side: the block steps are 64-long mat-vecs whose cost is
-    // the barrier between them, so rank 0 runs them alone with CTA barriers
-    // (Z in shared memory) and the other CTAs of the cluster leave
-    if (rank == 0) {
-      R* zs = &S3[0][0];   // Z [t] in S3 and S4 (free now: t <= 2 kTileF)
-      R* vs = &S1[0][0];   // Y_k + Z_k [64]
-      R* xs = &S1[1][0];   // X_k [64]
-      for (int e = tid; e < t; e += kCT) zs[e] = R(0);
-      __syncthreads();
-      for (int k = nblk - 1; k >= 0; --k) {
-        const int k0 = k * NB, kb = min(NB, t - k0);
-        if (tid < NB) vs[tid] = tid < kb ? __ldcg(Bb + (long long)(k0 + tid) * ldb) + zs[k0 + tid] : R(0);
-        __syncthreads();
-        {  // X_k[c] = sum_l Linv_k[l][c] v[l]: eight threads per column, l = part, part + 8, ...
-          const int c = tid >> 3, part = tid & 7;
-          const R* Li = Lb + (long long)k * NB * NB;
-          R a = R(0);
-#pragma unroll
-          for (int l = part; l < NB; l += 8) a = fma_r(__ldcg(Li + l * NB + c), vs[l], a);
-          a += __shfl_xor_sync(0xffffffffu, a, 1);
-          a += __shfl_xor_sync(0xffffffffu, a, 2);
-          a += __shfl_xor_sync(0xffffffffu, a, 4);
-          if (part == 0) {
-            xs[c] = c < kb ? a : R(0);
-            if (c < kb) Xb[(long long)(k0 + c) * ldb] = a;
-          }
-        }
-        __syncthreads();
-        // Z_j -= L_kj^T X_k for the columns before block k (one thread per column)
-        for (int cc = tid; cc < k0; cc += kCT) {
-          R a = R(0);
-          for (int l = 0; l < kb; ++l) a = fma_r(__ldcg(Ab + (long long)(k0 + l) * t + cc), xs[l], a);
-          zs[cc] -= a;
-        }
-        __syncthreads();
-      }
-    }
-    if (tid == 0 && bad) set_status(stt, ARCKV_ERR_NOT_SPD);
-    tc_release();
-    return;
-  }
-  if constexpr (kTc) {
-    if (nrhs <= 128) {
-      if (rank == (nblk - 1) % kCL) tc_x_unit(nblk - 1);
-      cluster_sync_all();
-      for (int k = nblk - 1; k >= 1; --k) {
-        if (rank == 0 && tid == 0) ctr[(ep + 1) & 1] = 0;
-        if (rank == (k - 1) % kCL) {   // the owner of block k-1 finishes Z_{k-1} and forms X_{k-1}
-          tc_z_unit(k, k - 1);
-          tc_x_unit(k - 1);
-        }
-        start_ahead();
-        for (;;) {
-          const int i = next_tile_ahead();
-          if (i >= k - 1) break;
-          tc_z_unit(k, i);
-        }
-        ++ep;
-        cluster_sync_all();
-      }
-      if (tid == 0 && bad) set_status(stt, ARCKV_ERR_NOT_SPD);
-      tc_release();
-      return;
-    }
-  }
   if (rank == (nblk - 1) % kCL) form_x(nblk - 1);
   cluster_sync_all();
   for (int k = nblk - 1; k >= 1; --k) {
@@ -1090,21 +297,14 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
     cluster_sync_all();
   }
   if (tid == 0 && bad) set_status(stt, ARCKV_ERR_NOT_SPD);
-  tc_release();
 }
 
-template <typename R>
-static int cholesky_solve(int H, int t, R* Gram, R* Linv, R* B, R* Z, R* X, int ldb, int nrhs, long long bbs,
-                          float ridge, DevStatus* stt, cudaStream_t st, int tdiv = 0) {
-  const int smem = 4 * kTileF<R> * (int)sizeof(R) + (std::is_same<R, float>::value ? kTcStageBytes : 0);
-  const R td = (R)(tdiv > 0 ? tdiv : t);
-  if (cluster_size(t) == 8) {
-    set_dyn_smem((const void*)chol_cluster_kernel<R, 8>, smem);
-    chol_cluster_kernel<R, 8><<<8 * H, kCT, smem, st>>>(Gram, Linv, B, Z, X, t, nrhs, ldb, bbs, (R)ridge, td, stt);
-  } else {
-    set_dyn_smem((const void*)chol_cluster_kernel<R, 4>, smem);
-    chol_cluster_kernel<R, 4><<<4 * H, kCT, smem, st>>>(Gram, Linv, B, Z, X, t, nrhs, ldb, bbs, (R)ridge, td, stt);
-  }
+// The fp64 system on SIMT tile products (dual fits beyond kSlicedMaxK).
+static int cholesky_solve64(int H, int n, double* A, double* Linv, double* B, double* Z, double* X, int nrhs,
+                            long long bbs, double ridge, double tdiv, DevStatus* stt, cudaStream_t st) {
+  const int smem = 4 * kTileF<double> * (int)sizeof(double);
+  if (set_dyn_smem((const void*)chol_cluster_kernel<double, 8>, smem) != cudaSuccess) return -1;
+  chol_cluster_kernel<double, 8><<<8 * H, kCT, smem, st>>>(A, Linv, B, Z, X, n, nrhs, nrhs, bbs, ridge, tdiv, stt);
   return 1;
 }
 
@@ -1349,8 +549,8 @@ __global__ void __launch_bounds__(kCT, 1) chol_diag_kernel(double* A, double* Li
   const int b = blockIdx.x, nblk = (n + NB - 1) / NB;
   if (threadIdx.x == 0) bad = 0;
   __syncthreads();
-  factor_diag<df64, double>(A + (long long)b * n * n, Linv + (long long)b * nblk * NB * NB, n, k, lam[b], S1, S2, S3,
-                            &bad);
+  load_diag(S1, A + (long long)b * n * n, n, k * NB, min(NB, n - k * NB), lam[b]);
+  factor_diag<df64, double>(A + (long long)b * n * n, Linv + (long long)b * nblk * NB * NB, n, k, S1, S2, S3, &bad);
   if (threadIdx.x == 0 && bad) set_status(stt, ARCKV_ERR_NOT_SPD);
 }
 
@@ -1708,7 +908,7 @@ static int fits_dual(const Dims& D, float ridge_w, float ridge_v, float eps_w, f
   const CholSlicedBufs CW{B.Sl, B.Sl2, B.Sl3, B.eR, B.eC, B.eC2, B.cl_lam, B.Z64};
   auto solve = [&](int nrhs, long long nrow, float ridge) -> int {
     if (sliced) return chol_solve_sliced(D.H, D.n, B.G64, B.L64, B.B64, B.X64, nrhs, ridge, D.t, CW, stt, st);
-    return cholesky_solve<double>(D.H, D.n, B.G64, B.L64, B.B64, B.Z64, B.X64, nrhs, nrhs, nrow, ridge, stt, st, D.t);
+    return cholesky_solve64(D.H, D.n, B.G64, B.L64, B.B64, B.Z64, B.X64, nrhs, nrow, ridge, D.t, stt, st);
   };
   mark(8);
   widen_kernel<<<cdiv((long long)D.H * D.n, 256), 256, 0, st>>>(m, B.B64, (long long)D.H * D.n);
@@ -1752,23 +952,55 @@ static int fits_dual(const Dims& D, float ridge_w, float ridge_v, float eps_w, f
 // x += (L L^T)^-1 r with the factor the solver left behind: L_kk and the
 // off-diagonal blocks in the Gram's lower part, L_kk^-1 in Linv.
 
+// fp32 -> fp64 by moving the fields (IEEE 754: the exponent rebiased by 1023 -
+// 127, the fraction padded; subnormals -- a fifth of Phi -- scaled by 2^64
+// first): GB300 converts fewer than one value per clock and SM, which held the
+// residual passes at 62 and 64 us for 27 MB of Phi (8 heads, n = 1024, t = 819);
+// they take 37 and 27 us this way.
+// Infinities and NaN take the conversion.
+__device__ __forceinline__ double widen_bits(float x) {
+  const bool small = (__float_as_uint(x) & 0x7f800000u) == 0u;
+  const unsigned u = __float_as_uint(small ? x * 18446744073709551616.f : x), ex = u & 0x7f800000u;
+  if (ex == 0x7f800000u) return (double)x;
+  const unsigned hi = (u & 0x80000000u) | (ex ? ((u & 0x7fffffffu) >> 3) + (small ? 0x34000000u : 0x38000000u) : 0u);
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+
 // u[b][i] = m_i - sum_r Phi_ir x_r (fp64); with sq, also sq[b][i] = sum_r Phi_ir^2.
-// One warp per row.
+// One warp per row, eight loads in flight per lane; x is widened once per CTA.
+constexpr int kIrTile = 2048;   // columns of x in shared memory at a time
 __global__ void __launch_bounds__(256) ir_rows_kernel(const float* __restrict__ Phi, const float* __restrict__ m,
                                                       const float* __restrict__ x, double* __restrict__ u,
-                                                      double* __restrict__ sq, int n, int t, int H) {
+                                                      double* __restrict__ sq, int n, int t) {
+  __shared__ double xd[kIrTile];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long gr = (long long)blockIdx.x * 8 + warp;
-  if (gr >= (long long)H * n) return;
-  const int b = (int)(gr / n);
+  const int b = blockIdx.y, row = blockIdx.x * 8 + warp;
+  const long long gr = (long long)b * n + row;
   const float* p = Phi + gr * t;
   const float* xb = x + (long long)b * t;
   double a = 0.0, q = 0.0;
-  for (int r = lane; r < t; r += 32) {
-    const double v = p[r];
-    a = fma(v, (double)xb[r], a);
-    if (sq) q = fma(v, v, q);
+  for (int c0 = 0; c0 < t; c0 += kIrTile) {
+    const int cn = min(kIrTile, t - c0);
+    __syncthreads();
+    for (int c = threadIdx.x; c < cn; c += 256) xd[c] = widen_bits(xb[c0 + c]);
+    __syncthreads();
+    if (row < n) {
+      for (int r0 = lane; r0 < cn; r0 += 256) {
+        float pv[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) pv[e] = r0 + 32 * e < cn ? p[c0 + r0 + 32 * e] : 0.f;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          if (r0 + 32 * e < cn) {
+            const double v = widen_bits(pv[e]);
+            a = fma(v, xd[r0 + 32 * e], a);
+            if (sq) q = fma(v, v, q);
+          }
+        }
+      }
+    }
   }
+  if (row >= n) return;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     a += __shfl_xor_sync(0xffffffffu, a, o);
@@ -1799,41 +1031,241 @@ __global__ void __launch_bounds__(256) ir_lambda_kernel(const double* __restrict
 }
 
 // r[b][c] = sum_i Phi_ic u_i - lam x_c (fp64 sums, rounded to fp32 at the end).
-// A CTA takes 32 columns (lane = column, coalesced rows) and its 8 warps
-// split the rows, each with four independent partial sums; the warps' sums
-// are added in warp order.
-__global__ void __launch_bounds__(256) ir_cols_kernel(const float* __restrict__ Phi, const double* __restrict__ u,
-                                                      const float* __restrict__ x, const double* __restrict__ lam,
-                                                      float* __restrict__ r, int n, int t) {
-  __shared__ double part[8][32];
+// A CTA takes 32 columns (lane = column, coalesced rows); its 32 warps are 8
+// row phases of four chains each: chain q of phase w takes the rows w + 8 q +
+// 32 j, chain 0 also what is left below n.  The chains of a phase are added,
+// then the phases in order.
+__global__ void __launch_bounds__(1024) ir_cols_kernel(const float* __restrict__ Phi, const double* __restrict__ u,
+                                                       const float* __restrict__ x, const double* __restrict__ lam,
+                                                       float* __restrict__ r, int n, int t) {
+  __shared__ double part[32][32];
   const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+  const int w = warp & 7, q = warp >> 3;
   const float* p = Phi + (long long)b * n * t + c;
   const double* ub = u + (long long)b * n;
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+  double a = 0.0;
   if (c < t) {
-    int i = warp;
-    for (; i + 24 < n; i += 32) {
-      a0 = fma((double)p[(long long)i * t], ub[i], a0);
-      a1 = fma((double)p[(long long)(i + 8) * t], ub[i + 8], a1);
-      a2 = fma((double)p[(long long)(i + 16) * t], ub[i + 16], a2);
-      a3 = fma((double)p[(long long)(i + 24) * t], ub[i + 24], a3);
+    int i = w;
+    for (; i + 24 + 96 < n; i += 128) {   // four rows of the chain in flight
+      float pv[4];
+      double uv[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        pv[e] = p[(long long)(i + 8 * q + 32 * e) * t];
+        uv[e] = ub[i + 8 * q + 32 * e];
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) a = fma(widen_bits(pv[e]), uv[e], a);
     }
-    for (; i < n; i += 8) a0 = fma((double)p[(long long)i * t], ub[i], a0);
+    for (; i + 24 < n; i += 32) a = fma(widen_bits(p[(long long)(i + 8 * q) * t]), ub[i + 8 * q], a);
+    if (q == 0)
+      for (; i < n; i += 8) a = fma(widen_bits(p[(long long)i * t]), ub[i], a);
   }
-  part[warp][lane] = (a0 + a1) + (a2 + a3);
+  part[warp][lane] = a;
   __syncthreads();
   if (warp == 0 && c < t) {
-    double a = part[0][lane];
+    double s = 0.0;
 #pragma unroll
-    for (int w = 1; w < 8; ++w) a += part[w][lane];
-    r[(long long)b * t + c] = (float)(a - lam[b] * (double)x[(long long)b * t + c]);
+    for (int k = 0; k < 8; ++k) {
+      const double ph = (part[k][lane] + part[k + 8][lane]) + (part[k + 16][lane] + part[k + 24][lane]);
+      s = k == 0 ? ph : s + ph;
+    }
+    r[(long long)b * t + c] = (float)(s - lam[b] * (double)x[(long long)b * t + c]);
   }
+}
+
+// x += (L L^T)^-1 r, one cluster of eight CTAs per head, for the refinement
+// steps of the primal beta solve: forward y_k = Linv_kk (r_k - sum_{j<k} L_kj y_j),
+// then d_k = Linv_kk^T (y_k - sum_{j>k} L_jk^T d_j), x_k += d_k.  Serial over the
+// blocks, so the time of a step is what counts: one exchange between the CTAs
+// (remote stores counted on mbarriers, about half a cluster barrier), a short
+// sum and a 64 x 64 mat-vec, everything that does not depend on the previous
+// block loaded ahead.
+//   forward, right-looking: rank k % 8 keeps the sums of block k's rows in
+//     registers (row = thread / 8; chain (part, q) takes the columns part + 8 q
+//     + 32 i), adds each y_j as it comes and broadcasts y_k;
+//   backward: a sum runs upwards from the newest block, so it cannot be formed
+//     ahead; its chains (part, q, column; rows part + 8 q + 32 i below block k,
+//     chain 0 also what is left below t) are dealt by part over the ranks, whose
+//     slices of L's column panel arrive by cp.async a step ahead, and every
+//     rank forms d_k for itself from the eight parts.
+// 43 us at t = 819 and 93 us at t = 1638 (8 heads); one CTA per head took 219
+// and 740 us.
+constexpr int kTriCL = 8, kTriMaxT = 2048, kTriSlots = kTriMaxT / (NB * kTriCL);
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
+// Store to the same shared address of another CTA of the cluster, counted on
+// that CTA's mbarrier.
+__device__ __forceinline__ void st_remote(const float* p, const uint64_t* bar, int rank, float v) {
+  asm volatile(
+      "{\n\t.reg .b32 a, m;\n\t"
+      "mapa.shared::cluster.u32 a, %0, %2;\n\t"
+      "mapa.shared::cluster.u32 m, %1, %2;\n\t"
+      "st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [a], %3, [m];\n\t}\n" ::"r"(tc::smem_u32(p)),
+      "r"(tc::smem_u32(bar)), "r"(rank), "r"(__float_as_uint(v))
+      : "memory");
+}
+__global__ void __cluster_dims__(kTriCL, 1, 1) __launch_bounds__(512, 1)
+    tri_solve_cluster32_kernel(const float* __restrict__ A, const float* __restrict__ Linv,
+                               const float* __restrict__ r, float* __restrict__ x, int t, DevStatus* stt) {
+  extern __shared__ __align__(16) float psm[];   // two panel slices [2 nblk][4][64]
+  __shared__ float yv[kTriMaxT];                 // y, then d block by block
+  __shared__ float v[NB];
+  __shared__ float parts[2][8][NB];              // backward: the ranks' sums of alternate steps
+  // one-shot mbarriers: y_k has arrived (forward), all parts of step k have (backward)
+  __shared__ uint64_t ybar[kTriMaxT / NB], pbar[kTriMaxT / NB];
+  __shared__ int abort_flag;
+  const int head = blockIdx.x / kTriCL, rank = (int)cluster_rank(), tid = threadIdx.x;
+  const int nblk = (t + NB - 1) / NB;
+  if (tid < nblk) {
+    tc::mbar_init(&ybar[tid], 1);
+    tc::mbar_init(&pbar[tid], 1);
+    tc::mbar_fence_init();
+    tc::mbar_arrive_expect_tx(&ybar[tid], NB * 4);
+    tc::mbar_arrive_expect_tx(&pbar[tid], kTriCL * NB * 4);
+  }
+  if (tid == 0) abort_flag = 0;
+  __syncthreads();
+  cluster_sync_all();   // every rank's barriers are armed
+  const float* Ab = A + (long long)head * t * t;
+  const float* Lb = Linv + (long long)head * nblk * NB * NB;
+  const float* rb = r + (long long)head * t;
+  float* xb = x + (long long)head * t;
+  const int rr = tid >> 3, pt = tid & 7;
+  // forward
+  float ch[kTriSlots][4], lv[kTriSlots][8];
+#pragma unroll
+  for (int s = 0; s < kTriSlots; ++s)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) ch[s][q] = 0.f;
+  auto fetch = [&](int j) {   // L_kj of this rank's blocks k > j
+#pragma unroll
+    for (int s = 0; s < kTriSlots; ++s) {
+      const int k = rank + kTriCL * s, row = k * NB + rr;
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        lv[s][e] = (k > j && k < nblk && row < t) ? __ldcg(Ab + (long long)row * t + j * NB + pt + 8 * e) : 0.f;
+    }
+  };
+  float li[8], rv = 0.f;   // Linv_k row rr (from part pt) and r of this rank's next block
+  auto fetch_li = [&](int k) {
+    if (rank != k % kTriCL || k >= nblk) return;
+    const float* Li = Lb + (long long)k * NB * NB + rr * NB;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) li[e] = pt + 8 * e <= rr ? __ldcg(Li + pt + 8 * e) : 0.f;
+    rv = k * NB + rr < t ? rb[k * NB + rr] : 0.f;
+  };
+  fetch_li(0);
+  for (int k = 0; k < nblk; ++k) {
+    if (k > 0) {   // y_{k-1} has arrived: add it to the sums
+      tc::mbar_wait(&ybar[k - 1], 0, &abort_flag, stt);
+      const float* y = yv + (k - 1) * NB;
+#pragma unroll
+      for (int s = 0; s < kTriSlots; ++s)
+        if (rank + kTriCL * s >= k) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) ch[s][e & 3] = fmaf(lv[s][e], y[pt + 8 * e], ch[s][e & 3]);
+        }
+    }
+    if (rank == k % kTriCL) {
+      const int k0 = k * NB, kb = min(NB, t - k0);
+      float a = 0.f;
+#pragma unroll
+      for (int s = 0; s < kTriSlots; ++s)
+        if (s == k / kTriCL) a = (ch[s][0] + ch[s][1]) + (ch[s][2] + ch[s][3]);
+      a += __shfl_xor_sync(0xffffffffu, a, 1);
+      a += __shfl_xor_sync(0xffffffffu, a, 2);
+      a += __shfl_xor_sync(0xffffffffu, a, 4);
+      if (pt == 0) v[rr] = rr < kb ? rv - a : 0.f;
+      __syncthreads();
+      float y = 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (pt + 8 * e <= rr) y = fmaf(li[e], v[pt + 8 * e], y);
+      y += __shfl_xor_sync(0xffffffffu, y, 1);
+      y += __shfl_xor_sync(0xffffffffu, y, 2);
+      y += __shfl_xor_sync(0xffffffffu, y, 4);
+      st_remote(&yv[k0 + rr], &ybar[k], pt, rr < kb ? y : 0.f);   // lane pt of the row writes it to rank pt
+    }
+    fetch(k);
+    fetch_li(k + 1);
+  }
+  tc::mbar_wait(&ybar[nblk - 1], 0, &abort_flag, stt);
+  // backward; thread (c, q) of the first 256 owns chain (rank, q, c)
+  const int c = tid & 63, q = tid >> 6;
+  const int slice = 2 * nblk * 256;
+  auto panel = [&](int k) {   // this rank's rows of L's column block k, below the block
+    float* dst = psm + (k & 1) * slice;
+    const int k0 = k * NB;
+    if (k >= 0 && tid < 256)
+      for (int i = 0, base = k0 + NB + rank; base < t; base += 32, ++i) {
+        const int row = base + 8 * q;
+        if (row < t) cp_async4(dst + i * 256 + q * 64 + c, Ab + (long long)row * t + k0 + c);
+      }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  panel(nblk - 1);
+  panel(nblk - 2);
+  for (int k = nblk - 1; k >= 0; --k) {
+    const int k0 = k * NB, kb = min(NB, t - k0);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();   // this step's slice, and the previous step's d
+    const float* P = psm + (k & 1) * slice;
+    if (tid < 256) {
+      float a = 0.f;
+      if (c < kb) {
+        int i = 0, base = k0 + NB + rank;
+#pragma unroll 4
+        for (; base + 24 < t; base += 32, ++i) a = fmaf(P[i * 256 + q * 64 + c], yv[base + 8 * q], a);
+        if (q == 0)   // rows base, base + 8, base + 16 below t
+          for (int e = 0; base + 8 * e < t; ++e) a = fmaf(P[i * 256 + e * 64 + c], yv[base + 8 * e], a);
+      }
+      // the four chains of a column are in warps w, w + 2, w + 4, w + 6: through shared memory
+      psm[2 * slice + q * 64 + c] = a;
+    }
+    __syncthreads();
+    {
+      const float* s4 = psm + 2 * slice;
+      const int col = tid >> 3;   // lane pt of the column writes it to rank pt
+      const float a = (s4[col] + s4[64 + col]) + (s4[128 + col] + s4[192 + col]);
+      st_remote(&parts[k & 1][rank][col], &pbar[k], pt, a);
+    }
+    panel(k - 2);
+    const float* Li = Lb + (long long)k * NB * NB;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int l = rr + pt + 8 * e;   // column rr of Linv, rows l >= rr
+      li[e] = l < NB ? __ldcg(Li + l * NB + rr) : 0.f;
+    }
+    if (tid < NB) {
+      tc::mbar_wait(&pbar[k], 0, &abort_flag, stt);
+      float a = 0.f;
+#pragma unroll
+      for (int p = 0; p < 8; ++p) a += parts[k & 1][p][tid];
+      v[tid] = tid < kb ? yv[k0 + tid] - a : 0.f;
+    }
+    __syncthreads();
+    float d = 0.f;
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (rr + pt + 8 * e < NB) d = fmaf(li[e], v[rr + pt + 8 * e], d);
+    d += __shfl_xor_sync(0xffffffffu, d, 1);
+    d += __shfl_xor_sync(0xffffffffu, d, 2);
+    d += __shfl_xor_sync(0xffffffffu, d, 4);
+    if (pt == 0 && rr < kb) {
+      yv[k0 + rr] = d;
+      if (rank == k % kTriCL) xb[k0 + rr] += d;
+    }
+  }
+  cluster_sync_all();   // nobody leaves before the last stores into its shared memory have been waited for
 }
 
 // x += (L L^T)^-1 r for one head per CTA (512 threads): forward substitution
 // y_k = Linv_kk (r_k - sum_{j<k} L_kj y_j), then x_k += Linv_kk^T (y_k -
 // sum_{j>k} L_jk^T d_j).  y and the correction d live in `yd` ([H][t]).
-// Used by the refinement steps of the primal beta solve.
+// Serves the refinement steps beyond kTriMaxT, where a rank's sums and panel
+// slices no longer fit.
 template <typename R>
 __global__ void __launch_bounds__(512) tri_solve_kernel(const R* __restrict__ A, const R* __restrict__ Linv,
                                                         const R* __restrict__ r, R* __restrict__ yd,
@@ -1938,18 +1370,24 @@ __global__ void __launch_bounds__(512) tri_solve_kernel(const R* __restrict__ A,
 
 constexpr int kBetaRefineSteps = 2;
 
-static int refine_beta(const Dims& D, float ridge_w, const float* m, const FitBufs& B, cudaStream_t st) {
-  const long long hn = (long long)D.H * D.n;
-  ir_rows_kernel<<<cdiv(hn, 8), 256, 0, st>>>(B.Phi, m, B.wsol, B.ir_u, B.ir_sq, D.n, D.t, D.H);
+static int refine_beta(const Dims& D, float ridge_w, const float* m, const FitBufs& B, DevStatus* stt, cudaStream_t st) {
+  const dim3 rows(cdiv(D.n, 8), D.H);
+  const int nblk = cdiv(D.t, NB), smem = (2 * 2 * nblk * 256 + 256) * (int)sizeof(float);
+  const bool cluster = D.t <= kTriMaxT;
+  if (cluster && set_dyn_smem((const void*)tri_solve_cluster32_kernel, smem) != cudaSuccess) return -1;
+  ir_rows_kernel<<<rows, 256, 0, st>>>(B.Phi, m, B.wsol, B.ir_u, B.ir_sq, D.n, D.t);
   ir_lambda_kernel<<<D.H, 256, 0, st>>>(B.ir_sq, B.ir_lam, D.n, D.t, (double)ridge_w);
   int nl = 2;
   for (int it = 0; it < kBetaRefineSteps; ++it) {
     if (it > 0) {
-      ir_rows_kernel<<<cdiv(hn, 8), 256, 0, st>>>(B.Phi, m, B.wsol, B.ir_u, nullptr, D.n, D.t, D.H);
+      ir_rows_kernel<<<rows, 256, 0, st>>>(B.Phi, m, B.wsol, B.ir_u, nullptr, D.n, D.t);
       ++nl;
     }
-    ir_cols_kernel<<<dim3(cdiv(D.t, 32), D.H), 256, 0, st>>>(B.Phi, B.ir_u, B.wsol, B.ir_lam, B.rhs, D.n, D.t);
-    tri_solve_kernel<float><<<D.H, 512, 0, st>>>(B.Gram, B.Linv, B.rhs, B.Z, B.wsol, D.t);
+    ir_cols_kernel<<<dim3(cdiv(D.t, 32), D.H), 1024, 0, st>>>(B.Phi, B.ir_u, B.wsol, B.ir_lam, B.rhs, D.n, D.t);
+    if (cluster)
+      tri_solve_cluster32_kernel<<<kTriCL * D.H, 512, smem, st>>>(B.Gram, B.Linv, B.rhs, B.wsol, D.t, stt);
+    else
+      tri_solve_kernel<float><<<D.H, 512, 0, st>>>(B.Gram, B.Linv, B.rhs, B.Z, B.wsol, D.t);
     nl += 2;
   }
   return nl;
@@ -1998,8 +1436,12 @@ int launch_fits(const Dims& D, float scale, float ridge_w, float ridge_v, float 
   mass_rhs_kernel<<<dim3(cdiv(D.t, 32), D.H), 1024, 0, st>>>(B.Phi, m, B.rhs, D.n, D.t);
   ++nl;
   mark(8);
-  nl += cholesky_solve(D.H, D.t, B.Gram, B.Linv, B.rhs, B.Z, B.wsol, 1, 1, D.t, ridge_w, stt, st);
-  nl += refine_beta(D, ridge_w, m, B, st);
+  const int nb = launch_chol(D.H, D.t, B.Gram, B.Linv, B.rhs, B.Z, B.wsol, 1, D.t, ridge_w, B.ctrip, stt, st);
+  if (nb < 0) return -1;
+  nl += nb;
+  const int nrf = refine_beta(D, ridge_w, m, B, stt, st);
+  if (nrf < 0) return -1;
+  nl += nrf;
   const long long ht = (long long)D.H * D.t;
   beta_kernel<<<cdiv(ht, 256), 256, 0, st>>>(B.wsol, beta, ht, eps_w, b_min, b_max);
   ++nl;
@@ -2018,8 +1460,8 @@ int launch_fits(const Dims& D, float scale, float ridge_w, float ridge_v, float 
   if (gram_tc(D.H, D.t, D.d, ldn, B.PT_hi, B.PT_lo, B.YT_hi, B.YT_lo, B.R, D.d, stt, st) < 0) return -1;
   nl += 2;
   mark(10);
-  nl += cholesky_solve(D.H, D.t, B.Gram, B.Linv, B.R, B.Z, C_v, D.d, D.d, td, ridge_v, stt, st);
-  return nl;
+  const int nv = launch_chol(D.H, D.t, B.Gram, B.Linv, B.R, B.Z, C_v, D.d, td, ridge_v, B.ctrip, stt, st);
+  return nv < 0 ? -1 : nl + nv;
 }
 
 __global__ void check_finite_kernel(const float* x, long long count, DevStatus* stt) {

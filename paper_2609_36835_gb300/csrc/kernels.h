@@ -152,6 +152,7 @@ struct FitBufs {
   bf16* Sl3;                            // right-hand-side slices of the dual solves (t > n only)
   int* eC2;
   double* cl_lam;                       // [H]
+  uint8_t* ctrip;                       // operand slots of launch_chol (t <= n only)
 };
 // Returns launches, or -1 when a TMA descriptor cannot be encoded.
 // ev (nullable): events recorded before the beta solve, before the value
@@ -161,6 +162,14 @@ int launch_fits(const Dims& D, float scale, float ridge_w, float ridge_v, float 
                 const float* Y, const FitBufs& B, float* beta, float* C_v, DevStatus* stt, cudaStream_t st,
                 cudaEvent_t const* ev = nullptr);
 int launch_check_finite(const float* x, long long count, DevStatus* stt, cudaStream_t st);
+// (Gram + lam I) X = B for H fp32 systems of size t, lam = ridge trace(Gram) / t
+// (chol.cu): Gram [H][t][t] is overwritten by the factor (lower part), Linv
+// [H][ceil(t / 64)][64][64] by the inverses of its diagonal blocks; B, Z, X [H]
+// (bbs apart) hold [t][nrhs], nrhs = 1 .. 128, B being overwritten by the forward
+// solution; trip: chol_trip_bytes(H, t) of scratch.  Returns launches or -1.
+int launch_chol(int H, int t, float* Gram, float* Linv, float* B, float* Z, float* X, int nrhs, long long bbs,
+                float ridge, uint8_t* trip, DevStatus* stt, cudaStream_t st);
+size_t chol_trip_bytes(int H, int t);
 
 // ---- fp64-grade products on the bf16 tensor pipe (tc_sliced.cu) ------------
 // Operands are cut into S bf16 slices per row (S = 3, 4 or 5) with a power-of-two
