@@ -19,7 +19,7 @@ constexpr size_t kAlign = 256;
 inline size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-  size_t status, kbar_hi, kbar_lo, vq, qpp, q_h, q_m, q_l, av, VT, p_h, p_m, p_l, vq3, av3, ukt, qbar_hi, qbar_lo, wts, NT, rA, rB, part, lse, s, anchors, z, m, invm, Y, logphi,
+  size_t status, kbar_hi, kbar_lo, vq, qpp, q_h, q_m, q_l, av, VT, vq3, av3, ukt, qbar_hi, qbar_lo, wts, NT, rA, rB, part, lse, s, anchors, z, m, invm, Y, logphi,
       qcat, wcat, Ut_hi, Ut_lo, S_hi, S_lo, best, kappa, kmap, perm, goff, cursor, LC, Phi, Gram, Linv, rhs, wsol, R, Z,
       ck3, YT_hi, YT_lo, G64, L64, B64, Z64, X64, Sl, Sl2, eR, eC, ir_u, ir_sq, ir_lam, Sl3, eC2, cl_lam, ctrip, total;
 };
@@ -78,10 +78,6 @@ Layout plan(const arckv_config& c) {
   L.q_l = take(H * n * 128 * 2);
   L.av = take(H * n * 128 * f);
   L.VT = take(H * 128 * ldT * 2);
-  const size_t ptrip = probs_fused((int)T) ? 0 : H * n * ldT * 2;   // probability triple (unfused path only)
-  L.p_h = take(ptrip);
-  L.p_m = take(ptrip);
-  L.p_l = take(ptrip);
   L.qcat = take(H * n * 512 * 2);
   L.vq3 = take(3 * H * n * 128 * 2);
   L.av3 = take(3 * H * n * 128 * 2);
@@ -90,7 +86,7 @@ Layout plan(const arckv_config& c) {
   L.qbar_hi = take(H * n * HD * 2);
   L.qbar_lo = take(H * n * HD * 2);
   L.wts = take(H * (size_t)D.n_pos * D.H_I * f);
-  L.NT = take(H * n * T * f);
+  L.NT = take(H * n * (size_t)logit_ld((int)T) * f);
   L.rA = take(H * n * f);
   L.rB = take(H * n * f);
   L.part = take(H * n * ntile * 8);
@@ -292,7 +288,7 @@ arckv_status arckv_compact(const arckv_config* cfg, const void* K, const void* V
   auto reference_attention = [&]() -> int {
     ref_done = true;
     return launch_reference_attention(D, scale, Qb, Kb, B16(L.VT), F(L.NT), (float2*)(w + L.part), F(L.z), F(L.m),
-                                      F(L.invm), B16(L.p_h), B16(L.p_m), B16(L.p_l), F(L.Y), stt, st);
+                                      F(L.invm), F(L.Y), stt, st);
   };
   if (!given_anchors && !use_indexer) {
     mark(1);
@@ -307,7 +303,7 @@ arckv_status arckv_compact(const arckv_config* cfg, const void* K, const void* V
       float* vq = F(L.vq);   // VI scratch: n-sized rows here, O^(-a) in L.qpp
       const size_t hn = (size_t)D.H * D.n;
       ViBufs VB{(int*)vq, vq + hn, vq + 2 * hn, vq + 3 * hn, vq + 4 * hn, F(L.qpp), F(L.best), F(L.Ut_hi),
-                B16(L.p_h), B16(L.p_m), B16(L.p_l), B16(L.q_h), B16(L.q_m), B16(L.q_l)};
+                B16(L.q_h), B16(L.q_m), B16(L.q_l)};
       const int nlv = launch_vi_scores(D, F(L.NT), F(L.z), F(L.m), F(L.Y), Vb, B16(L.VT), VB, F(L.s), 1e-6f, stt,
                                        st);
       if (nlv < 0) return ARCKV_ERR_CUDA;
@@ -321,7 +317,7 @@ arckv_status arckv_compact(const arckv_config* cfg, const void* K, const void* V
     if (nlk < 0) return ARCKV_ERR_CUDA;
     nl += nlk;
     QueryBufs QB{F(L.NT),    F(L.rA),    F(L.rB),    F(L.av),     B16(L.q_h),
-                 B16(L.q_m), B16(L.q_l), B16(L.p_h), B16(L.p_m), B16(L.p_l),
+                 B16(L.q_m), B16(L.q_l),
                  (float2*)(w + L.part),  B16(L.qcat), B16(L.wcat), B16(L.vq3), B16(L.av3),
                  B16(L.ukt)};
     const int nlq = launch_query_features(D, Qb, (const bf16*)X_ref, Kb, B16(L.VT), (const bf16*)idx->U_q,

@@ -1489,10 +1489,10 @@ int launch_check_finite(const float* x, long long count, DevStatus* stt, cudaStr
 // x += beta over each row, then shift = max, mul = 1 / sum exp(x - shift); one
 // warp per row of X [H][n][t].
 __global__ void __launch_bounds__(256) bias_rowstats_kernel(float* X, const float* beta, float* shift, float* mul,
-                                                            int n, int t) {
+                                                            int n, int t, int ld) {
   const int b = blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= n) return;
-  float* x = X + ((long long)b * n + row) * t;
+  float* x = X + ((long long)b * n + row) * ld;
   const float* be = beta + (long long)b * t;
   float mx = -INFINITY;
   for (int c = lane; c < t; c += 32) {
@@ -1523,13 +1523,12 @@ AttendLayout attend_layout(int H, int n, int t) {
   size_t o = 0;
   auto take = [&](size_t bytes) { const size_t r = o; o += (bytes + 255) / 256 * 256; return r; };
   L.status = take(256);
-  L.X = take(h * n * t * 4);
+  L.X = take(h * n * (size_t)logit_ld(t) * 4);
   L.shift = take(h * n * 4);
   L.mul = take(h * n * 4);
   L.ck3 = take(3 * h * t * 128 * 2);
   L.vt3 = take(3 * h * 128 * ldt * 2);
   L.parts = take(3 * h * n * 128 * 4);
-  L.p3 = take(probs_fused(t) ? 0 : 3 * h * n * ldt * 2);
   L.total = o;
   return L;
 }
@@ -1544,19 +1543,18 @@ int launch_attend(int H, int n, int t, float scale, const bf16* Q, const float* 
   bf16* ck = (bf16*)(ws + L.ck3);
   bf16* vt = (bf16*)(ws + L.vt3);
   float* parts = (float*)(ws + L.parts);
-  bf16* p3 = (bf16*)(ws + L.p3);
   int nl = launch_split3(C_k, ck, ck + htd, ck + 2 * htd, htd, st);
   {  // X^T = C_k Q^T, stored transposed as X [H][n][t] and scaled
     CUtensorMap mA, mA2, mA3, mB;
     if (!encode_bf16_map_3d(&mA, ck, 128, t, H, 128) || !encode_bf16_map_3d(&mA2, ck + htd, 128, t, H, 128) ||
         !encode_bf16_map_3d(&mA3, ck + 2 * htd, 128, t, H, 128) || !encode_bf16_map_3d(&mB, Q, 128, n, H, 128))
       return -1;
-    if (launch_tc_gemm<128, kSplit3A>(mA, mB, mA2, mA, TcEpiStoreT{X, (long long)n * t, t, scale}, H, t, n, 128, 128,
+    if (launch_tc_gemm<128, kSplit3A>(mA, mB, mA2, mA, TcEpiStoreT{X, (long long)n * logit_ld(t), logit_ld(t), scale}, H, t, n, 128, 128,
                                       stt, st, 0, &mA3) != cudaSuccess)
       return -1;
     ++nl;
   }
-  bias_rowstats_kernel<<<dim3(cdiv(n, 8), H), 256, 0, st>>>(X, beta, shift, mul, n, t);
+  bias_rowstats_kernel<<<dim3(cdiv(n, 8), H), 256, 0, st>>>(X, beta, shift, mul, n, t, logit_ld(t));
   // C_v^T as a bf16 triple [H][128][ldt] (zero pad)
   transpose_split3_kernel<<<dim3(cdiv(128, 32), cdiv(ldt, 32), H), 256, 0, st>>>(
       C_v, t, 128, vt, vt + (long long)H * 128 * ldt, vt + 2LL * H * 128 * ldt, (int)ldt);
@@ -1566,10 +1564,9 @@ int launch_attend(int H, int n, int t, float scale, const bf16* Q, const float* 
   D.n = n;
   D.T = t;
   D.d = 128;
-  const long long hnd = (long long)H * n * 128, pl = (long long)H * n * ldt;
+  const long long hnd = (long long)H * n * 128;
   for (int p = 0; p < 3; ++p) {
-    const int r = launch_probs_v_tc(D, X, shift, mul, p3, p3 + pl, p3 + 2 * pl, vt + p * (long long)H * 128 * ldt,
-                                    parts + p * hnd, stt, st);
+    const int r = launch_probs_v_tc(D, X, shift, mul, vt + p * (long long)H * 128 * ldt, parts + p * hnd, stt, st);
     if (r < 0) return -1;
     nl += r;
   }

@@ -82,7 +82,7 @@ int launch_query_features(const Dims& D, const bf16* Q, const bf16* X, const bf1
   nl += launch_part_stats(D.H, D.n, cdiv(D.T, kRowPartW), B.part, B.rshift, B.rmul, nullptr, st);
   // A^V V on the tensor cores, then c = (A^V V) U_v^T = A^V (U_v V), written as
   // the bf16 triple that the q_bar GEMM reads (columns 128.. of its A operand)
-  r = launch_probs_v_tc(D, B.logits, B.rshift, B.rmul, B.p_h, B.p_m, B.p_l, VT, B.av, stt, st);
+  r = launch_probs_v_tc(D, B.logits, B.rshift, B.rmul, VT, B.av, stt, st);
   if (r < 0) return -1;
   nl += r;
   bf16 *av_h = B.av3, *av_m = B.av3 + hn, *av_l = B.av3 + 2 * hn;
@@ -118,27 +118,28 @@ __global__ void lse_reduce_kernel(const float2* part, float* lse, int n, int nti
 // s_j = sqrt(mean_i exp(2 (I_ij - lse_i))).  A CTA owns 32 columns; warp w
 // sums the rows i = w, w+8, ... of its column (four independent partial sums
 // per thread) and the eight warp sums are added in warp order.
-__global__ void __launch_bounds__(256) pool_kernel(const float* I, const float* lse, float* s, int n, int T) {
+__global__ void __launch_bounds__(256) pool_kernel(const float* I, const float* lse, float* s, int n, int T,
+                                                   int ld) {
   const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int j = blockIdx.x * 32 + lane;
   __shared__ float red[8][33];
-  const float* Ib = I + (long long)b * n * T + j;
+  const float* Ib = I + (long long)b * n * ld + j;
   const float* lb = lse + (long long)b * n;
   float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
   if (j < T) {
     int i = warp;
     for (; i + 24 < n; i += 32) {
-      const float p0 = expf(Ib[(long long)i * T] - lb[i]);
-      const float p1 = expf(Ib[(long long)(i + 8) * T] - lb[i + 8]);
-      const float p2 = expf(Ib[(long long)(i + 16) * T] - lb[i + 16]);
-      const float p3 = expf(Ib[(long long)(i + 24) * T] - lb[i + 24]);
+      const float p0 = expf(Ib[(long long)i * ld] - lb[i]);
+      const float p1 = expf(Ib[(long long)(i + 8) * ld] - lb[i + 8]);
+      const float p2 = expf(Ib[(long long)(i + 16) * ld] - lb[i + 16]);
+      const float p3 = expf(Ib[(long long)(i + 24) * ld] - lb[i + 24]);
       a0 = fmaf(p0, p0, a0);
       a1 = fmaf(p1, p1, a1);
       a2 = fmaf(p2, p2, a2);
       a3 = fmaf(p3, p3, a3);
     }
     for (; i < n; i += 8) {
-      const float p0 = expf(Ib[(long long)i * T] - lb[i]);
+      const float p0 = expf(Ib[(long long)i * ld] - lb[i]);
       a0 = fmaf(p0, p0, a0);
     }
   }
@@ -210,7 +211,7 @@ int launch_index_pool(const Dims& D, const float* I, const float2* part, int nti
   if ((D.T & 3) == 0 && (((uintptr_t)I | (uintptr_t)s) & 15u) == 0)
     pool4_kernel<<<dim3(cdiv(D.T, 128), D.H), 256, 0, st>>>(I, lse, s, D.n, D.T);
   else
-    pool_kernel<<<dim3(cdiv(D.T, 32), D.H), 256, 0, st>>>(I, lse, s, D.n, D.T);
+    pool_kernel<<<dim3(cdiv(D.T, 32), D.H), 256, 0, st>>>(I, lse, s, D.n, D.T, logit_ld(D.T));
   return 2;
 }
 

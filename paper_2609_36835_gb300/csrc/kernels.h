@@ -22,9 +22,11 @@ __host__ __device__ inline int chunk_budget(int T, int t, int Tc) {
   if (2 * r > T || (2 * r == T && (q & 1))) ++q;
   return (int)(q < 1 ? 1 : (q > Tc ? Tc : q));
 }
-// softmax(X) V products run fused (no probability triple in memory) when the
-// fp32 logit rows can be tiled by TMA: T a multiple of 4
-inline bool probs_fused(int T) { return (T & 3) == 0; }
+// Row pitch (elements) of an fp32 [n][T] logit matrix: T rounded up to the 16
+// bytes that TMA wants, so that every T is stored and read in tiles (before,
+// T % 4 != 0 went through per-thread stores and a probability triple in memory:
+// 0.55 + 0.41 ms against 0.09 + 0.23 for 8 heads, n = 512, T = 20011).
+inline int logit_ld(int T) { return (T + 3) & ~3; }
 inline int effective_chunk(int T, int chunk_len) { return (chunk_len > 0 && T > kChunkThreshold) ? chunk_len : 0; }
 inline int realized_anchors(int T, int t, int chunk_len) {
   const int L = effective_chunk(T, chunk_len);
@@ -60,7 +62,7 @@ int launch_key_features_tc(const Dims& D, const bf16* K, const bf16* V, const bf
 // Scratch of the query-side features.
 struct QueryBufs {
   float *logits, *rshift, *rmul, *av;
-  bf16 *q_h, *q_m, *q_l, *p_h, *p_m, *p_l;
+  bf16 *q_h, *q_m, *q_l;
   float2* part;        // per-(row, 128-column tile) softmax partials of the logits
   bf16 *qcat, *wcat;   // K-concatenated operands of the q_bar GEMM ([n][512], [HD][512])
   bf16 *vq3, *av3;     // bf16 triples of U_q q and A^V V (parts [H][n][128], one after another)
@@ -77,10 +79,9 @@ int launch_transpose_v(const Dims& D, const bf16* V, bf16* VT, cudaStream_t st);
 // value logits [H][n][T] from the q'' triple and the bf16 keys, with row partials
 int launch_value_logits_tc(const Dims& D, const bf16* q_h, const bf16* q_m, const bf16* q_l, const bf16* K,
                            float* logits, float2* part, DevStatus* stt, cudaStream_t st);
-// out [H][n][128] = (exp(X - shift) * mul) V over rows of X [H][n][T].
-int launch_probs_v_tc(const Dims& D, const float* X, const float* shift, const float* mul, bf16* p_h, bf16* p_m,
-                      bf16* p_l, const bf16* VT, float* out, DevStatus* stt, cudaStream_t st,
-                      const int* skip = nullptr);
+// out [H][n][128] = (exp(X - shift) * mul) V over rows of X [H][n][logit_ld(T)].
+int launch_probs_v_tc(const Dims& D, const float* X, const float* shift, const float* mul, const bf16* VT, float* out,
+                      DevStatus* stt, cudaStream_t st, const int* skip = nullptr);
 // x (count floats) -> bf16 triple h + m + l
 int launch_split3(const float* x, bf16* h, bf16* m, bf16* l, long long count, cudaStream_t st);
 // I (Eq. pairwise_index_score) on tcgen05 with split-bf16 operands, and the
@@ -108,8 +109,8 @@ int launch_check_anchors(const Dims& D, int* anchors, DevStatus* stt, cudaStream
 // (tcgen05, split-3 probabilities against VT); column statistics log phi,
 // M_j and 1/||e^{l_:j - M_j}||.  -1 when a TMA descriptor cannot be encoded.
 int launch_reference_attention(const Dims& D, float scale, const bf16* Q, const bf16* K, const bf16* VT,
-                               float* L, float2* part, float* z, float* m, float* invm, bf16* p_h, bf16* p_m,
-                               bf16* p_l, float* Y, DevStatus* stt, cudaStream_t st);
+                               float* L, float2* part, float* z, float* m, float* invm, float* Y,
+                               DevStatus* stt, cudaStream_t st);
 int launch_ref_logits_tc(const Dims& D, float scale, const bf16* Q, const bf16* K, float* L, float2* part,
                          DevStatus* stt, cudaStream_t st);
 // Column statistics of the reference logits L: log phi [H][T] (mass weights of
@@ -207,7 +208,7 @@ int launch_sliced_product_f32(int S, const bf16* As, const int* eA, int M, const
 // Scratch of launch_attend: byte offsets from one 256-byte aligned base (the
 // first 256 bytes are the status word) and the total size.
 struct AttendLayout {
-  size_t status, X, shift, mul, ck3, vt3, parts, p3, total;
+  size_t status, X, shift, mul, ck3, vt3, parts, total;
 };
 AttendLayout attend_layout(int H, int n, int t);
 // O [H][n][128] = softmax(scale Q C_k^T + beta) C_v on the tensor pipe; `ws` is
@@ -222,12 +223,11 @@ int launch_truncated_error(int H, int n, int T, int t, float scale, float eps, c
                            const bf16* V, const int* S, float* E, unsigned char* inS, float* err, DevStatus* stt,
                            cudaStream_t st);
 // Scratch of launch_vi_scores: per row amax, z2, mul2, Da, oo [H][n]; O^(-a) Om
-// [H][n][128]; the split probabilities p_* [H][n][ldT] and Y's split y_*
-// [H][n][128]; vv [H][T]; colpart [H][ceil(n/32)][T].
+// [H][n][128]; Y's split y_* [H][n][128]; vv [H][T]; colpart [H][ceil(n/32)][T].
 struct ViBufs {
   int* amax;
   float *z2, *mul2, *Da, *oo, *Om, *vv, *colpart;
-  bf16 *p_h, *p_m, *p_l, *y_h, *y_m, *y_l;
+  bf16 *y_h, *y_m, *y_l;
 };
 // s [H][T] = VI scores from the reference logits L, row stats z, m, Y = softmax(L) V.
 int launch_vi_scores(const Dims& D, const float* L, const float* z, const float* m, const float* Y, const bf16* V,

@@ -26,12 +26,12 @@ namespace arckv {
 
 // Per row of l [H][n][T]: a_i, z2_i = max_{u != a_i} l_iu, mul2_i = 1 / sum_{u != a_i} e^{l_iu - z2_i}
 // (0 when T = 1).  One warp per row.
-__global__ void __launch_bounds__(256) vi_row_kernel(const float* L, int n, int T, int* amax, float* z2,
+__global__ void __launch_bounds__(256) vi_row_kernel(const float* L, int n, int T, int ld, int* amax, float* z2,
                                                      float* mul2) {
   const int b = blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= n) return;
   const long long r = (long long)b * n + row;
-  const float* x = L + r * T;
+  const float* x = L + r * ld;
   float mx = -INFINITY;
   int ai = INT_MAX;
   for (int j = lane; j < T; j += 32) {
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(256) row_norm2_kernel(const bf16* V, long long
 // D_ij^2 / (||O_i||^2 + eps), summed over the warp's 32 rows; lane q writes the
 // column sum into part[b][row / 32][col].
 struct TcEpiVI {
-  const float* L;     // [H][n][T] reference logits
+  const float* L;     // [H][n][T] reference logits (rows ld apart)
   const float* z;     // [H][n] row max
   const float* m;     // [H][n] sum_u e^{l_iu - z_i}
   const int* amax;    // [H][n]
@@ -106,7 +106,7 @@ struct TcEpiVI {
   const float* oo;    // [H][n] ||O_i||^2
   const float* vv;    // [H][T] ||v_j||^2
   float* part;        // [H][ceil(n / 32)][T]
-  int n, T, nb;
+  int n, T, ld, nb;
   float eps;
   struct State {
     const float* lrow;
@@ -120,7 +120,7 @@ struct TcEpiVI {
     s.row_ok = row < M;
     s.blk_ok = (row & ~31) < M;
     const long long r = (long long)b * n + (s.row_ok ? row : 0);
-    s.lrow = L + r * T + n0;
+    s.lrow = L + r * ld + n0;
     s.vvb = vv + (long long)b * T + n0;
     s.prow = part + ((long long)b * nb + (s.blk_ok ? row / 32 : 0)) * T + n0;
     s.zi = z[r];
@@ -179,10 +179,10 @@ __global__ void vi_reduce_kernel(const float* part, int nb, int n, int T, float*
 int launch_vi_scores(const Dims& D, const float* L, const float* z, const float* m, const float* Y, const bf16* V,
                      const bf16* VT, const ViBufs& B, float* s, float eps, DevStatus* stt, cudaStream_t st) {
   int nl = 0;
-  vi_row_kernel<<<dim3(cdiv(D.n, 8), D.H), 256, 0, st>>>(L, D.n, D.T, B.amax, B.z2, B.mul2);
+  vi_row_kernel<<<dim3(cdiv(D.n, 8), D.H), 256, 0, st>>>(L, D.n, D.T, logit_ld(D.T), B.amax, B.z2, B.mul2);
   ++nl;
   // O^(-a): softmax over the keys other than a_i, times V
-  const int r = launch_probs_v_tc(D, L, B.z2, B.mul2, B.p_h, B.p_m, B.p_l, VT, B.Om, stt, st, B.amax);
+  const int r = launch_probs_v_tc(D, L, B.z2, B.mul2, VT, B.Om, stt, st, B.amax);
   if (r < 0) return -1;
   nl += r;
   vi_rowfinish_kernel<<<dim3(cdiv(D.n, 8), D.H), 256, 0, st>>>(z, B.amax, B.z2, B.mul2, V, B.Om, Y, D.n, D.T, B.Da,
@@ -195,7 +195,7 @@ int launch_vi_scores(const Dims& D, const float* L, const float* z, const float*
       !encode_bf16_map_3d(&mA3, B.y_l, 128, D.n, D.H, 128) || !encode_bf16_map_3d(&mB, V, 128, D.T, D.H, 128))
     return -1;
   const int nb = cdiv(D.n, 32);
-  TcEpiVI epi{L, z, m, B.amax, B.Da, B.oo, B.vv, B.colpart, D.n, D.T, nb, eps};
+  TcEpiVI epi{L, z, m, B.amax, B.Da, B.oo, B.vv, B.colpart, D.n, D.T, logit_ld(D.T), nb, eps};
   if (launch_tc_gemm<128, kSplit3A>(mA, mB, mA2, mA, epi, D.H, D.n, D.T, 128, 128, stt, st, 0, &mA3) != cudaSuccess)
     return -1;
   vi_reduce_kernel<<<dim3(cdiv(D.T, 256), D.H), 256, 0, st>>>(B.colpart, nb, D.n, D.T, s);

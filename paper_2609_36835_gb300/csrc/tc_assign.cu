@@ -105,7 +105,7 @@ struct ProfileOut {
 //     columns n..ldn-1 are written as zeros).
 // e^x is taken as 2^(x log2 e) after the subtraction.
 __global__ void __launch_bounds__(512) col_profiles_kernel(const float* L, float* logphi, ProfileOut po, int n, int T,
-                                                           int ldn) {
+                                                           int ld, int ldn) {
   const int b = blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int j0 = blockIdx.x * 32, j = j0 + lane;
   __shared__ float red[3][16][32];
@@ -114,13 +114,13 @@ __global__ void __launch_bounds__(512) col_profiles_kernel(const float* L, float
   __shared__ long long orow[32];   // element offset of each column's output row
   if (po.Ut_hi != nullptr && w == 0 && j < T)
     orow[lane] = profile_row(po.anchors + (long long)b * po.t, po.t, T, b, j, ldn, po.kmap);
-  const float* Lb = L + (long long)b * n * T + j;
+  const float* Lb = L + (long long)b * n * ld + j;
   float mx = -INFINITY, s1 = 0.f, s2 = 0.f;
   if (j < T) {
     int i = w;
     for (; i + 48 < n; i += 64) {   // rows i, i + 16, i + 32, i + 48: one rescale per step
-      const float v0 = Lb[(long long)i * T], v1 = Lb[(long long)(i + 16) * T];
-      const float v2 = Lb[(long long)(i + 32) * T], v3 = Lb[(long long)(i + 48) * T];
+      const float v0 = Lb[(long long)i * ld], v1 = Lb[(long long)(i + 16) * ld];
+      const float v2 = Lb[(long long)(i + 32) * ld], v3 = Lb[(long long)(i + 48) * ld];
       const float m4 = fmaxf(fmaxf(v0, v1), fmaxf(v2, v3));
       if (m4 > mx) {
         const float r = (mx == -INFINITY) ? 0.f : ex2_approx((mx - m4) * kLog2e);
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(512) col_profiles_kernel(const float* L, float
       s2 += (e0 * e0 + e1 * e1) + (e2 * e2 + e3 * e3);
     }
     for (; i < n; i += 16) {
-      const float v = Lb[(long long)i * T];
+      const float v = Lb[(long long)i * ld];
       if (v > mx) {
         const float r = (mx == -INFINITY) ? 0.f : ex2_approx((mx - v) * kLog2e);
         s1 = fmaf(s1, r, 1.f);
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(512) col_profiles_kernel(const float* L, float
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int r = w + 16 * k, i = i0 + r;
-      tile[r][lane] = (i < n && j < T) ? ex2_approx((Lb[(long long)i * T] - cm) * kLog2e) * ci : 0.f;
+      tile[r][lane] = (i < n && j < T) ? ex2_approx((Lb[(long long)i * ld] - cm) * kLog2e) * ci : 0.f;
     }
     __syncthreads();
     // warp w writes columns 2w and 2w + 1, lane l rows i0 + 2l and i0 + 2l + 1 (ldn even)
@@ -354,7 +354,7 @@ static int col_profiles(const Dims& D, const float* L, float* logphi, const Prof
   if (smem > 0 && set_dyn_smem((const void*)col_profiles_kernel, smem) !=
                       cudaSuccess)
     return -1;
-  col_profiles_kernel<<<dim3(cdiv(D.T, 32), D.H), 512, smem, st>>>(L, logphi, po, D.n, D.T, ldn);
+  col_profiles_kernel<<<dim3(cdiv(D.T, 32), D.H), 512, smem, st>>>(L, logphi, po, D.n, D.T, logit_ld(D.T), ldn);
   return 1;
 }
 

@@ -19,22 +19,6 @@ __global__ void split3_kernel(const float* x, bf16* h, bf16* m, bf16* l, long lo
     split3_bf16(x[k], h[k], m[k], l[k]);
 }
 
-// P = exp(X - shift_row) * mul_row as a bf16 triple [H][rows][ldc] (zero in the
-// pad columns cols..ldc-1, and in column skip[row] when skip is given).
-__global__ void probs_split3_kernel(const float* X, const float* shift, const float* mul, const int* skip, bf16* h,
-                                    bf16* m, bf16* l, int rows, int cols, int ldc) {
-  const int b = blockIdx.z, row = blockIdx.y;
-  const long long rr = (long long)b * rows + row;
-  const float sh = shift[rr], mu = mul[rr];
-  const int sk = skip ? skip[rr] : -1;
-  const float* x = X + rr * cols;
-  const long long o = rr * ldc;
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ldc; c += gridDim.x * blockDim.x) {
-    const float p = (c < cols && c != sk) ? expf(x[c] - sh) * mu : 0.f;
-    split3_bf16(p, h[o + c], m[o + c], l[o + c]);
-  }
-}
-
 // VT[b][d][j] = V[b][j][d] (bf16), zero for T <= j < ldT.
 __global__ void __launch_bounds__(256) transpose_v_kernel(const bf16* V, bf16* VT, int T, int ldT) {
   const int b = blockIdx.z, j0 = blockIdx.x * 32, d0 = blockIdx.y * 32;
@@ -50,20 +34,6 @@ __global__ void __launch_bounds__(256) transpose_v_kernel(const bf16* V, bf16* V
     const int j = j0 + tx;
     if (j < ldT) VT[((long long)b * 128 + d0 + q) * ldT + j] = tile[tx][q];
   }
-}
-
-// C[b] (rows x 128 or rows x N) = A3 B^T with A3 = (h, m, l) [H][rows][K] and B [H][N][K].
-static int gemm_split3a(int H, int rows, int N, int K, int ldk, const bf16* h, const bf16* m, const bf16* l,
-                        const bf16* B, float* C, int ldc, float alpha, DevStatus* stt, cudaStream_t st) {
-  CUtensorMap mA, mA2, mA3, mB;
-  if (!encode_bf16_map_3d(&mA, h, ldk, rows, H, 128) || !encode_bf16_map_3d(&mA2, m, ldk, rows, H, 128) ||
-      !encode_bf16_map_3d(&mA3, l, ldk, rows, H, 128) || !encode_bf16_map_3d(&mB, B, ldk, N, H, 128))
-    return -1;
-  TcEpiStore epi{C, (long long)rows * ldc, ldc, alpha};
-  const int kfull = (K + 63) / 64 * 64;
-  if (launch_tc_gemm<128, kSplit3A>(mA, mB, mA2, mA, epi, H, rows, N, K, kfull, stt, st, 0, &mA3) != cudaSuccess)
-    return -1;
-  return 1;
 }
 
 int launch_value_logits_tc(const Dims& D, const bf16* q_h, const bf16* q_m, const bf16* q_l, const bf16* K,
@@ -96,28 +66,34 @@ int launch_transpose_v(const Dims& D, const bf16* V, bf16* VT, cudaStream_t st) 
 // warps form P there (e^x as 2^(x log2 e), one MUFU op per element), split it into the bf16 triple (h, m, l) and write the
 // three operand tiles straight into the 128-byte-swizzled K-major layout the
 // MMA reads; one thread issues h V + m V + l V per 16-wide K step into a
-// 128 x 128 fp32 TMEM accumulator; a fifth warp streams the V^T slabs.  The
-// products are those of the unfused split-3 GEMM, in the same order.
+// 128 x 128 fp32 TMEM accumulator; a fifth warp streams the V^T slabs.
 //
-// CTA = (row tile of 128, K split); with two K splits the halves are added
-// into a zeroed output with fp32 atomics (two addends onto 0: the sum does not
-// depend on their order).
+// kExpf takes e^x by expf after the subtraction: the form that T % 4 != 0 has
+// always had, kept so that its anchors stay what they were.
+//
+// CTA = (row tile, K split); with two K splits the halves are added into a
+// zeroed output with fp32 atomics (two addends onto 0: the sum does not depend
+// on their order).  A row tile has kRows = 128, 64 or 32 rows: a slab's time is
+// the converters', so a call that leaves SMs idle takes shorter tiles, each
+// still one M = 128 MMA whose other rows are ignored (the results keep their
+// bits; 2 row tiles x 2 at n = 256, T = 1024: 20 us, as 8 x 2: 11).
 namespace {
-constexpr int kPvRawBytes = 128 * 64 * 4;   // one fp32 slab of X
 constexpr int kPvTile = 128 * 128;          // one bf16 128 x 64 operand tile
 constexpr int kPvRS = 3;                    // raw ring depth
 constexpr int kPvOS = 2;                    // operand ring depth (h, m, l, V^T)
 constexpr int kPvOpBytes = 4 * kPvTile;
-constexpr int kPvConv = 16;                 // converter warps 2..17, 8 rows each
+constexpr int kPvConv = 16;                 // converter warps 2..17, kRows / 16 rows each
 constexpr int kPvThreads = 32 * (kPvConv + 3);
-constexpr int kPvSmem = kPvRS * kPvRawBytes + kPvOS * kPvOpBytes + 1024;
+constexpr int kPvSmem = kPvRS * 128 * 64 * 4 + kPvOS * kPvOpBytes + 1024;
 }  // namespace
 
-template <bool kSkip>
+template <bool kSkip, bool kExpf, int kRows>
 __global__ void __launch_bounds__(kPvThreads, 1)
     probs_v_kernel(const __grid_constant__ CUtensorMap mX, const __grid_constant__ CUtensorMap mVT,
                    const float* shift, const float* mul, const int* skip, float* O, int rows, int T, int splits,
                    DevStatus* stt) {
+  constexpr int kPvRawBytes = kRows * 64 * 4;   // one fp32 slab of X
+  constexpr int kSteps = kRows / 32;            // two rows of a warp at a time
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t rfull[kPvRS], rempty[kPvRS], vfull[kPvOS], ofull[kPvOS], oempty[kPvOS], accf, drain;
   __shared__ uint32_t tmem_slot;
@@ -126,9 +102,9 @@ __global__ void __launch_bounds__(kPvThreads, 1)
   uint8_t* rbase = smem_raw + (((r0 + 1023u) & ~1023u) - r0);
   uint8_t* obase = rbase + kPvRS * kPvRawBytes;   // 1024-byte aligned: the ring is a multiple of 1 KB
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int mt = (rows + 127) / 128;
+  const int mt = (rows + kRows - 1) / kRows;
   const int tile = blockIdx.x / splits, sp = blockIdx.x - tile * splits;
-  const int b = tile / mt, m0 = (tile - b * mt) * 128;
+  const int b = tile / mt, m0 = (tile - b * mt) * kRows;
   const int nk = (T + 63) / 64;
   const int kb0 = (int)((long long)nk * sp / splits), kb1 = (int)((long long)nk * (sp + 1) / splits);
   const int nkb = kb1 - kb0;
@@ -212,20 +188,20 @@ __global__ void __launch_bounds__(kPvThreads, 1)
       tc::mbar_wait(&drain, 0, &never, stt);
     }
   } else {
-    // converters: warp cw owns rows 8 cw .. 8 cw + 7 of the tile, two rows per
+    // converters: warp cw owns kRows / 16 consecutive rows of the tile, two rows per
     // step (lanes 0-15 the first, 16-31 the second), four columns per lane
     const int cw = warp - 2, hl = lane >> 4, cl = lane & 15;
-    float zl[4], mu[4];   // per step: shift * log2 e and scale of this lane's row (0, 0 past the end: P = 0)
-    int sk[4];
+    float zl[kSteps], mu[kSteps];   // per step: shift * log2 e and scale of this lane's row (0, 0 past the end: P = 0)
+    int sk[kSteps];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int row = m0 + cw * 8 + 2 * u + hl;
+    for (int u = 0; u < kSteps; ++u) {
+      const int row = m0 + cw * (kRows / 16) + 2 * u + hl;
       zl[u] = 0.f;
       mu[u] = 0.f;
       sk[u] = -1;
       if (row < rows) {
         const long long rr = (long long)b * rows + row;
-        zl[u] = shift[rr] * kLog2e;
+        zl[u] = kExpf ? shift[rr] : shift[rr] * kLog2e;
         mu[u] = mul[rr];
         if (kSkip) sk[u] = skip[rr];
       }
@@ -242,11 +218,13 @@ __global__ void __launch_bounds__(kPvThreads, 1)
       const int c = (kb0 + g) * 64 + 4 * cl;   // this lane's first column
       const bool edge = kSkip || c + 4 > T;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int r = cw * 8 + 2 * u + hl;
+      for (int u = 0; u < kSteps; ++u) {
+        const int r = cw * (kRows / 16) + 2 * u + hl;
         const float4 x = *(const float4*)(R + r * 64 + 4 * cl);
-        float p[4] = {ex2_approx(fmaf(x.x, kLog2e, -zl[u])) * mu[u], ex2_approx(fmaf(x.y, kLog2e, -zl[u])) * mu[u],
-                      ex2_approx(fmaf(x.z, kLog2e, -zl[u])) * mu[u], ex2_approx(fmaf(x.w, kLog2e, -zl[u])) * mu[u]};
+        auto prob = [&](float v) {
+          return (kExpf ? expf(v - zl[u]) : ex2_approx(fmaf(v, kLog2e, -zl[u]))) * mu[u];
+        };
+        float p[4] = {prob(x.x), prob(x.y), prob(x.z), prob(x.w)};
         if (edge) {
 #pragma unroll
           for (int e = 0; e < 4; ++e)
@@ -271,7 +249,7 @@ __global__ void __launch_bounds__(kPvThreads, 1)
     }
     if (ok) ok = tc::mbar_wait(&accf, 0, abortp, stt);
     ok = __all_sync(0xffffffffu, ok);
-    if (ok) {
+    if (ok && (warp & 3) * 32 < kRows) {
       tc::fence_after_sync();
       const int qd = warp & 3, cg = cw >> 2;   // TMEM lane quarter; 32-column group
       const int row = m0 + qd * 32 + lane;
@@ -297,33 +275,39 @@ __global__ void __launch_bounds__(kPvThreads, 1)
   }
 }
 
-// The fused product (probs_fused(T): X rows tileable by TMA); returns the
-// launches issued or -1 (also for base pointers off the 16-byte grid).
-static int launch_probs_v_fused(const Dims& D, const float* X, const float* shift, const float* mul, const int* skip,
-                                const bf16* VT, float* out, DevStatus* stt, cudaStream_t st) {
-  if (((uintptr_t)X & 15u) != 0 || ((uintptr_t)out & 15u) != 0) return -1;
-  const int ldT = (D.T + 7) / 8 * 8;
-  CUtensorMap mX, mVT;
-  if (!encode_f32_map_3d(&mX, X, D.T, D.n, D.H, 64, 128) || !encode_bf16_map_3d(&mVT, VT, ldT, 128, D.H, 128))
-    return -1;
-  const int tiles = D.H * cdiv(D.n, 128), nk = cdiv(D.T, 64);
-  const int splits = (2 * tiles <= tc_gemm_sm_count() && nk >= 2) ? 2 : 1;
-  auto kern = skip ? probs_v_kernel<true> : probs_v_kernel<false>;
-  if (set_dyn_smem((const void*)kern, kPvSmem) != cudaSuccess) return -1;
-  if (splits > 1 && cudaMemsetAsync(out, 0, sizeof(float) * (size_t)D.H * D.n * 128, st) != cudaSuccess) return -1;
-  kern<<<tiles * splits, kPvThreads, kPvSmem, st>>>(mX, mVT, shift, mul, skip, out, D.n, D.T, splits, stt);
-  return cudaGetLastError() == cudaSuccess ? 1 : -1;
+template <int kRows>
+static cudaError_t launch_probs_v_rows(const Dims& D, const float* X, const float* shift, const float* mul,
+                                       const CUtensorMap& mVT, float* out, int splits, DevStatus* stt, cudaStream_t st,
+                                       const int* skip) {
+  const int ld = logit_ld(D.T);
+  CUtensorMap mX;
+  if (!encode_f32_map_3d(&mX, X, D.T, D.n, D.H, 64, kRows, ld, (uint64_t)D.n * ld)) return cudaErrorInvalidValue;
+  const bool odd = (D.T & 3) != 0;
+  auto kern = skip ? (odd ? probs_v_kernel<true, true, kRows> : probs_v_kernel<true, false, kRows>)
+                   : (odd ? probs_v_kernel<false, true, kRows> : probs_v_kernel<false, false, kRows>);
+  const cudaError_t e = set_dyn_smem((const void*)kern, kPvSmem);
+  if (e != cudaSuccess) return e;
+  kern<<<D.H * cdiv(D.n, kRows) * splits, kPvThreads, kPvSmem, st>>>(mX, mVT, shift, mul, skip, out, D.n, D.T, splits,
+                                                                     stt);
+  return cudaGetLastError();
 }
 
-int launch_probs_v_tc(const Dims& D, const float* X, const float* shift, const float* mul, bf16* p_h, bf16* p_m,
-                      bf16* p_l, const bf16* VT, float* out, DevStatus* stt, cudaStream_t st, const int* skip) {
-  if (probs_fused(D.T)) return launch_probs_v_fused(D, X, shift, mul, skip, VT, out, stt, st);
-  // X rows not TMA-tileable: P as a bf16 triple in memory, then the split-3 GEMM
-  const int ldT = (D.T + 7) / 8 * 8;
-  probs_split3_kernel<<<dim3(cdiv(ldT, 256 * 4), D.n, D.H), 256, 0, st>>>(X, shift, mul, skip, p_h, p_m, p_l, D.n,
-                                                                          D.T, ldT);
-  if (gemm_split3a(D.H, D.n, 128, ldT, ldT, p_h, p_m, p_l, VT, out, 128, 1.f, stt, st) < 0) return -1;
-  return 2;
+int launch_probs_v_tc(const Dims& D, const float* X, const float* shift, const float* mul, const bf16* VT, float* out,
+                      DevStatus* stt, cudaStream_t st, const int* skip) {
+  if (((uintptr_t)X & 15u) != 0 || ((uintptr_t)out & 15u) != 0) return -1;
+  const int ldT = (D.T + 7) / 8 * 8, sms = tc_gemm_sm_count();
+  CUtensorMap mVT;
+  if (!encode_bf16_map_3d(&mVT, VT, ldT, 128, D.H, 128)) return -1;
+  const int tiles = D.H * cdiv(D.n, 128), nk = cdiv(D.T, 64);
+  // (T % 4 != 0 never had its sums split, and the fits amplify their rounding a
+  // hundredfold: it keeps one K range and takes shorter row tiles alone)
+  const int splits = (2 * tiles <= sms && nk >= 2 && (D.T & 3) == 0) ? 2 : 1;
+  if (splits > 1 && cudaMemsetAsync(out, 0, sizeof(float) * (size_t)D.H * D.n * 128, st) != cudaSuccess) return -1;
+  const cudaError_t e =
+      4 * tiles * splits <= sms   ? launch_probs_v_rows<32>(D, X, shift, mul, mVT, out, splits, stt, st, skip)
+      : 2 * tiles * splits <= sms ? launch_probs_v_rows<64>(D, X, shift, mul, mVT, out, splits, stt, st, skip)
+                                  : launch_probs_v_rows<128>(D, X, shift, mul, mVT, out, splits, stt, st, skip);
+  return e == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace arckv

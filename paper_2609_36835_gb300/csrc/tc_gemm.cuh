@@ -56,6 +56,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "kernels.h"
 #include "tc.cuh"
 
 namespace arckv {
@@ -333,11 +334,6 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
   }
 }
 
-// Resident CTAs of the persistent GEMM: one per SM (the stage ring takes most
-// of the shared memory), looked up once per device.
-int tc_gemm_sm_count();
-cudaError_t set_dyn_smem(const void* kern, int bytes);
-
 // Host: launch over H batches; maps are built by the caller (encode_bf16_map_3d,
 // box rows 128 for A and BN for B).
 template <int BN, int MODE, class Epi>
@@ -513,7 +509,7 @@ struct TcEpiStoreTmaT {
   __device__ __forceinline__ void finish(State&, int, int, int, int, int) const {}
 };
 
-// A store epilogue (TcEpiStore or TcEpiStoreTma) that also writes each row's
+// A store epilogue (TcEpiStoreTmaT) that also writes each row's
 // softmax partials over each kRowPartW = 64 columns: part[b][row][col / 64] =
 // (max, sum exp(x - max)) of alpha * acc (exp as 2^(x log2 e) on the MUFU
 // unit).  Eight epilogue warps, each draining 64 columns of a 128-wide tile.
@@ -568,31 +564,23 @@ struct TcEpiRowPartT {
     if (s.row_ok && s.ncols > 0) part[s.prow] = make_float2(s.mx, s.sm);
   }
 };
-using TcEpiStoreRowPart = TcEpiRowPartT<TcEpiStore>;
 using TcEpiStoreRowPartTma = TcEpiRowPartT<TcEpiStoreTmaT<1>>;
 
-// Row-partial logits L = alpha * (A B^T) [H][M][N] (row stride N) through the
-// TMA-store epilogue when N is a multiple of 4 (row pitch on the 16-byte grid),
-// else through plain stores.
+// Row-partial logits L = alpha * (A B^T) [H][M][N] (row pitch logit_ld(N)).
 template <int MODE>
 inline cudaError_t launch_tc_logits_rowpart(const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mA2,
                                             const CUtensorMap& mB2, const CUtensorMap* mA3, float* L, float alpha,
                                             float2* part, int H, int M, int N, int K, DevStatus* stt,
                                             cudaStream_t st) {
-  const int ntiles = cdiv(N, 64);
-  if ((N & 3) == 0 && (((uintptr_t)L) & 15u) == 0) {
-    TcEpiStoreRowPartTma epi{};
-    epi.st.alpha = alpha;
-    epi.st.M = M;
-    epi.st.N = N;
-    epi.part = part;
-    epi.ntiles = ntiles;
-    epi.BNt = 64;
-    if (!encode_f32_map_3d(&epi.st.map, L, N, M, H, 32, 32, N, (uint64_t)M * N, true))
-      return cudaErrorInvalidValue;
-    return launch_tc_gemm<128, MODE>(mA, mB, mA2, mB2, epi, H, M, N, K, K, stt, st, 0, mA3);
-  }
-  TcEpiStoreRowPart epi{{L, (long long)M * N, N, alpha}, part, ntiles, 64};
+  const int ld = logit_ld(N);
+  TcEpiStoreRowPartTma epi{};
+  epi.st.alpha = alpha;
+  epi.st.M = M;
+  epi.st.N = N;
+  epi.part = part;
+  epi.ntiles = cdiv(N, 64);
+  epi.BNt = 64;
+  if (!encode_f32_map_3d(&epi.st.map, L, N, M, H, 32, 32, ld, (uint64_t)M * ld, true)) return cudaErrorInvalidValue;
   return launch_tc_gemm<128, MODE>(mA, mB, mA2, mB2, epi, H, M, N, K, K, stt, st, 0, mA3);
 }
 

@@ -17,20 +17,19 @@ namespace arckv {
 // Each epilogue thread folds one row of kW columns of a kBN-wide tile (kBN / kW
 // warps per TMEM lane quarter: four epilogue warps for 128-wide tiles, eight
 // for 256-wide ones) and writes their row-softmax partials,
-// part[b][row][n0 / kW].  kTma: the I tile leaves through TMA stores staged in
+// part[b][row][n0 / kW].  The I tile leaves through TMA stores staged in
 // shared memory (32 x 32 boxes; two buffers per warp with four warps, one
-// with eight); else each row writes its kW values.
-template <bool kTma, int kW_, int kBN = 128>
+// with eight).
+template <int kW_, int kBN = 128>
 struct TcEpiIndexT {
   static constexpr int kW = kW_;
   static constexpr int kEpiWarps = kBN / kW * 4;
   static constexpr int kNBuf = kEpiWarps == 4 ? 2 : 1;
-  static constexpr int kStageBytes = kTma ? kNBuf * 32 * 128 : 0;
+  static constexpr int kStageBytes = kNBuf * 32 * 128;
   const float* wts;  // [H][n_pos][H_I]
-  float* I;          // [H][n][T]
   float2* part;      // [H][n][ntiles], ntiles = ceil(T / kW)
   int n, T, H_I, G, n_pos, ntiles;
-  CUtensorMap map;   // kTma: I as [H][n][T], box {32, 32, 1}, 128-byte swizzle
+  CUtensorMap map;   // I as [H][n][T] (rows logit_ld(T) apart), box {32, 32, 1}, 128-byte swizzle
   struct State {
     float acc[kW];
     const float* wrow;
@@ -93,25 +92,11 @@ struct TcEpiIndexT {
       const float sm = ((a8[0] + a8[1]) + (a8[2] + a8[3])) + ((a8[4] + a8[5]) + (a8[6] + a8[7]));
       part[((long long)b * n + row) * ntiles + n0 / kW] = make_float2(mx, sm);
     }
-    if constexpr (kTma) {
-      // rows past n and columns past T fall outside the tensor map: not written
-      const int y = row & ~31;
+    // rows past n and columns past T fall outside the tensor map: not written
+    const int y = row & ~31;
 #pragma unroll
-      for (int j = 0; j < kW / 32; ++j)
-        staged_store_32x32<kNBuf>(&map, s.stage, s.stores, n0 + 32 * j, y, b, n, T, s.acc + 32 * j, 1.f);
-    } else {
-      if (!s.row_ok || nc <= 0) return;
-      float* dst = I + ((long long)b * n + row) * T + n0;
-      if ((T & 3) == 0 && nc == kW) {
-#pragma unroll
-        for (int q = 0; q < kW; q += 4)
-          *(float4*)(dst + q) = make_float4(s.acc[q], s.acc[q + 1], s.acc[q + 2], s.acc[q + 3]);
-      } else {
-#pragma unroll
-        for (int q = 0; q < kW; ++q)
-          if (q < nc) dst[q] = s.acc[q];
-      }
-    }
+    for (int j = 0; j < kW / 32; ++j)
+      staged_store_32x32<kNBuf>(&map, s.stage, s.stores, n0 + 32 * j, y, b, n, T, s.acc + 32 * j, 1.f);
   }
 };
 
@@ -126,29 +111,19 @@ int launch_index_logits(const Dims& D, const bf16* qbar_hi, const bf16* qbar_lo,
   if (!encode_bf16_map_3d(&mA, qbar_hi, D.HD, D.n, D.H, 128) || !encode_bf16_map_3d(&mA2, qbar_lo, D.HD, D.n, D.H, 128) ||
       !encode_bf16_map_3d(&mB, kbar_hi, D.HD, D.T, D.H, bB) || !encode_bf16_map_3d(&mB2, kbar_lo, D.HD, D.T, D.H, bB))
     return -1;
-  if ((D.T & 3) == 0 && ((uintptr_t)I & 15u) == 0) {
-    if (wide) {
-      TcEpiIndexT<true, kIndexPartW, 256> epi{wts, I, part, D.n, D.T, D.H_I, D.G, D.n_pos, cdiv(D.T, kIndexPartW), {}};
-      if (!encode_f32_map_3d(&epi.map, I, D.T, D.n, D.H, 32, 32, D.T, (uint64_t)D.n * D.T, true)) return -1;
-      if (launch_tc_gemm<256, kSplit>(mA, mB, mA2, mB2, epi, D.H, D.n, D.T, D.HD, 128, stt, st) != cudaSuccess)
-        return -1;
-      return 1;
-    }
-    TcEpiIndexT<true, kIndexPartW> epi{wts, I, part, D.n, D.T, D.H_I, D.G, D.n_pos, cdiv(D.T, kIndexPartW), {}};
-    if (!encode_f32_map_3d(&epi.map, I, D.T, D.n, D.H, 32, 32, D.T, (uint64_t)D.n * D.T, true)) return -1;
-    if (launch_tc_gemm<128, kSplit>(mA, mB, mA2, mB2, epi, D.H, D.n, D.T, D.HD, 128, stt, st) != cudaSuccess)
-      return -1;
-    return 1;
-  }
+  const int ld = logit_ld(D.T);
+  CUtensorMap mI;
+  if (!encode_f32_map_3d(&mI, I, D.T, D.n, D.H, 32, 32, ld, (uint64_t)D.n * ld, true)) return -1;
+  const int ntiles = cdiv(D.T, kIndexPartW);
+  cudaError_t e;
   if (wide) {
-    TcEpiIndexT<false, kIndexPartW, 256> epi{wts, I, part, D.n, D.T, D.H_I, D.G, D.n_pos, cdiv(D.T, kIndexPartW), {}};
-    if (launch_tc_gemm<256, kSplit>(mA, mB, mA2, mB2, epi, D.H, D.n, D.T, D.HD, 128, stt, st) != cudaSuccess)
-      return -1;
-    return 1;
+    TcEpiIndexT<kIndexPartW, 256> epi{wts, part, D.n, D.T, D.H_I, D.G, D.n_pos, ntiles, mI};
+    e = launch_tc_gemm<256, kSplit>(mA, mB, mA2, mB2, epi, D.H, D.n, D.T, D.HD, 128, stt, st);
+  } else {
+    TcEpiIndexT<kIndexPartW> epi{wts, part, D.n, D.T, D.H_I, D.G, D.n_pos, ntiles, mI};
+    e = launch_tc_gemm<128, kSplit>(mA, mB, mA2, mB2, epi, D.H, D.n, D.T, D.HD, 128, stt, st);
   }
-  TcEpiIndexT<false, kIndexPartW> epi{wts, I, part, D.n, D.T, D.H_I, D.G, D.n_pos, cdiv(D.T, kIndexPartW), {}};
-  if (launch_tc_gemm<128, kSplit>(mA, mB, mA2, mB2, epi, D.H, D.n, D.T, D.HD, 128, stt, st) != cudaSuccess) return -1;
-  return 1;
+  return e == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace arckv

@@ -24,7 +24,9 @@ def _gpu(lib):
 # one block (full, short, one row), its edge, the cluster sizes 4 / 8 / 12 or 16
 # (5 and 9 blocks; 8 heads at a time), and one above the clustered substitution's 2048
 @pytest.mark.parametrize("H,T,n_pos,t", [(2, 200, 40, 1), (2, 200, 40, 64), (2, 203, 40, 65), (1, 400, 90, 257),
-                                         (3, 801, 160, 513), (8, 900, 161, 577), (1, 2500, 600, 2049)])
+                                         (3, 801, 160, 513), (8, 900, 161, 577), (1, 2500, 600, 2049),
+                                         # reference attention: 64-row tiles (split and odd T), 32-row tiles at odd T
+                                         (8, 704, 128, 70), (4, 705, 290, 60), (8, 701, 128, 70)])
 def test_primal_fits_on_given_groups(H, T, n_pos, t):
     w = synth.WORKLOADS["llama8b_layer_T8192"]
     arr = workload.layer_inputs_np(w, 0, list(range(H)), T=T, n_pos=n_pos)
