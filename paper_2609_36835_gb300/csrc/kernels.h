@@ -216,12 +216,18 @@ AttendLayout attend_layout(int H, int n, int t);
 int launch_attend(int H, int n, int t, float scale, const bf16* Q, const float* C_k, const float* beta,
                   const float* C_v, float* O, char* ws, DevStatus* stt, cudaStream_t st);
 
+// Key splits of the split-key attention pass (deterministic in the sizes).
+struct JointSplit {
+  int per_split, nsplit;
+};
+
 // ---- HA / VI anchor scores (App. B.1) ----------------------------------
 // E[h] = mean_i ||O_i - O~_i(S)|| / (||O_i|| + eps) (Eq. background_truncated_error);
-// scratch inS [H][T] bytes, err [H][n].
+// scratch inS [H][T] bytes, err [H][n], Opart [H][nsplit][n][2][128], ml
+// [H][nsplit][n] (trunc_split); non-finite results are recorded in stt.
 int launch_truncated_error(int H, int n, int T, int t, float scale, float eps, const bf16* Q, const bf16* K,
-                           const bf16* V, const int* S, float* E, unsigned char* inS, float* err, DevStatus* stt,
-                           cudaStream_t st);
+                           const bf16* V, const int* S, float* E, unsigned char* inS, float* err, float* Opart,
+                           float2* ml, DevStatus* stt, cudaStream_t st);
 // Scratch of launch_vi_scores: per row amax, z2, mul2, Da, oo [H][n]; O^(-a) Om
 // [H][n][128]; Y's split y_* [H][n][128]; vv [H][T]; colpart [H][ceil(n/32)][T].
 struct ViBufs {
@@ -234,14 +240,12 @@ int launch_vi_scores(const Dims& D, const float* L, const float* z, const float*
                      const bf16* VT, const ViBufs& B, float* s, float eps, DevStatus* stt, cudaStream_t st);
 
 // ---- joint attention with an uncompressed block (App. A.7) -------------
-// Key splits of the split-key pass (deterministic in H, n, t, F).
-struct JointSplit {
-  int per_split, nsplit;
-};
 JointSplit joint_split(int H, int n, int t, int F);
+JointSplit trunc_split(int H, int n, int T);
 // O [H][n][128] fp32 = softmax(scale Q [C_k; K_f]^T + [beta; 0]) [C_v; V_f];
 // C_k, C_v fp32 or (compact_bf16) bf16 [H][t][128]; K_f, V_f bf16 [H][F][128];
-// scratch Opart [H][nsplit][n][128] fp32 and ml [H][nsplit][n].
+// scratch Opart [H][nsplit][n][128] fp32 and ml [H][nsplit][n]; non-finite
+// results are recorded in stt.
 int launch_attend_joint(int H, int n, int t, int F, float scale, const bf16* Q, const void* Ck, const float* beta,
                         const void* Cv, bool compact_bf16, const bf16* Kf, const bf16* Vf, float* O, float* Opart,
                         float2* ml, DevStatus* stt, cudaStream_t st);
