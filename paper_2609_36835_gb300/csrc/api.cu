@@ -19,7 +19,7 @@ constexpr size_t kAlign = 256;
 inline size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-  size_t status, kbar_hi, kbar_lo, vq, qpp, q_h, q_m, q_l, av, VT, vq3, av3, ukt, qbar_hi, qbar_lo, wts, NT, rA, rB, part, lse, s, anchors, z, m, invm, Y, logphi,
+  size_t status, kbar_hi, kbar_lo, vq, qpp, q_h, q_m, q_l, av, VT, spare, vq3, av3, ukt, qbar_hi, qbar_lo, wts, NT, rA, rB, part, lse, s, anchors, z, m, invm, Y, logphi,
       qcat, wcat, Ut_hi, Ut_lo, S_hi, S_lo, best, kappa, kmap, perm, goff, cursor, LC, Phi, Gram, Linv, rhs, wsol, R, Z,
       ck3, YT_hi, YT_lo, G64, L64, B64, Z64, X64, Sl, Sl2, eR, eC, ir_u, ir_sq, ir_lam, Sl3, eC2, cl_lam, ctrip, total;
 };
@@ -78,6 +78,9 @@ Layout plan(const arckv_config& c) {
   L.q_l = take(H * n * 128 * 2);
   L.av = take(H * n * 128 * f);
   L.VT = take(H * 128 * ldT * 2);
+  // with T % 4 != 0 a workspace has always held three bf16 [n][T] arrays here,
+  // and keeps its size
+  L.spare = take((T & 3) ? 3 * H * n * ldT * 2 : 0);
   L.qcat = take(H * n * 512 * 2);
   L.vq3 = take(3 * H * n * 128 * 2);
   L.av3 = take(3 * H * n * 128 * 2);
@@ -142,7 +145,10 @@ Layout plan(const arckv_config& c) {
   L.Sl3 = take(dual ? 5 * H * 128 * sliced_ld((int)n) * 2 : 0);
   L.eC2 = take(dual ? H * 128 * 4 : 0);
   L.cl_lam = take(dual ? H * 8 : 0);
-  L.ctrip = take(dual ? 0 : chol_trip_bytes(c.H_kv, (int)t));
+  // the solver's operand slots: over the reference logits (not read after the
+  // assignment) unless the problem is tiny
+  const size_t trip = dual ? 0 : chol_trip_bytes(c.H_kv, (int)t);
+  L.ctrip = trip <= H * n * (size_t)logit_ld((int)T) * f ? L.NT : take(trip);
   L.total = o;
   return L;
 }
@@ -424,7 +430,6 @@ arckv_status arckv_attend(int32_t H_kv, int32_t n, int32_t t, int32_t d, float l
   cudaGetLastError();
   if (cudaMemsetAsync(stt, 0, sizeof(DevStatus), st) != cudaSuccess) return ARCKV_ERR_CUDA;
   if (launch_attend(H_kv, n, t, scale, (const bf16*)Q, C_k, beta, C_v, O, w, stt, st) < 0) return ARCKV_ERR_CUDA;
-  launch_check_finite(O, (long long)H_kv * n * d, stt, st);
   if (cudaGetLastError() != cudaSuccess) return ARCKV_ERR_CUDA;
   if (flags & ARCKV_FLAG_NONBLOCKING) return ARCKV_OK;
   return read_status(ws, st);

@@ -99,7 +99,6 @@ arckv_status arckv_attend_static(int32_t H_kv, int32_t n, int32_t t, int32_t d, 
   if (cudaMemsetAsync(stt, 0, sizeof(arckv::DevStatus), st) != cudaSuccess) return ARCKV_ERR_CUDA;
   if (arckv::launch_attend(H_kv, n, t, scale, (const arckv::bf16*)Q, C_k, beta, C_v, O, (char*)base, stt, st) < 0)
     return ARCKV_ERR_CUDA;
-  arckv::launch_check_finite(O, (long long)H_kv * n * d, stt, st);
   if (cudaGetLastError() != cudaSuccess) return ARCKV_ERR_CUDA;
   unsigned int code = 0;
   if (cudaMemcpyAsync(&code, stt, sizeof(code), cudaMemcpyDeviceToHost, st) != cudaSuccess) return ARCKV_ERR_CUDA;

@@ -212,7 +212,8 @@ struct AttendLayout {
 };
 AttendLayout attend_layout(int H, int n, int t);
 // O [H][n][128] = softmax(scale Q C_k^T + beta) C_v on the tensor pipe; `ws` is
-// the scratch base of attend_layout.  Returns launches or -1.
+// the scratch base of attend_layout; a non-finite result is recorded in stt.
+// Returns launches or -1.
 int launch_attend(int H, int n, int t, float scale, const bf16* Q, const float* C_k, const float* beta,
                   const float* C_v, float* O, char* ws, DevStatus* stt, cudaStream_t st);
 

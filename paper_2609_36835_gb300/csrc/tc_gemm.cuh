@@ -24,6 +24,8 @@
 //              within 2^-24 relative (mA, mA2, mA3) and B is exact bf16 (mB):
 //              every K step issues h*B + m*B + l*B, fp32-grade products for an
 //              fp32 operand against a bf16 input;
+//   kSplit3B -- the same with the triple on the B side (mB, mB2, mA3) and exact A
+//              (mA): A*h + A*m + A*l;
 //   kSplit3S -- a Gram of one fp32 operand with itself: A and B are both the
 //              triple (mA, mA2, mA3), read at rows m0 and n0, and every K step
 //              issues hh + hm + mh + hl + lh + mm (the dropped ml, lm, ll terms
@@ -61,7 +63,7 @@
 
 namespace arckv {
 
-enum TcMode { kPlain = 0, kSplit = 1, kConcat = 2, kSplit3A = 3, kSplit3S = 4 };
+enum TcMode { kPlain = 0, kSplit = 1, kConcat = 2, kSplit3A = 3, kSplit3S = 4, kSplit3B = 5 };
 
 template <class E, class = void>
 struct EpiWarps {
@@ -99,9 +101,10 @@ struct TcCfg {
   static constexpr int TILE_B = BN * 128;
   static constexpr int STAGE = MODE == kSplit     ? 2 * (TILE_A + TILE_B)
                                : MODE == kSplit3A ? 3 * TILE_A + TILE_B
+                               : MODE == kSplit3B ? TILE_A + 3 * TILE_B
                                : MODE == kSplit3S ? 3 * (TILE_A + TILE_B)
                                                   : TILE_A + TILE_B;
-  static constexpr int STAGES_WANT = MODE == kSplit3S ? 2 : (MODE == kSplit || MODE == kSplit3A) ? 3 : 4;
+  static constexpr int STAGES_WANT = MODE == kSplit3S ? 2 : (MODE == kSplit || MODE == kSplit3A || MODE == kSplit3B) ? 3 : 4;
   // as many of those as fit beside the epilogue staging (wide tiles take fewer)
   static constexpr int STAGES = STAGES_WANT * STAGE <= 200 * 1024 ? STAGES_WANT : (200 * 1024) / STAGE;
   static constexpr int SMEM = STAGES * STAGE + 1024;
@@ -173,6 +176,10 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
         tc::tma_prefetch(&mA2);
         tc::tma_prefetch(&mB2);
       }
+      if (MODE == kSplit3B) {
+        tc::tma_prefetch(&mB2);
+        tc::tma_prefetch(&mA3);
+      }
       if (MODE == kSplit3A || MODE == kSplit3S) {
         tc::tma_prefetch(&mA2);
         tc::tma_prefetch(&mA3);
@@ -212,6 +219,10 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
           if (MODE == kSplit3A) {
             tc::tma_load_3d(st + C::TILE_A + C::TILE_B, &mA2, kb * 64, m0, b, &full[s]);
             tc::tma_load_3d(st + 2 * C::TILE_A + C::TILE_B, &mA3, kb * 64, m0, b, &full[s]);
+          }
+          if (MODE == kSplit3B) {
+            tc::tma_load_3d(st + C::TILE_A + C::TILE_B, &mB2, kb * 64, n0, b, &full[s]);
+            tc::tma_load_3d(st + C::TILE_A + 2 * C::TILE_B, &mA3, kb * 64, n0, b, &full[s]);
           }
           ++g;
         }
@@ -259,6 +270,10 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
                 const uint64_t al = tc::sdesc_k128(a + 2 * C::TILE_A + C::TILE_B + ks * 32);
                 tc::mma_f16(d, am, bd, idesc, 1u);
                 tc::mma_f16(d, al, bd, idesc, 1u);
+              }
+              if (MODE == kSplit3B) {
+                tc::mma_f16(d, ad, tc::sdesc_k128(bb + C::TILE_B + ks * 32), idesc, 1u);
+                tc::mma_f16(d, ad, tc::sdesc_k128(bb + 2 * C::TILE_B + ks * 32), idesc, 1u);
               }
               if (MODE == kSplit3S) {
                 constexpr uint32_t P = C::TILE_A + C::TILE_B;

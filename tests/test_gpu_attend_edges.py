@@ -1,5 +1,5 @@
-"""Joint attention and the truncated-output error at the edges of their tiles
-(16 keys a warp, four warps, the key splits): every head against the oracle,
+"""Joint and compact attention and the truncated-output error at the edges of
+their tiles (16 keys a warp, four warps; 32 or 64 rows, 64 keys): every head against the oracle,
 with the bound of the other joint-attention tests (1e-4)."""
 import numpy as np
 import pytest
@@ -49,6 +49,18 @@ def test_joint_tile_edges(H, n, t, F, dtype):
         x = np.concatenate([_np(Q[h]) @ _np(Ck[h]).T * SCALE + _np(beta[h]), _np(Q[h]) @ _np(Kf[h]).T * SCALE], axis=1)
         p = np.exp(x - x.max(axis=1, keepdims=True))
         ref = p / p.sum(axis=1, keepdims=True) @ np.concatenate([_np(Cv[h]), _np(Vf[h])])
+        assert _rel(O[h], ref) <= 1e-4, h
+
+
+# (H, n, t): 32-row tiles with key splits, 64-row tiles, odd pitches, a slab's edge, one key
+@pytest.mark.parametrize("H,n,t", [(1, 1, 1), (2, 33, 63), (1, 70, 1027), (8, 900, 65), (3, 5, 4097)])
+def test_compact_attention_tile_edges(H, n, t):
+    Q, Ck, Cv = _draw(1, H, n, 128) * 2, _draw(4, H, t, 128, dtype=torch.float32), _draw(5, H, t, 128, dtype=torch.float32)
+    beta = _draw(6, H, t, dtype=torch.float32)
+    beta[:, 1::3] = -20.0
+    O = pk.attend(Q.cuda(), Ck.cuda(), beta.cuda(), Cv.cuda()).cpu().numpy()
+    for h in range(H):
+        ref = oracle.compact_attention(_np(Q[h]), _np(Ck[h]), _np(beta[h]), _np(Cv[h]), SCALE)
         assert _rel(O[h], ref) <= 1e-4, h
 
 
