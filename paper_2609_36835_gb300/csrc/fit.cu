@@ -553,27 +553,30 @@ __global__ void __launch_bounds__(kCT, 1) chol_diag_kernel(double* A, double* Li
   if (threadIdx.x == 0 && bad) set_status(stt, ARCKV_ERR_NOT_SPD);
 }
 
-// X_k = Linv_kk^T (Y_k - Z_k) for block k of every head, 32 right-hand sides
-// per CTA (grid: head x column group): V = Y_k - Z_k and Linv_kk go through
-// shared memory, X[k0 + c][j] = sum_{l >= c} Linv_k[l][c] V[l][j].
+// X_k = Linv_kk^T (Y_k - Z_k) for block k of every head, kBackCols right-hand
+// sides per CTA (grid: head x column group): V = Y_k - Z_k and Linv_kk go through
+// shared memory, X[k0 + c][j] = sum_{l >= c} Linv_k[l][c] V[l][j].  Bound by the
+// fp64 pipe (two multiply-adds per clock and SM): 8 columns a CTA spread 8 heads
+// x 128 columns over 128 SMs, 32 left three quarters of them idle (30 us a block).
+constexpr int kBackCols = 8;
 __global__ void __launch_bounds__(256) chol_back_block_kernel(const double* Linv, const double* Y, const double* Z,
                                                               double* X, int n, int k, int nrhs, int useZ) {
   __shared__ double Ls[NB][NB + 1];
-  __shared__ double Vs[NB][33];
-  const int b = blockIdx.x, j0 = blockIdx.y * 32, nblk = (n + NB - 1) / NB, k0 = k * NB, kb = min(NB, n - k0);
-  const int nj = min(32, nrhs - j0);
+  __shared__ double Vs[NB][kBackCols + 1];
+  const int b = blockIdx.x, j0 = blockIdx.y * kBackCols, nblk = (n + NB - 1) / NB, k0 = k * NB, kb = min(NB, n - k0);
+  const int nj = min(kBackCols, nrhs - j0);
   const double* Li = Linv + ((long long)b * nblk + k) * NB * NB;
   const double* Yb = Y + ((long long)b * n + k0) * nrhs + j0;
   const double* Zb = Z + (long long)b * NB * nrhs + j0;
   double* Xb = X + ((long long)b * n + k0) * nrhs + j0;
   for (int e = threadIdx.x; e < NB * NB; e += 256) Ls[e / NB][e % NB] = Li[e];
-  for (int e = threadIdx.x; e < NB * 32; e += 256) {
-    const int l = e >> 5, j = e & 31;
+  for (int e = threadIdx.x; e < NB * kBackCols; e += 256) {
+    const int l = e / kBackCols, j = e % kBackCols;
     Vs[l][j] = (l < kb && j < nj) ? Yb[(long long)l * nrhs + j] - (useZ ? Zb[(long long)l * nrhs + j] : 0.0) : 0.0;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < kb * 32; e += 256) {
-    const int c = e >> 5, j = e & 31;
+  for (int e = threadIdx.x; e < kb * kBackCols; e += 256) {
+    const int c = e / kBackCols, j = e % kBackCols;
     double a = 0.0;
     for (int l = c; l < kb; ++l) a = fma(Ls[l][c], Vs[l][j], a);
     if (j < nj) Xb[(long long)c * nrhs + j] = a;
@@ -585,18 +588,21 @@ __global__ void __launch_bounds__(256) chol_back_block_kernel(const double* Linv
 // terms cancel heavily (|a| |Phi| exceeds |w| by ~1e4 on 128K caches), so the
 // sum runs in double-float arithmetic: each product Phi a_hi + Phi a_lo is
 // formed exactly up to the lo part's rounding and added with an error-free
-// sum; a is split into fp32 (hi, lo) pairs in shared memory, 1024 rows at a time.
-__global__ void __launch_bounds__(256) phi_t_vec_kernel(const float* __restrict__ Phi, const double* __restrict__ a,
+// sum; a is split into fp32 (hi, lo) pairs in shared memory, 1024 rows at a time,
+// and sixteen rows of Phi are in flight per thread (128 threads a CTA: at t = 2001
+// the columns fill the SMs).
+constexpr int kPtThreads = 128;
+__global__ void __launch_bounds__(kPtThreads) phi_t_vec_kernel(const float* __restrict__ Phi, const double* __restrict__ a,
                                                         float* __restrict__ w, int n, int t) {
   __shared__ float ah[1024], al[1024];
-  const int b = blockIdx.y, r = blockIdx.x * 256 + threadIdx.x;
+  const int b = blockIdx.y, r = blockIdx.x * kPtThreads + threadIdx.x;
   const float* p = Phi + (long long)b * n * t + min(r, t - 1);
   const double* ab = a + (long long)b * n;
   df64 sum(0.f, 0.f);
   for (int i0 = 0; i0 < n; i0 += 1024) {
     const int cnt = min(1024, n - i0);
     __syncthreads();
-    for (int i = threadIdx.x; i < cnt; i += 256) {
+    for (int i = threadIdx.x; i < cnt; i += kPtThreads) {
       const double v = ab[i0 + i];
       const float h = __double2float_rn(v);
       ah[i] = h;
@@ -604,14 +610,22 @@ __global__ void __launch_bounds__(256) phi_t_vec_kernel(const float* __restrict_
     }
     __syncthreads();
     if (r < t) {
-      for (int i = 0; i < cnt; ++i) {
-        const float x = p[(long long)(i0 + i) * t];
+      auto add = [&](float x, int i) {
         const float ph = x * ah[i];
         const float pl = fmaf(x, al[i], fmaf(x, ah[i], -ph));
         df64 s2 = df_two(sum.hi, ph);
         s2.lo += sum.lo + pl;
         sum = df_fast2(s2.hi, s2.lo);
+      };
+      int i = 0;
+      for (; i + 16 <= cnt; i += 16) {
+        float x[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] = p[(long long)(i0 + i + e) * t];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) add(x[e], i + e);
       }
+      for (; i < cnt; ++i) add(p[(long long)(i0 + i) * t], i);
     }
   }
   if (r < t) w[(long long)b * t + r] = sum.hi + sum.lo;
@@ -860,7 +874,7 @@ static int chol_solve_sliced(int H, int n, double* A, double* Linv, double* B, d
                                 false, stt, st)))
         return -1;
     }
-    chol_back_block_kernel<<<dim3(H, cdiv(nrhs, 32)), 256, 0, st>>>(Linv, B, W.Z, X, n, k, nrhs, m > 0 ? 1 : 0);
+    chol_back_block_kernel<<<dim3(H, cdiv(nrhs, kBackCols)), 256, 0, st>>>(Linv, B, W.Z, X, n, k, nrhs, m > 0 ? 1 : 0);
     ++nl;
   }
   return nl;
@@ -914,7 +928,7 @@ static int fits_dual(const Dims& D, float ridge_w, float ridge_v, float eps_w, f
   r = solve(1, D.n, ridge_w);
   if (r < 0) return -1;
   nl += 1 + r;
-  phi_t_vec_kernel<<<dim3(cdiv(D.t, 256), D.H), 256, 0, st>>>(B.Phi, B.X64, B.rhs, D.n, D.t);   // w = Phi^T a
+  phi_t_vec_kernel<<<dim3(cdiv(D.t, kPtThreads), D.H), kPtThreads, 0, st>>>(B.Phi, B.X64, B.rhs, D.n, D.t);   // w = Phi^T a
   const long long ht = (long long)D.H * D.t;
   beta_kernel<<<cdiv(ht, 256), 256, 0, st>>>(B.rhs, beta, ht, eps_w, b_min, b_max);
   softmax_bias_kernel<<<dim3(cdiv(D.n, 8), D.H), 256, 0, st>>>(B.LC, beta, B.Phi, D.n, D.t);
@@ -950,20 +964,6 @@ static int fits_dual(const Dims& D, float ridge_w, float ridge_v, float eps_w, f
 // (the exact normal matrix of the fp32 Phi, no Gram rounding) and corrects
 // x += (L L^T)^-1 r with the factor the solver left behind: L_kk and the
 // off-diagonal blocks in the Gram's lower part, L_kk^-1 in Linv.
-
-// fp32 -> fp64 by moving the fields (IEEE 754: the exponent rebiased by 1023 -
-// 127, the fraction padded; subnormals -- a fifth of Phi -- scaled by 2^64
-// first): GB300 converts fewer than one value per clock and SM, which held the
-// residual passes at 62 and 64 us for 27 MB of Phi (8 heads, n = 1024, t = 819);
-// they take 37 and 27 us this way.
-// Infinities and NaN take the conversion.
-__device__ __forceinline__ double widen_bits(float x) {
-  const bool small = (__float_as_uint(x) & 0x7f800000u) == 0u;
-  const unsigned u = __float_as_uint(small ? x * 18446744073709551616.f : x), ex = u & 0x7f800000u;
-  if (ex == 0x7f800000u) return (double)x;
-  const unsigned hi = (u & 0x80000000u) | (ex ? ((u & 0x7fffffffu) >> 3) + (small ? 0x34000000u : 0x38000000u) : 0u);
-  return __hiloint2double((int)hi, (int)(u << 29));
-}
 
 // u[b][i] = m_i - sum_r Phi_ir x_r (fp64); with sq, also sq[b][i] = sum_r Phi_ir^2.
 // One warp per row, eight loads in flight per lane; x is widened once per CTA.
