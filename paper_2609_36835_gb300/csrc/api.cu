@@ -207,6 +207,7 @@ arckv_status arckv_query_status(void* ws, void* stream) {
 // wait of the tensor-core kernels with a limit of limit_ns: the wait gives up
 // and records ARCKV_ERR_TIMEOUT in the status word, and the CTA returns.
 __global__ void wait_probe_kernel(DevStatus* stt, unsigned long long limit_ns) {
+  chain_wait();
   __shared__ uint64_t bar;
   __shared__ int abort_flag;
   if (threadIdx.x == 0) {
@@ -227,7 +228,7 @@ arckv_status arckv_wait_probe(void* ws, size_t ws_bytes, uint32_t limit_us, void
   cudaGetLastError();
   DevStatus* stt = (DevStatus*)ws;
   if (cudaMemsetAsync(stt, 0, sizeof(DevStatus), st) != cudaSuccess) return ARCKV_ERR_CUDA;
-  wait_probe_kernel<<<1, 32, 0, st>>>(stt, (unsigned long long)limit_us * 1000ull);
+  launch_chained(wait_probe_kernel, 1, 32, 0, st, stt, (unsigned long long)limit_us * 1000ull);
   if (cudaGetLastError() != cudaSuccess) return ARCKV_ERR_CUDA;
   return read_status(ws, st);
 }

@@ -20,6 +20,7 @@ namespace arckv {
 // columns zero (32 x 32 tiles).
 __global__ void __launch_bounds__(256) attend_operands_kernel(const float* Ck, const float* Cv, bf16* ck, bf16* vt,
                                                               int H, int t, int ldt, int ncopy) {
+  chain_wait();
   if ((int)blockIdx.x < ncopy) {
     const long long count = (long long)H * t * 128;
     for (long long e = 4 * ((long long)blockIdx.x * 256 + threadIdx.x); e < count; e += 4LL * ncopy * 256) {
@@ -99,6 +100,7 @@ struct TcEpiBias {
 // warp per row, 16-byte loads (the columns of the last one past t are skipped).
 __global__ void __launch_bounds__(256) row_stats_kernel(const float* X, float* shift, float* mul, long long rows, int t,
                                                         int ld) {
+  chain_wait();
   const long long row = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
@@ -184,6 +186,7 @@ __global__ void __launch_bounds__(kAvThreads, 1)
     tc::mbar_fence_init();
   }
   constexpr int kCols = kR < 32 ? 32 : kR;
+  chain_wait();
   if (warp == 1) tc::tmem_alloc(&tmem_slot, kCols);
   tc::fence_before_sync();
   __syncthreads();
@@ -325,6 +328,7 @@ __global__ void __launch_bounds__(kAvThreads, 1)
 // O = the splits' products added in order; non-finite sums are recorded.
 __global__ void __launch_bounds__(256) sum_parts_kernel(const float* P, float* O, long long count, int splits,
                                                         DevStatus* stt) {
+  chain_wait();
   bool bad = false;
   for (long long k = blockIdx.x * 256LL + threadIdx.x; k < count; k += 256LL * gridDim.x) {
     float a = P[k];
@@ -365,7 +369,7 @@ static cudaError_t launch_attend_pv(int H, int n, int t, const float* X, const f
   auto kern = attend_pv_kernel<kR>;
   const cudaError_t e = set_dyn_smem((const void*)kern, kAvSmem<kR>);
   if (e != cudaSuccess) return e;
-  kern<<<H * cdiv(n, kR) * splits, kAvThreads, kAvSmem<kR>, st>>>(mX, mV, shift, mul, O, parts, H, n, t, splits, stt);
+  launch_chained(kern, H * cdiv(n, kR) * splits, kAvThreads, kAvSmem<kR>, st, mX, mV, shift, mul, O, parts, H, n, t, splits, stt);
   return cudaGetLastError();
 }
 
@@ -381,7 +385,7 @@ int launch_attend(int H, int n, int t, float scale, const bf16* Q, const float* 
   bf16* vt = (bf16*)(ws + L.vt3);
   float* parts = (float*)(ws + L.parts);
   const int ncopy = stride_grid(htd, 4 * 256, 4);
-  attend_operands_kernel<<<ncopy + 4 * H * cdiv(ldt, 32), 256, 0, st>>>(C_k, C_v, ck, vt, H, t, ldt, ncopy);
+  launch_chained(attend_operands_kernel, ncopy + 4 * H * cdiv(ldt, 32), 256, 0, st, C_k, C_v, ck, vt, H, t, ldt, ncopy);
   {
     CUtensorMap mA, mB, mB2, mB3;
     TcEpiBias epi{};
@@ -396,7 +400,7 @@ int launch_attend(int H, int n, int t, float scale, const bf16* Q, const float* 
     if (launch_tc_gemm<128, kSplit3B>(mA, mB, mA, mB2, epi, H, n, t, 128, 128, stt, st, 0, &mB3) != cudaSuccess)
       return -1;
   }
-  row_stats_kernel<<<(unsigned)cdiv(rows, 8), 256, 0, st>>>(X, shift, mul, rows, t, ld);
+  launch_chained(row_stats_kernel, (unsigned)cdiv(rows, 8), 256, 0, st, X, shift, mul, rows, t, ld);
   // 64-row tiles where they fill the SMs, else 32-row ones, and key splits
   // (of four slabs or more) for what is still idle
   const int tiles64 = H * cdiv(n, 64), tiles32 = H * cdiv(n, 32), nk = cdiv(t, 64);
@@ -406,7 +410,7 @@ int launch_attend(int H, int n, int t, float scale, const bf16* Q, const float* 
                               : launch_attend_pv<64>(H, n, t, X, shift, mul, vt, O, parts, splits, stt, st);
   if (e != cudaSuccess) return -1;
   if (splits == 1) return 4;
-  sum_parts_kernel<<<stride_grid(rows * 128, 256, 8), 256, 0, st>>>(parts, O, rows * 128, splits, stt);
+  launch_chained(sum_parts_kernel, stride_grid(rows * 128, 256, 8), 256, 0, st, parts, O, rows * 128, splits, stt);
   return 5;
 }
 

@@ -146,6 +146,7 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
     bad = 0;
     tc::mbar_fence_init();
   }
+  chain_wait();
   if (warp == 0) tc::tmem_alloc(&tmem_slot, 128);
   tc::fence_before_sync();
   __syncthreads();
@@ -610,7 +611,7 @@ static bool chol_launch(int H, int t, float* Gram, float* Linv, float* B, float*
     }
     if (it->second < H) return false;
   }
-  chol_tc_kernel<kCL><<<kCL * H, kCT, kCholSmem, st>>>(Gram, Linv, B, Z, X, trip, t, nrhs, nrhs, bbs, ridge, (float)t,
+  launch_chained(chol_tc_kernel<kCL>, kCL * H, kCT, kCholSmem, st, Gram, Linv, B, Z, X, trip, t, nrhs, nrhs, bbs, ridge, (float)t,
                                                        stt);
   return true;
 }

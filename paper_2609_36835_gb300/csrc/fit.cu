@@ -22,6 +22,7 @@
 namespace arckv {
 
 __global__ void phi_kernel(const float* LC, const float* z, float* Phi, int n, int t, long long count) {
+  chain_wait();
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count;
        k += (long long)gridDim.x * blockDim.x) {
     const long long row = k / t;  // = b * n + i
@@ -33,6 +34,7 @@ __global__ void phi_kernel(const float* LC, const float* z, float* Phi, int n, i
 // columns; warp w sums the rows i = w, w+8, ... (four partial sums) and the
 // eight warp sums are added in warp order.
 __global__ void __launch_bounds__(1024) mass_rhs_kernel(const float* Phi, const float* m, float* rhs, int n, int t) {
+  chain_wait();
   // 32 columns per CTA, the rows split over 32 warps (four loads in flight each)
   const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int r = blockIdx.x * 32 + lane;
@@ -81,6 +83,7 @@ template <typename R, int kCL>
 __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
     chol_cluster_kernel(R* A, R* Linv, R* B, R* Z, R* X, int t, int nrhs, int ldb, long long bbs, R ridge, R tdiv,
                         DevStatus* stt) {
+  chain_wait();
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char smraw[];
   R* sm = (R*)smraw;
@@ -303,11 +306,12 @@ static int cholesky_solve64(int H, int n, double* A, double* Linv, double* B, do
                             long long bbs, double ridge, double tdiv, DevStatus* stt, cudaStream_t st) {
   const int smem = 4 * kTileF<double> * (int)sizeof(double);
   if (set_dyn_smem((const void*)chol_cluster_kernel<double, 8>, smem) != cudaSuccess) return -1;
-  chol_cluster_kernel<double, 8><<<8 * H, kCT, smem, st>>>(A, Linv, B, Z, X, n, nrhs, nrhs, bbs, ridge, tdiv, stt);
+  launch_chained(chol_cluster_kernel<double, 8>, 8 * H, kCT, smem, st, A, Linv, B, Z, X, n, nrhs, nrhs, bbs, ridge, tdiv, stt);
   return 1;
 }
 
 __global__ void beta_kernel(const float* w, float* beta, long long count, float eps_w, float b_min, float b_max) {
+  chain_wait();
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count;
        k += (long long)gridDim.x * blockDim.x) {
     const float ws = fmaxf(w[k], 0.f);
@@ -317,6 +321,7 @@ __global__ void beta_kernel(const float* w, float* beta, long long count, float 
 
 // P[row] = softmax(LC[row] + beta), one warp per row (rows = H * n).
 __global__ void softmax_bias_kernel(const float* LC, const float* beta, float* P, int n, int t) {
+  chain_wait();
   const int b = blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= n) return;
   const float* x = LC + ((long long)b * n + row) * t;
@@ -336,6 +341,7 @@ __global__ void softmax_bias_kernel(const float* LC, const float* beta, float* P
 // the transposed, K-major split-bf16 operand of the Gram GEMMs.
 __global__ void __launch_bounds__(256) transpose_split_kernel(const float* src, int rows, int cols, bf16* dst_hi,
                                                               bf16* dst_lo, int ldr) {
+  chain_wait();
   const int b = blockIdx.z, c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   __shared__ float tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -361,6 +367,7 @@ __global__ void __launch_bounds__(256) transpose_split_kernel(const float* src, 
 // (row stride ldr >= rows; the pad r in [rows, ldr) is written as zeros).
 __global__ void __launch_bounds__(256) transpose_split3_kernel(const float* src, int rows, int cols, bf16* dh, bf16* dm,
                                                                bf16* dl, int ldr) {
+  chain_wait();
   const int b = blockIdx.z, c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   __shared__ float tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -410,6 +417,7 @@ static int gram_tc(int H, int M, int N, int ldn, const bf16* Xh, const bf16* Xl,
 
 // C[b] = X X^T in fp64 (X fp32 [rows][K]); 64 x 64 lower tiles, mirrored.
 __global__ void __launch_bounds__(256) syrk64_kernel(const float* X, double* C, int rows, int K) {
+  chain_wait();
   const int b = blockIdx.z, i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
   if (j0 > i0) return;
   const float* Xb = X + (long long)b * rows * K;
@@ -453,6 +461,7 @@ __global__ void __launch_bounds__(256) syrk64_kernel(const float* X, double* C, 
 }
 
 __global__ void widen_kernel(const float* x, double* y, long long count) {
+  chain_wait();
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count;
        k += (long long)gridDim.x * blockDim.x)
     y[k] = (double)x[k];
@@ -462,6 +471,7 @@ __global__ void widen_kernel(const float* x, double* y, long long count) {
 // Y fp64 [n][ncol], out fp32 [t][ncol]); 64 x 32 output tiles.
 __global__ void __launch_bounds__(256) xty64_kernel(const float* X, const double* Y, float* out, int n, int t,
                                                     int ncol) {
+  chain_wait();
   const int b = blockIdx.z, r0 = blockIdx.x * 64, c0 = blockIdx.y * 32;
   const float* Xb = X + (long long)b * n * t;
   const double* Yb = Y + (long long)b * n * ncol;
@@ -518,6 +528,7 @@ __global__ void __launch_bounds__(256) xty64_kernel(const float* X, const double
 constexpr int kCholSlices = 5;
 
 __global__ void chol_lambda_kernel(const double* A, int n, double ridge, double tdiv, double* lam, DevStatus* stt) {
+  chain_wait();
   __shared__ double red[8];
   const int b = blockIdx.x;
   const double* Ab = A + (long long)b * n * n;
@@ -539,6 +550,7 @@ __global__ void chol_lambda_kernel(const double* A, int n, double ridge, double 
 // non-positive pivot records ARCKV_ERR_NOT_SPD.
 __global__ void __launch_bounds__(kCT, 1) chol_diag_kernel(double* A, double* Linv, int n, int k, const double* lam,
                                                            DevStatus* stt) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   df64* sm = (df64*)smraw;
   Tile<df64> S1 = (Tile<df64>)sm;
@@ -561,6 +573,7 @@ __global__ void __launch_bounds__(kCT, 1) chol_diag_kernel(double* A, double* Li
 constexpr int kBackCols = 8;
 __global__ void __launch_bounds__(256) chol_back_block_kernel(const double* Linv, const double* Y, const double* Z,
                                                               double* X, int n, int k, int nrhs, int useZ) {
+  chain_wait();
   __shared__ double Ls[NB][NB + 1];
   __shared__ double Vs[NB][kBackCols + 1];
   const int b = blockIdx.x, j0 = blockIdx.y * kBackCols, nblk = (n + NB - 1) / NB, k0 = k * NB, kb = min(NB, n - k0);
@@ -594,6 +607,7 @@ __global__ void __launch_bounds__(256) chol_back_block_kernel(const double* Linv
 constexpr int kPtThreads = 128;
 __global__ void __launch_bounds__(kPtThreads) phi_t_vec_kernel(const float* __restrict__ Phi, const double* __restrict__ a,
                                                         float* __restrict__ w, int n, int t) {
+  chain_wait();
   __shared__ float ah[1024], al[1024];
   const int b = blockIdx.y, r = blockIdx.x * kPtThreads + threadIdx.x;
   const float* p = Phi + (long long)b * n * t + min(r, t - 1);
@@ -643,6 +657,7 @@ constexpr int kTsCL = 8;
 __global__ void __cluster_dims__(kTsCL, 1, 1) __launch_bounds__(256, 1)
     tri_solve_cluster_kernel(const double* __restrict__ A, const double* __restrict__ Linv,
                              const double* __restrict__ r, double* __restrict__ yd, double* __restrict__ x, int n) {
+  chain_wait();
   namespace cg = cooperative_groups;
   __shared__ double red[kTsCL][NB];   // rank 0: the ranks' partial sums
   __shared__ double part[4][NB];
@@ -807,7 +822,7 @@ static int chol_solve_sliced(int H, int n, double* A, double* Linv, double* B, d
   // L_ik = A_ik Linv_kk^T below it and the panel's slices (on stream s)
   auto diag_panel = [&](int k, cudaStream_t s) -> bool {
     const int k0 = k * NB, kb = std::min(NB, n - k0), m = n - k0 - kb;
-    chol_diag_kernel<<<H, kCT, dsm, s>>>(A, Linv, n, k, W.lam, stt);
+    launch_chained(chol_diag_kernel, H, kCT, dsm, s, A, Linv, n, k, W.lam, stt);
     ++nl;
     if (!ok(launch_slice_rows(S, Linv + (long long)k * NB * NB, kb, kb, NB, lb, H, SB(k), EB(k), s))) return false;
     if (m > 0) {
@@ -820,7 +835,7 @@ static int chol_solve_sliced(int H, int n, double* A, double* Linv, double* B, d
     }
     return true;
   };
-  chol_lambda_kernel<<<H, 256, 0, st>>>(A, n, ridge, tdiv, W.lam, stt);
+  launch_chained(chol_lambda_kernel, H, 256, 0, st, A, n, ridge, tdiv, W.lam, stt);
   ++nl;
   if (!diag_panel(0, st)) return -1;
   for (int k = 0; k < nblk; ++k) {
@@ -860,7 +875,7 @@ static int chol_solve_sliced(int H, int n, double* A, double* Linv, double* B, d
   if (nrhs == 1) {
     // one right-hand side: both substitutions by a cluster per head (fp64,
     // n^2 multiply-adds spread over its SMs), the forward result left in W.Z
-    tri_solve_cluster_kernel<<<H * kTsCL, 256, 0, st>>>(A, Linv, B, W.Z, X, n);
+    launch_chained(tri_solve_cluster_kernel, H * kTsCL, 256, 0, st, A, Linv, B, W.Z, X, n);
     return nl + 1;
   }
   for (int k = nblk - 1; k >= 0; --k) {
@@ -874,7 +889,7 @@ static int chol_solve_sliced(int H, int n, double* A, double* Linv, double* B, d
                                 false, stt, st)))
         return -1;
     }
-    chol_back_block_kernel<<<dim3(H, cdiv(nrhs, kBackCols)), 256, 0, st>>>(Linv, B, W.Z, X, n, k, nrhs, m > 0 ? 1 : 0);
+    launch_chained(chol_back_block_kernel, dim3(H, cdiv(nrhs, kBackCols)), 256, 0, st, Linv, B, W.Z, X, n, k, nrhs, m > 0 ? 1 : 0);
     ++nl;
   }
   return nl;
@@ -907,7 +922,7 @@ static int fits_dual(const Dims& D, float ridge_w, float ridge_v, float eps_w, f
   int nl = 0;
   auto gram = [&](int S) -> int {   // B.G64 = X X^T for X = B.Phi [n][t]
     if (!sliced) {
-      syrk64_kernel<<<sgrid, 256, 0, st>>>(B.Phi, B.G64, D.n, D.t);
+      launch_chained(syrk64_kernel, sgrid, 256, 0, st, B.Phi, B.G64, D.n, D.t);
       return 1;
     }
     const int a = launch_slice_rows(S, B.Phi, D.n, D.t, D.t, nt, D.H, B.Sl, B.eR, st);
@@ -924,14 +939,14 @@ static int fits_dual(const Dims& D, float ridge_w, float ridge_v, float eps_w, f
     return cholesky_solve64(D.H, D.n, B.G64, B.L64, B.B64, B.Z64, B.X64, nrhs, nrow, ridge, D.t, stt, st);
   };
   mark(8);
-  widen_kernel<<<cdiv((long long)D.H * D.n, 256), 256, 0, st>>>(m, B.B64, (long long)D.H * D.n);
+  launch_chained(widen_kernel, cdiv((long long)D.H * D.n, 256), 256, 0, st, m, B.B64, (long long)D.H * D.n);
   r = solve(1, D.n, ridge_w);
   if (r < 0) return -1;
   nl += 1 + r;
-  phi_t_vec_kernel<<<dim3(cdiv(D.t, kPtThreads), D.H), kPtThreads, 0, st>>>(B.Phi, B.X64, B.rhs, D.n, D.t);   // w = Phi^T a
+  launch_chained(phi_t_vec_kernel, dim3(cdiv(D.t, kPtThreads), D.H), kPtThreads, 0, st, B.Phi, B.X64, B.rhs, D.n, D.t);   // w = Phi^T a
   const long long ht = (long long)D.H * D.t;
-  beta_kernel<<<cdiv(ht, 256), 256, 0, st>>>(B.rhs, beta, ht, eps_w, b_min, b_max);
-  softmax_bias_kernel<<<dim3(cdiv(D.n, 8), D.H), 256, 0, st>>>(B.LC, beta, B.Phi, D.n, D.t);
+  launch_chained(beta_kernel, cdiv(ht, 256), 256, 0, st, B.rhs, beta, ht, eps_w, b_min, b_max);
+  launch_chained(softmax_bias_kernel, dim3(cdiv(D.n, 8), D.H), 256, 0, st, B.LC, beta, B.Phi, D.n, D.t);
   nl += 3;
   // value system
   mark(9);
@@ -939,12 +954,12 @@ static int fits_dual(const Dims& D, float ridge_w, float ridge_v, float eps_w, f
   if (r < 0) return -1;
   nl += r;
   mark(10);
-  widen_kernel<<<cdiv((long long)D.H * nd, 256), 256, 0, st>>>(Y, B.B64, (long long)D.H * nd);
+  launch_chained(widen_kernel, cdiv((long long)D.H * nd, 256), 256, 0, st, Y, B.B64, (long long)D.H * nd);
   r = solve(D.d, nd, ridge_v);
   if (r < 0) return -1;
   nl += 1 + r;
   if (!sliced) {
-    xty64_kernel<<<dim3(cdiv(D.t, 64), cdiv(D.d, 32), D.H), 256, 0, st>>>(B.Phi, B.X64, C_v, D.n, D.t, D.d);
+    launch_chained(xty64_kernel, dim3(cdiv(D.t, 64), cdiv(D.d, 32), D.H), 256, 0, st, B.Phi, B.X64, C_v, D.n, D.t, D.d);
     return nl + 1;
   }
   // C_v = P^T A: the rows of P^T (columns of P) and of A^T, 4 slices each
@@ -971,6 +986,7 @@ constexpr int kIrTile = 2048;   // columns of x in shared memory at a time
 __global__ void __launch_bounds__(256) ir_rows_kernel(const float* __restrict__ Phi, const float* __restrict__ m,
                                                       const float* __restrict__ x, double* __restrict__ u,
                                                       double* __restrict__ sq, int n, int t) {
+  chain_wait();
   __shared__ double xd[kIrTile];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = blockIdx.y, row = blockIdx.x * 8 + warp;
@@ -1014,6 +1030,7 @@ __global__ void __launch_bounds__(256) ir_rows_kernel(const float* __restrict__ 
 // lam[b] = ridge * sum_i sq[b][i] / t, summed in a fixed order (one CTA per head).
 __global__ void __launch_bounds__(256) ir_lambda_kernel(const double* __restrict__ sq, double* __restrict__ lam, int n,
                                                         int t, double ridge) {
+  chain_wait();
   __shared__ double red[8];
   const int b = blockIdx.x;
   double a = 0.0;
@@ -1037,6 +1054,7 @@ __global__ void __launch_bounds__(256) ir_lambda_kernel(const double* __restrict
 __global__ void __launch_bounds__(1024) ir_cols_kernel(const float* __restrict__ Phi, const double* __restrict__ u,
                                                        const float* __restrict__ x, const double* __restrict__ lam,
                                                        float* __restrict__ r, int n, int t) {
+  chain_wait();
   __shared__ double part[32][32];
   const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
   const int w = warp & 7, q = warp >> 3;
@@ -1108,6 +1126,7 @@ __device__ __forceinline__ void st_remote(const float* p, const uint64_t* bar, i
 __global__ void __cluster_dims__(kTriCL, 1, 1) __launch_bounds__(512, 1)
     tri_solve_cluster32_kernel(const float* __restrict__ A, const float* __restrict__ Linv,
                                const float* __restrict__ r, float* __restrict__ x, int t, DevStatus* stt) {
+  chain_wait();
   extern __shared__ __align__(16) float psm[];   // two panel slices [2 nblk][4][64]
   __shared__ float yv[kTriMaxT];                 // y, then d block by block
   __shared__ float v[NB];
@@ -1269,6 +1288,7 @@ template <typename R>
 __global__ void __launch_bounds__(512) tri_solve_kernel(const R* __restrict__ A, const R* __restrict__ Linv,
                                                         const R* __restrict__ r, R* __restrict__ yd,
                                                         R* __restrict__ x, int t) {
+  chain_wait();
   constexpr int NBk = kCholNB;
   __shared__ R v[NBk];
   __shared__ R part[8][NBk];
@@ -1374,19 +1394,19 @@ static int refine_beta(const Dims& D, float ridge_w, const float* m, const FitBu
   const int nblk = cdiv(D.t, NB), smem = (2 * 2 * nblk * 256 + 256) * (int)sizeof(float);
   const bool cluster = D.t <= kTriMaxT;
   if (cluster && set_dyn_smem((const void*)tri_solve_cluster32_kernel, smem) != cudaSuccess) return -1;
-  ir_rows_kernel<<<rows, 256, 0, st>>>(B.Phi, m, B.wsol, B.ir_u, B.ir_sq, D.n, D.t);
-  ir_lambda_kernel<<<D.H, 256, 0, st>>>(B.ir_sq, B.ir_lam, D.n, D.t, (double)ridge_w);
+  launch_chained(ir_rows_kernel, rows, 256, 0, st, B.Phi, m, B.wsol, B.ir_u, B.ir_sq, D.n, D.t);
+  launch_chained(ir_lambda_kernel, D.H, 256, 0, st, B.ir_sq, B.ir_lam, D.n, D.t, (double)ridge_w);
   int nl = 2;
   for (int it = 0; it < kBetaRefineSteps; ++it) {
     if (it > 0) {
-      ir_rows_kernel<<<rows, 256, 0, st>>>(B.Phi, m, B.wsol, B.ir_u, nullptr, D.n, D.t);
+      launch_chained(ir_rows_kernel, rows, 256, 0, st, B.Phi, m, B.wsol, B.ir_u, nullptr, D.n, D.t);
       ++nl;
     }
-    ir_cols_kernel<<<dim3(cdiv(D.t, 32), D.H), 1024, 0, st>>>(B.Phi, B.ir_u, B.wsol, B.ir_lam, B.rhs, D.n, D.t);
+    launch_chained(ir_cols_kernel, dim3(cdiv(D.t, 32), D.H), 1024, 0, st, B.Phi, B.ir_u, B.wsol, B.ir_lam, B.rhs, D.n, D.t);
     if (cluster)
-      tri_solve_cluster32_kernel<<<kTriCL * D.H, 512, smem, st>>>(B.Gram, B.Linv, B.rhs, B.wsol, D.t, stt);
+      launch_chained(tri_solve_cluster32_kernel, kTriCL * D.H, 512, smem, st, B.Gram, B.Linv, B.rhs, B.wsol, D.t, stt);
     else
-      tri_solve_kernel<float><<<D.H, 512, 0, st>>>(B.Gram, B.Linv, B.rhs, B.Z, B.wsol, D.t);
+      launch_chained(tri_solve_kernel<float>, D.H, 512, 0, st, B.Gram, B.Linv, B.rhs, B.Z, B.wsol, D.t);
     nl += 2;
   }
   return nl;
@@ -1417,7 +1437,7 @@ int launch_fits(const Dims& D, float scale, float ridge_w, float ridge_v, float 
     ++nl;
   }
   const long long cnt = (long long)D.H * nt;
-  phi_kernel<<<stride_grid(cnt, 256, 16), 256, 0, st>>>(B.LC, z, B.Phi, D.n, D.t, cnt);
+  launch_chained(phi_kernel, stride_grid(cnt, 256, 16), 256, 0, st, B.LC, z, B.Phi, D.n, D.t, cnt);
   ++nl;
   if (D.t > D.n) {
     const int nd = fits_dual(D, ridge_w, ridge_v, eps_w, b_min, b_max, m, Y, B, beta, C_v, stt, st, ev);
@@ -1429,10 +1449,10 @@ int launch_fits(const Dims& D, float scale, float ridge_w, float ridge_v, float 
   // tensor-core Gram keeps every product term down to 2^-24 (kSplit3S).
   const int ldn = (D.n + 7) / 8 * 8;
   const dim3 tgrid(cdiv(D.t, 32), cdiv(ldn, 32), D.H);
-  transpose_split3_kernel<<<tgrid, 256, 0, st>>>(B.Phi, D.n, D.t, B.PT_hi, B.PT_mid, B.PT_lo, ldn);
+  launch_chained(transpose_split3_kernel, tgrid, 256, 0, st, B.Phi, D.n, D.t, B.PT_hi, B.PT_mid, B.PT_lo, ldn);
   if (gram3_tc(D.H, D.t, ldn, B.PT_hi, B.PT_mid, B.PT_lo, B.Gram, stt, st) < 0) return -1;
   nl += 2;
-  mass_rhs_kernel<<<dim3(cdiv(D.t, 32), D.H), 1024, 0, st>>>(B.Phi, m, B.rhs, D.n, D.t);
+  launch_chained(mass_rhs_kernel, dim3(cdiv(D.t, 32), D.H), 1024, 0, st, B.Phi, m, B.rhs, D.n, D.t);
   ++nl;
   mark(8);
   const int nb = launch_chol(D.H, D.t, B.Gram, B.Linv, B.rhs, B.Z, B.wsol, 1, D.t, ridge_w, B.ctrip, stt, st);
@@ -1442,15 +1462,15 @@ int launch_fits(const Dims& D, float scale, float ridge_w, float ridge_v, float 
   if (nrf < 0) return -1;
   nl += nrf;
   const long long ht = (long long)D.H * D.t;
-  beta_kernel<<<cdiv(ht, 256), 256, 0, st>>>(B.wsol, beta, ht, eps_w, b_min, b_max);
+  launch_chained(beta_kernel, cdiv(ht, 256), 256, 0, st, B.wsol, beta, ht, eps_w, b_min, b_max);
   ++nl;
   // value system: P^ over the compact keys with the fitted bias; its Gram and
   // P^T Y on the tensor cores from transposed split-bf16 operands
   mark(9);
-  softmax_bias_kernel<<<dim3(cdiv(D.n, 8), D.H), 256, 0, st>>>(B.LC, beta, B.Phi, D.n, D.t);
+  launch_chained(softmax_bias_kernel, dim3(cdiv(D.n, 8), D.H), 256, 0, st, B.LC, beta, B.Phi, D.n, D.t);
   ++nl;
-  transpose_split_kernel<<<tgrid, 256, 0, st>>>(B.Phi, D.n, D.t, B.PT_hi, B.PT_lo, ldn);
-  transpose_split_kernel<<<dim3(cdiv(D.d, 32), cdiv(ldn, 32), D.H), 256, 0, st>>>(Y, D.n, D.d, B.YT_hi, B.YT_lo,
+  launch_chained(transpose_split_kernel, tgrid, 256, 0, st, B.Phi, D.n, D.t, B.PT_hi, B.PT_lo, ldn);
+  launch_chained(transpose_split_kernel, dim3(cdiv(D.d, 32), cdiv(ldn, 32), D.H), 256, 0, st, Y, D.n, D.d, B.YT_hi, B.YT_lo,
                                                                                     ldn);
   nl += 2;
   if (gram_tc(D.H, D.t, D.t, ldn, B.PT_hi, B.PT_lo, B.PT_hi, B.PT_lo, B.Gram, D.t, stt, st) < 0) return -1;
@@ -1464,6 +1484,7 @@ int launch_fits(const Dims& D, float scale, float ridge_w, float ridge_v, float 
 }
 
 __global__ void check_finite_kernel(const float* x, long long count, DevStatus* stt) {
+  chain_wait();
   bool bad = false;
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count;
        k += (long long)gridDim.x * blockDim.x)
@@ -1472,7 +1493,7 @@ __global__ void check_finite_kernel(const float* x, long long count, DevStatus* 
 }
 
 int launch_check_finite(const float* x, long long count, DevStatus* stt, cudaStream_t st) {
-  check_finite_kernel<<<stride_grid(count, 256, 8), 256, 0, st>>>(x, count, stt);
+  launch_chained(check_finite_kernel, stride_grid(count, 256, 8), 256, 0, st, x, count, stt);
   return 1;
 }
 

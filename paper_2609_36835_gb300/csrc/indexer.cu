@@ -15,6 +15,7 @@ namespace arckv {
 // w[b][r][a] = L_x[b][a] . x_r + b_x[b][a]: one CTA per (position, head).
 __global__ void __launch_bounds__(512) index_weights_kernel(const bf16* X, const bf16* L_x, const bf16* b_x,
                                                             float* wts, int d_x, int H_I, int n_pos) {
+  chain_wait();
   // one warp per index head a: w_ra = L_x[a] . x_r + b_x[a]
   const int r = blockIdx.x, b = blockIdx.y, a = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (a >= H_I) return;
@@ -95,13 +96,14 @@ int launch_query_features(const Dims& D, const bf16* Q, const bf16* X, const bf1
   r = launch_query_proj_tc(D, Q, L_q, L_c, B.qcat, B.wcat, qbar_hi, qbar_lo, stt, st);
   if (r < 0) return -1;
   nl += r;
-  index_weights_kernel<<<dim3(D.n_pos, D.H), 32 * D.H_I, 0, st>>>(X, L_x, b_x, wts, D.d_x, D.H_I, D.n_pos);
+  launch_chained(index_weights_kernel, dim3(D.n_pos, D.H), 32 * D.H_I, 0, st, X, L_x, b_x, wts, D.d_x, D.H_I, D.n_pos);
   ++nl;
   return nl;
 }
 
 // lse[b][i] = log sum_j exp(I_ij) from the column-tile partials; one warp per row.
 __global__ void lse_reduce_kernel(const float2* part, float* lse, int n, int ntiles) {
+  chain_wait();
   const int b = blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= n) return;
   const float2* p = part + ((long long)b * n + row) * ntiles;
@@ -120,6 +122,7 @@ __global__ void lse_reduce_kernel(const float2* part, float* lse, int n, int nti
 // per thread) and the eight warp sums are added in warp order.
 __global__ void __launch_bounds__(256) pool_kernel(const float* I, const float* lse, float* s, int n, int T,
                                                    int ld) {
+  chain_wait();
   const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int j = blockIdx.x * 32 + lane;
   __shared__ float red[8][33];
@@ -156,6 +159,7 @@ __global__ void __launch_bounds__(256) pool_kernel(const float* I, const float* 
 // 4l..4l+3 (16-byte loads), warp w the rows w, w+8, ... with four rows in
 // flight, and pi^2 = e^{2 (I - lse)} = 2^(2 log2 e (I - lse)) is one MUFU op.
 __global__ void __launch_bounds__(256) pool4_kernel(const float* I, const float* lse, float* s, int n, int T) {
+  chain_wait();
   const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int j = blockIdx.x * 128 + lane * 4;
   __shared__ float4 red[8][32];
@@ -207,11 +211,11 @@ __global__ void __launch_bounds__(256) pool4_kernel(const float* I, const float*
 
 int launch_index_pool(const Dims& D, const float* I, const float2* part, int ntiles, float* lse, float* s,
                       cudaStream_t st) {
-  lse_reduce_kernel<<<dim3(cdiv(D.n, 8), D.H), 256, 0, st>>>(part, lse, D.n, ntiles);
+  launch_chained(lse_reduce_kernel, dim3(cdiv(D.n, 8), D.H), 256, 0, st, part, lse, D.n, ntiles);
   if ((D.T & 3) == 0 && (((uintptr_t)I | (uintptr_t)s) & 15u) == 0)
-    pool4_kernel<<<dim3(cdiv(D.T, 128), D.H), 256, 0, st>>>(I, lse, s, D.n, D.T);
+    launch_chained(pool4_kernel, dim3(cdiv(D.T, 128), D.H), 256, 0, st, I, lse, s, D.n, D.T);
   else
-    pool_kernel<<<dim3(cdiv(D.T, 32), D.H), 256, 0, st>>>(I, lse, s, D.n, D.T, logit_ld(D.T));
+    launch_chained(pool_kernel, dim3(cdiv(D.T, 32), D.H), 256, 0, st, I, lse, s, D.n, D.T, logit_ld(D.T));
   return 2;
 }
 

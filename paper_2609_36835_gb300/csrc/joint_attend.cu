@@ -98,6 +98,7 @@ constexpr int kJSmem = kJWarps * kJStages * kJStageBytes<TC>;
 
 template <typename TC, bool kErr>
 __global__ void __launch_bounds__(32 * kJWarps, kErr ? 2 : 3) attend_warp_kernel(const JointArgs a) {
+  chain_wait();
   extern __shared__ __align__(128) unsigned char smraw[];
   __shared__ __align__(8) uint64_t bar[kJWarps][kJStages];
   __shared__ __align__(16) float sP[kJWarps][kJKeys][kJR];
@@ -341,6 +342,7 @@ __global__ void __launch_bounds__(32 * kJWarps, kErr ? 2 : 3) attend_warp_kernel
 // O[h][i] = sum_s e^{m_s - m} Opart_s / sum_s e^{m_s - m} l_s (one warp per row, lane dims 4l..4l+3)
 __global__ void __launch_bounds__(128) attend_combine_kernel(const float* Opart, const float2* ml, int n, int nsplit,
                                                              long long rows, float* O, DevStatus* stt) {
+  chain_wait();
   const long long g = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (g >= rows) return;
@@ -376,6 +378,7 @@ __global__ void __launch_bounds__(128) attend_combine_kernel(const float* Opart,
 // T = 8192: 0.17 ms a call; one CTA per four rows over all keys took 0.88 ms.
 __global__ void __launch_bounds__(128) trunc_combine_kernel(const float* Opart, const float2* ml, int n, int nsplit,
                                                             long long rows, float eps, float* err) {
+  chain_wait();
   const long long g = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (g >= rows) return;
@@ -410,6 +413,7 @@ __global__ void __launch_bounds__(128) trunc_combine_kernel(const float* Opart, 
 
 // inS[h][j] = 1 for the anchors S[h][:] (clamped into [0, T); out-of-range entries record INVALID_ARG)
 __global__ void anchor_mask_kernel(const int* S, int t, int T, int H, unsigned char* inS, DevStatus* stt) {
+  chain_wait();
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < (long long)H * t;
        k += (long long)gridDim.x * blockDim.x) {
     const long long h = k / t;
@@ -424,6 +428,7 @@ __global__ void anchor_mask_kernel(const int* S, int t, int T, int H, unsigned c
 
 // E[h] = mean_i err[h][i] (fixed order: lane sums, then the butterfly), one warp per head
 __global__ void __launch_bounds__(32) row_mean_kernel(const float* err, int n, float* E, DevStatus* stt) {
+  chain_wait();
   const int h = blockIdx.x, lane = threadIdx.x;
   float a = 0.f;
   for (int i = lane; i < n; i += 32) a += err[(long long)h * n + i];
@@ -466,15 +471,15 @@ int launch_truncated_error(int H, int n, int T, int t, float scale, float eps, c
                            float2* ml, DevStatus* stt, cudaStream_t st) {
   cudaMemsetAsync(inS, 0, (size_t)H * T, st);
   if (t > 0)
-    anchor_mask_kernel<<<stride_grid((long long)H * t, 256, 4), 256, 0, st>>>(S, t, T, H, inS, stt);
+    launch_chained(anchor_mask_kernel, stride_grid((long long)H * t, 256, 4), 256, 0, st, S, t, T, H, inS, stt);
   const JointSplit s = trunc_split(H, n, T);
   const JointArgs a{Q, n, nullptr, nullptr, nullptr, 0, K, V, T, inS, scale, s.per_split, s.nsplit, Opart, ml, nullptr,
                     stt};
   set_dyn_smem((const void*)attend_warp_kernel<bf16, true>, kJSmem<bf16>);
-  attend_warp_kernel<bf16, true><<<dim3(s.nsplit, cdiv(n, kJR), H), 32 * kJWarps, kJSmem<bf16>, st>>>(a);
+  launch_chained(attend_warp_kernel<bf16, true>, dim3(s.nsplit, cdiv(n, kJR), H), 32 * kJWarps, kJSmem<bf16>, st, a);
   const long long rows = (long long)H * n;
-  trunc_combine_kernel<<<(unsigned)cdiv(rows, 4), 128, 0, st>>>(Opart, ml, n, s.nsplit, rows, eps, err);
-  row_mean_kernel<<<H, 32, 0, st>>>(err, n, E, stt);
+  launch_chained(trunc_combine_kernel, (unsigned)cdiv(rows, 4), 128, 0, st, Opart, ml, n, s.nsplit, rows, eps, err);
+  launch_chained(row_mean_kernel, H, 32, 0, st, err, n, E, stt);
   return t > 0 ? 4 : 3;
 }
 
@@ -486,14 +491,14 @@ int launch_attend_joint(int H, int n, int t, int F, float scale, const bf16* Q, 
   const JointArgs a{Q, n, Ck, beta, Cv, t, Kf, Vf, F, nullptr, scale, s.per_split, s.nsplit, Opart, ml, O, stt};
   if (compact_bf16 || t == 0) {
     set_dyn_smem((const void*)attend_warp_kernel<bf16, false>, kJSmem<bf16>);
-    attend_warp_kernel<bf16, false><<<grid, 32 * kJWarps, kJSmem<bf16>, st>>>(a);
+    launch_chained(attend_warp_kernel<bf16, false>, grid, 32 * kJWarps, kJSmem<bf16>, st, a);
   } else {
     set_dyn_smem((const void*)attend_warp_kernel<float, false>, kJSmem<float>);
-    attend_warp_kernel<float, false><<<grid, 32 * kJWarps, kJSmem<float>, st>>>(a);
+    launch_chained(attend_warp_kernel<float, false>, grid, 32 * kJWarps, kJSmem<float>, st, a);
   }
   if (s.nsplit == 1) return 1;
   const long long rows = (long long)H * n;
-  attend_combine_kernel<<<(unsigned)cdiv(rows, 4), 128, 0, st>>>(Opart, ml, n, s.nsplit, rows, O, stt);
+  launch_chained(attend_combine_kernel, (unsigned)cdiv(rows, 4), 128, 0, st, Opart, ml, n, s.nsplit, rows, O, stt);
   return 2;
 }
 

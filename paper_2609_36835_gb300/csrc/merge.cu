@@ -31,6 +31,7 @@ int launch_reference_attention(const Dims& D, float scale, const bf16* Q, const 
 // so anchors are already inside [0, T).  Two kernels: the anchor rows are
 // read only after every clamp has landed.
 __global__ void check_assign_range_kernel(int* kappa, int t, long long total, DevStatus* stt) {
+  chain_wait();
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total;
        k += (long long)gridDim.x * blockDim.x) {
     const int v = kappa[k];
@@ -42,6 +43,7 @@ __global__ void check_assign_range_kernel(int* kappa, int t, long long total, De
 }
 
 __global__ void check_assign_anchor_kernel(const int* kappa, const int* anchors, int T, int t, int H, DevStatus* stt) {
+  chain_wait();
   const long long ta = (long long)H * t;
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < ta;
        k += (long long)gridDim.x * blockDim.x) {
@@ -52,8 +54,8 @@ __global__ void check_assign_anchor_kernel(const int* kappa, const int* anchors,
 
 int launch_check_assign(const Dims& D, int* kappa, const int* anchors, DevStatus* stt, cudaStream_t st) {
   const long long total = (long long)D.H * D.T;
-  check_assign_range_kernel<<<stride_grid(total, 256, 8), 256, 0, st>>>(kappa, D.t, total, stt);
-  check_assign_anchor_kernel<<<stride_grid((long long)D.H * D.t, 256, 8), 256, 0, st>>>(kappa, anchors, D.T, D.t,
+  launch_chained(check_assign_range_kernel, stride_grid(total, 256, 8), 256, 0, st, kappa, D.t, total, stt);
+  launch_chained(check_assign_anchor_kernel, stride_grid((long long)D.H * D.t, 256, 8), 256, 0, st, kappa, anchors, D.T, D.t,
                                                                                      D.H, stt);
   return 2;
 }
@@ -89,6 +91,7 @@ __device__ __forceinline__ int block_excl_scan_1024_m(int v, int* sc, int& total
 // goff[r] .. goff[r+1] delimits G_r.
 __global__ void __launch_bounds__(1024) group_sort_kernel(const int* kappa, int T, int t, int* perm, int* goff,
                                                           int* cursor) {
+  chain_wait();
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int* kb = kappa + (long long)b * T;
   int* pb = perm + (long long)b * T;
@@ -138,6 +141,7 @@ __global__ void __launch_bounds__(1024) group_sort_kernel(const int* kappa, int 
 // identical to group_sort_kernel's.  cnt is [H][t][C], C = ceil(T / kSortChunk).
 __global__ void __launch_bounds__(1024) sort_hist_kernel(const int* __restrict__ kappa, int T, int t, int C,
                                                          int* __restrict__ cnt) {
+  chain_wait();
   extern __shared__ int hist[];
   const int c = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
   for (int g = tid; g < t; g += 1024) hist[g] = 0;
@@ -155,6 +159,7 @@ __global__ void __launch_bounds__(1024) sort_hist_kernel(const int* __restrict__
 // tot[b][g] = sum over chunks of cnt[b][g][.]
 __global__ void __launch_bounds__(256) sort_totals_kernel(const int* __restrict__ cnt, int t, int C, int H,
                                                           int* __restrict__ tot) {
+  chain_wait();
   const long long gi = (long long)blockIdx.x * 256 + threadIdx.x;
   if (gi >= (long long)H * t) return;
   const int* row = cnt + gi * C;
@@ -165,6 +170,7 @@ __global__ void __launch_bounds__(256) sort_totals_kernel(const int* __restrict_
 
 // goff[b] = exclusive scan of tot[b] (one CTA per head); goff[b][t] = T
 __global__ void __launch_bounds__(1024) sort_scan_kernel(const int* __restrict__ tot, int t, int* __restrict__ goff) {
+  chain_wait();
   __shared__ int sc[32];
   const int b = blockIdx.x, tid = threadIdx.x;
   const int* tb = tot + (long long)b * t;
@@ -183,6 +189,7 @@ __global__ void __launch_bounds__(1024) sort_scan_kernel(const int* __restrict__
 // cnt[b][g][c] <- the first slot of chunk c's members of group g
 __global__ void __launch_bounds__(256) sort_slots_kernel(int* __restrict__ cnt, const int* __restrict__ goff, int t,
                                                          int C, int H) {
+  chain_wait();
   const long long gi = (long long)blockIdx.x * 256 + threadIdx.x;
   if (gi >= (long long)H * t) return;
   const int b = (int)(gi / t), g = (int)(gi - (long long)b * t);
@@ -198,6 +205,7 @@ __global__ void __launch_bounds__(256) sort_slots_kernel(int* __restrict__ cnt, 
 // each chunk's positions, ascending, to their groups' slots
 __global__ void __launch_bounds__(1024) sort_scatter_kernel(const int* __restrict__ kappa, int T, int t, int C,
                                                             const int* __restrict__ cnt, int* __restrict__ perm) {
+  chain_wait();
   extern __shared__ int cur[];
   const int c = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int* cb = cnt + (long long)b * t * C + c;
@@ -235,6 +243,7 @@ constexpr int kMergeWarpMax = 128;
 __global__ void __launch_bounds__(256) group_merge_cta_kernel(const bf16* K, const int* anchors, const int* perm,
                                                               const int* goff, const float* logphi, float lambda_m,
                                                               float* C_k, int T, int t) {
+  chain_wait();
   const int b = blockIdx.y, r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int* pb = perm + (long long)b * T;
   const int* gb = goff + (long long)b * (t + 1);
@@ -309,6 +318,7 @@ __global__ void __launch_bounds__(256) group_merge_cta_kernel(const bf16* K, con
 __global__ void __launch_bounds__(256) group_merge_kernel(const bf16* K, const int* anchors, const int* perm,
                                                           const int* goff, const float* logphi, float lambda_m,
                                                           float* C_k, int T, int t) {
+  chain_wait();
   const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = blockIdx.x * 8 + warp;
   if (r >= t) return;
@@ -375,19 +385,19 @@ int launch_merge(const Dims& D, float lambda_m, const bf16* K, const int* anchor
       set_dyn_smem((const void*)sort_scatter_kernel, hsm) == cudaSuccess) {
     // cursor: the chunk counts [H][t][C], then the group totals [H][t]
     int* tot = cursor + (long long)D.H * D.t * C;
-    sort_hist_kernel<<<dim3(C, D.H), 1024, hsm, st>>>(kappa, D.T, D.t, C, cursor);
-    sort_totals_kernel<<<hb, 256, 0, st>>>(cursor, D.t, C, D.H, tot);
-    sort_scan_kernel<<<D.H, 1024, 0, st>>>(tot, D.t, goff);
-    sort_slots_kernel<<<hb, 256, 0, st>>>(cursor, goff, D.t, C, D.H);
-    sort_scatter_kernel<<<dim3(C, D.H), 1024, hsm, st>>>(kappa, D.T, D.t, C, cursor, perm);
+    launch_chained(sort_hist_kernel, dim3(C, D.H), 1024, hsm, st, kappa, D.T, D.t, C, cursor);
+    launch_chained(sort_totals_kernel, hb, 256, 0, st, cursor, D.t, C, D.H, tot);
+    launch_chained(sort_scan_kernel, D.H, 1024, 0, st, tot, D.t, goff);
+    launch_chained(sort_slots_kernel, hb, 256, 0, st, cursor, goff, D.t, C, D.H);
+    launch_chained(sort_scatter_kernel, dim3(C, D.H), 1024, hsm, st, kappa, D.T, D.t, C, cursor, perm);
     nl += 5;
   } else {
-    group_sort_kernel<<<D.H, 1024, 0, st>>>(kappa, D.T, D.t, perm, goff, cursor);
+    launch_chained(group_sort_kernel, D.H, 1024, 0, st, kappa, D.T, D.t, perm, goff, cursor);
     ++nl;
   }
-  group_merge_kernel<<<dim3(cdiv(D.t, 8), D.H), 256, 0, st>>>(K, anchors, perm, goff, logphi, lambda_m, C_k, D.T,
+  launch_chained(group_merge_kernel, dim3(cdiv(D.t, 8), D.H), 256, 0, st, K, anchors, perm, goff, logphi, lambda_m, C_k, D.T,
                                                               D.t);
-  group_merge_cta_kernel<<<dim3(D.t, D.H), 256, 0, st>>>(K, anchors, perm, goff, logphi, lambda_m, C_k, D.T, D.t);
+  launch_chained(group_merge_cta_kernel, dim3(D.t, D.H), 256, 0, st, K, anchors, perm, goff, logphi, lambda_m, C_k, D.T, D.t);
   return nl;
 }
 

@@ -41,6 +41,7 @@ constexpr int kSelE = 8;   // consecutive scores per thread per round
 
 __global__ void __launch_bounds__(1024) top_t_kernel(const float* s, int Tall, int tb, int L, int tp, int* anchors,
                                                      DevStatus* stt) {
+  chain_wait();
   const int b = blockIdx.y, c = blockIdx.x, tid = threadIdx.x;
   int cstart = 0, T = Tall, t = tb, off = 0;   // chunk start, length, budget, output offset
   if (L > 0) {
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(1024) top_t_kernel(const float* s, int Tall, i
 
 int launch_top_t(const Dims& D, int t_budget, const float* s, int* anchors, DevStatus* stt, cudaStream_t st) {
   const int nch = D.chunk > 0 ? cdiv(D.T, D.chunk) : 1;
-  top_t_kernel<<<dim3(nch, D.H), 1024, 0, st>>>(s, D.T, D.chunk > 0 ? t_budget : D.t, D.chunk, D.t, anchors, stt);
+  launch_chained(top_t_kernel, dim3(nch, D.H), 1024, 0, st, s, D.T, D.chunk > 0 ? t_budget : D.t, D.chunk, D.t, anchors, stt);
   return 1;
 }
 
@@ -133,6 +134,7 @@ int launch_top_t(const Dims& D, int t_budget, const float* s, int* anchors, DevS
 // ARCKV_ERR_INVALID_ARG and every entry is clamped to [0, T) so that later
 // kernels never index outside the cache.  One CTA per head.
 __global__ void check_anchors_kernel(int* anchors, int T, int t, DevStatus* stt) {
+  chain_wait();
   int* a = anchors + (long long)blockIdx.x * t;
   bool bad = false;
   for (int r = threadIdx.x; r < t; r += blockDim.x) {
@@ -145,13 +147,14 @@ __global__ void check_anchors_kernel(int* anchors, int T, int t, DevStatus* stt)
 }
 
 int launch_check_anchors(const Dims& D, int* anchors, DevStatus* stt, cudaStream_t st) {
-  check_anchors_kernel<<<D.H, 256, 0, st>>>(anchors, D.T, D.t, stt);
+  launch_chained(check_anchors_kernel, D.H, 256, 0, st, anchors, D.T, D.t, stt);
   return 1;
 }
 
 // Row statistics from per-tile softmax partials part[b][row][tile] = (max, sum):
 // shift = max, sum = total sum of exp(x - shift), mul = 1 / sum.  One warp per row.
 __global__ void part_stats_kernel(const float2* part, float* shift, float* mul, float* sum, int rows, int ntiles) {
+  chain_wait();
   const int b = blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= rows) return;
   const float2* p = part + ((long long)b * rows + row) * ntiles;
@@ -172,7 +175,7 @@ __global__ void part_stats_kernel(const float2* part, float* shift, float* mul, 
 
 int launch_part_stats(int H, int rows, int ntiles, const float2* part, float* shift, float* mul, float* sum,
                       cudaStream_t st) {
-  part_stats_kernel<<<dim3(cdiv(rows, 8), H), 256, 0, st>>>(part, shift, mul, sum, rows, ntiles);
+  launch_chained(part_stats_kernel, dim3(cdiv(rows, 8), H), 256, 0, st, part, shift, mul, sum, rows, ntiles);
   return 1;
 }
 

@@ -28,6 +28,7 @@ namespace arckv {
 // (0 when T = 1).  One warp per row.
 __global__ void __launch_bounds__(256) vi_row_kernel(const float* L, int n, int T, int ld, int* amax, float* z2,
                                                      float* mul2) {
+  chain_wait();
   const int b = blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= n) return;
   const long long r = (long long)b * n + row;
@@ -62,6 +63,7 @@ __global__ void __launch_bounds__(256) vi_row_kernel(const float* L, int n, int 
 __global__ void __launch_bounds__(256) vi_rowfinish_kernel(const float* z, const int* amax, const float* z2,
                                                            const float* mul2, const bf16* V, const float* Om,
                                                            const float* Y, int n, int T, float* Da, float* oo) {
+  chain_wait();
   const int b = blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= n) return;
   const long long r = (long long)b * n + row;
@@ -85,6 +87,7 @@ __global__ void __launch_bounds__(256) vi_rowfinish_kernel(const float* z, const
 
 // out[k] = ||v_k||^2 for the cache rows V [rows][128] (one warp per row)
 __global__ void __launch_bounds__(256) row_norm2_kernel(const bf16* V, long long rows, float* out) {
+  chain_wait();
   const long long k = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (k >= rows) return;
@@ -169,6 +172,7 @@ struct TcEpiVI {
 
 // s_j = (sum_r part[r][j] / n)^(1/2)
 __global__ void vi_reduce_kernel(const float* part, int nb, int n, int T, float* s) {
+  chain_wait();
   const int b = blockIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= T) return;
   float a = 0.f;
@@ -179,15 +183,15 @@ __global__ void vi_reduce_kernel(const float* part, int nb, int n, int T, float*
 int launch_vi_scores(const Dims& D, const float* L, const float* z, const float* m, const float* Y, const bf16* V,
                      const bf16* VT, const ViBufs& B, float* s, float eps, DevStatus* stt, cudaStream_t st) {
   int nl = 0;
-  vi_row_kernel<<<dim3(cdiv(D.n, 8), D.H), 256, 0, st>>>(L, D.n, D.T, logit_ld(D.T), B.amax, B.z2, B.mul2);
+  launch_chained(vi_row_kernel, dim3(cdiv(D.n, 8), D.H), 256, 0, st, L, D.n, D.T, logit_ld(D.T), B.amax, B.z2, B.mul2);
   ++nl;
   // O^(-a): softmax over the keys other than a_i, times V
   const int r = launch_probs_v_tc(D, L, B.z2, B.mul2, VT, B.Om, stt, st, B.amax);
   if (r < 0) return -1;
   nl += r;
-  vi_rowfinish_kernel<<<dim3(cdiv(D.n, 8), D.H), 256, 0, st>>>(z, B.amax, B.z2, B.mul2, V, B.Om, Y, D.n, D.T, B.Da,
+  launch_chained(vi_rowfinish_kernel, dim3(cdiv(D.n, 8), D.H), 256, 0, st, z, B.amax, B.z2, B.mul2, V, B.Om, Y, D.n, D.T, B.Da,
                                                               B.oo);
-  row_norm2_kernel<<<cdiv((long long)D.H * D.T, 8), 256, 0, st>>>(V, (long long)D.H * D.T, B.vv);
+  launch_chained(row_norm2_kernel, cdiv((long long)D.H * D.T, 8), 256, 0, st, V, (long long)D.H * D.T, B.vv);
   nl += 2;
   nl += launch_split3(Y, B.y_h, B.y_m, B.y_l, (long long)D.H * D.n * 128, st);
   CUtensorMap mA, mA2, mA3, mB;
@@ -198,7 +202,7 @@ int launch_vi_scores(const Dims& D, const float* L, const float* z, const float*
   TcEpiVI epi{L, z, m, B.amax, B.Da, B.oo, B.vv, B.colpart, D.n, D.T, logit_ld(D.T), nb, eps};
   if (launch_tc_gemm<128, kSplit3A>(mA, mB, mA2, mA, epi, D.H, D.n, D.T, 128, 128, stt, st, 0, &mA3) != cudaSuccess)
     return -1;
-  vi_reduce_kernel<<<dim3(cdiv(D.T, 256), D.H), 256, 0, st>>>(B.colpart, nb, D.n, D.T, s);
+  launch_chained(vi_reduce_kernel, dim3(cdiv(D.T, 256), D.H), 256, 0, st, B.colpart, nb, D.n, D.T, s);
   return nl + 2;
 }
 

@@ -106,6 +106,7 @@ struct ProfileOut {
 // e^x is taken as 2^(x log2 e) after the subtraction.
 __global__ void __launch_bounds__(512) col_profiles_kernel(const float* L, float* logphi, ProfileOut po, int n, int T,
                                                            int ld, int ldn) {
+  chain_wait();
   const int b = blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int j0 = blockIdx.x * 32, j = j0 + lane;
   __shared__ float red[3][16][32];
@@ -204,6 +205,7 @@ template <int W>
 __global__ void __launch_bounds__(512) col_profiles_tma_kernel(const __grid_constant__ CUtensorMap mL, float* logphi,
                                                                ProfileOut po, int n, int T, int ldn, int nbox,
                                                                DevStatus* stt) {
+  chain_wait();
   constexpr int PH = 512 / W;   // row phases
   extern __shared__ uint8_t smem_raw[];
   const uint32_t r0 = tc::smem_u32(smem_raw);
@@ -334,7 +336,7 @@ static int launch_col_profiles_tma(const Dims& D, const float* L, float* logphi,
   if (set_dyn_smem((const void*)col_profiles_tma_kernel<W>, smem) !=
       cudaSuccess)
     return -1;
-  col_profiles_tma_kernel<W><<<dim3(cdiv(D.T, W), D.H), 512, smem, st>>>(m, logphi, po, D.n, D.T, ldn, nbox, stt);
+  launch_chained(col_profiles_tma_kernel<W>, dim3(cdiv(D.T, W), D.H), 512, smem, st, m, logphi, po, D.n, D.T, ldn, nbox, stt);
   return 1;
 }
 
@@ -354,7 +356,7 @@ static int col_profiles(const Dims& D, const float* L, float* logphi, const Prof
   if (smem > 0 && set_dyn_smem((const void*)col_profiles_kernel, smem) !=
                       cudaSuccess)
     return -1;
-  col_profiles_kernel<<<dim3(cdiv(D.T, 32), D.H), 512, smem, st>>>(L, logphi, po, D.n, D.T, logit_ld(D.T), ldn);
+  launch_chained(col_profiles_kernel, dim3(cdiv(D.T, 32), D.H), 512, smem, st, L, logphi, po, D.n, D.T, logit_ld(D.T), ldn);
   return 1;
 }
 
@@ -366,6 +368,7 @@ int launch_col_profiles(const Dims& D, const float* L, float* logphi, DevStatus*
 // (rows c < T - t of head b; kmap gives the key)
 __global__ void decode_assign_kernel2(const unsigned long long* best, const int* kmap, int* kappa, int T, int Tm,
                                       long long count) {
+  chain_wait();
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count;
        k += (long long)gridDim.x * blockDim.x) {
     const long long b = k / Tm, o = b * T + (k - b * Tm);
@@ -376,6 +379,7 @@ __global__ void decode_assign_kernel2(const unsigned long long* best, const int*
 }
 
 __global__ void anchor_self_assign_kernel2(const int* anchors, int* kappa, int T, int t, int H) {
+  chain_wait();
   const long long total = (long long)H * t;
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total;
        k += (long long)gridDim.x * blockDim.x) {
@@ -421,10 +425,10 @@ int launch_assign_gemm(const Dims& D, const int* anchors, const bf16* Ut_hi, con
         cudaSuccess)
       return -1;
     const long long cnt = (long long)D.H * Tm;
-    decode_assign_kernel2<<<stride_grid(cnt, 256, 8), 256, 0, st>>>(best, kmap, kappa, D.T, Tm, cnt);
+    launch_chained(decode_assign_kernel2, stride_grid(cnt, 256, 8), 256, 0, st, best, kmap, kappa, D.T, Tm, cnt);
     nl += 2;
   }
-  anchor_self_assign_kernel2<<<cdiv((long long)D.H * D.t, 256), 256, 0, st>>>(anchors, kappa, D.T, D.t, D.H);
+  launch_chained(anchor_self_assign_kernel2, cdiv((long long)D.H * D.t, 256), 256, 0, st, anchors, kappa, D.T, D.t, D.H);
   return nl;
 }
 

@@ -14,6 +14,7 @@
 namespace arckv {
 
 __global__ void split3_kernel(const float* x, bf16* h, bf16* m, bf16* l, long long count) {
+  chain_wait();
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count;
        k += (long long)gridDim.x * blockDim.x)
     split3_bf16(x[k], h[k], m[k], l[k]);
@@ -21,6 +22,7 @@ __global__ void split3_kernel(const float* x, bf16* h, bf16* m, bf16* l, long lo
 
 // VT[b][d][j] = V[b][j][d] (bf16), zero for T <= j < ldT.
 __global__ void __launch_bounds__(256) transpose_v_kernel(const bf16* V, bf16* VT, int T, int ldT) {
+  chain_wait();
   const int b = blockIdx.z, j0 = blockIdx.x * 32, d0 = blockIdx.y * 32;
   __shared__ bf16 tile[32][34];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -49,13 +51,13 @@ int launch_value_logits_tc(const Dims& D, const bf16* q_h, const bf16* q_m, cons
 }
 
 int launch_split3(const float* x, bf16* h, bf16* m, bf16* l, long long count, cudaStream_t st) {
-  split3_kernel<<<stride_grid(count, 256, 8), 256, 0, st>>>(x, h, m, l, count);
+  launch_chained(split3_kernel, stride_grid(count, 256, 8), 256, 0, st, x, h, m, l, count);
   return 1;
 }
 
 int launch_transpose_v(const Dims& D, const bf16* V, bf16* VT, cudaStream_t st) {
   const int ldT = (D.T + 7) / 8 * 8;
-  transpose_v_kernel<<<dim3(cdiv(ldT, 32), 4, D.H), 256, 0, st>>>(V, VT, D.T, ldT);
+  launch_chained(transpose_v_kernel, dim3(cdiv(ldT, 32), 4, D.H), 256, 0, st, V, VT, D.T, ldT);
   return 1;
 }
 
@@ -124,6 +126,7 @@ __global__ void __launch_bounds__(kPvThreads, 1)
     abort_flag = 0;
     tc::mbar_fence_init();
   }
+  chain_wait();
   if (warp == 1) tc::tmem_alloc(&tmem_slot, 128);
   tc::fence_before_sync();
   __syncthreads();
@@ -287,7 +290,7 @@ static cudaError_t launch_probs_v_rows(const Dims& D, const float* X, const floa
                    : (odd ? probs_v_kernel<false, true, kRows> : probs_v_kernel<false, false, kRows>);
   const cudaError_t e = set_dyn_smem((const void*)kern, kPvSmem);
   if (e != cudaSuccess) return e;
-  kern<<<D.H * cdiv(D.n, kRows) * splits, kPvThreads, kPvSmem, st>>>(mX, mVT, shift, mul, skip, out, D.n, D.T, splits,
+  launch_chained(kern, D.H * cdiv(D.n, kRows) * splits, kPvThreads, kPvSmem, st, mX, mVT, shift, mul, skip, out, D.n, D.T, splits,
                                                                      stt);
   return cudaGetLastError();
 }

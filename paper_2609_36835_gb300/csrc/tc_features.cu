@@ -104,12 +104,14 @@ int launch_key_features_tc(const Dims& D, const bf16* K, const bf16* V, const bf
 // and one plain GEMM gives L_q q + L_c (c_h + c_m + c_l) with exact bf16 products.
 // The c triple is written into A by the GEMM that forms c; qcat_kernel adds q.
 __global__ void __launch_bounds__(256) qcat_kernel(const bf16* Q, bf16* A, int n) {
+  chain_wait();
   const int b = blockIdx.y, i = blockIdx.x * 16 + (threadIdx.x >> 4), k = (threadIdx.x & 15) * 8;
   if (i >= n) return;
   const long long r = (long long)b * n + i;
   *(uint4*)(A + r * 512 + k) = *(const uint4*)(Q + r * 128 + k);
 }
 __global__ void __launch_bounds__(256) wcat_kernel(const bf16* L_q, const bf16* L_c, bf16* W, long long rows) {
+  chain_wait();
   const long long r = blockIdx.x * 2ll + (threadIdx.x >> 7);
   const int k = threadIdx.x & 127;
   if (r >= rows) return;
@@ -123,9 +125,9 @@ __global__ void __launch_bounds__(256) wcat_kernel(const bf16* L_q, const bf16* 
 
 int launch_query_proj_tc(const Dims& D, const bf16* Q, const bf16* L_q, const bf16* L_c, bf16* qcat, bf16* wcat,
                          bf16* qbar_hi, bf16* qbar_lo, DevStatus* stt, cudaStream_t st) {
-  qcat_kernel<<<dim3(cdiv(D.n, 16), D.H), 256, 0, st>>>(Q, qcat, D.n);
+  launch_chained(qcat_kernel, dim3(cdiv(D.n, 16), D.H), 256, 0, st, Q, qcat, D.n);
   const long long wrows = (long long)D.H * D.HD;
-  wcat_kernel<<<(unsigned)cdiv(wrows, 2), 256, 0, st>>>(L_q, L_c, wcat, wrows);
+  launch_chained(wcat_kernel, (unsigned)cdiv(wrows, 2), 256, 0, st, L_q, L_c, wcat, wrows);
   CUtensorMap mA, mB;
   if (!encode_bf16_map_3d(&mA, qcat, 512, D.n, D.H, 128) || !encode_bf16_map_3d(&mB, wcat, 512, D.HD, D.H, 128))
     return -1;

@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
     abort_flag = 0;
     tc::mbar_fence_init();
   }
+  chain_wait();
   if (warp == 1) tc::tmem_alloc(&tmem_slot, C::TMEM_COLS);
   tc::fence_before_sync();
   __syncthreads();
@@ -365,7 +366,7 @@ inline cudaError_t launch_tc_gemm(const CUtensorMap& mA, const CUtensorMap& mB, 
   if (e != cudaSuccess) return e;
   const long long ntiles = (long long)cdiv(N, BN) * cdiv(M, 128) * H;
   const int grid = (int)std::min<long long>(ntiles, tc_gemm_sm_count());
-  kern<<<grid, 64 + 32 * NE, smem, st>>>(mA, mB, mA2, mB2, mA3 ? *mA3 : mA, epi, H, M, N, K, chunk_k, K1, stt,
+  launch_chained(kern, grid, 64 + 32 * NE, smem, st, mA, mB, mA2, mB2, mA3 ? *mA3 : mA, epi, H, M, N, K, chunk_k, K1, stt,
                                          col_group);
   return cudaGetLastError();
 }

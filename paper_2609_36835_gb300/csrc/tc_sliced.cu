@@ -266,6 +266,7 @@ __global__ void __launch_bounds__(SlShape<BN>::THREADS, 1)
   }
   // TMEM: exact levels 2..4 of two alternating chunks at columns (buf * 3 + lvl) * 64,
   // the levels above 4 of two alternating tiles at columns 384 + 64 (tile & 1)
+  chain_wait();
   if (warp == 1) tc::tmem_alloc(&tmem_slot, 512);
   tc::fence_before_sync();
   __syncthreads();
@@ -547,6 +548,7 @@ template <int S, typename T>
 __global__ void __launch_bounds__(256) slice_rows_kernel(const T* __restrict__ X, int R, int K, int ldx, long long xbs,
                                                          int H, bf16* __restrict__ out, int ldo,
                                                          int* __restrict__ ex) {
+  chain_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long gr = (long long)blockIdx.x * 8 + warp;   // row over all batches
   if (gr >= (long long)H * R) return;
@@ -598,6 +600,7 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(const T* __restrict__ X
 template <typename T>
 __global__ void __launch_bounds__(1024) col_exp_kernel(const T* __restrict__ X, int K, int R, int ldx, long long xbs,
                                                        int* __restrict__ ex) {
+  chain_wait();
   __shared__ unsigned long long part[32][33];
   const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = blockIdx.x * 32 + lane;
   const T* x = X + (long long)b * xbs + r;
@@ -629,6 +632,7 @@ template <int S, typename T>
 __global__ void __launch_bounds__(256) slice_cols_kernel(const T* __restrict__ X, int K, int R, int ldx, long long xbs,
                                                          int H, const int* __restrict__ ex, bf16* __restrict__ out,
                                                          int ldo) {
+  chain_wait();
   const int b = blockIdx.z, r0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
   __shared__ T tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -679,7 +683,7 @@ int launch_sliced(const bf16* As, const int* eA, int M, const bf16* Bs, const in
   if (per == 0) return 0;   // no tile in the column range
   int grid = (int)std::min<long long>(per * H, tc_gemm_sm_count());
   if (max_ctas > 0) grid = std::min(grid, max_ctas);
-  kern<<<grid, Sh::THREADS, C::SMEM, st>>>(mA, mB, out, eA, eB, H, M, N, K, lower ? 1 : 0, nt0, nt1, stt);
+  launch_chained(kern, grid, Sh::THREADS, C::SMEM, st, mA, mB, out, eA, eB, H, M, N, K, lower ? 1 : 0, nt0, nt1, stt);
   const cudaError_t el = cudaGetLastError();
   if (el != cudaSuccess) g_sliced_fail = 1000 + (int)el;
   return el == cudaSuccess ? 1 : -1;
@@ -698,11 +702,11 @@ static int slice_rows_t(int S, const T* X, int R, int K, int ldx, long long xbs,
                         cudaStream_t st) {
   const int grid = cdiv((long long)H * R, 8), ldo = (int)sliced_ld(K);
   if (S == 3)
-    slice_rows_kernel<3, T><<<grid, 256, 0, st>>>(X, R, K, ldx, xbs, H, out, ldo, ex);
+    launch_chained(slice_rows_kernel<3, T>, grid, 256, 0, st, X, R, K, ldx, xbs, H, out, ldo, ex);
   else if (S == 4)
-    slice_rows_kernel<4, T><<<grid, 256, 0, st>>>(X, R, K, ldx, xbs, H, out, ldo, ex);
+    launch_chained(slice_rows_kernel<4, T>, grid, 256, 0, st, X, R, K, ldx, xbs, H, out, ldo, ex);
   else if (S == 5)
-    slice_rows_kernel<5, T><<<grid, 256, 0, st>>>(X, R, K, ldx, xbs, H, out, ldo, ex);
+    launch_chained(slice_rows_kernel<5, T>, grid, 256, 0, st, X, R, K, ldx, xbs, H, out, ldo, ex);
   else
     return -1;
   return 1;
@@ -722,14 +726,14 @@ template <typename T>
 static int slice_cols_t(int S, const T* X, int K, int R, int ldx, long long xbs, int H, bf16* out, int* ex,
                         cudaStream_t st) {
   const int ldo = (int)sliced_ld(K);
-  col_exp_kernel<T><<<dim3(cdiv(R, 32), H), 1024, 0, st>>>(X, K, R, ldx, xbs, ex);
+  launch_chained(col_exp_kernel<T>, dim3(cdiv(R, 32), H), 1024, 0, st, X, K, R, ldx, xbs, ex);
   const dim3 grid(cdiv(R, 32), cdiv(K, 32), H);
   if (S == 3)
-    slice_cols_kernel<3, T><<<grid, 256, 0, st>>>(X, K, R, ldx, xbs, H, ex, out, ldo);
+    launch_chained(slice_cols_kernel<3, T>, grid, 256, 0, st, X, K, R, ldx, xbs, H, ex, out, ldo);
   else if (S == 4)
-    slice_cols_kernel<4, T><<<grid, 256, 0, st>>>(X, K, R, ldx, xbs, H, ex, out, ldo);
+    launch_chained(slice_cols_kernel<4, T>, grid, 256, 0, st, X, K, R, ldx, xbs, H, ex, out, ldo);
   else if (S == 5)
-    slice_cols_kernel<5, T><<<grid, 256, 0, st>>>(X, K, R, ldx, xbs, H, ex, out, ldo);
+    launch_chained(slice_cols_kernel<5, T>, grid, 256, 0, st, X, K, R, ldx, xbs, H, ex, out, ldo);
   else
     return -1;
   return 2;
