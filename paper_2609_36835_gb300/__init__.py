@@ -156,16 +156,26 @@ def attend_workspace_bytes(H_kv: int, n: int, t: int, d: int = 128) -> int:
     return int(load_library().arckv_attend_workspace_bytes(H_kv, n, t, d))
 
 
+# The helpers below run between a caller's arguments and a few tens of
+# microseconds of kernels, so their passing paths are kept short.
+
 def _ptr(x) -> Optional[int]:
-    if x is None:
-        return None
-    if isinstance(x, int):
+    if x is None or isinstance(x, int):
         return x
     if not x.is_contiguous():
         # the C ABI takes dense row-major arrays; a strided view would be read with the wrong layout
         raise ValueError("arckv: tensor arguments must be contiguous (row-major); got strides %s"
                          % (tuple(x.stride()),))
     return x.data_ptr()
+
+
+def _fits(got, want) -> bool:
+    if len(got) != len(want):
+        return False
+    for g, w in zip(got, want):
+        if w is not None and g != w:
+            return False
+    return True
 
 
 def _expect(name: str, x, dtypes, shape=None):
@@ -176,8 +186,7 @@ def _expect(name: str, x, dtypes, shape=None):
         raise ValueError("arckv: %s must be a torch tensor" % name)
     if x.dtype not in dtypes:
         raise ValueError("arckv: %s must be %s, got %s" % (name, " or ".join(map(str, dtypes)), x.dtype))
-    if shape is not None and (x.dim() != len(shape) or
-                              any(w is not None and int(g) != int(w) for g, w in zip(x.shape, shape))):
+    if shape is not None and not _fits(x.shape, shape):
         raise ValueError("arckv: %s must have shape %s, got %s" % (
             name, tuple("*" if w is None else w for w in shape), tuple(x.shape)))
     if not x.is_contiguous():
@@ -191,17 +200,19 @@ def _on_one_cuda_device(**tensors):
     for name, x in tensors.items():
         if x is None:
             continue
-        if x.device.type != "cuda":
+        if not x.is_cuda:
             raise ValueError("arckv: %s must be on a CUDA device, got %s (there is no CPU path)" % (name, x.device))
-        if dev is not None and x.device != dev:
-            raise ValueError("arckv: %s is on %s but the other arguments on %s" % (name, x.device, dev))
-        dev = x.device
+        i = x.get_device()
+        if dev is not None and i != dev:
+            raise ValueError("arckv: %s is on %s but the other arguments on cuda:%d" % (name, x.device, dev))
+        dev = i
 
 
 def _stream_handle(stream) -> Optional[int]:
     if stream is None:
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        # the current stream's handle without the Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
