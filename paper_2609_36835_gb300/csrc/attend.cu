@@ -3,7 +3,7 @@
 //                                  C_k (kSplit3B), beta added in the epilogue;
 //   O = softmax(X) C_v             attend_pv_kernel: the probabilities formed on
 //                                  the fly as a bf16 triple against the triple
-//                                  of C_v, nine products (fp32-grade).
+//                                  of C_v, eight products (fp32-grade).
 // Four launches (a fifth sums key splits): the operands' split, X, its row
 // statistics, the products.  8 heads, n = 1024, t = 819: 51 us of kernels (5 + 12
 // + 10 + 24); 207 before, with beta and the statistics in a pass of 58 us and the
@@ -137,8 +137,10 @@ __global__ void __launch_bounds__(256) row_stats_kernel(const float* X, float* s
 // O = P C_v with P = exp(X - shift) mul formed on the fly.  CTA = (kR query
 // rows, key split): TMA streams kR x 64 slabs of X into a raw ring; sixteen
 // converter warps form P and its bf16 triple in the K-major layout of an MMA
-// operand; per 16-wide K step one thread issues the nine products of the two
-// triples, D [128 dims x kR rows] += C_v^T P^T -- the value side as M, so that
+// operand; per 16-wide K step one thread issues the products of the two
+// triples (all but l l, 2^-32 of the result), D [128 dims x kR rows] += C_v^T
+// P^T: h h into one accumulator, the others, at most 2^-8 of it, into a second,
+// so that the leading sum is rounded once per step.  The value side is M, so that
 // a short row tile makes a narrow MMA instead of an idle half.  The products
 // are bound by operand bytes (6 KB of shared memory per MMA at kR = 64), a CTA
 // by them and the conversion about alike.
@@ -185,7 +187,7 @@ __global__ void __launch_bounds__(kAvThreads, 1)
     abort_flag = 0;
     tc::mbar_fence_init();
   }
-  constexpr int kCols = kR < 32 ? 32 : kR;
+  constexpr int kCols = 2 * kR;
   chain_wait();
   if (warp == 1) tc::tmem_alloc(&tmem_slot, kCols);
   tc::fence_before_sync();
@@ -240,8 +242,10 @@ __global__ void __launch_bounds__(kAvThreads, 1)
           for (int i = 0; i < 3; ++i)
 #pragma unroll
             for (int j = 0; j < 3; ++j)
-              tc::mma_f16(tmem, tc::sdesc_k128(v + i * kAvVTile + ks * 32), tc::sdesc_k128(p + j * kR * 128 + ks * 32),
-                          idesc, (g > 0 || ks > 0 || i > 0 || j > 0) ? 1u : 0u);
+              if (i + j < 4)
+                tc::mma_f16(tmem + (i + j > 0 ? kR : 0), tc::sdesc_k128(v + i * kAvVTile + ks * 32),
+                            tc::sdesc_k128(p + j * kR * 128 + ks * 32), idesc,
+                            (g > 0 || ks > 0 || i + j > 1 || (i == 1 && j == 0)) ? 1u : 0u);
         tc::mma_commit(&oempty[s]);
       }
       if (ok) tc::mma_commit(&accf);
@@ -303,15 +307,17 @@ __global__ void __launch_bounds__(kAvThreads, 1)
       tc::fence_after_sync();
       bool bad = false;
       for (int g16 = cg * 16; g16 < kR; g16 += 64) {
-        float v[16];
+        float v[16], u[16];
         tc::tmem_ld16(tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)g16, v);
+        tc::tmem_ld16(tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(kR + g16), u);
         float* d = (splits > 1 ? parts + (long long)sp * H * rows * 128 : O) + ((long long)b * rows + m0 + g16) * 128 +
                    qd * 32 + lane;
 #pragma unroll
         for (int e = 0; e < 16; ++e)
           if (m0 + g16 + e < rows) {
-            d[e * 128] = v[e];
-            bad |= !isfinite(v[e]);
+            const float o = v[e] + u[e];
+            d[e * 128] = o;
+            bad |= !isfinite(o);
           }
       }
       if (bad) set_status(stt, ARCKV_ERR_NONFINITE);
