@@ -235,10 +235,15 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      constexpr uint32_t idesc = tc::idesc_bf16_f32(BN);
       bool ok = true;
       int g = 0, cg = 0;   // K slabs and chunks consumed by this CTA, across tiles
       for (int tl = blockIdx.x; tl < ntiles && ok; tl += gridDim.x) {
+        // the last column tile is as wide as the matrix needs (819 columns in
+        // tiles of 256 are 3.2 tiles of MMA time, not 4); the accumulator's
+        // columns past N keep what they held, which no epilogue uses
+        int tb, tm0, tn0;
+        tile_coords(tl, tb, tm0, tn0);
+        const uint32_t idesc = tc::idesc_bf16_f32(min(BN, (N - tn0 + 15) & ~15));
         for (int c = 0; c < nchunks && ok; ++c, ++cg) {
           const int buf = cg & 1;
           if (cg >= 2 && !tc::mbar_wait(&acce[buf], ((cg >> 1) - 1) & 1, abortp, stt)) {
