@@ -358,12 +358,16 @@ arckv_status arckv_compact(const arckv_config* cfg, const void* K, const void* V
   int* kappa = I32(L.kappa);
   mark(4);
   if (!given_assign) {
+    // the filter's bounds and lists go over the index features, which are done
+    const bool filtered = assign_filtered(D);
+    float2* fb = filtered ? (float2*)(w + L.kbar_hi) : nullptr;
+    char* fs = filtered ? w + L.kbar_lo : nullptr;
     const int nla = launch_assign_prep(D, F(L.NT), F(L.logphi), anchors, B16(L.Ut_hi), B16(L.Ut_lo), B16(L.S_hi),
-                                       B16(L.S_lo), I32(L.kmap), stt, st);
+                                       B16(L.S_lo), I32(L.kmap), fs, stt, st);
     if (nla < 0) return ARCKV_ERR_CUDA;
     mark(5);
     const int nlg = launch_assign_gemm(D, anchors, B16(L.Ut_hi), B16(L.Ut_lo), B16(L.S_hi), B16(L.S_lo),
-                                       I32(L.kmap), (unsigned long long*)(w + L.best), kappa, stt, st);
+                                       I32(L.kmap), (unsigned long long*)(w + L.best), kappa, fb, fs, stt, st);
     if (nlg < 0) return ARCKV_ERR_CUDA;
     nl += nla + nlg;
   } else {

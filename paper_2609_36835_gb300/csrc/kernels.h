@@ -122,10 +122,14 @@ int launch_col_profiles(const Dims& D, const float* L, float* logphi, DevStatus*
 // then the argmax GEMM over the compacted rows (the anchors' own kappa(s_r) = r
 // is set directly).
 int launch_assign_prep(const Dims& D, const float* L, float* logphi, const int* anchors, bf16* Ut_hi, bf16* Ut_lo,
-                       bf16* S_hi, bf16* S_lo, int* kmap, DevStatus* stt, cudaStream_t st);
+                       bf16* S_hi, bf16* S_lo, int* kmap, char* filter_scratch, DevStatus* stt, cudaStream_t st);
 int launch_assign_gemm(const Dims& D, const int* anchors, const bf16* Ut_hi, const bf16* Ut_lo, const bf16* S_hi,
-                       const bf16* S_lo, const int* kmap, unsigned long long* best, int* kappa, DevStatus* stt,
-                       cudaStream_t st);
+                       const bf16* S_lo, const int* kmap, unsigned long long* best, int* kappa, float2* filter_bounds,
+                       char* filter_scratch, DevStatus* stt, cudaStream_t st);
+// Whether the assignment runs in two passes (one product per pair, then split
+// products where they can decide); then filter_bounds and filter_scratch of both
+// calls are buffers of H T HD bf16 each, else null.
+bool assign_filtered(const Dims& D);
 int launch_check_assign(const Dims& D, int* kappa, const int* anchors, DevStatus* stt, cudaStream_t st);
 // The counting sort of the merge runs over chunks of kSortChunk positions
 // when a group histogram fits shared memory; its scratch (`cursor`) then

@@ -90,7 +90,18 @@ struct ProfileOut {
   int* kmap;           // [H][T]: key of compacted row c (c < T - t)
   const int* anchors;  // [H][t]
   int t;
+  // filter (nullable): upper bounds of ||u - bf16(u)|| of the key rows [H][T]
+  // (compacted like Ut) and of the anchor rows [H][ldr]
+  float *rho_k, *rho_s;
+  int ldr;
 };
+
+// The bound of one profile row (output offset ro) from its residual's sum of squares.
+__device__ __forceinline__ void write_rho(const ProfileOut& po, int b, int T, int ldn, long long ro, float sq) {
+  const float r = sqrtf(sq) * 1.001f;   // (the fp32 sum of squares is good to 1e-4)
+  if (ro >= 0) po.rho_k[(long long)b * T + (ro / ldn - (long long)b * T)] = r;
+  else po.rho_s[(long long)b * po.ldr + ((-1 - ro) / ldn - (long long)b * po.t)] = r;
+}
 
 // Column statistics of the reference logits and the transposed response
 // profiles (Sec. 3.4, Eq. response_profile), one CTA per (32 columns, head):
@@ -169,6 +180,7 @@ __global__ void __launch_bounds__(512) col_profiles_kernel(const float* L, float
   __syncthreads();
   if (po.Ut_hi == nullptr) return;
   const float cm = cstat[0][lane], ci = cstat[1][lane];
+  float rsq[2] = {0.f, 0.f};
   for (int i0 = 0; i0 < ldn; i0 += 64) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -184,6 +196,8 @@ __global__ void __launch_bounds__(512) col_profiles_kernel(const float* L, float
         bf16 h0, l0, h1, l1;
         split_bf16(tile[2 * lane][c], h0, l0);
         split_bf16(tile[2 * lane + 1][c], h1, l1);
+        const float e0 = tile[2 * lane][c] - __bfloat162float(h0), e1 = tile[2 * lane + 1][c] - __bfloat162float(h1);
+        rsq[c & 1] = fmaf(e0, e0, fmaf(e1, e1, rsq[c & 1]));
         const long long ro = orow[c];
         bf16* dh = ro >= 0 ? po.Ut_hi + ro : po.S_hi + (-1 - ro);
         bf16* dl = ro >= 0 ? po.Ut_lo + ro : po.S_lo + (-1 - ro);
@@ -192,6 +206,14 @@ __global__ void __launch_bounds__(512) col_profiles_kernel(const float* L, float
       }
     }
     __syncthreads();
+  }
+  if (po.rho_k != nullptr) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float sq = warp_sum(rsq[k]);
+      const int c = 2 * w + k;
+      if (lane == 0 && j0 + c < T && orow[c] != kNoRow) write_rho(po, b, T, ldn, orow[c], sq);
+    }
   }
 }
 
@@ -302,6 +324,7 @@ __global__ void __launch_bounds__(512) col_profiles_tma_kernel(const __grid_cons
   // pass 3: U_ij = e_ij invN_j, transposed through a padded tile 64 rows at a time
   constexpr int RPT = (64 + PH - 1) / PH;   // tile rows per thread: rows ph + k PH below 64
   const float inv = cstat[1][c];
+  float rsq = 0.f;   // of column `warp` (W <= 16: one column per warp)
   for (int i0 = 0; i0 < ldn; i0 += 64) {
 #pragma unroll
     for (int k = 0; k < RPT; ++k) {
@@ -316,6 +339,7 @@ __global__ void __launch_bounds__(512) col_profiles_tma_kernel(const __grid_cons
         const float x0 = tile[2 * lane][cc], x1 = tile[2 * lane + 1][cc];
         const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
         const float2 hf = __bfloat1622float2(h);
+        rsq = fmaf(x0 - hf.x, x0 - hf.x, fmaf(x1 - hf.y, x1 - hf.y, rsq));
         const long long ro = orow[cc];
         bf16* dh = ro >= 0 ? po.Ut_hi + ro : po.S_hi + (-1 - ro);
         bf16* dl = ro >= 0 ? po.Ut_lo + ro : po.S_lo + (-1 - ro);
@@ -324,6 +348,11 @@ __global__ void __launch_bounds__(512) col_profiles_tma_kernel(const __grid_cons
       }
     }
     __syncthreads();
+  }
+  static_assert(W <= 16, "one column per warp");
+  if (po.rho_k != nullptr && warp < W) {
+    rsq = warp_sum(rsq);
+    if (lane == 0 && j0 + warp < T && orow[warp] != kNoRow) write_rho(po, b, T, ldn, orow[warp], rsq);
   }
 }
 
@@ -361,7 +390,7 @@ static int col_profiles(const Dims& D, const float* L, float* logphi, const Prof
 }
 
 int launch_col_profiles(const Dims& D, const float* L, float* logphi, DevStatus* stt, cudaStream_t st) {
-  return col_profiles(D, L, logphi, ProfileOut{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, D.t}, stt, st);
+  return col_profiles(D, L, logphi, ProfileOut{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, D.t, nullptr, nullptr, 0}, stt, st);
 }
 
 // kappa of the non-anchor keys from the argmax of their compacted rows
@@ -388,14 +417,420 @@ __global__ void anchor_self_assign_kernel2(const int* anchors, int* kappa, int T
   }
 }
 
+// ---------------------------------------------------------------------------
+// Filtered assignment, for many anchors.  The argmax needs the split products
+// (three MMAs) only where two anchors are close: a first pass scores every
+// (key, anchor) pair by one product of the leading parts, h_j . h_r, which
+// misses the split product by at most
+//     |rho_j| + |rho_r| + B0,   rho = u - h (Cauchy-Schwarz, ||u|| = ||h|| = 1),
+// B0 covering what the split product itself leaves out and the fp32 sums of
+// both.  Per key and 128 anchors its epilogue keeps the largest upper and lower
+// bound; a tile of anchors whose upper bound reaches the key's largest lower
+// bound may hold the argmax.  The second pass computes the split products of
+// those (key, tile) pairs alone, with the MMA sequence of the full GEMM, so the
+// scores it compares, and the result, have the same bits.
+//   prefilter_kernel   (tc_gemm, kPlain, TcEpiFilter)  bounds per (key, tile)
+//   candidates_kernel  per (head, key chunk, tile): the list of its keys
+//   items_kernel       lists -> work items of 128 keys
+//   rescore_kernel     gathered keys x 128 anchors, argmax into `best`
+// Keys go in chunks whose profiles stay in L2 while all anchor tiles pass them
+// (a key is a candidate in 16 of 103 tiles on average at 128K).
+// 128K layer (t = 13107, n = 2048, 8 heads): 75.1 ms for the full GEMM.
+struct FilterDims {
+  int Nt, Tp, CR, nch;   // anchor tiles, pitch of the bounds, keys per chunk, chunks
+};
+static FilterDims filter_dims(const Dims& D) {
+  const int ldn = (D.n + 7) / 8 * 8, Tm = D.T - D.t;
+  FilterDims f;
+  f.Nt = 2 * cdiv(D.t, 256);   // the first pass takes anchors 256 at a time
+  f.Tp = (Tm + 31) / 32 * 32;
+  const long long rows = (48LL << 20) / (4LL * ldn) / 256 * 256;   // 48 MB of split profiles
+  f.CR = (int)std::max<long long>(256, std::min<long long>(8192, rows));
+  f.nch = cdiv(std::max(Tm, 1), f.CR);
+  return f;
+}
+// byte offsets in the scratch (the index features' second half, free by then)
+struct FilterLayout {
+  size_t list, cnt, off, items, rho_k, rho_s, total;
+};
+static FilterLayout filter_layout(const Dims& D, const FilterDims& f) {
+  FilterLayout L;
+  size_t o = 0;
+  auto take = [&](size_t bytes) { const size_t r = o; o += (bytes + 255) / 256 * 256; return r; };
+  const size_t E = (size_t)D.H * f.nch * f.Nt;
+  L.list = take(E * f.CR * 4);
+  L.cnt = take(E * 4);
+  L.off = take((E + 1) * 4);
+  L.items = take(E * (f.CR / 128) * 4);
+  L.rho_k = take((size_t)D.H * D.T * 4);
+  L.rho_s = take((size_t)D.H * f.Nt * 128 * 4);
+  L.total = o;
+  return L;
+}
+// Where the filter is used: from 24 tiles of 128 anchors up (a tile of few is
+// more often a candidate: 0.15 of all (key, tile) pairs at t = 13107, 0.37 at
+// 1638, 0.39 at 819, and the passes cost 0.35 + 1.3 times that share of the
+// full GEMM), when the bounds and lists fit the two halves of the index
+// features' buffer.
+bool assign_filtered(const Dims& D) {
+  const FilterDims f = filter_dims(D);
+  const size_t half = (size_t)D.H * D.T * D.HD * 2;
+  return D.t > 23 * 128 && D.T - D.t >= 4096 && f.CR % 256 == 0 && (size_t)D.H * f.Nt * f.Tp * 8 <= half &&
+         filter_layout(D, f).total <= half;
+}
+
+// Bounds of a row over its warp's 128 anchors (eight warps, 256-wide tiles).
+// rho_s is NaN past the last anchor: fmaxf skips those columns.
+struct TcEpiFilter {
+  static constexpr int kEpiWarps = 8;
+  const float* rho_s;   // [H][Nt * 128]
+  float2* bounds;       // [H][Nt][Tp] (upper, lower)
+  int Nt, Tp;
+  struct State {
+    float ub, lb;
+    const float4* r;
+  };
+  __device__ __forceinline__ void init(State& s, int b, int, int n0, int, int) const {
+    s.ub = s.lb = -INFINITY;
+    s.r = (const float4*)(rho_s + (long long)b * Nt * 128 + n0);
+  }
+  __device__ __forceinline__ void consume(State& s, int, int j, float (&v)[32]) const {
+    float u[4] = {s.ub, -INFINITY, -INFINITY, -INFINITY}, l[4] = {s.lb, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float4 r = __ldg(s.r + j * 8 + q);
+      u[0] = fmaxf(u[0], v[4 * q] + r.x);
+      l[0] = fmaxf(l[0], v[4 * q] - r.x);
+      u[1] = fmaxf(u[1], v[4 * q + 1] + r.y);
+      l[1] = fmaxf(l[1], v[4 * q + 1] - r.y);
+      u[2] = fmaxf(u[2], v[4 * q + 2] + r.z);
+      l[2] = fmaxf(l[2], v[4 * q + 2] - r.z);
+      u[3] = fmaxf(u[3], v[4 * q + 3] + r.w);
+      l[3] = fmaxf(l[3], v[4 * q + 3] - r.w);
+    }
+    s.ub = fmaxf(fmaxf(u[0], u[1]), fmaxf(u[2], u[3]));
+    s.lb = fmaxf(fmaxf(l[0], l[1]), fmaxf(l[2], l[3]));
+  }
+  __device__ __forceinline__ void finish(State& s, int b, int row, int n0, int M, int) const {
+    if (row < M) bounds[((long long)b * Nt + n0 / 128) * Tp + row] = make_float2(s.ub, s.lb);
+  }
+};
+
+// One thread per key: the tiles that may hold its argmax, appended to their
+// lists (one atomic per warp and tile; the order within a list does not matter).
+__global__ void __launch_bounds__(256) candidates_kernel(const float2* bounds, const float* rho_k, float B0, int T, int Tm,
+                                                         FilterDims f, int* list, int* cnt) {
+  chain_wait();
+  const int b = blockIdx.y, row = blockIdx.x * 256 + threadIdx.x, lane = threadIdx.x & 31;
+  const int ch = blockIdx.x * 256 / f.CR;
+  const float2* bd = bounds + (long long)b * f.Nt * f.Tp + row;
+  const bool in = row < Tm;
+  float lb = -INFINITY;
+#pragma unroll 8
+  for (int k = 0; k < f.Nt; ++k)
+    if (in) lb = fmaxf(lb, bd[(long long)k * f.Tp].y);
+  // upper + (rho_j + B0) >= lower - (rho_j + B0); no finite bound (a NaN profile): no candidate
+  const float thr = in ? lb - 2.f * (rho_k[(long long)b * T + row] + B0) : 0.f;
+  const bool any = in && lb > -INFINITY;
+  const long long e0 = ((long long)b * f.nch + ch) * f.Nt;
+#pragma unroll 4
+  for (int k = 0; k < f.Nt; ++k) {
+    const bool c = any && bd[(long long)k * f.Tp].x >= thr;
+    const unsigned m = __ballot_sync(0xffffffffu, c);
+    if (m == 0) continue;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(cnt + e0 + k, __popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (c) list[(e0 + k) * f.CR + base + __popc(m & ((1u << lane) - 1))] = row;
+  }
+}
+
+// off = exclusive sums of the lists' 128-key blocks; items[i] = list * (CR / 128) + block.
+__global__ void __launch_bounds__(1024) items_kernel(const int* cnt, int E, int per, int* off, int* items) {
+  chain_wait();
+  __shared__ int part[1024];
+  const int tid = threadIdx.x, step = (E + 1023) / 1024, e0 = min(E, tid * step), e1 = min(E, e0 + step);
+  int sum = 0;
+  for (int e = e0; e < e1; ++e) sum += (cnt[e] + 127) / 128;
+  part[tid] = sum;
+  __syncthreads();
+  for (int o = 1; o < 1024; o <<= 1) {
+    const int v = tid >= o ? part[tid - o] : 0;
+    __syncthreads();
+    part[tid] += v;
+    __syncthreads();
+  }
+  int at = part[tid] - sum;
+  for (int e = e0; e < e1; ++e) {
+    off[e] = at;
+    const int nb = (cnt[e] + 127) / 128;
+    for (int k = 0; k < nb; ++k) items[at + k] = e * per + k;
+    at += nb;
+  }
+  if (tid == 1023) off[E] = part[1023];
+}
+
+// 128 gathered keys x 128 anchors per work item, split products over the whole
+// K in one accumulator, row argmax (lowest index on ties) merged into `best`.
+// Persistent, one CTA per SM: warp 0 streams the anchor slabs by TMA, warps 6-9
+// gather the keys' (16-byte cp.async into the same swizzled layout; a thread
+// serves one 16-byte chunk of eight rows), warp 1 issues the MMAs, warps 2-5
+// drain the accumulators.
+constexpr int kRsStages = 3, kRsTile = 128 * 128, kRsStage = 4 * kRsTile;   // [keys hi][anchors hi][keys lo][anchors lo]
+constexpr int kRsThreads = 320;
+__global__ void __launch_bounds__(kRsThreads, 1)
+    rescore_kernel(const __grid_constant__ CUtensorMap mB, const __grid_constant__ CUtensorMap mB2, const bf16* Ut_hi,
+                   const bf16* Ut_lo, const int* list, const int* cnt, const int* off, const int* items, FilterDims f,
+                   int H, int T, int t, int ldn, unsigned long long* best, DevStatus* stt) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ uint64_t full[kRsStages], empty[kRsStages], accf[2], acce[2], drain;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag;
+  const uint32_t raw = tc::smem_u32(smem_raw);
+  uint8_t* base = smem_raw + (((raw + 1023u) & ~1023u) - raw);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nk = (ldn + 63) / 64, per = f.CR / 128, E = H * f.nch * f.Nt;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kRsStages; ++s) {
+      tc::mbar_init(&full[s], 1 + 4);
+      tc::mbar_init(&empty[s], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      tc::mbar_init(&accf[i], 1);
+      tc::mbar_init(&acce[i], 4);
+    }
+    tc::mbar_init(&drain, 1);
+    abort_flag = 0;
+    tc::mbar_fence_init();
+  }
+  chain_wait();
+  if (warp == 1) tc::tmem_alloc(&tmem_slot, 256);
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = tmem_slot;
+  volatile int* abortp = &abort_flag;
+  const int nitems = off[E];
+  // item -> list e of (head b, chunk, tile nt), its first key and key count
+  auto item = [&](int i, int& e, int& b, int& n0, int& k0, int& nkeys) {
+    const int v = items[i];
+    e = v / per;
+    k0 = (v - e * per) * 128;
+    b = e / (f.nch * f.Nt);
+    n0 = (e % f.Nt) * 128;
+    nkeys = min(128, cnt[e] - k0);
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      tc::tma_prefetch(&mB);
+      tc::tma_prefetch(&mB2);
+      int g = 0;
+      bool ok = true;
+      for (int i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
+        int e, b, n0, k0, nkeys;
+        item(i, e, b, n0, k0, nkeys);
+        for (int kb = 0; kb < nk; ++kb, ++g) {
+          const int s = g % kRsStages;
+          if (g >= kRsStages && !tc::mbar_wait(&empty[s], ((g / kRsStages) - 1) & 1, abortp, stt)) {
+            ok = false;
+            break;
+          }
+          uint8_t* st = base + s * kRsStage;
+          tc::mbar_arrive_expect_tx(&full[s], 2 * kRsTile);
+          tc::tma_load_3d(st + kRsTile, &mB, kb * 64, n0, b, &full[s]);
+          tc::tma_load_3d(st + 3 * kRsTile, &mB2, kb * 64, n0, b, &full[s]);
+        }
+      }
+      // every issued copy lands before the CTA may exit: the last slabs' barriers
+      // complete once the key gatherers have arrived too (they issue the same slabs)
+      volatile int never = 0;
+      for (int k = g > kRsStages ? g - kRsStages : 0; k < g; ++k)
+        tc::mbar_wait(&full[k % kRsStages], (k / kRsStages) & 1, &never, stt);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      bool ok = true;
+      int g = 0, c = 0;
+      for (int i = blockIdx.x; i < nitems && ok; i += gridDim.x, ++c) {
+        int e, b, n0, k0, nkeys;
+        item(i, e, b, n0, k0, nkeys);
+        const uint32_t idesc = tc::idesc_bf16_f32(min(128, (t - n0 + 15) & ~15));
+        const int buf = c & 1;
+        if (c >= 2 && !tc::mbar_wait(&acce[buf], ((c >> 1) - 1) & 1, abortp, stt)) break;
+        tc::fence_after_sync();
+        const uint32_t d = tmem + (uint32_t)(buf * 128);
+        for (int kb = 0; kb < nk; ++kb, ++g) {
+          const int s = g % kRsStages;
+          if (!tc::mbar_wait(&full[s], (g / kRsStages) & 1, abortp, stt)) {
+            ok = false;
+            break;
+          }
+          tc::fence_after_sync();
+          const uint32_t a = tc::smem_u32(base + s * kRsStage), bb = a + kRsTile;
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks) {   // the sequence of tc_gemm's kSplit
+            const uint64_t ad = tc::sdesc_k128(a + ks * 32), bd = tc::sdesc_k128(bb + ks * 32);
+            tc::mma_f16(d, ad, bd, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+            tc::mma_f16(d, ad, tc::sdesc_k128(bb + 2 * kRsTile + ks * 32), idesc, 1u);
+            tc::mma_f16(d, tc::sdesc_k128(a + 2 * kRsTile + ks * 32), bd, idesc, 1u);
+          }
+          tc::mma_commit(&empty[s]);
+        }
+        if (ok) tc::mma_commit(&accf[buf]);
+      }
+      tc::mma_commit(&drain);
+      volatile int never = 0;
+      tc::mbar_wait(&drain, 0, &never, stt);
+    }
+  } else if (warp < 6) {
+    const int q = warp & 3;
+    bool ok = true;
+    int c = 0;
+    for (int i = blockIdx.x; i < nitems; i += gridDim.x, ++c) {
+      int e, b, n0, k0, nkeys;
+      item(i, e, b, n0, k0, nkeys);
+      const int r = q * 32 + lane;
+      const int key = r < nkeys ? list[(long long)e * f.CR + k0 + r] : -1;
+      ok = tc::mbar_wait(&accf[c & 1], (c >> 1) & 1, abortp, stt);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc::fence_after_sync();
+      float bv = -INFINITY;
+      int bi = -1;
+      const int ncols = t - n0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float v[32];
+        tc::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((c & 1) * 128 + j * 32), v);
+#pragma unroll
+        for (int k = 0; k < 32; ++k)
+          if (j * 32 + k < ncols && v[k] > bv) {
+            bv = v[k];
+            bi = n0 + j * 32 + k;
+          }
+      }
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&acce[c & 1]);
+      if (key >= 0 && bi >= 0)
+        atomicMax(best + (long long)b * T + key,
+                  ((unsigned long long)f32_ordered(bv) << 32) | (unsigned long long)(0xffffffffu - (unsigned int)bi));
+    }
+  } else {
+    // gather: 16-byte chunk `ch` of rows rr, rr + 16, .. of the key tiles; a
+    // slab is handed over two slabs later, when its copies have landed
+    const int p = threadIdx.x - 192, ch = p & 7, rr = p >> 3;
+    const long long lo = Ut_lo - Ut_hi;
+    int g = 0;
+    bool ok = true;
+    auto hand_over = [&](int q) {   // slab q's copies are complete
+      tc::fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&full[q % kRsStages]);
+    };
+    for (int i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
+      int e, b, n0, k0, nkeys;
+      item(i, e, b, n0, k0, nkeys);
+      const bf16* src[8];
+      uint32_t dst[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int r = rr + 16 * u;
+        // rows past the list's end repeat its first (their results are dropped)
+        const int key = list[(long long)e * f.CR + k0 + (r < nkeys ? r : 0)];
+        src[u] = Ut_hi + ((long long)b * T + key) * ldn + ch * 8;
+        dst[u] = (uint32_t)(r * 128 + ((ch ^ (r & 7)) << 4));
+      }
+      for (int kb = 0; kb < nk; ++kb, ++g) {
+        const int s = g % kRsStages;
+        if (g >= kRsStages) {
+          ok = tc::mbar_wait(&empty[s], ((g / kRsStages) - 1) & 1, abortp, stt);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+        }
+        const uint32_t st = tc::smem_u32(base + s * kRsStage);
+        const int n16 = kb * 64 + ch * 8 < ldn ? 16 : 0;   // past the row's end: zeros
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const bf16* x = src[u] + (n16 ? kb * 64 : 0);
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(st + dst[u]), "l"(x), "r"(n16) : "memory");
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(st + 2 * kRsTile + dst[u]), "l"(x + lo),
+                       "r"(n16)
+                       : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (g >= 2) {
+          asm volatile("cp.async.wait_group 2;" ::: "memory");
+          hand_over(g - 2);
+        }
+      }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    for (int q = g >= 2 ? g - 2 : 0; q < g; ++q) hand_over(q);
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 1) {
+    tc::fence_after_sync();
+    tc::tmem_dealloc(tmem, 256);
+  }
+}
+
 int launch_assign_prep(const Dims& D, const float* L, float* logphi, const int* anchors, bf16* Ut_hi, bf16* Ut_lo,
-                       bf16* S_hi, bf16* S_lo, int* kmap, DevStatus* stt, cudaStream_t st) {
-  return col_profiles(D, L, logphi, ProfileOut{Ut_hi, Ut_lo, S_hi, S_lo, kmap, anchors, D.t}, stt, st);
+                       bf16* S_hi, bf16* S_lo, int* kmap, char* filter_scratch, DevStatus* stt, cudaStream_t st) {
+  ProfileOut po{Ut_hi, Ut_lo, S_hi, S_lo, kmap, anchors, D.t, nullptr, nullptr, 0};
+  if (filter_scratch) {
+    const FilterDims f = filter_dims(D);
+    const FilterLayout L2 = filter_layout(D, f);
+    po.rho_k = (float*)(filter_scratch + L2.rho_k);
+    po.rho_s = (float*)(filter_scratch + L2.rho_s);
+    po.ldr = f.Nt * 128;
+    // NaN past the anchors (TcEpiFilter)
+    if (cudaMemsetAsync(po.rho_s, 0xff, (size_t)D.H * po.ldr * 4, st) != cudaSuccess) return -1;
+  }
+  return col_profiles(D, L, logphi, po, stt, st);
+}
+
+// The two passes of the filtered assignment: `best` of every compacted row.
+static int filtered_argmax(const Dims& D, const bf16* Ut_hi, const bf16* Ut_lo, const bf16* S_hi, const bf16* S_lo,
+                           float2* bounds, char* scratch, unsigned long long* best, DevStatus* stt, cudaStream_t st) {
+  const FilterDims f = filter_dims(D);
+  const FilterLayout L = filter_layout(D, f);
+  const int ldn = (D.n + 7) / 8 * 8, Tm = D.T - D.t, E = D.H * f.nch * f.Nt;
+  const float* rho_k = (const float*)(scratch + L.rho_k);
+  const float* rho_s = (const float*)(scratch + L.rho_s);
+  int* list = (int*)(scratch + L.list);
+  int* cnt = (int*)(scratch + L.cnt);
+  int* off = (int*)(scratch + L.off);
+  int* items = (int*)(scratch + L.items);
+  CUtensorMap mA, mB, mC, mC2;
+  if (!encode_bf16_map_3d(&mA, Ut_hi, ldn, D.T, D.H, 128) || !encode_bf16_map_3d(&mB, S_hi, ldn, D.t, D.H, 256) ||
+      !encode_bf16_map_3d(&mC, S_hi, ldn, D.t, D.H, 128) || !encode_bf16_map_3d(&mC2, S_lo, ldn, D.t, D.H, 128))
+    return -1;
+  if (cudaMemsetAsync(cnt, 0, (size_t)E * 4, st) != cudaSuccess) return -1;
+  const int group = (int)std::max<long long>(1, (40LL << 20) / (512LL * ldn));   // 40 MB of anchor rows stay in L2
+  const TcEpiFilter epi{rho_s, bounds, f.Nt, f.Tp};
+  if (launch_tc_gemm<256, kPlain>(mA, mB, mA, mB, epi, D.H, Tm, D.t, ldn, (ldn + 63) / 64 * 64, stt, st, 0, nullptr,
+                                  group) != cudaSuccess)
+    return -1;
+  // B0: the split product drops lo lo and the lo parts' own rounding (2^-15 in
+  // all); an fp32 accumulation step errs by at most 2^-20 of a sum below 1, and
+  // the two passes take 4 n / 16 of them
+  const float B0 = 0x1p-15f + (float)D.n * 0x1p-22f;
+  launch_chained(candidates_kernel, dim3(cdiv(Tm, 256), D.H), 256, 0, st, bounds, rho_k, B0, D.T, Tm, f, list, cnt);
+  launch_chained(items_kernel, 1, 1024, 0, st, cnt, E, f.CR / 128, off, items);
+  const int smem = kRsStages * kRsStage + 1024;
+  if (set_dyn_smem((const void*)rescore_kernel, smem) != cudaSuccess) return -1;
+  if (launch_chained(rescore_kernel, tc_gemm_sm_count(), kRsThreads, smem, st, mC, mC2, Ut_hi, Ut_lo, list, cnt, off,
+                     items, f, D.H, D.T, D.t, ldn, best, stt) != cudaSuccess)
+    return -1;
+  return 4;
 }
 
 int launch_assign_gemm(const Dims& D, const int* anchors, const bf16* Ut_hi, const bf16* Ut_lo, const bf16* S_hi,
-                       const bf16* S_lo, const int* kmap, unsigned long long* best, int* kappa, DevStatus* stt,
-                       cudaStream_t st) {
+                       const bf16* S_lo, const int* kmap, unsigned long long* best, int* kappa, float2* filter_bounds,
+                       char* filter_scratch, DevStatus* stt, cudaStream_t st) {
   const int ldn = (D.n + 7) / 8 * 8;
   const int Tm = D.T - D.t;   // the non-anchor keys, compacted (none when t = T)
   int nl = 1;
@@ -404,6 +839,11 @@ int launch_assign_gemm(const Dims& D, const int* anchors, const bf16* Ut_hi, con
   cudaMemsetAsync(kappa, 0, sizeof(int) * (size_t)D.H * D.T, st);
   if (Tm > 0) {
     cudaMemsetAsync(best, 0, sizeof(unsigned long long) * (size_t)D.H * D.T, st);
+    if (filter_scratch) {
+      const int r = filtered_argmax(D, Ut_hi, Ut_lo, S_hi, S_lo, filter_bounds, filter_scratch, best, stt, st);
+      if (r < 0) return -1;
+      nl += r - 1;
+    } else {
     // 128 keys x 256 anchors per tile (M = 128, N = 256 MMAs): half the key-side
     // operand bytes per flop of a 128-wide tile.  The key map spans all T rows
     // of a head (its plane stride); the GEMM takes the first Tm.
@@ -424,6 +864,7 @@ int launch_assign_gemm(const Dims& D, const int* anchors, const bf16* Ut_hi, con
     if (launch_tc_gemm<BN, kSplit>(mA, mB, mA2, mB2, epi, D.H, Tm, D.t, ldn, kfull, stt, st, 0, nullptr, group) !=
         cudaSuccess)
       return -1;
+    }
     const long long cnt = (long long)D.H * Tm;
     launch_chained(decode_assign_kernel2, stride_grid(cnt, 256, 8), 256, 0, st, best, kmap, kappa, D.T, Tm, cnt);
     nl += 2;
