@@ -574,10 +574,17 @@ __global__ void __launch_bounds__(1024) items_kernel(const int* cnt, int E, int 
 // K in one accumulator, row argmax (lowest index on ties) merged into `best`.
 // Persistent, one CTA per SM: warp 0 streams the anchor slabs by TMA, warps 6-9
 // gather the keys' (16-byte cp.async into the same swizzled layout; a thread
-// serves one 16-byte chunk of eight rows), warp 1 issues the MMAs, warps 2-5
-// drain the accumulators.
-constexpr int kRsStages = 3, kRsTile = 128 * 128, kRsStage = 4 * kRsTile;   // [keys hi][anchors hi][keys lo][anchors lo]
+// serves one 16-byte chunk of four rows), warp 1 issues the MMAs, warps 2-5
+// drain the accumulators.  What bounds it is the latency of the gathered rows
+// against the 192 KB a CTA can have in flight, so the slabs are short (32 of K,
+// six stages, a slab handed over four later) and every role looks its next item
+// up while it works on the current one.
+constexpr int kRsStages = 6, kRsLag = 4, kRsK = 32;
+constexpr int kRsTile = 128 * kRsK * 2, kRsStage = 4 * kRsTile;   // [keys hi][anchors hi][keys lo][anchors lo]
 constexpr int kRsThreads = 320;
+struct RsItem {
+  int e, b, n0, k0, nkeys;   // list, head, first anchor, first key of the list, keys
+};
 __global__ void __launch_bounds__(kRsThreads, 1)
     rescore_kernel(const __grid_constant__ CUtensorMap mB, const __grid_constant__ CUtensorMap mB2, const bf16* Ut_hi,
                    const bf16* Ut_lo, const int* list, const int* cnt, const int* off, const int* items, FilterDims f,
@@ -589,7 +596,7 @@ __global__ void __launch_bounds__(kRsThreads, 1)
   const uint32_t raw = tc::smem_u32(smem_raw);
   uint8_t* base = smem_raw + (((raw + 1023u) & ~1023u) - raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nk = (ldn + 63) / 64, per = f.CR / 128, E = H * f.nch * f.Nt;
+  const int nk = 2 * ((ldn + 63) / 64), per = f.CR / 128, E = H * f.nch * f.Nt;   // whole 64-wide slabs, as the full GEMM
   if (threadIdx.x == 0) {
     for (int s = 0; s < kRsStages; ++s) {
       tc::mbar_init(&full[s], 1 + 4);
@@ -611,14 +618,17 @@ __global__ void __launch_bounds__(kRsThreads, 1)
   const uint32_t tmem = tmem_slot;
   volatile int* abortp = &abort_flag;
   const int nitems = off[E];
-  // item -> list e of (head b, chunk, tile nt), its first key and key count
-  auto item = [&](int i, int& e, int& b, int& n0, int& k0, int& nkeys) {
-    const int v = items[i];
-    e = v / per;
-    k0 = (v - e * per) * 128;
-    b = e / (f.nch * f.Nt);
-    n0 = (e % f.Nt) * 128;
-    nkeys = min(128, cnt[e] - k0);
+  auto item = [&](int i) {
+    RsItem x{};
+    if (i < nitems) {
+      const int v = items[i];
+      x.e = v / per;
+      x.k0 = (v - x.e * per) * 128;
+      x.b = x.e / (f.nch * f.Nt);
+      x.n0 = (x.e % f.Nt) * 128;
+      x.nkeys = min(128, cnt[x.e] - x.k0);
+    }
+    return x;
   };
 
   if (warp == 0) {
@@ -627,9 +637,10 @@ __global__ void __launch_bounds__(kRsThreads, 1)
       tc::tma_prefetch(&mB2);
       int g = 0;
       bool ok = true;
+      RsItem nx = item(blockIdx.x);
       for (int i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
-        int e, b, n0, k0, nkeys;
-        item(i, e, b, n0, k0, nkeys);
+        const RsItem x = nx;
+        nx = item(i + gridDim.x);
         for (int kb = 0; kb < nk; ++kb, ++g) {
           const int s = g % kRsStages;
           if (g >= kRsStages && !tc::mbar_wait(&empty[s], ((g / kRsStages) - 1) & 1, abortp, stt)) {
@@ -638,8 +649,8 @@ __global__ void __launch_bounds__(kRsThreads, 1)
           }
           uint8_t* st = base + s * kRsStage;
           tc::mbar_arrive_expect_tx(&full[s], 2 * kRsTile);
-          tc::tma_load_3d(st + kRsTile, &mB, kb * 64, n0, b, &full[s]);
-          tc::tma_load_3d(st + 3 * kRsTile, &mB2, kb * 64, n0, b, &full[s]);
+          tc::tma_load_3d(st + kRsTile, &mB, kb * kRsK, x.n0, x.b, &full[s]);
+          tc::tma_load_3d(st + 3 * kRsTile, &mB2, kb * kRsK, x.n0, x.b, &full[s]);
         }
       }
       // every issued copy lands before the CTA may exit: the last slabs' barriers
@@ -652,10 +663,11 @@ __global__ void __launch_bounds__(kRsThreads, 1)
     if (lane == 0) {
       bool ok = true;
       int g = 0, c = 0;
+      RsItem nx = item(blockIdx.x);
       for (int i = blockIdx.x; i < nitems && ok; i += gridDim.x, ++c) {
-        int e, b, n0, k0, nkeys;
-        item(i, e, b, n0, k0, nkeys);
-        const uint32_t idesc = tc::idesc_bf16_f32(min(128, (t - n0 + 15) & ~15));
+        const RsItem x = nx;
+        nx = item(i + gridDim.x);
+        const uint32_t idesc = tc::idesc_bf16_f32(min(128, (t - x.n0 + 15) & ~15));
         const int buf = c & 1;
         if (c >= 2 && !tc::mbar_wait(&acce[buf], ((c >> 1) - 1) & 1, abortp, stt)) break;
         tc::fence_after_sync();
@@ -669,11 +681,11 @@ __global__ void __launch_bounds__(kRsThreads, 1)
           tc::fence_after_sync();
           const uint32_t a = tc::smem_u32(base + s * kRsStage), bb = a + kRsTile;
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks) {   // the sequence of tc_gemm's kSplit
-            const uint64_t ad = tc::sdesc_k128(a + ks * 32), bd = tc::sdesc_k128(bb + ks * 32);
+          for (int ks = 0; ks < kRsK / 16; ++ks) {   // the sequence of tc_gemm's kSplit
+            const uint64_t ad = tc::sdesc_k64(a + ks * 32), bd = tc::sdesc_k64(bb + ks * 32);
             tc::mma_f16(d, ad, bd, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
-            tc::mma_f16(d, ad, tc::sdesc_k128(bb + 2 * kRsTile + ks * 32), idesc, 1u);
-            tc::mma_f16(d, tc::sdesc_k128(a + 2 * kRsTile + ks * 32), bd, idesc, 1u);
+            tc::mma_f16(d, ad, tc::sdesc_k64(bb + 2 * kRsTile + ks * 32), idesc, 1u);
+            tc::mma_f16(d, tc::sdesc_k64(a + 2 * kRsTile + ks * 32), bd, idesc, 1u);
           }
           tc::mma_commit(&empty[s]);
         }
@@ -688,10 +700,9 @@ __global__ void __launch_bounds__(kRsThreads, 1)
     bool ok = true;
     int c = 0;
     for (int i = blockIdx.x; i < nitems; i += gridDim.x, ++c) {
-      int e, b, n0, k0, nkeys;
-      item(i, e, b, n0, k0, nkeys);
-      const int r = q * 32 + lane;
-      const int key = r < nkeys ? list[(long long)e * f.CR + k0 + r] : -1;
+      const RsItem x = item(i);   // (in the shadow of the item's MMAs)
+      const int r = q * 32 + lane, n0 = x.n0, b = x.b;
+      const int key = r < x.nkeys ? list[(long long)x.e * f.CR + x.k0 + r] : -1;
       ok = tc::mbar_wait(&accf[c & 1], (c >> 1) & 1, abortp, stt);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
@@ -718,10 +729,16 @@ __global__ void __launch_bounds__(kRsThreads, 1)
                   ((unsigned long long)f32_ordered(bv) << 32) | (unsigned long long)(0xffffffffu - (unsigned int)bi));
     }
   } else {
-    // gather: 16-byte chunk `ch` of rows rr, rr + 16, .. of the key tiles; a
-    // slab is handed over two slabs later, when its copies have landed
-    const int p = threadIdx.x - 192, ch = p & 7, rr = p >> 3;
+    // gather: 16-byte chunk `ch` of rows rr, rr + 32, .. of the key tiles; a
+    // slab is handed over kRsLag slabs later, when its copies have landed
+    const int p = threadIdx.x - 192, ch = p & 3, rr = p >> 2;
     const long long lo = Ut_lo - Ut_hi;
+    uint32_t dst[4];   // 64-byte swizzle: chunk ch of row r at ch ^ (r / 2 % 4)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = rr + 32 * u;
+      dst[u] = (uint32_t)(r * 64 + ((ch ^ ((r >> 1) & 3)) << 4));
+    }
     int g = 0;
     bool ok = true;
     auto hand_over = [&](int q) {   // slab q's copies are complete
@@ -729,20 +746,24 @@ __global__ void __launch_bounds__(kRsThreads, 1)
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&full[q % kRsStages]);
     };
-    for (int i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
-      int e, b, n0, k0, nkeys;
-      item(i, e, b, n0, k0, nkeys);
-      const bf16* src[8];
-      uint32_t dst[8];
+    // rows past the list's end repeat its first (their results are dropped)
+    auto keys_of = [&](const RsItem& x, int (&key)[4]) {
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int r = rr + 16 * u;
-        // rows past the list's end repeat its first (their results are dropped)
-        const int key = list[(long long)e * f.CR + k0 + (r < nkeys ? r : 0)];
-        src[u] = Ut_hi + ((long long)b * T + key) * ldn + ch * 8;
-        dst[u] = (uint32_t)(r * 128 + ((ch ^ (r & 7)) << 4));
+      for (int u = 0; u < 4; ++u) {
+        const int r = rr + 32 * u;
+        key[u] = x.nkeys > 0 ? list[(long long)x.e * f.CR + x.k0 + (r < x.nkeys ? r : 0)] : 0;
       }
+    };
+    RsItem x = item(blockIdx.x);
+    int key[4];
+    keys_of(x, key);
+    for (int i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
+      const bf16* src[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) src[u] = Ut_hi + ((long long)x.b * T + key[u]) * ldn + ch * 8;
+      RsItem nx = item(i + gridDim.x);
       for (int kb = 0; kb < nk; ++kb, ++g) {
+        if (kb == nk / 2) keys_of(nx, key);
         const int s = g % kRsStages;
         if (g >= kRsStages) {
           ok = tc::mbar_wait(&empty[s], ((g / kRsStages) - 1) & 1, abortp, stt);
@@ -750,24 +771,25 @@ __global__ void __launch_bounds__(kRsThreads, 1)
           if (!ok) break;
         }
         const uint32_t st = tc::smem_u32(base + s * kRsStage);
-        const int n16 = kb * 64 + ch * 8 < ldn ? 16 : 0;   // past the row's end: zeros
+        const int n16 = kb * kRsK + ch * 8 < ldn ? 16 : 0;   // past the row's end: zeros
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const bf16* x = src[u] + (n16 ? kb * 64 : 0);
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(st + dst[u]), "l"(x), "r"(n16) : "memory");
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(st + 2 * kRsTile + dst[u]), "l"(x + lo),
+        for (int u = 0; u < 4; ++u) {
+          const bf16* y = src[u] + (n16 ? kb * kRsK : 0);
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(st + dst[u]), "l"(y), "r"(n16) : "memory");
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(st + 2 * kRsTile + dst[u]), "l"(y + lo),
                        "r"(n16)
                        : "memory");
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
-        if (g >= 2) {
-          asm volatile("cp.async.wait_group 2;" ::: "memory");
-          hand_over(g - 2);
+        if (g >= kRsLag) {
+          asm volatile("cp.async.wait_group %0;" ::"n"(kRsLag) : "memory");
+          hand_over(g - kRsLag);
         }
       }
+      x = nx;
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    for (int q = g >= 2 ? g - 2 : 0; q < g; ++q) hand_over(q);
+    for (int q = g > kRsLag ? g - kRsLag : 0; q < g; ++q) hand_over(q);
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -806,7 +828,8 @@ static int filtered_argmax(const Dims& D, const bf16* Ut_hi, const bf16* Ut_lo, 
   int* items = (int*)(scratch + L.items);
   CUtensorMap mA, mB, mC, mC2;
   if (!encode_bf16_map_3d(&mA, Ut_hi, ldn, D.T, D.H, 128) || !encode_bf16_map_3d(&mB, S_hi, ldn, D.t, D.H, 256) ||
-      !encode_bf16_map_3d(&mC, S_hi, ldn, D.t, D.H, 128) || !encode_bf16_map_3d(&mC2, S_lo, ldn, D.t, D.H, 128))
+      !encode_bf16_map_3d_sw64(&mC, S_hi, ldn, D.t, D.H, ldn, 128) ||
+      !encode_bf16_map_3d_sw64(&mC2, S_lo, ldn, D.t, D.H, ldn, 128))
     return -1;
   if (cudaMemsetAsync(cnt, 0, (size_t)E * 4, st) != cudaSuccess) return -1;
   const int group = (int)std::max<long long>(1, (40LL << 20) / (512LL * ldn));   // 40 MB of anchor rows stay in L2
