@@ -380,7 +380,7 @@ arckv_status arckv_compact(const arckv_config* cfg, const void* K, const void* V
   }
   mark(6);
   nl += launch_merge(D, cfg->lambda_m, Kb, anchors, kappa, F(L.logphi), I32(L.perm), I32(L.goff), I32(L.cursor),
-                     C_k, st);
+                     I32(L.kmap), C_k, st);   // (kmap: free after the assignment)
   mark(7);
   FitBufs B{F(L.LC),  F(L.Phi), F(L.Gram), F(L.Linv), F(L.rhs), F(L.wsol), F(L.R), F(L.Z),
             (bf16*)(w + L.S_hi), (bf16*)(w + L.S_lo), (bf16*)(w + L.YT_hi), (bf16*)(w + L.YT_lo),

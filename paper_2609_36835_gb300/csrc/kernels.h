@@ -141,8 +141,9 @@ inline long long sort_scratch_ints(int H, int T, int t) {
   const long long C = (T + kSortChunk - 1) / kSortChunk;
   return sort_chunked(T, t) ? (long long)H * t * (C + 1) : (long long)H * t;
 }
+// big [H][T]: scratch (the list of each head's large groups).
 int launch_merge(const Dims& D, float lambda_m, const bf16* K, const int* anchors, const int* kappa,
-                 const float* logphi, int* perm, int* goff, int* cursor, float* C_k, cudaStream_t st);
+                 const float* logphi, int* perm, int* goff, int* cursor, int* big, float* C_k, cudaStream_t st);
 
 // ---- fits (App. A.9) -----------------------------------------------------
 struct FitBufs {

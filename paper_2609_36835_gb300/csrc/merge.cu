@@ -90,7 +90,7 @@ __device__ __forceinline__ int block_excl_scan_1024_m(int v, int* sc, int& total
 // perm lists the members of G_0, G_1, ... each in ascending position order;
 // goff[r] .. goff[r+1] delimits G_r.
 __global__ void __launch_bounds__(1024) group_sort_kernel(const int* kappa, int T, int t, int* perm, int* goff,
-                                                          int* cursor) {
+                                                          int* cursor, int* big) {
   chain_wait();
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int* kb = kappa + (long long)b * T;
@@ -111,7 +111,10 @@ __global__ void __launch_bounds__(1024) group_sort_kernel(const int* kappa, int 
     if (r < t) { gb[r] = ex; cb[r] = ex; }
     base += tot;
   }
-  if (tid == 0) gb[t] = base;
+  if (tid == 0) {
+    gb[t] = base;
+    big[(long long)b * T] = 0;
+  }
   __syncthreads();
   const unsigned int lt = (1u << lane) - 1u;
   for (int j0 = 0; j0 < T; j0 += 1024) {
@@ -169,7 +172,8 @@ __global__ void __launch_bounds__(256) sort_totals_kernel(const int* __restrict_
 }
 
 // goff[b] = exclusive scan of tot[b] (one CTA per head); goff[b][t] = T
-__global__ void __launch_bounds__(1024) sort_scan_kernel(const int* __restrict__ tot, int t, int* __restrict__ goff) {
+__global__ void __launch_bounds__(1024) sort_scan_kernel(const int* __restrict__ tot, int t, int* __restrict__ goff,
+                                                         int* __restrict__ big, int T) {
   chain_wait();
   __shared__ int sc[32];
   const int b = blockIdx.x, tid = threadIdx.x;
@@ -183,7 +187,10 @@ __global__ void __launch_bounds__(1024) sort_scan_kernel(const int* __restrict__
     if (r < t) gb[r] = ex;
     base += total;
   }
-  if (tid == 0) gb[t] = base;
+  if (tid == 0) {
+    gb[t] = base;
+    big[(long long)b * T] = 0;   // the list of large groups starts empty
+  }
 }
 
 // cnt[b][g][c] <- the first slot of chunk c's members of group g
@@ -236,73 +243,99 @@ __global__ void __launch_bounds__(1024) sort_scatter_kernel(const int* __restric
 
 constexpr int kMergeWarpMax = 128;
 
-// Groups of more than kMergeWarpMax members (this launch skips the others),
-// one CTA per group with the member layout of group_merge_kernel in each of
-// its eight warps (32 members in flight); the warps' partial sums are added in
-// warp order, so the result does not depend on scheduling.
-__global__ void __launch_bounds__(256) group_merge_cta_kernel(const bf16* K, const int* anchors, const int* perm,
-                                                              const int* goff, const float* logphi, float lambda_m,
-                                                              float* C_k, int T, int t) {
+// Groups of more than kMergeWarpMax members, listed by group_merge_kernel in
+// big[b * T ..] (their count, then the groups in any order): a CTA takes 32 of a
+// group's 128 dimensions.  Its eight warps have four members each (eight lanes of
+// four dimensions per member), so member q of the group is summed by slot q % 32
+// in ascending order and the slots are combined by a fixed tree, whatever the
+// scheduling.  Sixteen members per slot are in flight: one at a time, a member
+// costs two dependent round trips, and one CTA per group left the largest group
+// to a single SM, 64 us of an 8K layer and 0.24 ms of a 32K one.
+constexpr int kBigParts = 4, kBigCtas = 64, kB = 16;
+__global__ void __launch_bounds__(256) group_merge_cta_kernel(const bf16* __restrict__ K, const int* __restrict__ anchors,
+                                                              const int* __restrict__ perm, const int* __restrict__ goff,
+                                                              const float* __restrict__ logphi, float lambda_m,
+                                                              float* C_k, const int* __restrict__ big, int T, int t) {
   chain_wait();
-  const int b = blockIdx.y, r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int* pb = perm + (long long)b * T;
   const int* gb = goff + (long long)b * (t + 1);
   const float* lp = logphi + (long long)b * T;
   const bf16* Kb = K + (long long)b * T * 128;
-  const int beg = gb[r], end = gb[r + 1];
-  if (end - beg <= kMergeWarpMax) return;
-  __shared__ float red[8][129];
+  const int* bg = big + (long long)b * T;
+  __shared__ float red[8][33];
   __shared__ float gmax_s[8];
-  float gm = -INFINITY;
-  for (int q = beg + threadIdx.x; q < end; q += 256) gm = fmaxf(gm, lp[pb[q]]);
-  gm = warp_max(gm);
-  if (lane == 0) gmax_s[warp] = gm;
-  __syncthreads();
-  gm = gmax_s[0];
-  for (int w = 1; w < 8; ++w) gm = fmaxf(gm, gmax_s[w]);
-  const int slot = lane >> 3, d0 = (lane & 7) * 16;
-  float acc[16], ws = 0.f;
+  const int count = bg[0];
+  for (int i = blockIdx.x; i < count * kBigParts; i += kBigCtas) {
+    const int r = bg[1 + i / kBigParts], dbase = (i % kBigParts) * 32;
+    const int beg = gb[r], end = gb[r + 1];
+    float gm = -INFINITY;
+    for (int q = beg + threadIdx.x; q < end; q += 256 * kB) {
+      int j[kB];
 #pragma unroll
-  for (int e = 0; e < 16; ++e) acc[e] = 0.f;
-  for (int q = beg + warp * 4 + slot; q < end; q += 32) {
-    const int j = pb[q];
-    const float om = ex2_approx((lp[j] - gm) * kLog2e);
-    const uint4* src = (const uint4*)(Kb + (long long)j * 128 + d0);
-    const uint4 u0 = src[0], u1 = src[1];
-    const __nv_bfloat162* h0 = (const __nv_bfloat162*)&u0;
-    const __nv_bfloat162* h1 = (const __nv_bfloat162*)&u1;
+      for (int u = 0; u < kB; ++u) j[u] = pb[min(q + 256 * u, end - 1)];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 f0 = __bfloat1622float2(h0[e]), f1 = __bfloat1622float2(h1[e]);
-      acc[2 * e] = fmaf(om, f0.x, acc[2 * e]);
-      acc[2 * e + 1] = fmaf(om, f0.y, acc[2 * e + 1]);
-      acc[8 + 2 * e] = fmaf(om, f1.x, acc[8 + 2 * e]);
-      acc[8 + 2 * e + 1] = fmaf(om, f1.y, acc[8 + 2 * e + 1]);
+      for (int u = 0; u < kB; ++u) gm = fmaxf(gm, lp[j[u]]);
     }
-    ws += om;
-  }
+    gm = warp_max(gm);
+    if (lane == 0) gmax_s[warp] = gm;
+    __syncthreads();
+    gm = gmax_s[0];
+    for (int w = 1; w < 8; ++w) gm = fmaxf(gm, gmax_s[w]);
+    const int slot = lane >> 3, d0 = dbase + (lane & 7) * 4;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f}, ws = 0.f;
+    int j[kB];   // the batch's members, looked up a batch ahead
+    const int q0 = beg + warp * 4 + slot;
 #pragma unroll
-  for (int o = 8; o < 32; o <<= 1) {
+    for (int u = 0; u < kB; ++u) j[u] = pb[min(q0 + 32 * u, end - 1)];
+    for (int q = q0; q < end; q += 32 * kB) {
+      float lv[kB];
+      uint2 x[kB];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
-    ws += __shfl_xor_sync(0xffffffffu, ws, o);
-  }
-  if (lane < 8) {
+      for (int u = 0; u < kB; ++u) {
+        lv[u] = lp[j[u]];
+        x[u] = *(const uint2*)(Kb + (long long)j[u] * 128 + d0);
+      }
 #pragma unroll
-    for (int e = 0; e < 16; ++e) red[warp][d0 + e] = acc[e];
-    if (lane == 0) red[warp][128] = ws;
+      for (int u = 0; u < kB; ++u) j[u] = pb[min(q + 32 * (kB + u), end - 1)];
+#pragma unroll
+      for (int u = 0; u < kB; ++u) {
+        // weight 0 past the end, not a branch: loads used in one alone are sunk
+        // into it, and then wait for one another
+        const float om = q + 32 * u < end ? ex2_approx((lv[u] - gm) * kLog2e) : 0.f;
+        const float2 f0 = __bfloat1622float2(*(const __nv_bfloat162*)&x[u].x);
+        const float2 f1 = __bfloat1622float2(*(const __nv_bfloat162*)&x[u].y);
+        acc[0] = fmaf(om, f0.x, acc[0]);
+        acc[1] = fmaf(om, f0.y, acc[1]);
+        acc[2] = fmaf(om, f1.x, acc[2]);
+        acc[3] = fmaf(om, f1.y, acc[3]);
+        ws += om;
+      }
+    }
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+      ws += __shfl_xor_sync(0xffffffffu, ws, o);
+    }
+    if (lane < 8) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) red[warp][lane * 4 + e] = acc[e];
+      if (lane == 0) red[warp][32] = ws;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      float a = 0.f, wsum = 0.f;
+      for (int w = 0; w < 8; ++w) {
+        a += red[w][threadIdx.x];
+        wsum += red[w][32];
+      }
+      const int s = anchors[(long long)b * t + r], dcol = dbase + threadIdx.x;
+      const float k = to_f32(Kb[(long long)s * 128 + dcol]);
+      C_k[((long long)b * t + r) * 128 + dcol] = fmaf(lambda_m, a * (1.0f / wsum) - k, k);
+    }
+    __syncthreads();   // red and gmax_s are free
   }
-  __syncthreads();
-  if (threadIdx.x >= 128) return;
-  const int dcol = threadIdx.x;
-  float a = 0.f, wsum = 0.f;
-  for (int w = 0; w < 8; ++w) {
-    a += red[w][dcol];
-    wsum += red[w][128];
-  }
-  const int s = anchors[(long long)b * t + r];
-  const float k = to_f32(Kb[(long long)s * 128 + dcol]);
-  C_k[((long long)b * t + r) * 128 + dcol] = fmaf(lambda_m, a * (1.0f / wsum) - k, k);
 }
 
 // Groups of up to kMergeWarpMax members, one warp per group r:
@@ -317,7 +350,7 @@ __global__ void __launch_bounds__(256) group_merge_cta_kernel(const bf16* K, con
 // group avoids the block barriers and idle warps of a CTA per group.
 __global__ void __launch_bounds__(256) group_merge_kernel(const bf16* K, const int* anchors, const int* perm,
                                                           const int* goff, const float* logphi, float lambda_m,
-                                                          float* C_k, int T, int t) {
+                                                          float* C_k, int* big, int T, int t) {
   chain_wait();
   const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = blockIdx.x * 8 + warp;
@@ -327,7 +360,10 @@ __global__ void __launch_bounds__(256) group_merge_kernel(const bf16* K, const i
   const float* lp = logphi + (long long)b * T;
   const bf16* Kb = K + (long long)b * T * 128;
   const int beg = gb[r], end = gb[r + 1];
-  if (end - beg > kMergeWarpMax) return;   // group_merge_cta_kernel
+  if (end - beg > kMergeWarpMax) {   // group_merge_cta_kernel's
+    if (lane == 0) big[(long long)b * T + 1 + atomicAdd(big + (long long)b * T, 1)] = r;
+    return;
+  }
   float gm = -INFINITY;
   for (int q = beg + lane; q < end; q += 32) gm = fmaxf(gm, lp[pb[q]]);
   gm = warp_max(gm);
@@ -335,22 +371,34 @@ __global__ void __launch_bounds__(256) group_merge_kernel(const bf16* K, const i
   float acc[16], ws = 0.f;
 #pragma unroll
   for (int e = 0; e < 16; ++e) acc[e] = 0.f;
-  for (int q = beg + slot; q < end; q += 4) {
-    const int j = pb[q];
-    const float om = ex2_approx((lp[j] - gm) * kLog2e);
-    const uint4* src = (const uint4*)(Kb + (long long)j * 128 + d0);
-    const uint4 u0 = src[0], u1 = src[1];
-    const __nv_bfloat162* h0 = (const __nv_bfloat162*)&u0;
-    const __nv_bfloat162* h1 = (const __nv_bfloat162*)&u1;
+  for (int q = beg + slot; q < end; q += 16) {   // four members of the slot in flight (weight 0 past the end)
+    int j[4];
+    float lv[4];
+    uint4 u0[4], u1[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 f0 = __bfloat1622float2(h0[e]), f1 = __bfloat1622float2(h1[e]);
-      acc[2 * e] = fmaf(om, f0.x, acc[2 * e]);
-      acc[2 * e + 1] = fmaf(om, f0.y, acc[2 * e + 1]);
-      acc[8 + 2 * e] = fmaf(om, f1.x, acc[8 + 2 * e]);
-      acc[8 + 2 * e + 1] = fmaf(om, f1.y, acc[8 + 2 * e + 1]);
+    for (int u = 0; u < 4; ++u) j[u] = pb[min(q + 4 * u, end - 1)];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint4* src = (const uint4*)(Kb + (long long)j[u] * 128 + d0);
+      lv[u] = lp[j[u]];
+      u0[u] = src[0];
+      u1[u] = src[1];
     }
-    ws += om;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float om = q + 4 * u < end ? ex2_approx((lv[u] - gm) * kLog2e) : 0.f;
+      const __nv_bfloat162* h0 = (const __nv_bfloat162*)&u0[u];
+      const __nv_bfloat162* h1 = (const __nv_bfloat162*)&u1[u];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 f0 = __bfloat1622float2(h0[e]), f1 = __bfloat1622float2(h1[e]);
+        acc[2 * e] = fmaf(om, f0.x, acc[2 * e]);
+        acc[2 * e + 1] = fmaf(om, f0.y, acc[2 * e + 1]);
+        acc[8 + 2 * e] = fmaf(om, f1.x, acc[8 + 2 * e]);
+        acc[8 + 2 * e + 1] = fmaf(om, f1.y, acc[8 + 2 * e + 1]);
+      }
+      ws += om;
+    }
   }
 #pragma unroll
   for (int o = 8; o < 32; o <<= 1) {
@@ -377,7 +425,7 @@ __global__ void __launch_bounds__(256) group_merge_kernel(const bf16* K, const i
 }
 
 int launch_merge(const Dims& D, float lambda_m, const bf16* K, const int* anchors, const int* kappa,
-                 const float* logphi, int* perm, int* goff, int* cursor, float* C_k, cudaStream_t st) {
+                 const float* logphi, int* perm, int* goff, int* cursor, int* big, float* C_k, cudaStream_t st) {
   int nl = 2;
   const int C = cdiv(D.T, kSortChunk), hb = (int)cdiv((long long)D.H * D.t, 256);
   const int hsm = D.t * (int)sizeof(int);
@@ -387,17 +435,18 @@ int launch_merge(const Dims& D, float lambda_m, const bf16* K, const int* anchor
     int* tot = cursor + (long long)D.H * D.t * C;
     launch_chained(sort_hist_kernel, dim3(C, D.H), 1024, hsm, st, kappa, D.T, D.t, C, cursor);
     launch_chained(sort_totals_kernel, hb, 256, 0, st, cursor, D.t, C, D.H, tot);
-    launch_chained(sort_scan_kernel, D.H, 1024, 0, st, tot, D.t, goff);
+    launch_chained(sort_scan_kernel, D.H, 1024, 0, st, tot, D.t, goff, big, D.T);
     launch_chained(sort_slots_kernel, hb, 256, 0, st, cursor, goff, D.t, C, D.H);
     launch_chained(sort_scatter_kernel, dim3(C, D.H), 1024, hsm, st, kappa, D.T, D.t, C, cursor, perm);
     nl += 5;
   } else {
-    launch_chained(group_sort_kernel, D.H, 1024, 0, st, kappa, D.T, D.t, perm, goff, cursor);
+    launch_chained(group_sort_kernel, D.H, 1024, 0, st, kappa, D.T, D.t, perm, goff, cursor, big);
     ++nl;
   }
-  launch_chained(group_merge_kernel, dim3(cdiv(D.t, 8), D.H), 256, 0, st, K, anchors, perm, goff, logphi, lambda_m, C_k, D.T,
-                                                              D.t);
-  launch_chained(group_merge_cta_kernel, dim3(D.t, D.H), 256, 0, st, K, anchors, perm, goff, logphi, lambda_m, C_k, D.T, D.t);
+  launch_chained(group_merge_kernel, dim3(cdiv(D.t, 8), D.H), 256, 0, st, K, anchors, perm, goff, logphi, lambda_m, C_k,
+                 big, D.T, D.t);
+  launch_chained(group_merge_cta_kernel, dim3(kBigCtas, D.H), 256, 0, st, K, anchors, perm, goff, logphi, lambda_m, C_k,
+                 big, D.T, D.t);
   return nl;
 }
 

@@ -9,6 +9,8 @@
 // row's head weight w_ia before the next head is added.  The epilogue then
 // writes the row-softmax partials (max, sum of exp) of each kIndexPartW
 // columns and the I tile.
+#include <algorithm>
+
 #include "kernels.h"
 #include "tc_gemm.cuh"
 
@@ -115,13 +117,20 @@ int launch_index_logits(const Dims& D, const bf16* qbar_hi, const bf16* qbar_lo,
   CUtensorMap mI;
   if (!encode_f32_map_3d(&mI, I, D.T, D.n, D.H, 32, 32, ld, (uint64_t)D.n * ld, true)) return -1;
   const int ntiles = cdiv(D.T, kIndexPartW);
+  // key tiles in groups whose split features (bB rows x HD x 4 bytes each) take
+  // about 40 MB, so that a group stays in L2 while every row tile passes it (at T
+  // = 131072 a head's k_bar, 0.5 GB, was streamed once per row tile: 69 GB in
+  // all, 11.1 ms)
+  const int group = (int)std::max<long long>(1, (40LL << 20) / ((long long)bB * D.HD * 4));
   cudaError_t e;
   if (wide) {
     TcEpiIndexT<kIndexPartW, 256> epi{wts, part, D.n, D.T, D.H_I, D.G, D.n_pos, ntiles, mI};
-    e = launch_tc_gemm<256, kSplit>(mA, mB, mA2, mB2, epi, D.H, D.n, D.T, D.HD, 128, stt, st);
+    e = launch_tc_gemm<256, kSplit>(mA, mB, mA2, mB2, epi, D.H, D.n, D.T, D.HD, 128, stt, st, 0, nullptr,
+                                     group);
   } else {
     TcEpiIndexT<kIndexPartW> epi{wts, part, D.n, D.T, D.H_I, D.G, D.n_pos, ntiles, mI};
-    e = launch_tc_gemm<128, kSplit>(mA, mB, mA2, mB2, epi, D.H, D.n, D.T, D.HD, 128, stt, st);
+    e = launch_tc_gemm<128, kSplit>(mA, mB, mA2, mB2, epi, D.H, D.n, D.T, D.HD, 128, stt, st, 0, nullptr,
+                                     group);
   }
   return e == cudaSuccess ? 1 : -1;
 }
