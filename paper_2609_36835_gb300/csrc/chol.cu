@@ -27,8 +27,8 @@
 // blocks are dealt over the cluster, X_k broadcast through distributed shared
 // memory.
 //
-// Eight heads on a GB300, one right-hand side / 128: 0.29 / 0.41 ms at t = 819,
-// 0.78 / 1.05 ms at t = 1638; 0.67 / 0.81 and 1.88 / 2.09 ms before, with the
+// Eight heads on a GB300, one right-hand side / 128: 0.28 / 0.34 ms at t = 819,
+// 0.77 / 0.98 ms at t = 1638; 0.67 / 0.81 and 1.88 / 2.09 ms before, with the
 // split redone in every unit, 4 (8) CTAs a head and a 40 K cycle factor.  At t =
 // 819 a step is its owner's chain, 36 K cycles: L_{k+1,k} 8.5, diagonal update
 // 5, factor and inverse 21.
@@ -492,85 +492,137 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
   // right-hand-side columns, its columns n the rows of the block
   //   Z_i -= L_ki^T X_k:     D = X_k^T L_ki,          Z_i[n][m] -= D[m][n]
   //   X_k = Linv^T (Y + Z):  D = (Y_k + Z_k)^T Linv,  X_k[n][m] = D[m][n]
-  // Operand rows r < rows of a triple from a column-major source: element
-  // (r, l) = G[l * ld + r] (+ G2[...] when given) for r < rvalid, l < kvalid,
-  // zero elsewhere; consecutive threads take consecutive r (coalesced).
-  uint8_t *Ah = stage, *Bh = stage + 3 * kStageA;
-  auto stage_cols = [&](uint8_t* h, int part, int rows, const float* G, const float* G2, long long ld, int rvalid,
-                        int kvalid) {
-    for (int task = tid; task < rows * 8; task += kCT) {
-      const int r = task % rows, ch = task / rows;
+  // Serial over the blocks: the owner of block k - 1 stages the two operands that
+  // do not depend on X_k while it waits for the others, takes X_k as the triple
+  // its owner left in a slot (alternate slots), adds the update to Y + Z on the
+  // way from TMEM to the second product's operand, and leaves X_{k-1} as a triple
+  // in turn; the other CTAs apply X_k to their blocks of Z.
+  uint8_t* const SA = stage;                               // X_k^T
+  uint8_t* const SB = stage + 3 * kStageA;                 // L_ki
+  uint8_t* const SA2 = stage + kStageBytes;                // (Y + Z)^T
+  uint8_t* const SB2 = stage + kStageBytes + 3 * kStageA;  // Linv
+  constexpr int kXSlot = 3 * kStageA;                      // triple of a 128 x 64 operand
+  static_assert(2 * kXSlot <= 4 * kOpSlot, "two X slots in the operand slots of two blocks");
+  const int mrow = dq * 32 + lane, ncol = dg * 16;
+  // operand rows r < 64 of a triple from a column-major source: element (r, l) =
+  // G[l * ld + r] for l < kvalid, zero elsewhere; consecutive threads take consecutive r
+  auto stage_cols = [&](uint8_t* h, const float* G, long long ld, int kvalid) {
+    const int r = tid & 63, ch = tid >> 6;
+    float xv[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) xv[q] = 8 * ch + q < kvalid ? __ldcg(G + (long long)(8 * ch + q) * ld + r) : 0.f;
+    put_split3_chunk(h, h + kOpPart, h + 2 * kOpPart, r, ch, xv);
+  };
+  // this thread's 16 values of row mrow as operand elements l = ncol .. of a 128-row triple
+  auto put_row = [&](uint8_t* h, const float (&x)[16]) {
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
       float xv[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int kk = 8 * ch + q;
-        float v = 0.f;
-        if (r < rvalid && kk < kvalid) {
-          v = __ldcg(G + (long long)kk * ld + r);
-          if (G2) v += __ldcg(G2 + (long long)kk * ld + r);
-        }
-        xv[q] = v;
-      }
-      put_split3_chunk(h, h + part, h + 2 * part, r, ch, xv);
+      for (int q = 0; q < 8; ++q) xv[q] = x[8 * half + q];
+      put_split3_chunk(h, h + kStageA, h + 2 * kStageA, mrow, ncol / 8 + half, xv);
     }
   };
-  auto run_mma = [&]() -> bool {
+  auto run_mma = [&](const uint8_t* A_, const uint8_t* B_, bool wait_x) -> bool {
     tc::fence_proxy_async_smem();
     __syncthreads();
     if (tid == 0) {
-      tc::fence_after_sync();
-      issue_mma(Ah, kStageA, Bh, kOpPart, qm);
+      if (!wait_x || tc::mbar_wait(&fullb[ql & 1], (ql >> 1) & 1, abp, stt)) {
+        tc::fence_after_sync();
+        issue_mma(A_, kStageA, B_, kOpPart, qm);
+      }
     }
     return wait_acc();
   };
-  auto z_unit = [&](int k, int i) {
-    const int k0 = k * NB, kb = min(NB, t - k0), i0 = i * NB;
-    const int mrow = dq * 32 + lane, ncol = dg * 16;
-    stage_cols(Ah, kStageA, 128, Xb + (long long)k0 * ldb, nullptr, ldb, nrhs, kb);
-    stage_cols(Bh, kOpPart, 64, Ab + (long long)k0 * t + i0, nullptr, t, 64, kb);
-    float* dst = Zb + (long long)(i0 + ncol) * ldb + mrow;   // block i < k is full
-    const bool ok = run_mma();
-    float v[16];
-    ld_slice(v);
-    if (ok && mrow < nrhs) {
-#pragma unroll
-      for (int c = 0; c < 16; ++c) red_sub(dst + (long long)c * ldb, v[c]);
-    }
+  auto mma_done = [&]() {   // the accumulator and its operands are free
     tc::fence_before_sync();
     __syncthreads();
     ++qm;
   };
-  auto x_unit = [&](int k) {
+  // X_k from y = Y_k + Z_k (this thread's 16 rows of column mrow) with Linv_k in SB2
+  auto form_x = [&](int k, const float (&y)[16]) {
     const int k0 = k * NB, kb = min(NB, t - k0);
-    const int mrow = dq * 32 + lane, ncol = dg * 16;
-    stage_cols(Ah, kStageA, 128, Bb + (long long)k0 * ldb, Zb + (long long)k0 * ldb, ldb, nrhs, kb);
-    stage_cols(Bh, kOpPart, 64, Lb + (long long)k * NB * NB, nullptr, NB, 64, NB);
-    const bool ok = run_mma();
+    put_row(SA2, y);
+    const bool ok = run_mma(SA2, SB2, false);
     float v[16];
     ld_slice(v);
+#pragma unroll
+    for (int c = 0; c < 16; ++c) v[c] = ok && ncol + c < kb ? v[c] : 0.f;
+    put_row(tb + (k & 1) * kXSlot, v);
     if (ok && mrow < nrhs) {
       float* dst = Xb + (long long)(k0 + ncol) * ldb + mrow;
 #pragma unroll
       for (int c = 0; c < 16; ++c)
         if (ncol + c < kb) dst[(long long)c * ldb] = v[c];
     }
-    tc::fence_before_sync();
-    __syncthreads();
-    ++qm;
+    asm volatile("fence.proxy.async;" ::: "memory");   // the slot, for the other CTAs' bulk copies
+    mma_done();
   };
-  if (rank == (nblk - 1) % kCL) x_unit(nblk - 1);
-  cluster_sync_all();
-  for (int k = nblk - 1; k >= 1; --k) {
-    // the owner of block k-1 finishes Z_{k-1} and forms X_{k-1}; the others share the rest
-    const int own = (k - 1) % kCL;
-    if (rank == own) {
-      z_unit(k, k - 1);
-      x_unit(k - 1);
-    } else {
-      for (int i = (rank - own - 1 + kCL) % kCL; i < k - 1; i += kCL - 1) z_unit(k, i);
+  auto load_yz = [&](int k, float (&y)[16], float (&z)[16]) {
+    const int k0 = k * NB, kb = min(NB, t - k0);
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+      const bool in = mrow < nrhs && ncol + c < kb;
+      const long long o = (long long)(k0 + ncol + c) * ldb + mrow;
+      y[c] = in ? __ldcg(Bb + o) : 0.f;
+      z[c] = in ? __ldcg(Zb + o) : 0.f;
     }
-    cluster_sync_all();
+  };
+  if (rank == (nblk - 1) % kCL) {
+    stage_cols(SB2, Lb + (long long)(nblk - 1) * NB * NB, NB, NB);
+    float y[16], z[16];
+    load_yz(nblk - 1, y, z);
+#pragma unroll
+    for (int c = 0; c < 16; ++c) y[c] += z[c];
+    form_x(nblk - 1, y);
   }
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  for (int k = nblk - 1; k >= 1; --k) {
+    const int k0 = k * NB, kb = min(NB, t - k0), own = (k - 1) % kCL;
+    const bool owner = rank == own;
+    // this CTA's first block of Z: k - 1 for its owner, the others share i < k - 1
+    int i = owner ? k - 1 : (rank - own - 1 + kCL) % kCL;
+    const bool any = owner || i < k - 1;
+    if (any) stage_cols(SB, Ab + (long long)k0 * t + i * NB, t, kb);
+    if (owner) stage_cols(SB2, Lb + (long long)(k - 1) * NB * NB, NB, NB);
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (any && tid == 0) {
+      asm volatile("fence.proxy.async;" ::: "memory");
+      tc::mbar_arrive_expect_tx(&fullb[ql & 1], kXSlot);
+      tc::bulk_load(SA, tb + (k & 1) * kXSlot, kXSlot, &fullb[ql & 1]);
+      ++issued;
+    }
+    if (owner) {
+      float y[16], z[16], v[16];
+      load_yz(k - 1, y, z);
+      const bool ok = run_mma(SA, SB, true);
+      ld_slice(v);
+#pragma unroll
+      for (int c = 0; c < 16; ++c) y[c] += ok ? z[c] - v[c] : z[c];
+      mma_done();
+      form_x(k - 1, y);
+    } else {
+      bool first = true;
+      for (; i < k - 1; i += kCL - 1) {
+        if (!first) stage_cols(SB, Ab + (long long)k0 * t + i * NB, t, kb);
+        const bool ok = run_mma(SA, SB, first);
+        float v[16];
+        ld_slice(v);
+        float* dst = Zb + (long long)(i * NB + ncol) * ldb + mrow;   // block i < k is full
+        if (ok && mrow < nrhs) {
+#pragma unroll
+          for (int c = 0; c < 16; ++c) red_sub(dst + (long long)c * ldb, v[c]);
+        }
+        mma_done();
+        first = false;
+      }
+    }
+    if (any) ++ql;
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  }
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (tid == 0 && bad) set_status(stt, ARCKV_ERR_NOT_SPD);
   release();
 }
