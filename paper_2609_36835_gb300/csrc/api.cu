@@ -393,9 +393,8 @@ arckv_status arckv_compact(const arckv_config* cfg, const void* K, const void* V
                               F(L.z), F(L.m), F(L.Y), B, beta, C_v, stt, st, ev);
   if (nlf < 0) return ARCKV_ERR_CUDA;
   nl += nlf;
-  nl += launch_check_finite(C_k, (long long)D.H * D.t * D.d, stt, st);
-  nl += launch_check_finite(beta, (long long)D.H * D.t, stt, st);
-  nl += launch_check_finite(C_v, (long long)D.H * D.t * D.d, stt, st);
+  nl += launch_check_finite(C_k, (long long)D.H * D.t * D.d, beta, (long long)D.H * D.t, C_v,
+                            (long long)D.H * D.t * D.d, stt, st);
   mark(ARCKV_NUM_STAGES);
   if (aux) {
     if (aux->scores && !given_anchors)

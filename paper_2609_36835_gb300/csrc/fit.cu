@@ -1483,17 +1483,22 @@ int launch_fits(const Dims& D, float scale, float ridge_w, float ridge_v, float 
   return nv < 0 ? -1 : nl + nv;
 }
 
-__global__ void check_finite_kernel(const float* x, long long count, DevStatus* stt) {
+// NaN or Inf in any of three arrays, one after another in the grid's stride
+__global__ void check_finite_kernel(const float* x, long long nx, const float* y, long long ny, const float* z,
+                                    long long nz, DevStatus* stt) {
   chain_wait();
   bool bad = false;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count;
-       k += (long long)gridDim.x * blockDim.x)
-    bad |= !isfinite(x[k]);
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+  for (long long k = i; k < nx; k += step) bad |= !isfinite(x[k]);
+  for (long long k = i; k < ny; k += step) bad |= !isfinite(y[k]);
+  for (long long k = i; k < nz; k += step) bad |= !isfinite(z[k]);
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) set_status(stt, ARCKV_ERR_NONFINITE);
 }
 
-int launch_check_finite(const float* x, long long count, DevStatus* stt, cudaStream_t st) {
-  launch_chained(check_finite_kernel, stride_grid(count, 256, 8), 256, 0, st, x, count, stt);
+int launch_check_finite(const float* x, long long nx, const float* y, long long ny, const float* z, long long nz,
+                        DevStatus* stt, cudaStream_t st) {
+  launch_chained(check_finite_kernel, stride_grid(std::max(nx, std::max(ny, nz)), 256, 8), 256, 0, st, x, nx, y, ny, z, nz,
+                 stt);
   return 1;
 }
 

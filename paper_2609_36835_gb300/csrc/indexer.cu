@@ -66,9 +66,7 @@ int launch_query_features(const Dims& D, const bf16* Q, const bf16* X, const bf1
   // vq = U_q q (exact products of bf16 inputs) and q'' = U_k^T vq, so that
   // (U_q q_i).(U_k k_j) = q''_i . k_j; both leave their GEMM as bf16 triples
   // (vq for the q'' product, q'' as the A operand of the value logits)
-  Dims Dw = D;
-  Dw.T = 128;
-  nl += launch_transpose_v(Dw, U_k, B.ukt, st);   // U_k^T [H][d][d_A]
+  nl += launch_query_operands(D, Q, L_q, L_c, U_k, B.qcat, B.wcat, B.ukt, st);
   bf16 *vq_h = B.vq3, *vq_m = B.vq3 + hn, *vq_l = B.vq3 + 2 * hn;
   int r = gemm_rows128(D, Q, nullptr, nullptr, U_q, TcEpiSplit3{vq_h, vq_m, vq_l, nd, 128}, stt, st);
   if (r < 0) return -1;
@@ -93,7 +91,7 @@ int launch_query_features(const Dims& D, const bf16* Q, const bf16* X, const bf1
   if (r < 0) return -1;
   nl += r;
   // q_bar = N(L_q q + L_c c) per block, as a split-bf16 pair
-  r = launch_query_proj_tc(D, Q, L_q, L_c, B.qcat, B.wcat, qbar_hi, qbar_lo, stt, st);
+  r = launch_query_proj_tc(D, B.qcat, B.wcat, qbar_hi, qbar_lo, stt, st);
   if (r < 0) return -1;
   nl += r;
   launch_chained(index_weights_kernel, dim3(D.n_pos, D.H), 32 * D.H_I, 0, st, X, L_x, b_x, wts, D.d_x, D.H_I, D.n_pos);

@@ -55,8 +55,11 @@ constexpr int kCholNB = 64;  // Cholesky block size
 // ---- indexer (Sec. 3.3, App. A.1) --------------------------------------
 // k_bar = N(L_k k + L_v v) per d_I block, as a split-bf16 pair (one tcgen05
 // GEMM over [K | V] against [L_k | L_v]).
-int launch_query_proj_tc(const Dims& D, const bf16* Q, const bf16* L_q, const bf16* L_c, bf16* qcat, bf16* wcat,
-                         bf16* qbar_hi, bf16* qbar_lo, DevStatus* stt, cudaStream_t st);
+int launch_query_proj_tc(const Dims& D, const bf16* qcat, const bf16* wcat, bf16* qbar_hi, bf16* qbar_lo,
+                         DevStatus* stt, cudaStream_t st);
+// the inputs' part of the query side's operands: qcat, wcat and U_k^T
+int launch_query_operands(const Dims& D, const bf16* Q, const bf16* L_q, const bf16* L_c, const bf16* U_k, bf16* qcat,
+                          bf16* wcat, bf16* ukt, cudaStream_t st);
 int launch_key_features_tc(const Dims& D, const bf16* K, const bf16* V, const bf16* L_k, const bf16* L_v,
                            bf16* kbar_hi, bf16* kbar_lo, DevStatus* stt, cudaStream_t st);
 // Scratch of the query-side features.
@@ -167,7 +170,8 @@ int launch_fits(const Dims& D, float scale, float ridge_w, float ridge_v, float 
                 float b_max, const bf16* Q, const float* C_k, const float* z, const float* m,
                 const float* Y, const FitBufs& B, float* beta, float* C_v, DevStatus* stt, cudaStream_t st,
                 cudaEvent_t const* ev = nullptr);
-int launch_check_finite(const float* x, long long count, DevStatus* stt, cudaStream_t st);
+int launch_check_finite(const float* x, long long nx, const float* y, long long ny, const float* z, long long nz,
+                        DevStatus* stt, cudaStream_t st);
 // (Gram + lam I) X = B for H fp32 systems of size t, lam = ridge trace(Gram) / t
 // (chol.cu): Gram [H][t][t] is overwritten by the factor (lower part), Linv
 // [H][ceil(t / 64)][64][64] by the inverses of its diagonal blocks; B, Z, X [H]

@@ -393,27 +393,22 @@ int launch_col_profiles(const Dims& D, const float* L, float* logphi, DevStatus*
   return col_profiles(D, L, logphi, ProfileOut{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, D.t, nullptr, nullptr, 0}, stt, st);
 }
 
-// kappa of the non-anchor keys from the argmax of their compacted rows
-// (rows c < T - t of head b; kmap gives the key)
-__global__ void decode_assign_kernel2(const unsigned long long* best, const int* kmap, int* kappa, int T, int Tm,
-                                      long long count) {
+// kappa of the non-anchor keys from the argmax of their compacted rows (rows c <
+// Tm of head b; kmap gives the key), then the anchors' own, kappa(s_r) = r
+__global__ void decode_assign_kernel(const unsigned long long* best, const int* kmap, const int* anchors, int* kappa,
+                                     int T, int Tm, int t, long long keys, long long total) {
   chain_wait();
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count;
-       k += (long long)gridDim.x * blockDim.x) {
-    const long long b = k / Tm, o = b * T + (k - b * Tm);
-    const unsigned long long v = best[o];
-    const int j = kmap[o];
-    if ((unsigned)j < (unsigned)T) kappa[b * T + j] = v ? (int)(0xffffffffu - (unsigned int)(v & 0xffffffffull)) : 0;
-  }
-}
-
-__global__ void anchor_self_assign_kernel2(const int* anchors, int* kappa, int T, int t, int H) {
-  chain_wait();
-  const long long total = (long long)H * t;
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total;
        k += (long long)gridDim.x * blockDim.x) {
-    const long long b = k / t;
-    kappa[b * T + anchors[k]] = (int)(k - b * t);
+    if (k < keys) {
+      const long long b = k / Tm, o = b * T + (k - b * Tm);
+      const unsigned long long v = best[o];
+      const int j = kmap[o];
+      if ((unsigned)j < (unsigned)T) kappa[b * T + j] = v ? (int)(0xffffffffu - (unsigned int)(v & 0xffffffffull)) : 0;
+    } else {
+      const long long a = k - keys, b = a / t;
+      kappa[b * T + anchors[a]] = (int)(a - b * t);
+    }
   }
 }
 
@@ -867,32 +862,31 @@ int launch_assign_gemm(const Dims& D, const int* anchors, const bf16* Ut_hi, con
       if (r < 0) return -1;
       nl += r - 1;
     } else {
-    // 128 keys x 256 anchors per tile (M = 128, N = 256 MMAs): half the key-side
-    // operand bytes per flop of a 128-wide tile.  The key map spans all T rows
-    // of a head (its plane stride); the GEMM takes the first Tm.
-    constexpr int BN = 256;
-    CUtensorMap mA, mA2, mB, mB2;
-    if (!encode_bf16_map_3d(&mA, Ut_hi, ldn, D.T, D.H, 128) || !encode_bf16_map_3d(&mA2, Ut_lo, ldn, D.T, D.H, 128) ||
-        !encode_bf16_map_3d(&mB, S_hi, ldn, D.t, D.H, BN) || !encode_bf16_map_3d(&mB2, S_lo, ldn, D.t, D.H, BN))
-      return -1;
-    TcEpiArgmax8 epi;
-    epi.best = best;
-    epi.bbs = D.T;
-    const int kfull = (ldn + 63) / 64 * 64;
-    // anchor tiles in groups whose split profiles (BN rows x ldn x 4 bytes per
-    // tile) take about 40 MB, so each group stays in L2 while the key profiles
-    // stream past it (one pass over them per group instead of one per wave)
-    const long long tile_bytes = (long long)BN * ldn * 4;
-    const int group = (int)std::max<long long>(1, (40LL << 20) / tile_bytes);
-    if (launch_tc_gemm<BN, kSplit>(mA, mB, mA2, mB2, epi, D.H, Tm, D.t, ldn, kfull, stt, st, 0, nullptr, group) !=
-        cudaSuccess)
-      return -1;
+      // 128 keys x 256 anchors per tile (M = 128, N = 256 MMAs): half the key-side
+      // operand bytes per flop of a 128-wide tile.  The key map spans all T rows
+      // of a head (its plane stride); the GEMM takes the first Tm.
+      constexpr int BN = 256;
+      CUtensorMap mA, mA2, mB, mB2;
+      if (!encode_bf16_map_3d(&mA, Ut_hi, ldn, D.T, D.H, 128) || !encode_bf16_map_3d(&mA2, Ut_lo, ldn, D.T, D.H, 128) ||
+          !encode_bf16_map_3d(&mB, S_hi, ldn, D.t, D.H, BN) || !encode_bf16_map_3d(&mB2, S_lo, ldn, D.t, D.H, BN))
+        return -1;
+      TcEpiArgmax8 epi;
+      epi.best = best;
+      epi.bbs = D.T;
+      const int kfull = (ldn + 63) / 64 * 64;
+      // anchor tiles in groups whose split profiles (BN rows x ldn x 4 bytes per
+      // tile) take about 40 MB, so each group stays in L2 while the key profiles
+      // stream past it (one pass over them per group instead of one per wave)
+      const long long tile_bytes = (long long)BN * ldn * 4;
+      const int group = (int)std::max<long long>(1, (40LL << 20) / tile_bytes);
+      if (launch_tc_gemm<BN, kSplit>(mA, mB, mA2, mB2, epi, D.H, Tm, D.t, ldn, kfull, stt, st, 0, nullptr, group) !=
+          cudaSuccess)
+        return -1;
     }
-    const long long cnt = (long long)D.H * Tm;
-    launch_chained(decode_assign_kernel2, stride_grid(cnt, 256, 8), 256, 0, st, best, kmap, kappa, D.T, Tm, cnt);
-    nl += 2;
   }
-  launch_chained(anchor_self_assign_kernel2, cdiv((long long)D.H * D.t, 256), 256, 0, st, anchors, kappa, D.T, D.t, D.H);
+  const long long keys = (long long)D.H * Tm, total = keys + (long long)D.H * D.t;
+  launch_chained(decode_assign_kernel, stride_grid(total, 256, 8), 256, 0, st, best, kmap, anchors, kappa, D.T,
+                 std::max(Tm, 1), D.t, keys, total);
   return nl;
 }
 

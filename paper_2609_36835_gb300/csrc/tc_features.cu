@@ -102,39 +102,62 @@ int launch_key_features_tc(const Dims& D, const bf16* K, const bf16* V, const bf
 // are concatenated along K as
 //   A = [q | c_h | c_m | c_l]  [n][4 * 128],   B = [L_q | L_c | L_c | L_c]  [HD][4 * 128]
 // and one plain GEMM gives L_q q + L_c (c_h + c_m + c_l) with exact bf16 products.
-// The c triple is written into A by the GEMM that forms c; qcat_kernel adds q.
-__global__ void __launch_bounds__(256) qcat_kernel(const bf16* Q, bf16* A, int n) {
+// The c triple is written into A by the GEMM that forms c; query_operands_kernel adds q.
+// One launch for what depends on the inputs alone: CTAs below nq copy q (16 rows
+// each), the next nw write two rows of W, the last 16 H transpose U_k by 32 x 32.
+__global__ void __launch_bounds__(256) query_operands_kernel(const bf16* Q, const bf16* L_q, const bf16* L_c,
+                                                             const bf16* U_k, bf16* A, bf16* W, bf16* ukt,
+                                                             long long qrows, long long wrows, int nq, int nw) {
   chain_wait();
-  const int b = blockIdx.y, i = blockIdx.x * 16 + (threadIdx.x >> 4), k = (threadIdx.x & 15) * 8;
-  if (i >= n) return;
-  const long long r = (long long)b * n + i;
-  *(uint4*)(A + r * 512 + k) = *(const uint4*)(Q + r * 128 + k);
-}
-__global__ void __launch_bounds__(256) wcat_kernel(const bf16* L_q, const bf16* L_c, bf16* W, long long rows) {
-  chain_wait();
-  const long long r = blockIdx.x * 2ll + (threadIdx.x >> 7);
-  const int k = threadIdx.x & 127;
-  if (r >= rows) return;
-  bf16* w = W + r * 512;
-  const bf16 c = L_c[r * 128 + k];
-  w[k] = L_q[r * 128 + k];
-  w[128 + k] = c;
-  w[256 + k] = c;
-  w[384 + k] = c;
+  int i = blockIdx.x;
+  if (i < nq) {
+    const long long r = i * 16ll + (threadIdx.x >> 4);
+    const int k = (threadIdx.x & 15) * 8;
+    if (r < qrows) *(uint4*)(A + r * 512 + k) = *(const uint4*)(Q + r * 128 + k);
+    return;
+  }
+  i -= nq;
+  if (i < nw) {
+    const long long r = i * 2ll + (threadIdx.x >> 7);
+    const int k = threadIdx.x & 127;
+    if (r >= wrows) return;
+    bf16* w = W + r * 512;
+    const bf16 c = L_c[r * 128 + k];
+    w[k] = L_q[r * 128 + k];
+    w[128 + k] = c;
+    w[256 + k] = c;
+    w[384 + k] = c;
+    return;
+  }
+  i -= nw;
+  __shared__ bf16 tile[32][34];
+  const long long b = i >> 4;
+  const int j0 = (i & 3) * 32, d0 = ((i >> 2) & 3) * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = ty; q < 32; q += 8) tile[q][tx] = U_k[(b * 128 + j0 + q) * 128 + d0 + tx];
+  __syncthreads();
+#pragma unroll
+  for (int q = ty; q < 32; q += 8) ukt[(b * 128 + d0 + q) * 128 + j0 + tx] = tile[tx][q];
 }
 
-int launch_query_proj_tc(const Dims& D, const bf16* Q, const bf16* L_q, const bf16* L_c, bf16* qcat, bf16* wcat,
-                         bf16* qbar_hi, bf16* qbar_lo, DevStatus* stt, cudaStream_t st) {
-  launch_chained(qcat_kernel, dim3(cdiv(D.n, 16), D.H), 256, 0, st, Q, qcat, D.n);
-  const long long wrows = (long long)D.H * D.HD;
-  launch_chained(wcat_kernel, (unsigned)cdiv(wrows, 2), 256, 0, st, L_q, L_c, wcat, wrows);
+int launch_query_operands(const Dims& D, const bf16* Q, const bf16* L_q, const bf16* L_c, const bf16* U_k, bf16* qcat,
+                          bf16* wcat, bf16* ukt, cudaStream_t st) {
+  const long long qrows = (long long)D.H * D.n, wrows = (long long)D.H * D.HD;
+  const int nq = cdiv(qrows, 16), nw = cdiv(wrows, 2);
+  launch_chained(query_operands_kernel, nq + nw + 16 * D.H, 256, 0, st, Q, L_q, L_c, U_k, qcat, wcat, ukt, qrows, wrows,
+                 nq, nw);
+  return 1;
+}
+
+int launch_query_proj_tc(const Dims& D, const bf16* qcat, const bf16* wcat, bf16* qbar_hi, bf16* qbar_lo,
+                         DevStatus* stt, cudaStream_t st) {
   CUtensorMap mA, mB;
   if (!encode_bf16_map_3d(&mA, qcat, 512, D.n, D.H, 128) || !encode_bf16_map_3d(&mB, wcat, 512, D.HD, D.H, 128))
     return -1;
   TcEpiBlockNorm epi{};
   if (!block_norm_epi(epi, qbar_hi, qbar_lo, D.H, D.n, D.HD)) return -1;
   if (launch_tc_gemm<128, kPlain>(mA, mB, mA, mB, epi, D.H, D.n, D.HD, 512, 512, stt, st) != cudaSuccess) return -1;
-  return 3;
+  return 1;
 }
 
 }  // namespace arckv

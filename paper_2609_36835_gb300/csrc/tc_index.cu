@@ -107,8 +107,10 @@ int launch_index_logits(const Dims& D, const bf16* qbar_hi, const bf16* qbar_lo,
                         cudaStream_t st) {
   CUtensorMap mA, mA2, mB, mB2;
   // 128 x 256 tiles (M = 128, N = 256 MMAs: a quarter fewer operand bytes per
-  // flop than 128 x 128) where T fills them; the key operand's box is 256 rows
-  const bool wide = D.T >= 256;
+  // flop than 128 x 128); the key operand's box is 256 rows.  A call whose 128-wide
+  // tiles fit the SMs in one wave is as long as one tile and takes those (1 head,
+  // n = 256, T = 1024: 25 us on 8 SMs with 256-wide tiles, 17 on 16).
+  const bool wide = (long long)D.H * cdiv(D.n, 128) * cdiv(D.T, 128) > tc_gemm_sm_count();
   const int bB = wide ? 256 : 128;
   if (!encode_bf16_map_3d(&mA, qbar_hi, D.HD, D.n, D.H, 128) || !encode_bf16_map_3d(&mA2, qbar_lo, D.HD, D.n, D.H, 128) ||
       !encode_bf16_map_3d(&mB, kbar_hi, D.HD, D.T, D.H, bB) || !encode_bf16_map_3d(&mB2, kbar_lo, D.HD, D.T, D.H, bB))
