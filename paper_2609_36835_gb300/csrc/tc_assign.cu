@@ -424,13 +424,15 @@ __global__ void decode_assign_kernel(const unsigned long long* best, const int* 
 // bound may hold the argmax.  The second pass computes the split products of
 // those (key, tile) pairs alone, with the MMA sequence of the full GEMM, so the
 // scores it compares, and the result, have the same bits.
-//   prefilter_kernel   (tc_gemm, kPlain, TcEpiFilter)  bounds per (key, tile)
+//   tc_gemm (kPlain, TcEpiFilter)  bounds per (key, tile)
 //   candidates_kernel  per (head, key chunk, tile): the list of its keys
-//   items_kernel       lists -> work items of 128 keys
+//   items_kernel       lists -> work items of 256 keys
 //   rescore_kernel     gathered keys x 128 anchors, argmax into `best`
 // Keys go in chunks whose profiles stay in L2 while all anchor tiles pass them
 // (a key is a candidate in 16 of 103 tiles on average at 128K).
-// 128K layer (t = 13107, n = 2048, 8 heads): 75.1 ms for the full GEMM.
+// 128K layer (t = 13107, n = 2048, 8 heads): 26.6 + 0.5 + 22.6 ms (filter, lists,
+// second pass); 75.1 ms for the full GEMM.
+constexpr int kRsKeys = 256;   // keys per work item of the second pass
 struct FilterDims {
   int Nt, Tp, CR, nch;   // anchor tiles, pitch of the bounds, keys per chunk, chunks
 };
@@ -456,21 +458,24 @@ static FilterLayout filter_layout(const Dims& D, const FilterDims& f) {
   L.list = take(E * f.CR * 4);
   L.cnt = take(E * 4);
   L.off = take((E + 1) * 4);
-  L.items = take(E * (f.CR / 128) * 4);
+  L.items = take(E * (f.CR / kRsKeys) * 4);
   L.rho_k = take((size_t)D.H * D.T * 4);
   L.rho_s = take((size_t)D.H * f.Nt * 128 * 4);
   L.total = o;
   return L;
 }
 // Where the filter is used: from 24 tiles of 128 anchors up (a tile of few is
-// more often a candidate: 0.15 of all (key, tile) pairs at t = 13107, 0.37 at
-// 1638, 0.39 at 819, and the passes cost 0.35 + 1.3 times that share of the
+// more often a candidate: 0.16 of all (key, tile) pairs at t = 13107, 0.37 at
+// 1638, 0.39 at 819, and the passes cost 0.35 + 1.9 times that share of the
 // full GEMM), when the bounds and lists fit the two halves of the index
-// features' buffer.
+// features' buffer.  ms, 8 heads, with the filter (indexer's, highest-attention
+// anchors) against the full GEMM: T = 16384, n = 1024, t = 3000 0.87, 0.92
+// against 1.01; T = 32768, n = 2048, t = 3276 3.7, 4.0 against 4.7; T = 49152,
+// n = 2048, t = 4915 8.3, 9.0 against 10.5.
 bool assign_filtered(const Dims& D) {
   const FilterDims f = filter_dims(D);
   const size_t half = (size_t)D.H * D.T * D.HD * 2;
-  return D.t > 23 * 128 && D.T - D.t >= 4096 && f.CR % 256 == 0 && (size_t)D.H * f.Nt * f.Tp * 8 <= half &&
+  return D.t > 23 * 128 && D.T - D.t >= 4096 && f.CR % kRsKeys == 0 && (size_t)D.H * f.Nt * f.Tp * 8 <= half &&
          filter_layout(D, f).total <= half;
 }
 
@@ -540,13 +545,13 @@ __global__ void __launch_bounds__(256) candidates_kernel(const float2* bounds, c
   }
 }
 
-// off = exclusive sums of the lists' 128-key blocks; items[i] = list * (CR / 128) + block.
+// off = exclusive sums of the lists' kRsKeys-key blocks; items[i] = list * (CR / kRsKeys) + block.
 __global__ void __launch_bounds__(1024) items_kernel(const int* cnt, int E, int per, int* off, int* items) {
   chain_wait();
   __shared__ int part[1024];
   const int tid = threadIdx.x, step = (E + 1023) / 1024, e0 = min(E, tid * step), e1 = min(E, e0 + step);
   int sum = 0;
-  for (int e = e0; e < e1; ++e) sum += (cnt[e] + 127) / 128;
+  for (int e = e0; e < e1; ++e) sum += (cnt[e] + kRsKeys - 1) / kRsKeys;
   part[tid] = sum;
   __syncthreads();
   for (int o = 1; o < 1024; o <<= 1) {
@@ -558,24 +563,29 @@ __global__ void __launch_bounds__(1024) items_kernel(const int* cnt, int E, int 
   int at = part[tid] - sum;
   for (int e = e0; e < e1; ++e) {
     off[e] = at;
-    const int nb = (cnt[e] + 127) / 128;
+    const int nb = (cnt[e] + kRsKeys - 1) / kRsKeys;
     for (int k = 0; k < nb; ++k) items[at + k] = e * per + k;
     at += nb;
   }
   if (tid == 1023) off[E] = part[1023];
 }
 
-// 128 gathered keys x 128 anchors per work item, split products over the whole
-// K in one accumulator, row argmax (lowest index on ties) merged into `best`.
-// Persistent, one CTA per SM: warp 0 streams the anchor slabs by TMA, warps 6-9
-// gather the keys' (16-byte cp.async into the same swizzled layout; a thread
-// serves one 16-byte chunk of four rows), warp 1 issues the MMAs, warps 2-5
-// drain the accumulators.  What bounds it is the latency of the gathered rows
-// against the 192 KB a CTA can have in flight, so the slabs are short (32 of K,
-// six stages, a slab handed over four later) and every role looks its next item
-// up while it works on the current one.
-constexpr int kRsStages = 6, kRsLag = 4, kRsK = 32;
-constexpr int kRsTile = 128 * kRsK * 2, kRsStage = 4 * kRsTile;   // [keys hi][anchors hi][keys lo][anchors lo]
+// 256 gathered keys x 128 anchors per work item (two M = 128 halves on the same
+// anchor slab; the second is left out when its list has no key for it), split
+// products over the whole K, row argmax (lowest index on ties) merged into
+// `best`.  Persistent, one CTA per SM: warp 0 streams the anchor slabs by TMA,
+// warps 6-9 gather the keys' (16-byte cp.async into the same swizzled layout; a
+// thread serves one 16-byte chunk of eight rows), warp 1 issues the MMAs, warps
+// 2-5 drain the accumulators.  What bounds it is the operand bytes from L2, so
+// an anchor slab serves as many keys as TMEM has accumulators for, in short
+// slabs (32 of K, four stages, a slab handed over kRsLag later: 22.6 ms of the
+// 128K layer; 1 later 23.8, 3 later, when the gather waits for the MMAs, 37), and
+// every role looks its next item up while it works on the current one.  With 128
+// keys an item (six stages) 26.6 ms.
+constexpr int kRsStages = 4, kRsLag = 2, kRsK = 32;
+constexpr int kRsTile = 128 * kRsK * 2;          // 128 rows of one part
+constexpr int kRsA = 2 * kRsTile;                // 256 keys of one part
+constexpr int kRsLo = kRsA + kRsTile, kRsStage = 2 * kRsLo;   // [keys hi][anchors hi][keys lo][anchors lo]
 constexpr int kRsThreads = 320;
 struct RsItem {
   int e, b, n0, k0, nkeys;   // list, head, first anchor, first key of the list, keys
@@ -591,7 +601,7 @@ __global__ void __launch_bounds__(kRsThreads, 1)
   const uint32_t raw = tc::smem_u32(smem_raw);
   uint8_t* base = smem_raw + (((raw + 1023u) & ~1023u) - raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nk = 2 * ((ldn + 63) / 64), per = f.CR / 128, E = H * f.nch * f.Nt;   // whole 64-wide slabs, as the full GEMM
+  const int nk = 2 * ((ldn + 63) / 64), per = f.CR / kRsKeys, E = H * f.nch * f.Nt;   // whole 64-wide slabs, as the full GEMM
   if (threadIdx.x == 0) {
     for (int s = 0; s < kRsStages; ++s) {
       tc::mbar_init(&full[s], 1 + 4);
@@ -606,7 +616,7 @@ __global__ void __launch_bounds__(kRsThreads, 1)
     tc::mbar_fence_init();
   }
   chain_wait();
-  if (warp == 1) tc::tmem_alloc(&tmem_slot, 256);
+  if (warp == 1) tc::tmem_alloc(&tmem_slot, 512);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -618,10 +628,10 @@ __global__ void __launch_bounds__(kRsThreads, 1)
     if (i < nitems) {
       const int v = items[i];
       x.e = v / per;
-      x.k0 = (v - x.e * per) * 128;
+      x.k0 = (v - x.e * per) * kRsKeys;
       x.b = x.e / (f.nch * f.Nt);
       x.n0 = (x.e % f.Nt) * 128;
-      x.nkeys = min(128, cnt[x.e] - x.k0);
+      x.nkeys = min(kRsKeys, cnt[x.e] - x.k0);
     }
     return x;
   };
@@ -644,8 +654,8 @@ __global__ void __launch_bounds__(kRsThreads, 1)
           }
           uint8_t* st = base + s * kRsStage;
           tc::mbar_arrive_expect_tx(&full[s], 2 * kRsTile);
-          tc::tma_load_3d(st + kRsTile, &mB, kb * kRsK, x.n0, x.b, &full[s]);
-          tc::tma_load_3d(st + 3 * kRsTile, &mB2, kb * kRsK, x.n0, x.b, &full[s]);
+          tc::tma_load_3d(st + kRsA, &mB, kb * kRsK, x.n0, x.b, &full[s]);
+          tc::tma_load_3d(st + kRsLo + kRsA, &mB2, kb * kRsK, x.n0, x.b, &full[s]);
         }
       }
       // every issued copy lands before the CTA may exit: the last slabs' barriers
@@ -666,7 +676,8 @@ __global__ void __launch_bounds__(kRsThreads, 1)
         const int buf = c & 1;
         if (c >= 2 && !tc::mbar_wait(&acce[buf], ((c >> 1) - 1) & 1, abortp, stt)) break;
         tc::fence_after_sync();
-        const uint32_t d = tmem + (uint32_t)(buf * 128);
+        const uint32_t d = tmem + (uint32_t)(buf * 256);
+        const int halves = x.nkeys > 128 ? 2 : 1;
         for (int kb = 0; kb < nk; ++kb, ++g) {
           const int s = g % kRsStages;
           if (!tc::mbar_wait(&full[s], (g / kRsStages) & 1, abortp, stt)) {
@@ -674,13 +685,16 @@ __global__ void __launch_bounds__(kRsThreads, 1)
             break;
           }
           tc::fence_after_sync();
-          const uint32_t a = tc::smem_u32(base + s * kRsStage), bb = a + kRsTile;
+          const uint32_t bb = tc::smem_u32(base + s * kRsStage) + kRsA;
+          for (int h = 0; h < halves; ++h) {
+            const uint32_t a = bb - kRsA + h * kRsTile, dh = d + h * 128;
 #pragma unroll
-          for (int ks = 0; ks < kRsK / 16; ++ks) {   // the sequence of tc_gemm's kSplit
-            const uint64_t ad = tc::sdesc_k64(a + ks * 32), bd = tc::sdesc_k64(bb + ks * 32);
-            tc::mma_f16(d, ad, bd, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
-            tc::mma_f16(d, ad, tc::sdesc_k64(bb + 2 * kRsTile + ks * 32), idesc, 1u);
-            tc::mma_f16(d, tc::sdesc_k64(a + 2 * kRsTile + ks * 32), bd, idesc, 1u);
+            for (int ks = 0; ks < kRsK / 16; ++ks) {   // the sequence of tc_gemm's kSplit
+              const uint64_t ad = tc::sdesc_k64(a + ks * 32), bd = tc::sdesc_k64(bb + ks * 32);
+              tc::mma_f16(dh, ad, bd, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+              tc::mma_f16(dh, ad, tc::sdesc_k64(bb + kRsLo + ks * 32), idesc, 1u);
+              tc::mma_f16(dh, tc::sdesc_k64(a + kRsLo + ks * 32), bd, idesc, 1u);
+            }
           }
           tc::mma_commit(&empty[s]);
         }
@@ -697,43 +711,46 @@ __global__ void __launch_bounds__(kRsThreads, 1)
     for (int i = blockIdx.x; i < nitems; i += gridDim.x, ++c) {
       const RsItem x = item(i);   // (in the shadow of the item's MMAs)
       const int r = q * 32 + lane, n0 = x.n0, b = x.b;
-      const int key = r < x.nkeys ? list[(long long)x.e * f.CR + x.k0 + r] : -1;
+      const int* lk = list + (long long)x.e * f.CR + x.k0;
+      const int key[2] = {r < x.nkeys ? lk[r] : -1, r + 128 < x.nkeys ? lk[r + 128] : -1};
       ok = tc::mbar_wait(&accf[c & 1], (c >> 1) & 1, abortp, stt);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc::fence_after_sync();
-      float bv = -INFINITY;
-      int bi = -1;
+      float bv[2] = {-INFINITY, -INFINITY};
+      int bi[2] = {-1, -1};
       const int ncols = t - n0;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float v[32];
-        tc::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((c & 1) * 128 + j * 32), v);
+      for (int h = 0; h < 2; ++h) {
+        if (h * 128 >= x.nkeys) continue;
 #pragma unroll
-        for (int k = 0; k < 32; ++k)
-          if (j * 32 + k < ncols && v[k] > bv) {
-            bv = v[k];
-            bi = n0 + j * 32 + k;
-          }
+        for (int j = 0; j < 4; ++j) {
+          float v[32];
+          tc::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((c & 1) * 256 + h * 128 + j * 32), v);
+#pragma unroll
+          for (int k = 0; k < 32; ++k)
+            if (j * 32 + k < ncols && v[k] > bv[h]) {
+              bv[h] = v[k];
+              bi[h] = n0 + j * 32 + k;
+            }
+        }
       }
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&acce[c & 1]);
-      if (key >= 0 && bi >= 0)
-        atomicMax(best + (long long)b * T + key,
-                  ((unsigned long long)f32_ordered(bv) << 32) | (unsigned long long)(0xffffffffu - (unsigned int)bi));
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (key[h] >= 0 && bi[h] >= 0)
+          atomicMax(best + (long long)b * T + key[h], ((unsigned long long)f32_ordered(bv[h]) << 32) |
+                                                          (unsigned long long)(0xffffffffu - (unsigned int)bi[h]));
     }
   } else {
     // gather: 16-byte chunk `ch` of rows rr, rr + 32, .. of the key tiles; a
     // slab is handed over kRsLag slabs later, when its copies have landed
     const int p = threadIdx.x - 192, ch = p & 3, rr = p >> 2;
     const long long lo = Ut_lo - Ut_hi;
-    uint32_t dst[4];   // 64-byte swizzle: chunk ch of row r at ch ^ (r / 2 % 4)
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int r = rr + 32 * u;
-      dst[u] = (uint32_t)(r * 64 + ((ch ^ ((r >> 1) & 3)) << 4));
-    }
+    // 64-byte swizzle: chunk ch of row r at ch ^ (r / 2 % 4); rows rr + 32 u keep rr's
+    const uint32_t dst = (uint32_t)(rr * 64 + ((ch ^ ((rr >> 1) & 3)) << 4));
     int g = 0;
     bool ok = true;
     auto hand_over = [&](int q) {   // slab q's copies are complete
@@ -742,21 +759,22 @@ __global__ void __launch_bounds__(kRsThreads, 1)
       if (lane == 0) tc::mbar_arrive(&full[q % kRsStages]);
     };
     // rows past the list's end repeat its first (their results are dropped)
-    auto keys_of = [&](const RsItem& x, int (&key)[4]) {
+    auto keys_of = [&](const RsItem& x, int (&key)[8]) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < 8; ++u) {
         const int r = rr + 32 * u;
         key[u] = x.nkeys > 0 ? list[(long long)x.e * f.CR + x.k0 + (r < x.nkeys ? r : 0)] : 0;
       }
     };
     RsItem x = item(blockIdx.x);
-    int key[4];
+    int key[8];
     keys_of(x, key);
     for (int i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
-      const bf16* src[4];
+      const bf16* src[8];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) src[u] = Ut_hi + ((long long)x.b * T + key[u]) * ldn + ch * 8;
+      for (int u = 0; u < 8; ++u) src[u] = Ut_hi + ((long long)x.b * T + key[u]) * ldn + ch * 8;
       RsItem nx = item(i + gridDim.x);
+      const bool both = x.nkeys > 128;
       for (int kb = 0; kb < nk; ++kb, ++g) {
         if (kb == nk / 2) keys_of(nx, key);
         const int s = g % kRsStages;
@@ -767,13 +785,18 @@ __global__ void __launch_bounds__(kRsThreads, 1)
         }
         const uint32_t st = tc::smem_u32(base + s * kRsStage);
         const int n16 = kb * kRsK + ch * 8 < ldn ? 16 : 0;   // past the row's end: zeros
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        auto copy = [&](int u) {
           const bf16* y = src[u] + (n16 ? kb * kRsK : 0);
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(st + dst[u]), "l"(y), "r"(n16) : "memory");
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(st + 2 * kRsTile + dst[u]), "l"(y + lo),
-                       "r"(n16)
+          const uint32_t to = st + dst + u * 2048;
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(y), "r"(n16) : "memory");
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to + kRsLo), "l"(y + lo), "r"(n16)
                        : "memory");
+        };
+#pragma unroll
+        for (int u = 0; u < 4; ++u) copy(u);
+        if (both) {
+#pragma unroll
+          for (int u = 4; u < 8; ++u) copy(u);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
         if (g >= kRsLag) {
@@ -790,7 +813,7 @@ __global__ void __launch_bounds__(kRsThreads, 1)
   __syncthreads();
   if (warp == 1) {
     tc::fence_after_sync();
-    tc::tmem_dealloc(tmem, 256);
+    tc::tmem_dealloc(tmem, 512);
   }
 }
 
@@ -837,7 +860,7 @@ static int filtered_argmax(const Dims& D, const bf16* Ut_hi, const bf16* Ut_lo, 
   // the two passes take 4 n / 16 of them
   const float B0 = 0x1p-15f + (float)D.n * 0x1p-22f;
   launch_chained(candidates_kernel, dim3(cdiv(Tm, 256), D.H), 256, 0, st, bounds, rho_k, B0, D.T, Tm, f, list, cnt);
-  launch_chained(items_kernel, 1, 1024, 0, st, cnt, E, f.CR / 128, off, items);
+  launch_chained(items_kernel, 1, 1024, 0, st, cnt, E, f.CR / kRsKeys, off, items);
   const int smem = kRsStages * kRsStage + 1024;
   if (set_dyn_smem((const void*)rescore_kernel, smem) != cudaSuccess) return -1;
   if (launch_chained(rescore_kernel, tc_gemm_sm_count(), kRsThreads, smem, st, mC, mC2, Ut_hi, Ut_lo, list, cnt, off,
