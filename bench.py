@@ -596,27 +596,32 @@ def run_gpu(args, dist: Dist):
         for k in range(pk.NUM_STAGES):
             iso_ms[k].append(iso_ev[k].elapsed_time(iso_ev[k + 1]))
 
-    # roofline of the dominant kernel: the assignment GEMM (Eq. anchor_assignment,
-    # one launch per layer, stage 5), a split-bf16 tcgen05 GEMM issuing three
-    # bf16 MMAs per useful product; 2 n (T - t) t useful flops per head (the
-    # anchors' own assignment is fixed, kappa(s_r) = r: the launch scores the
-    # T - t other keys against the t anchors)
+    # roofline of the dominant stage: the assignment (Eq. anchor_assignment,
+    # stage 5), 2 n (T - t) t useful flops per head (the anchors' own assignment
+    # is fixed, kappa(s_r) = r: the T - t other keys are scored against the t
+    # anchors).  One split-bf16 tcgen05 GEMM issuing three bf16 MMAs per useful
+    # product, or, from 24 anchor tiles up (tc_assign.cu, assign_filtered), a
+    # one-product filter over all pairs and split products over those that it
+    # leaves: how many those are depends on the data, so no issued rate is given
+    filtered = tp > 23 * 128 and w.T - tp >= 4096
     flops = 2.0 * w.H_kv * w.n * (w.T - tp) * tp
     avg_s = statistics.mean(stage_launch_ms[5]) / 1e3
     iso_s = statistics.median(iso_ms[5]) / 1e3
     peak, _, peak_src = measured_peaks()
     burst = measured_burst()
     achieved = flops / avg_s / 1e12
-    roofline = {"kernel": "tc_gemm_kernel<256, kSplit, TcEpiArgmax8> (assignment, Eq. anchor_assignment)",
+    roofline = {"kernel": ("tc_gemm_kernel<256, kPlain, TcEpiFilter> + rescore_kernel" if filtered else
+                           "tc_gemm_kernel<256, kSplit, TcEpiArgmax8>") + " (assignment, Eq. anchor_assignment)",
                 "bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": profiled_traffic(), "flops_per_launch": flops, "launch_ms": avg_s * 1e3,
-                "issued_tflops": 3.0 * achieved, "issued_frac": 3.0 * achieved / peak,
+                "issued_tflops": None if filtered else 3.0 * achieved,
+                "issued_frac": None if filtered else 3.0 * achieved / peak,
                 "launch_ms_isolated": iso_s * 1e3, "frac_isolated": flops / iso_s / 1e12 / burst,
                 "timing_note": "launch_ms: live CUDA events over the timed region, where %d streams share the GPU; "
                                "launch_ms_isolated: the same launch with the GPU to itself (median of 5), "
                                "frac_isolated against the burst peak" % n_str,
                 "peak_note": "bf16 dense, sustained, of %s (MEASURED_PEAKS.json); achieved counts useful flops, "
-                             "issued counts the 3 bf16 MMAs of each split-bf16 product" % peak_src}
+                             "issued (null with the filter) the 3 bf16 MMAs of each split-bf16 product" % peak_src}
     # the solvers of the two fits (stages 8 and 10), timed the same way
     dual = tp > w.n
     m_sys = w.n if dual else tp
@@ -635,7 +640,7 @@ def run_gpu(args, dist: Dist):
                                                "diagonal factors, 5-slice tensor-core block products "
                                                "(sliced_gemm_kernel<5>); the 4-slice Grams and back-projection "
                                                "are counted outside" if dual else
-                                               "chol_cluster_kernel<float, 4|8> (tcgen05 trailing updates) "
+                                               "chol_tc_kernel<4|8|12|16> (tcgen05 trailing updates) "
                                                "+ two refinement steps"),
                                note="Cholesky m^3 / 3 plus the triangular solves (m = %d, 1 and 128 right-hand "
                                     "sides), against the bf16 burst peak; vs_fp64_gemm against this GPU's own "
@@ -812,7 +817,7 @@ def run_decode(args, dist: Dist):
         "config": {"workload": "decode step: 64 sequences x 8 KV heads x 4 query rows, head_dim 128, t = 0.2 T",
                    "l2": "inputs larger than L2 at every context; calls back to back"},
         "contexts": rows,
-        "roofline": {"kernel": "attend_bulk_kernel (split-key decode attention, bulk-copy K/V ring)", "bound": "hbm",
+        "roofline": {"kernel": "attend_warp_kernel (split-key decode attention, a bulk-copy K/V ring per warp)", "bound": "hbm",
                      "achieved": last["compact_gbs"], "peak": hbm_peak, "unit": "GB/s",
                      "frac": last["compact_frac"], "traffic": None,
                      "peak_note": "HBM copy bandwidth, of %s (MEASURED_PEAKS.json)" % peak_src},

@@ -576,12 +576,14 @@ __global__ void __launch_bounds__(1024) items_kernel(const int* cnt, int E, int 
 // `best`.  Persistent, one CTA per SM: warp 0 streams the anchor slabs by TMA,
 // warps 6-9 gather the keys' (16-byte cp.async into the same swizzled layout; a
 // thread serves one 16-byte chunk of eight rows), warp 1 issues the MMAs, warps
-// 2-5 drain the accumulators.  What bounds it is the operand bytes from L2, so
-// an anchor slab serves as many keys as TMEM has accumulators for, in short
-// slabs (32 of K, four stages, a slab handed over kRsLag later: 22.6 ms of the
-// 128K layer; 1 later 23.8, 3 later, when the gather waits for the MMAs, 37), and
-// every role looks its next item up while it works on the current one.  With 128
-// keys an item (six stages) 26.6 ms.
+// 2-5 drain the accumulators.  What bounds it is the latency of the gathered
+// rows against the 192 KB a CTA can have in flight, so an anchor slab serves as
+// many keys as TMEM has accumulators for, in short slabs (32 of K, four stages, a
+// slab handed over kRsLag later: 22.6 ms of the 128K layer; 1 later 23.8, 3
+// later, when the gather waits for the MMAs, 37), and every role looks its next
+// item up while it works on the current one.  With 128 keys an item (six stages)
+// 26.6 ms.  86 GB of DRAM reads at 128K: the key chunks of 48 MB are read again
+// by part, but chunks of 16 to 160 MB stay within 7 % of this time.
 constexpr int kRsStages = 4, kRsLag = 2, kRsK = 32;
 constexpr int kRsTile = 128 * kRsK * 2;          // 128 rows of one part
 constexpr int kRsA = 2 * kRsTile;                // 256 keys of one part
