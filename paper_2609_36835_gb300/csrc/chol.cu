@@ -304,10 +304,9 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
       tc::fence_before_sync();
       ++qm;
       if (tid == 0) tc::bulk_wait_all();   // the slot is written
-      __syncwarp();
-      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      cluster_arrive();
       factor_diag<float>(Ab, Lb, t, k + 1, S1, S2, S3, &bad);
-      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      cluster_wait();
     } else {
       // panel tiles x = 1 .. m-1 (block rows k+1+x; x = 0 is the owner's) and the nct tiles of Y_k
       const int x0 = m > 0 ? 1 : 0, nx = m + nct;
@@ -451,12 +450,12 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
       for (int rk = part; rk < kCL; rk += 8) cl.map_shared_rank(&xs[0][0], rk)[(k % 3) * NB + c] = a;
     };
     if (rank == (nblk - 1) % kCL) form_x(nblk - 1);
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    cluster_arrive();
     for (int k = nblk - 1; k >= 1; --k) {
       const int k0 = k * NB, kb = min(NB, t - k0);
       const bool next = rank == (k - 1) % kCL;
       if (next) ld_tile(S1, (const float*)Ab, (long long)t, k0, k0 - NB, kb, NB, false);   // L_k,k-1
-      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      cluster_wait();
       const float* xk = xs[k % 3];
       if (next) {
         __syncthreads();
@@ -469,8 +468,7 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
         __syncthreads();
         form_x(k - 1);
       }
-      __syncwarp();
-      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      cluster_arrive();
       // this rank's other blocks j < k - 1, 64 threads each
       for (int j = rank + kCL * (tid >> 6); j < k - 1; j += kCL * (kCT / NB)) {
         const int c = tid & 63;
@@ -482,7 +480,7 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
       }
       __syncthreads();
     }
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // nobody leaves before the last write to its xs
+    cluster_wait();   // nobody leaves before the last write to its xs
     if (tid == 0 && bad) set_status(stt, ARCKV_ERR_NOT_SPD);
     release();
     return;
@@ -576,8 +574,7 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
     for (int c = 0; c < 16; ++c) y[c] += z[c];
     form_x(nblk - 1, y);
   }
-  __syncwarp();
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  cluster_arrive();
   for (int k = nblk - 1; k >= 1; --k) {
     const int k0 = k * NB, kb = min(NB, t - k0), own = (k - 1) % kCL;
     const bool owner = rank == own;
@@ -586,7 +583,7 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
     const bool any = owner || i < k - 1;
     if (any) stage_cols(SB, Ab + (long long)k0 * t + i * NB, t, kb);
     if (owner) stage_cols(SB2, Lb + (long long)(k - 1) * NB * NB, NB, NB);
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_wait();
     if (any && tid == 0) {
       asm volatile("fence.proxy.async;" ::: "memory");
       tc::mbar_arrive_expect_tx(&fullb[ql & 1], kXSlot);
@@ -619,10 +616,9 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kCT, 1)
       }
     }
     if (any) ++ql;
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    cluster_arrive();
   }
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_wait();
   if (tid == 0 && bad) set_status(stt, ARCKV_ERR_NOT_SPD);
   release();
 }

@@ -127,8 +127,20 @@ __device__ __forceinline__ R warp_sum_r(R v) {
   return v;
 }
 
+// The .aligned forms want the warp's threads together.  They often follow a loop
+// or a branch that lanes leave at different times, and reconvergence after one
+// is not promised, so each begins with a __syncwarp().
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 __device__ __forceinline__ unsigned cluster_rank() {
   unsigned r;
