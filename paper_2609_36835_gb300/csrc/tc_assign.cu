@@ -885,7 +885,7 @@ int launch_assign_gemm(const Dims& D, const int* anchors, const bf16* Ut_hi, con
     if (filter_scratch) {
       const int r = filtered_argmax(D, Ut_hi, Ut_lo, S_hi, S_lo, filter_bounds, filter_scratch, best, stt, st);
       if (r < 0) return -1;
-      nl += r - 1;
+      nl += r;
     } else {
       // 128 keys x 256 anchors per tile (M = 128, N = 256 MMAs): half the key-side
       // operand bytes per flop of a 128-wide tile.  The key map spans all T rows
@@ -907,6 +907,7 @@ int launch_assign_gemm(const Dims& D, const int* anchors, const bf16* Ut_hi, con
       if (launch_tc_gemm<BN, kSplit>(mA, mB, mA2, mB2, epi, D.H, Tm, D.t, ldn, kfull, stt, st, 0, nullptr, group) !=
           cudaSuccess)
         return -1;
+      ++nl;
     }
   }
   const long long keys = (long long)D.H * Tm, total = keys + (long long)D.H * D.t;
