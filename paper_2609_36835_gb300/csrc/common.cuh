@@ -26,7 +26,10 @@ __device__ __forceinline__ void set_status(DevStatus* st, unsigned int code) {
 // programmatic stream serialisation (launch_chained), so that a kernel's CTAs
 // are set up while the last ones of the kernel before still run, and begin with
 // chain_wait(): it returns when that kernel has completed and its writes are
-// visible.  Nothing but a CTA's own shared memory is touched before it.  1 head,
+// visible.  Nothing but a CTA's own shared memory is touched before it, and what
+// another kernel of the call writes is not read-only while this one runs: no
+// __ldg and no const __restrict__ parameter for it, either of which lets loads
+// take the non-coherent path and be moved above the wait.  1 head,
 // T = 1024 (53 launches): 600 -> 478 us; 8 heads, T = 20011 (226): 3.63 -> 3.25 ms.
 // (Releasing the next kernel at the start of this one as well is slower, 501 us
 // and 3.61 ms: its waiting CTAs hold threads and shared memory that this kernel's

@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(256) chol_back_block_kernel(const double* Linv
 // and sixteen rows of Phi are in flight per thread (128 threads a CTA: at t = 2001
 // the columns fill the SMs).
 constexpr int kPtThreads = 128;
-__global__ void __launch_bounds__(kPtThreads) phi_t_vec_kernel(const float* __restrict__ Phi, const double* __restrict__ a,
+__global__ void __launch_bounds__(kPtThreads) phi_t_vec_kernel(const float* Phi, const double* a,
                                                         float* __restrict__ w, int n, int t) {
   chain_wait();
   __shared__ float ah[1024], al[1024];
@@ -655,8 +655,8 @@ __global__ void __launch_bounds__(kPtThreads) phi_t_vec_kernel(const float* __re
 // runs the same fixed trip counts, so every cluster barrier is reached by all.
 constexpr int kTsCL = 8;
 __global__ void __cluster_dims__(kTsCL, 1, 1) __launch_bounds__(256, 1)
-    tri_solve_cluster_kernel(const double* __restrict__ A, const double* __restrict__ Linv,
-                             const double* __restrict__ r, double* __restrict__ yd, double* __restrict__ x, int n) {
+    tri_solve_cluster_kernel(const double* A, const double* Linv,
+                             const double* r, double* __restrict__ yd, double* __restrict__ x, int n) {
   chain_wait();
   namespace cg = cooperative_groups;
   __shared__ double red[kTsCL][NB];   // rank 0: the ranks' partial sums
@@ -983,8 +983,8 @@ static int fits_dual(const Dims& D, float ridge_w, float ridge_v, float eps_w, f
 // u[b][i] = m_i - sum_r Phi_ir x_r (fp64); with sq, also sq[b][i] = sum_r Phi_ir^2.
 // One warp per row, eight loads in flight per lane; x is widened once per CTA.
 constexpr int kIrTile = 2048;   // columns of x in shared memory at a time
-__global__ void __launch_bounds__(256) ir_rows_kernel(const float* __restrict__ Phi, const float* __restrict__ m,
-                                                      const float* __restrict__ x, double* __restrict__ u,
+__global__ void __launch_bounds__(256) ir_rows_kernel(const float* Phi, const float* m,
+                                                      const float* x, double* __restrict__ u,
                                                       double* __restrict__ sq, int n, int t) {
   chain_wait();
   __shared__ double xd[kIrTile];
@@ -1028,7 +1028,7 @@ __global__ void __launch_bounds__(256) ir_rows_kernel(const float* __restrict__ 
 }
 
 // lam[b] = ridge * sum_i sq[b][i] / t, summed in a fixed order (one CTA per head).
-__global__ void __launch_bounds__(256) ir_lambda_kernel(const double* __restrict__ sq, double* __restrict__ lam, int n,
+__global__ void __launch_bounds__(256) ir_lambda_kernel(const double* sq, double* __restrict__ lam, int n,
                                                         int t, double ridge) {
   chain_wait();
   __shared__ double red[8];
@@ -1051,8 +1051,8 @@ __global__ void __launch_bounds__(256) ir_lambda_kernel(const double* __restrict
 // row phases of four chains each: chain q of phase w takes the rows w + 8 q +
 // 32 j, chain 0 also what is left below n.  The chains of a phase are added,
 // then the phases in order.
-__global__ void __launch_bounds__(1024) ir_cols_kernel(const float* __restrict__ Phi, const double* __restrict__ u,
-                                                       const float* __restrict__ x, const double* __restrict__ lam,
+__global__ void __launch_bounds__(1024) ir_cols_kernel(const float* Phi, const double* u,
+                                                       const float* x, const double* lam,
                                                        float* __restrict__ r, int n, int t) {
   chain_wait();
   __shared__ double part[32][32];
@@ -1124,8 +1124,8 @@ __device__ __forceinline__ void st_remote(const float* p, const uint64_t* bar, i
       : "memory");
 }
 __global__ void __cluster_dims__(kTriCL, 1, 1) __launch_bounds__(512, 1)
-    tri_solve_cluster32_kernel(const float* __restrict__ A, const float* __restrict__ Linv,
-                               const float* __restrict__ r, float* __restrict__ x, int t, DevStatus* stt) {
+    tri_solve_cluster32_kernel(const float* A, const float* Linv,
+                               const float* r, float* __restrict__ x, int t, DevStatus* stt) {
   chain_wait();
   extern __shared__ __align__(16) float psm[];   // two panel slices [2 nblk][4][64]
   __shared__ float yv[kTriMaxT];                 // y, then d block by block
@@ -1285,8 +1285,8 @@ __global__ void __cluster_dims__(kTriCL, 1, 1) __launch_bounds__(512, 1)
 // Serves the refinement steps beyond kTriMaxT, where a rank's sums and panel
 // slices no longer fit.
 template <typename R>
-__global__ void __launch_bounds__(512) tri_solve_kernel(const R* __restrict__ A, const R* __restrict__ Linv,
-                                                        const R* __restrict__ r, R* __restrict__ yd,
+__global__ void __launch_bounds__(512) tri_solve_kernel(const R* A, const R* Linv,
+                                                        const R* r, R* __restrict__ yd,
                                                         R* __restrict__ x, int t) {
   chain_wait();
   constexpr int NBk = kCholNB;

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(1024) group_sort_kernel(const int* kappa, int 
 // slot in group-major, chunk-minor order, and each chunk then scatters its
 // positions in ascending order from those slots.  perm and goff come out
 // identical to group_sort_kernel's.  cnt is [H][t][C], C = ceil(T / kSortChunk).
-__global__ void __launch_bounds__(1024) sort_hist_kernel(const int* __restrict__ kappa, int T, int t, int C,
+__global__ void __launch_bounds__(1024) sort_hist_kernel(const int* kappa, int T, int t, int C,
                                                          int* __restrict__ cnt) {
   chain_wait();
   extern __shared__ int hist[];
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(1024) sort_hist_kernel(const int* __restrict__
 }
 
 // tot[b][g] = sum over chunks of cnt[b][g][.]
-__global__ void __launch_bounds__(256) sort_totals_kernel(const int* __restrict__ cnt, int t, int C, int H,
+__global__ void __launch_bounds__(256) sort_totals_kernel(const int* cnt, int t, int C, int H,
                                                           int* __restrict__ tot) {
   chain_wait();
   const long long gi = (long long)blockIdx.x * 256 + threadIdx.x;
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(256) sort_totals_kernel(const int* __restrict_
 }
 
 // goff[b] = exclusive scan of tot[b] (one CTA per head); goff[b][t] = T
-__global__ void __launch_bounds__(1024) sort_scan_kernel(const int* __restrict__ tot, int t, int* __restrict__ goff,
+__global__ void __launch_bounds__(1024) sort_scan_kernel(const int* tot, int t, int* __restrict__ goff,
                                                          int* __restrict__ big, int T) {
   chain_wait();
   __shared__ int sc[32];
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(1024) sort_scan_kernel(const int* __restrict__
 }
 
 // cnt[b][g][c] <- the first slot of chunk c's members of group g
-__global__ void __launch_bounds__(256) sort_slots_kernel(int* __restrict__ cnt, const int* __restrict__ goff, int t,
+__global__ void __launch_bounds__(256) sort_slots_kernel(int* __restrict__ cnt, const int* goff, int t,
                                                          int C, int H) {
   chain_wait();
   const long long gi = (long long)blockIdx.x * 256 + threadIdx.x;
@@ -210,8 +210,8 @@ __global__ void __launch_bounds__(256) sort_slots_kernel(int* __restrict__ cnt, 
 }
 
 // each chunk's positions, ascending, to their groups' slots
-__global__ void __launch_bounds__(1024) sort_scatter_kernel(const int* __restrict__ kappa, int T, int t, int C,
-                                                            const int* __restrict__ cnt, int* __restrict__ perm) {
+__global__ void __launch_bounds__(1024) sort_scatter_kernel(const int* kappa, int T, int t, int C,
+                                                            const int* cnt, int* __restrict__ perm) {
   chain_wait();
   extern __shared__ int cur[];
   const int c = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -252,10 +252,10 @@ constexpr int kMergeWarpMax = 128;
 // costs two dependent round trips, and one CTA per group left the largest group
 // to a single SM, 64 us of an 8K layer and 0.24 ms of a 32K one.
 constexpr int kBigParts = 4, kBigCtas = 64, kB = 16;
-__global__ void __launch_bounds__(256) group_merge_cta_kernel(const bf16* __restrict__ K, const int* __restrict__ anchors,
-                                                              const int* __restrict__ perm, const int* __restrict__ goff,
-                                                              const float* __restrict__ logphi, float lambda_m,
-                                                              float* C_k, const int* __restrict__ big, int T, int t) {
+__global__ void __launch_bounds__(256) group_merge_cta_kernel(const bf16* K, const int* anchors,
+                                                              const int* perm, const int* goff,
+                                                              const float* logphi, float lambda_m,
+                                                              float* C_k, const int* big, int T, int t) {
   chain_wait();
   const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int* pb = perm + (long long)b * T;

@@ -498,7 +498,7 @@ struct TcEpiFilter {
     float u[4] = {s.ub, -INFINITY, -INFINITY, -INFINITY}, l[4] = {s.lb, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const float4 r = __ldg(s.r + j * 8 + q);
+      const float4 r = s.r[j * 8 + q];
       u[0] = fmaxf(u[0], v[4 * q] + r.x);
       l[0] = fmaxf(l[0], v[4 * q] - r.x);
       u[1] = fmaxf(u[1], v[4 * q + 1] + r.y);

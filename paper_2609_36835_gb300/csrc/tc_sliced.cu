@@ -230,7 +230,7 @@ __device__ __forceinline__ void sl_tile(int tl, int Mt, int nt0, int nt1, bool l
 template <int S, class Out, int BN>
 __global__ void __launch_bounds__(SlShape<BN>::THREADS, 1)
     sliced_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB, const Out out,
-                       const int* __restrict__ eA, const int* __restrict__ eB, int H, int M, int N, int K, int lower,
+                       const int* eA, const int* eB, int H, int M, int N, int K, int lower,
                        int nt0, int nt1, DevStatus* stt) {
   using C = SlCfg<S, BN>;
   using Sh = SlShape<BN>;
@@ -545,7 +545,7 @@ __device__ __forceinline__ void digit_slices(T x, int e, bf16 (&o)[S]) {
 // as one 8-byte store (ldo is a multiple of 8, so every plane row is 16-byte
 // aligned).
 template <int S, typename T>
-__global__ void __launch_bounds__(256) slice_rows_kernel(const T* __restrict__ X, int R, int K, int ldx, long long xbs,
+__global__ void __launch_bounds__(256) slice_rows_kernel(const T* X, int R, int K, int ldx, long long xbs,
                                                          int H, bf16* __restrict__ out, int ldo,
                                                          int* __restrict__ ex) {
   chain_wait();
@@ -598,7 +598,7 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(const T* __restrict__ X
 // A CTA takes 32 columns (lane = column, coalesced rows); its 32 warps split
 // the rows (four loads in flight each) and meet in shared memory.
 template <typename T>
-__global__ void __launch_bounds__(1024) col_exp_kernel(const T* __restrict__ X, int K, int R, int ldx, long long xbs,
+__global__ void __launch_bounds__(1024) col_exp_kernel(const T* X, int K, int R, int ldx, long long xbs,
                                                        int* __restrict__ ex) {
   chain_wait();
   __shared__ unsigned long long part[32][33];
@@ -629,8 +629,8 @@ __global__ void __launch_bounds__(1024) col_exp_kernel(const T* __restrict__ X, 
 // [S][H][R][ldo] of X^T with the exponents of col_exp_kernel; 32 x 32 tiles
 // through shared memory.
 template <int S, typename T>
-__global__ void __launch_bounds__(256) slice_cols_kernel(const T* __restrict__ X, int K, int R, int ldx, long long xbs,
-                                                         int H, const int* __restrict__ ex, bf16* __restrict__ out,
+__global__ void __launch_bounds__(256) slice_cols_kernel(const T* X, int K, int R, int ldx, long long xbs,
+                                                         int H, const int* ex, bf16* __restrict__ out,
                                                          int ldo) {
   chain_wait();
   const int b = blockIdx.z, r0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
