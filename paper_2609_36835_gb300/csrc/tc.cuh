@@ -222,9 +222,10 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int n) {
 }  // namespace tc
 
 // Host: encode a 3-D tiled TMA map over a bf16 tensor [dim2][dim1][dim0]
-// (dim0 contiguous) with a box of {64, box1, 1} and 128-byte swizzle.
+// (dim0 contiguous; rows ld elements apart, batches bs, multiples of 8) with a
+// box of {64, box1, 1} and 128-byte swizzle.
 bool encode_bf16_map_3d(CUtensorMap* map, const void* base, uint64_t dim0, uint64_t dim1, uint64_t dim2,
-                        uint32_t box1);
+                        uint32_t box1, uint64_t ld = 0, uint64_t bs = 0);
 
 // Host: encode a 3-D tiled TMA map over a bf16 tensor [dim2][dim1][dim0] whose
 // rows are ld >= dim0 elements apart (ld a multiple of 8), with a box of

@@ -45,9 +45,12 @@ struct TcEpiArgmax {
 };
 
 // The same with eight epilogue warps, two per TMEM lane quarter, for 256-wide
-// tiles (each warp takes 128 columns).
+// tiles (each warp takes 128 columns).  gate (nullable): a non-zero word there
+// closes the launch (the filter has taken the call).
 struct TcEpiArgmax8 : TcEpiArgmax {
   static constexpr int kEpiWarps = 8;
+  const int* gate;
+  __device__ __forceinline__ bool closed() const { return gate != nullptr && __ldcg(gate) != 0; }
 };
 
 int launch_ref_logits_tc(const Dims& D, float scale, const bf16* Q, const bf16* K, float* L, float2* part,
@@ -424,10 +427,13 @@ __global__ void decode_assign_kernel(const unsigned long long* best, const int* 
 // bound may hold the argmax.  The second pass computes the split products of
 // those (key, tile) pairs alone, with the MMA sequence of the full GEMM, so the
 // scores it compares, and the result, have the same bits.
+//   tc_gemm (kPlain, TcEpiFilter), share_kernel  the bounds of 128 keys a head, and
+//                      whether few enough tiles are candidates for the rest to pay
 //   tc_gemm (kPlain, TcEpiFilter)  bounds per (key, tile)
 //   candidates_kernel  per (head, key chunk, tile): the list of its keys
 //   items_kernel       lists -> work items of 256 keys
 //   rescore_kernel     gathered keys x 128 anchors, argmax into `best`
+//   tc_gemm (kSplit, TcEpiArgmax8)  the full product, where the share said so
 // Keys go in chunks whose profiles stay in L2 while all anchor tiles pass them
 // (a key is a candidate in 16 of 103 tiles on average at 128K).
 // 128K layer (t = 13107, n = 2048, 8 heads): 26.6 + 0.5 + 22.6 ms (filter, lists,
@@ -448,7 +454,7 @@ static FilterDims filter_dims(const Dims& D) {
 }
 // byte offsets in the scratch (the index features' second half, free by then)
 struct FilterLayout {
-  size_t list, cnt, off, items, rho_k, rho_s, total;
+  size_t list, cnt, off, items, gate, rho_k, rho_s, total;
 };
 static FilterLayout filter_layout(const Dims& D, const FilterDims& f) {
   FilterLayout L;
@@ -459,25 +465,34 @@ static FilterLayout filter_layout(const Dims& D, const FilterDims& f) {
   L.cnt = take(E * 4);
   L.off = take((E + 1) * 4);
   L.items = take(E * (f.CR / kRsKeys) * 4);
+  L.gate = take(4);
   L.rho_k = take((size_t)D.H * D.T * 4);
   L.rho_s = take((size_t)D.H * f.Nt * 128 * 4);
   L.total = o;
   return L;
 }
-// Where the filter is used: from 24 tiles of 128 anchors up (a tile of few is
-// more often a candidate: 0.16 of all (key, tile) pairs at t = 13107, 0.37 at
-// 1638, 0.39 at 819, and the passes cost 0.35 + 1.9 times that share of the
-// full GEMM), when the bounds and lists fit the two halves of the index
-// features' buffer.  ms, 8 heads, with the filter (indexer's, highest-attention
-// anchors) against the full GEMM: T = 16384, n = 1024, t = 3000 0.87, 0.92
-// against 1.01; T = 32768, n = 2048, t = 3276 3.7, 4.0 against 4.7; T = 49152,
-// n = 2048, t = 4915 8.3, 9.0 against 10.5.
+// Where the filter is tried: from 24 tiles of 128 anchors, 512 reference rows
+// and n t = 2.2 M up, when its bounds and lists fit the two halves of the index
+// features' buffer.  Its passes over the bounds and lists do not shrink with n:
+// time of the stage with the filter over without, 8 heads, random anchors, at
+// n = 256, 512, 1024, 2048: t = 3000 1.25, 1.07, 0.98, 0.92 (768: 0.97); t = 6553
+// 1.19, 0.96, 0.86, 0.76; t = 13107 1.12, 0.95, 0.76, 0.73.
 bool assign_filtered(const Dims& D) {
   const FilterDims f = filter_dims(D);
   const size_t half = (size_t)D.H * D.T * D.HD * 2;
-  return D.t > 23 * 128 && D.T - D.t >= 4096 && f.CR % kRsKeys == 0 && (size_t)D.H * f.Nt * f.Tp * 8 <= half &&
-         filter_layout(D, f).total <= half;
+  return D.t > 23 * 128 && D.n >= 512 && (long long)D.n * D.t >= 2200000 && D.T - D.t >= 4096 && f.CR % kRsKeys == 0 &&
+         (size_t)D.H * f.Nt * f.Tp * 8 <= half && filter_layout(D, f).total <= half;
 }
+// The time over the full GEMM's grows by 1.2 to 1.4 times the share of (key,
+// tile) pairs that stay candidates, which is the data's: 0.2 to 0.4 for random
+// anchors, 1 for keys that are all alike (1.6 to 1.9 times the full GEMM's time).
+// The two take the same time at a share of about 0.35, 0.35 to 0.43 and 0.45 to
+// 0.55 for n = 512, 1024, 2048, so the rest of the filter runs where a sample of
+// kSampleKeys keys a head stays below the line here, else the full GEMM.  The stage
+// then takes 0.71 to 0.99 of the full GEMM's time where the filter's passes run, up
+// to 1.03 at a share near the line, and at most 1.02 where the sample turns it away.
+constexpr int kSampleKeys = 128;
+static float filter_share(int n) { return 0.5f - 80.f / n; }
 
 // Bounds of a row over its warp's 128 anchors (eight warps, 256-wide tiles).
 // rho_s is NaN past the last anchor: fmaxf skips those columns.
@@ -486,6 +501,8 @@ struct TcEpiFilter {
   const float* rho_s;   // [H][Nt * 128]
   float2* bounds;       // [H][Nt][Tp] (upper, lower)
   int Nt, Tp;
+  const int* gate;      // nullable: a zero word there closes the launch
+  __device__ __forceinline__ bool closed() const { return gate != nullptr && __ldcg(gate) == 0; }
   struct State {
     float ub, lb;
     const float4* r;
@@ -516,11 +533,45 @@ struct TcEpiFilter {
   }
 };
 
+// What a candidate's upper bound has to reach: upper + (rho_j + B0) >= lower -
+// (rho_j + B0) for the largest lower bound lb of a key's tiles.
+__device__ __forceinline__ float candidate_line(float lb, float rho, float B0) { return lb - 2.f * (rho + B0); }
+
+// gate = 1 where at most a share `most` of the (key, tile) pairs of the sample are
+// candidates: key k of a head is its compacted row k * step, its bounds at row k.
+__global__ void __launch_bounds__(1024) share_kernel(const float2* bounds, const float* rho_k, float B0, int T, int H,
+                                                     int step, int tiles, FilterDims f, float most, int* gate) {
+  chain_wait();
+  __shared__ int part[32];
+  int count = 0;
+  for (int k = threadIdx.x; k < H * kSampleKeys; k += 1024) {
+    const int b = k / kSampleKeys, row = k % kSampleKeys;
+    const float2* bd = bounds + (long long)b * f.Nt * f.Tp + row;
+    float lb = -INFINITY;
+#pragma unroll 8
+    for (int i = 0; i < tiles; ++i) lb = fmaxf(lb, bd[(long long)i * f.Tp].y);
+    const float thr = candidate_line(lb, rho_k[(long long)b * T + row * step], B0);
+    if (!(lb > -INFINITY)) continue;
+#pragma unroll 8
+    for (int i = 0; i < tiles; ++i) count += bd[(long long)i * f.Tp].x >= thr;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = count;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0.0;
+    for (int w = 0; w < 32; ++w) sum += part[w];
+    *gate = sum <= (double)most * H * kSampleKeys * tiles ? 1 : 0;
+  }
+}
+
 // One thread per key: the tiles that may hold its argmax, appended to their
 // lists (one atomic per warp and tile; the order within a list does not matter).
 __global__ void __launch_bounds__(256) candidates_kernel(const float2* bounds, const float* rho_k, float B0, int T, int Tm,
-                                                         FilterDims f, int* list, int* cnt) {
+                                                         FilterDims f, const int* gate, int* list, int* cnt) {
   chain_wait();
+  if (__ldcg(gate) == 0) return;   // (the lists stay empty)
   const int b = blockIdx.y, row = blockIdx.x * 256 + threadIdx.x, lane = threadIdx.x & 31;
   const int ch = blockIdx.x * 256 / f.CR;
   const float2* bd = bounds + (long long)b * f.Nt * f.Tp + row;
@@ -529,8 +580,8 @@ __global__ void __launch_bounds__(256) candidates_kernel(const float2* bounds, c
 #pragma unroll 8
   for (int k = 0; k < f.Nt; ++k)
     if (in) lb = fmaxf(lb, bd[(long long)k * f.Tp].y);
-  // upper + (rho_j + B0) >= lower - (rho_j + B0); no finite bound (a NaN profile): no candidate
-  const float thr = in ? lb - 2.f * (rho_k[(long long)b * T + row] + B0) : 0.f;
+  // (no finite bound, a NaN profile: no candidate)
+  const float thr = in ? candidate_line(lb, rho_k[(long long)b * T + row], B0) : 0.f;
   const bool any = in && lb > -INFINITY;
   const long long e0 = ((long long)b * f.nch + ch) * f.Nt;
 #pragma unroll 4
@@ -834,47 +885,83 @@ int launch_assign_prep(const Dims& D, const float* L, float* logphi, const int* 
   return col_profiles(D, L, logphi, po, stt, st);
 }
 
-// The two passes of the filtered assignment: `best` of every compacted row.
+// The full product: 128 keys x 256 anchors per tile (M = 128, N = 256 MMAs): half
+// the key-side operand bytes per flop of a 128-wide tile.  The key map spans all T
+// rows of a head (its plane stride); the GEMM takes the first Tm.
+static int full_argmax(const Dims& D, const bf16* Ut_hi, const bf16* Ut_lo, const bf16* S_hi, const bf16* S_lo,
+                       unsigned long long* best, const int* gate, DevStatus* stt, cudaStream_t st) {
+  constexpr int BN = 256;
+  const int ldn = (D.n + 7) / 8 * 8, Tm = D.T - D.t;
+  CUtensorMap mA, mA2, mB, mB2;
+  if (!encode_bf16_map_3d(&mA, Ut_hi, ldn, D.T, D.H, 128) || !encode_bf16_map_3d(&mA2, Ut_lo, ldn, D.T, D.H, 128) ||
+      !encode_bf16_map_3d(&mB, S_hi, ldn, D.t, D.H, BN) || !encode_bf16_map_3d(&mB2, S_lo, ldn, D.t, D.H, BN))
+    return -1;
+  TcEpiArgmax8 epi;
+  epi.best = best;
+  epi.bbs = D.T;
+  epi.gate = gate;
+  const int kfull = (ldn + 63) / 64 * 64;
+  // anchor tiles in groups whose split profiles (BN rows x ldn x 4 bytes per
+  // tile) take about 40 MB, so each group stays in L2 while the key profiles
+  // stream past it (one pass over them per group instead of one per wave)
+  const long long tile_bytes = (long long)BN * ldn * 4;
+  const int group = (int)std::max<long long>(1, (40LL << 20) / tile_bytes);
+  return launch_tc_gemm<BN, kSplit>(mA, mB, mA2, mB2, epi, D.H, Tm, D.t, ldn, kfull, stt, st, 0, nullptr, group) ==
+                 cudaSuccess
+             ? 1
+             : -1;
+}
+
+// The filtered assignment: `best` of every compacted row, by its two passes or,
+// where the sample says so, by the full product.
 static int filtered_argmax(const Dims& D, const bf16* Ut_hi, const bf16* Ut_lo, const bf16* S_hi, const bf16* S_lo,
                            float2* bounds, char* scratch, unsigned long long* best, DevStatus* stt, cudaStream_t st) {
   const FilterDims f = filter_dims(D);
   const FilterLayout L = filter_layout(D, f);
-  const int ldn = (D.n + 7) / 8 * 8, Tm = D.T - D.t, E = D.H * f.nch * f.Nt;
+  const int ldn = (D.n + 7) / 8 * 8, Tm = D.T - D.t, E = D.H * f.nch * f.Nt, step = Tm / kSampleKeys;
   const float* rho_k = (const float*)(scratch + L.rho_k);
   const float* rho_s = (const float*)(scratch + L.rho_s);
   int* list = (int*)(scratch + L.list);
   int* cnt = (int*)(scratch + L.cnt);
   int* off = (int*)(scratch + L.off);
   int* items = (int*)(scratch + L.items);
-  CUtensorMap mA, mB, mC, mC2;
-  if (!encode_bf16_map_3d(&mA, Ut_hi, ldn, D.T, D.H, 128) || !encode_bf16_map_3d(&mB, S_hi, ldn, D.t, D.H, 256) ||
+  int* gate = (int*)(scratch + L.gate);
+  CUtensorMap mS, mA, mB, mC, mC2;
+  // mS: every step-th compacted row of a head
+  if (!encode_bf16_map_3d(&mS, Ut_hi, ldn, kSampleKeys, D.H, 128, (uint64_t)step * ldn, (uint64_t)D.T * ldn) ||
+      !encode_bf16_map_3d(&mA, Ut_hi, ldn, D.T, D.H, 128) || !encode_bf16_map_3d(&mB, S_hi, ldn, D.t, D.H, 256) ||
       !encode_bf16_map_3d_sw64(&mC, S_hi, ldn, D.t, D.H, ldn, 128) ||
       !encode_bf16_map_3d_sw64(&mC2, S_lo, ldn, D.t, D.H, ldn, 128))
     return -1;
   if (cudaMemsetAsync(cnt, 0, (size_t)E * 4, st) != cudaSuccess) return -1;
+  const int kfull = (ldn + 63) / 64 * 64;
   const int group = (int)std::max<long long>(1, (40LL << 20) / (512LL * ldn));   // 40 MB of anchor rows stay in L2
-  const TcEpiFilter epi{rho_s, bounds, f.Nt, f.Tp};
-  if (launch_tc_gemm<256, kPlain>(mA, mB, mA, mB, epi, D.H, Tm, D.t, ldn, (ldn + 63) / 64 * 64, stt, st, 0, nullptr,
-                                  group) != cudaSuccess)
-    return -1;
   // B0: the split product drops lo lo and the lo parts' own rounding (2^-15 in
   // all); an fp32 accumulation step errs by at most 2^-20 of a sum below 1, and
   // the two passes take 4 n / 16 of them
   const float B0 = 0x1p-15f + (float)D.n * 0x1p-22f;
-  launch_chained(candidates_kernel, dim3(cdiv(Tm, 256), D.H), 256, 0, st, bounds, rho_k, B0, D.T, Tm, f, list, cnt);
+  TcEpiFilter epi{rho_s, bounds, f.Nt, f.Tp, nullptr};
+  if (launch_tc_gemm<256, kPlain>(mS, mB, mS, mB, epi, D.H, kSampleKeys, D.t, ldn, kfull, stt, st) != cudaSuccess)
+    return -1;
+  launch_chained(share_kernel, 1, 1024, 0, st, bounds, rho_k, B0, D.T, D.H, step, cdiv(D.t, 128), f, filter_share(D.n),
+                 gate);
+  epi.gate = gate;
+  if (launch_tc_gemm<256, kPlain>(mA, mB, mA, mB, epi, D.H, Tm, D.t, ldn, kfull, stt, st, 0, nullptr, group) !=
+      cudaSuccess)
+    return -1;
+  launch_chained(candidates_kernel, dim3(cdiv(Tm, 256), D.H), 256, 0, st, bounds, rho_k, B0, D.T, Tm, f, gate, list, cnt);
   launch_chained(items_kernel, 1, 1024, 0, st, cnt, E, f.CR / kRsKeys, off, items);
   const int smem = kRsStages * kRsStage + 1024;
   if (set_dyn_smem((const void*)rescore_kernel, smem) != cudaSuccess) return -1;
   if (launch_chained(rescore_kernel, tc_gemm_sm_count(), kRsThreads, smem, st, mC, mC2, Ut_hi, Ut_lo, list, cnt, off,
                      items, f, D.H, D.T, D.t, ldn, best, stt) != cudaSuccess)
     return -1;
-  return 4;
+  return full_argmax(D, Ut_hi, Ut_lo, S_hi, S_lo, best, gate, stt, st) < 0 ? -1 : 7;
 }
 
 int launch_assign_gemm(const Dims& D, const int* anchors, const bf16* Ut_hi, const bf16* Ut_lo, const bf16* S_hi,
                        const bf16* S_lo, const int* kmap, unsigned long long* best, int* kappa, float2* filter_bounds,
                        char* filter_scratch, DevStatus* stt, cudaStream_t st) {
-  const int ldn = (D.n + 7) / 8 * 8;
   const int Tm = D.T - D.t;   // the non-anchor keys, compacted (none when t = T)
   int nl = 1;
   // every key gets an assignment in [0, t) even when invalid caller anchors
@@ -882,33 +969,11 @@ int launch_assign_gemm(const Dims& D, const int* anchors, const bf16* Ut_hi, con
   cudaMemsetAsync(kappa, 0, sizeof(int) * (size_t)D.H * D.T, st);
   if (Tm > 0) {
     cudaMemsetAsync(best, 0, sizeof(unsigned long long) * (size_t)D.H * D.T, st);
-    if (filter_scratch) {
-      const int r = filtered_argmax(D, Ut_hi, Ut_lo, S_hi, S_lo, filter_bounds, filter_scratch, best, stt, st);
-      if (r < 0) return -1;
-      nl += r;
-    } else {
-      // 128 keys x 256 anchors per tile (M = 128, N = 256 MMAs): half the key-side
-      // operand bytes per flop of a 128-wide tile.  The key map spans all T rows
-      // of a head (its plane stride); the GEMM takes the first Tm.
-      constexpr int BN = 256;
-      CUtensorMap mA, mA2, mB, mB2;
-      if (!encode_bf16_map_3d(&mA, Ut_hi, ldn, D.T, D.H, 128) || !encode_bf16_map_3d(&mA2, Ut_lo, ldn, D.T, D.H, 128) ||
-          !encode_bf16_map_3d(&mB, S_hi, ldn, D.t, D.H, BN) || !encode_bf16_map_3d(&mB2, S_lo, ldn, D.t, D.H, BN))
-        return -1;
-      TcEpiArgmax8 epi;
-      epi.best = best;
-      epi.bbs = D.T;
-      const int kfull = (ldn + 63) / 64 * 64;
-      // anchor tiles in groups whose split profiles (BN rows x ldn x 4 bytes per
-      // tile) take about 40 MB, so each group stays in L2 while the key profiles
-      // stream past it (one pass over them per group instead of one per wave)
-      const long long tile_bytes = (long long)BN * ldn * 4;
-      const int group = (int)std::max<long long>(1, (40LL << 20) / tile_bytes);
-      if (launch_tc_gemm<BN, kSplit>(mA, mB, mA2, mB2, epi, D.H, Tm, D.t, ldn, kfull, stt, st, 0, nullptr, group) !=
-          cudaSuccess)
-        return -1;
-      ++nl;
-    }
+    const int r = filter_scratch
+                      ? filtered_argmax(D, Ut_hi, Ut_lo, S_hi, S_lo, filter_bounds, filter_scratch, best, stt, st)
+                      : full_argmax(D, Ut_hi, Ut_lo, S_hi, S_lo, best, nullptr, stt, st);
+    if (r < 0) return -1;
+    nl += r;
   }
   const long long keys = (long long)D.H * Tm, total = keys + (long long)D.H * D.t;
   launch_chained(decode_assign_kernel, stride_grid(total, 256, 8), 256, 0, st, best, kmap, anchors, kappa, D.T,

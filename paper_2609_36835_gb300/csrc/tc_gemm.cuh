@@ -94,6 +94,16 @@ struct EpiHalfLoads<E, std::void_t<decltype(E::kHalfLoads)>> {
   static constexpr bool value = E::kHalfLoads;
 };
 
+// An epilogue that declares closed() can have the launch return at once.
+template <class E, class = void>
+struct EpiGate {
+  static __device__ __forceinline__ bool closed(const E&) { return false; }
+};
+template <class E>
+struct EpiGate<E, std::void_t<decltype(&E::closed)>> {
+  static __device__ __forceinline__ bool closed(const E& e) { return e.closed(); }
+};
+
 template <int BN, int MODE>
 struct TcCfg {
   static constexpr bool SPLIT = MODE == kSplit;
@@ -162,6 +172,7 @@ __global__ void __launch_bounds__(64 + 32 * EpiWarps<Epi>::value, 1)
     tc::mbar_fence_init();
   }
   chain_wait();
+  if (EpiGate<Epi>::closed(epi)) return;   // (every thread reads the same word)
   if (warp == 1) tc::tmem_alloc(&tmem_slot, C::TMEM_COLS);
   tc::fence_before_sync();
   __syncthreads();

@@ -27,12 +27,14 @@ static bool encoder_ready() {
 }
 
 bool encode_bf16_map_3d(CUtensorMap* map, const void* base, uint64_t dim0, uint64_t dim1, uint64_t dim2,
-                        uint32_t box1) {
+                        uint32_t box1, uint64_t ld, uint64_t bs) {
   if (!encoder_ready()) return false;
+  if (ld == 0) ld = dim0;
+  if (bs == 0) bs = ld * dim1;
   // TMA requires a 16-byte aligned base and row strides that are multiples of 16 bytes
-  if (((uintptr_t)base & 15u) != 0 || (dim0 * 2) % 16 != 0) return false;
+  if (((uintptr_t)base & 15u) != 0 || (ld * 2) % 16 != 0 || (bs * 2) % 16 != 0 || ld < dim0) return false;
   const cuuint64_t gdim[3] = {dim0, dim1, dim2};
-  const cuuint64_t gstride[2] = {dim0 * 2, dim0 * dim1 * 2};
+  const cuuint64_t gstride[2] = {ld * 2, bs * 2};
   const cuuint32_t box[3] = {64, box1, 1};
   const cuuint32_t estride[3] = {1, 1, 1};
   const CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), gdim, gstride, box,
