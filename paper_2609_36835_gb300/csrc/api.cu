@@ -483,7 +483,8 @@ arckv_status arckv_attend_joint(int32_t H, int32_t n, int32_t t, int32_t F, int3
 size_t arckv_truncated_error_workspace_bytes(int32_t H, int32_t n, int32_t T, int32_t t, int32_t d) {
   if (H < 1 || n < 1 || T < 1 || t < 0 || t > T || d != 128) return 0;
   if ((long long)H * T >= (1LL << 40) || (long long)H * n >= (1LL << 31) || cdiv(n, 4) > 65535 || H > 65535) return 0;
-  const size_t rows = (size_t)H * trunc_split(H, n, T).nsplit * n;
+  const int nsplit = trunc_split(H, n, T).nsplit;
+  const size_t rows = nsplit > 1 ? (size_t)H * nsplit * n : 0;   // partial rows of the splits
   return up(sizeof(DevStatus)) + up((size_t)H * T) + up((size_t)H * n * 4) + up(rows * 256 * 4) + up(rows * 8);
 }
 
@@ -504,8 +505,9 @@ arckv_status arckv_truncated_error(int32_t H, int32_t n, int32_t T, int32_t t, i
   unsigned char* inS = (unsigned char*)(w + up(sizeof(DevStatus)));
   char* o = w + up(sizeof(DevStatus)) + up((size_t)H * T);
   float* err = (float*)o;
+  const int nsplit = trunc_split(H, n, T).nsplit;   // (one split: neither array is there, nor used)
   float* Opart = (float*)(o += up((size_t)H * n * 4));
-  float2* ml = (float2*)(o + up((size_t)H * trunc_split(H, n, T).nsplit * n * 256 * 4));
+  float2* ml = (float2*)(o + up((size_t)H * nsplit * n * 256 * 4));
   const float scale = logit_scale > 0.f ? logit_scale : 1.0f / sqrtf((float)d);
   cudaGetLastError();
   if (cudaMemsetAsync(stt, 0, sizeof(DevStatus), st) != cudaSuccess) return ARCKV_ERR_CUDA;

@@ -89,7 +89,25 @@ struct JointArgs {
   float2* ml;       // [H][nsplit][n] (running max, sum)
   float* O;         // one split: the result
   DevStatus* stt;
+  float* err;       // kErr, one split: the rows' errors [H][n]
+  float eps;
 };
+
+// ||o - o_S|| / (||o|| + eps) of a row, on lane 0: o and o_S at this lane's four
+// dims, unnormalised, over the same sum of weights l (one warp per row).
+__device__ __forceinline__ float row_error(const float (&o)[4], const float (&os)[4], float l, float eps) {
+  const float inv = 1.0f / l;
+  float dd = 0.f, oo = 0.f;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float x = o[e] * inv, y = os[e] * inv;
+    dd = fmaf(x - y, x - y, dd);
+    oo = fmaf(x, x, oo);
+  }
+  dd = warp_sum(dd);
+  oo = warp_sum(oo);
+  return sqrtf(dd) / (sqrtf(oo) + eps);
+}
 
 template <typename TC>
 constexpr int kJStageBytes = 2 * kJKeys * 128 * (int)sizeof(TC);   // K and V tile of one warp
@@ -306,6 +324,7 @@ __global__ void __launch_bounds__(32 * kJWarps, kErr ? 2 : 3) attend_warp_kernel
   __syncthreads();
   if (abort_flag) return;
   constexpr int kRing = kJStages * kJStageBytes<TC> / 4;   // floats between two warps' accumulators
+  __shared__ float sOut[kErr ? kJR : 1][2][128], sSum[kJR];   // kErr, one split: the merged rows
   bool bad = false;
 #pragma unroll
   for (int r = 0; r < kJR; ++r) {
@@ -330,13 +349,30 @@ __global__ void __launch_bounds__(32 * kJWarps, kErr ? 2 : 3) attend_warp_kernel
         o *= 1.0f / l;
         bad |= !isfinite(o);
         a.O[((long long)h * n + r0 + r) * 128 + tid] = o;
+      } else if (kErr && a.nsplit == 1) {
+        sOut[kErr ? r : 0][c][tid] = o;
       } else {
         a.Opart[(row * kA + c) * 128 + tid] = o;
       }
     }
-    if (tid == 0) a.ml[row] = make_float2(M, l);
+    if (tid == 0) {
+      if (a.nsplit > 1) a.ml[row] = make_float2(M, l);
+      else if (kErr) sSum[r] = l;
+    }
   }
   if (bad) set_status(a.stt, ARCKV_ERR_NONFINITE);
+  if (kErr && a.nsplit == 1) {   // one split: nothing to combine, warp w takes row r0 + w
+    __syncthreads();
+    if (r0 + w >= n) return;
+    float o[4], os[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      o[e] = sOut[kErr ? w : 0][0][lane * 4 + e];
+      os[e] = sOut[kErr ? w : 0][1][lane * 4 + e];
+    }
+    const float er = row_error(o, os, sSum[w], a.eps);
+    if (lane == 0) a.err[(long long)h * n + r0 + w] = er;
+  }
 }
 
 // O[h][i] = sum_s e^{m_s - m} Opart_s / sum_s e^{m_s - m} l_s (one warp per row, lane dims 4l..4l+3)
@@ -374,8 +410,10 @@ __global__ void __launch_bounds__(128) attend_combine_kernel(const float* Opart,
 //   O_i = sum_j p_ij v_j, O~_i(S) = sum_{j in S} p_ij v_j (p over the full cache),
 //   err_i = ||O_i - O~_i|| / (||O_i|| + eps).
 // The split-key pass above with two value accumulators (all keys; keys in S);
-// then one warp per row merges the splits and takes the norms.  8 heads, n = 64,
-// T = 8192: 0.17 ms a call; one CTA per four rows over all keys took 0.88 ms.
+// then one warp per row merges the splits and takes the norms (in the first kernel
+// where there is one split, so that the partial rows, 1 KB each, are kept only
+// where the rows are too few to fill the SMs).  8 heads, n = 64, T = 8192: 0.17 ms
+// a call; one CTA per four rows over all keys took 0.88 ms.
 __global__ void __launch_bounds__(128) trunc_combine_kernel(const float* Opart, const float2* ml, int n, int nsplit,
                                                             long long rows, float eps, float* err) {
   chain_wait();
@@ -398,17 +436,8 @@ __global__ void __launch_bounds__(128) trunc_combine_kernel(const float* Opart, 
     o[0] = fmaf(f, x.x, o[0]); o[1] = fmaf(f, x.y, o[1]); o[2] = fmaf(f, x.z, o[2]); o[3] = fmaf(f, x.w, o[3]);
     os[0] = fmaf(f, y.x, os[0]); os[1] = fmaf(f, y.y, os[1]); os[2] = fmaf(f, y.z, os[2]); os[3] = fmaf(f, y.w, os[3]);
   }
-  const float inv = 1.0f / l;
-  float dd = 0.f, oo = 0.f;
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const float x = o[e] * inv, y = os[e] * inv;
-    dd = fmaf(x - y, x - y, dd);
-    oo = fmaf(x, x, oo);
-  }
-  dd = warp_sum(dd);
-  oo = warp_sum(oo);
-  if (lane == 0) err[g] = sqrtf(dd) / (sqrtf(oo) + eps);
+  const float er = row_error(o, os, l, eps);
+  if (lane == 0) err[g] = er;
 }
 
 // inS[h][j] = 1 for the anchors S[h][:] (clamped into [0, T); out-of-range entries record INVALID_ARG)
@@ -474,13 +503,14 @@ int launch_truncated_error(int H, int n, int T, int t, float scale, float eps, c
     launch_chained(anchor_mask_kernel, stride_grid((long long)H * t, 256, 4), 256, 0, st, S, t, T, H, inS, stt);
   const JointSplit s = trunc_split(H, n, T);
   const JointArgs a{Q, n, nullptr, nullptr, nullptr, 0, K, V, T, inS, scale, s.per_split, s.nsplit, Opart, ml, nullptr,
-                    stt};
+                    stt, err, eps};
   set_dyn_smem((const void*)attend_warp_kernel<bf16, true>, kJSmem<bf16>);
   launch_chained(attend_warp_kernel<bf16, true>, dim3(s.nsplit, cdiv(n, kJR), H), 32 * kJWarps, kJSmem<bf16>, st, a);
   const long long rows = (long long)H * n;
-  launch_chained(trunc_combine_kernel, (unsigned)cdiv(rows, 4), 128, 0, st, Opart, ml, n, s.nsplit, rows, eps, err);
+  if (s.nsplit > 1)
+    launch_chained(trunc_combine_kernel, (unsigned)cdiv(rows, 4), 128, 0, st, Opart, ml, n, s.nsplit, rows, eps, err);
   launch_chained(row_mean_kernel, H, 32, 0, st, err, n, E, stt);
-  return t > 0 ? 4 : 3;
+  return 2 + (t > 0 ? 1 : 0) + (s.nsplit > 1 ? 1 : 0);
 }
 
 int launch_attend_joint(int H, int n, int t, int F, float scale, const bf16* Q, const void* Ck, const float* beta,
@@ -488,7 +518,7 @@ int launch_attend_joint(int H, int n, int t, int F, float scale, const bf16* Q, 
                         float2* ml, DevStatus* stt, cudaStream_t st) {
   const JointSplit s = joint_split(H, n, t, F);
   const dim3 grid(s.nsplit, cdiv(n, kJR), H);
-  const JointArgs a{Q, n, Ck, beta, Cv, t, Kf, Vf, F, nullptr, scale, s.per_split, s.nsplit, Opart, ml, O, stt};
+  const JointArgs a{Q, n, Ck, beta, Cv, t, Kf, Vf, F, nullptr, scale, s.per_split, s.nsplit, Opart, ml, O, stt, nullptr, 0.f};
   if (compact_bf16 || t == 0) {
     set_dyn_smem((const void*)attend_warp_kernel<bf16, false>, kJSmem<bf16>);
     launch_chained(attend_warp_kernel<bf16, false>, grid, 32 * kJWarps, kJSmem<bf16>, st, a);

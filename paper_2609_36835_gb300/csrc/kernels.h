@@ -233,8 +233,9 @@ struct JointSplit {
 
 // ---- HA / VI anchor scores (App. B.1) ----------------------------------
 // E[h] = mean_i ||O_i - O~_i(S)|| / (||O_i|| + eps) (Eq. background_truncated_error);
-// scratch inS [H][T] bytes, err [H][n], Opart [H][nsplit][n][2][128], ml
-// [H][nsplit][n] (trunc_split); non-finite results are recorded in stt.
+// scratch inS [H][T] bytes, err [H][n] and, with more than one split (trunc_split),
+// Opart [H][nsplit][n][2][128], ml [H][nsplit][n]; non-finite results are recorded
+// in stt.
 int launch_truncated_error(int H, int n, int T, int t, float scale, float eps, const bf16* Q, const bf16* K,
                            const bf16* V, const int* S, float* E, unsigned char* inS, float* err, float* Opart,
                            float2* ml, DevStatus* stt, cudaStream_t st);
