@@ -109,8 +109,10 @@ int launch_index_logits(const Dims& D, const bf16* qbar_hi, const bf16* qbar_lo,
   // 128 x 256 tiles (M = 128, N = 256 MMAs: a quarter fewer operand bytes per
   // flop than 128 x 128); the key operand's box is 256 rows.  A call whose 128-wide
   // tiles fit the SMs in one wave is as long as one tile and takes those (1 head,
-  // n = 256, T = 1024: 25 us on 8 SMs with 256-wide tiles, 17 on 16).
-  const bool wide = (long long)D.H * cdiv(D.n, 128) * cdiv(D.T, 128) > tc_gemm_sm_count();
+  // n = 256, T = 1024: 25 us on 8 SMs with 256-wide tiles, 17 on 16), and so does one
+  // whose keys fill no more than one (16 heads, n = 2048: T = 64 45 and 39 us, T = 128
+  // 49 and 41, but T = 200 53 and 60).
+  const bool wide = D.T > 128 && (long long)D.H * cdiv(D.n, 128) * cdiv(D.T, 128) > tc_gemm_sm_count();
   const int bB = wide ? 256 : 128;
   if (!encode_bf16_map_3d(&mA, qbar_hi, D.HD, D.n, D.H, 128) || !encode_bf16_map_3d(&mA2, qbar_lo, D.HD, D.n, D.H, 128) ||
       !encode_bf16_map_3d(&mB, kbar_hi, D.HD, D.T, D.H, bB) || !encode_bf16_map_3d(&mB2, kbar_lo, D.HD, D.T, D.H, bB))
