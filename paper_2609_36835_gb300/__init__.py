@@ -211,8 +211,10 @@ def _on_one_cuda_device(**tensors):
 def _stream_handle(stream) -> Optional[int]:
     if stream is None:
         import torch
-        # the current stream's handle without the Stream object around it
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        # the current stream's handle without the Stream object around it, where
+        # this torch has that (private) call
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        return raw(torch.cuda.current_device()) if raw is not None else torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
