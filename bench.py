@@ -349,6 +349,16 @@ def profiled_traffic():
     return float(m.group(1)) if h.group(1) == dominant_source_hash() else None
 
 
+def assignment_kernel(t):
+    """The kernels of the assignment stage at t anchors, and whether that is the
+    full product for certain.  The library tries the filter above 23 tiles of 128
+    anchors, by further sizes and by the data (tc_assign.cu): not restated here."""
+    full = "tc_gemm_kernel<256, kSplit, TcEpiArgmax8>"
+    if t <= 23 * 128:
+        return full, True
+    return "tc_gemm_kernel<256, kPlain, TcEpiFilter> + rescore_kernel, or %s where those would not pay" % full, False
+
+
 # ------------------------------------------------------------ reference arm
 
 def oracle_segments(w, pairs, selector="indexer", chunk_len=0):
@@ -600,28 +610,27 @@ def run_gpu(args, dist: Dist):
     # stage 5), 2 n (T - t) t useful flops per head (the anchors' own assignment
     # is fixed, kappa(s_r) = r: the T - t other keys are scored against the t
     # anchors).  One split-bf16 tcgen05 GEMM issuing three bf16 MMAs per useful
-    # product, or, from 24 anchor tiles up (tc_assign.cu, assign_filtered), a
-    # one-product filter over all pairs and split products over those that it
-    # leaves: how many those are depends on the data, so no issued rate is given
-    filtered = tp > 23 * 128 and w.T - tp >= 4096
+    # product, or a one-product filter over all pairs and split products over those
+    # that it leaves: which of them, and how many, depends on the data as well, so
+    # no issued rate is given where the filter may run
+    kernel, one_gemm = assignment_kernel(tp)
     flops = 2.0 * w.H_kv * w.n * (w.T - tp) * tp
     avg_s = statistics.mean(stage_launch_ms[5]) / 1e3
     iso_s = statistics.median(iso_ms[5]) / 1e3
     peak, _, peak_src = measured_peaks()
     burst = measured_burst()
     achieved = flops / avg_s / 1e12
-    roofline = {"kernel": ("tc_gemm_kernel<256, kPlain, TcEpiFilter> + rescore_kernel" if filtered else
-                           "tc_gemm_kernel<256, kSplit, TcEpiArgmax8>") + " (assignment, Eq. anchor_assignment)",
+    roofline = {"kernel": kernel + " (assignment, Eq. anchor_assignment)",
                 "bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": profiled_traffic(), "flops_per_launch": flops, "launch_ms": avg_s * 1e3,
-                "issued_tflops": None if filtered else 3.0 * achieved,
-                "issued_frac": None if filtered else 3.0 * achieved / peak,
+                "issued_tflops": 3.0 * achieved if one_gemm else None,
+                "issued_frac": 3.0 * achieved / peak if one_gemm else None,
                 "launch_ms_isolated": iso_s * 1e3, "frac_isolated": flops / iso_s / 1e12 / burst,
                 "timing_note": "launch_ms: live CUDA events over the timed region, where %d streams share the GPU; "
                                "launch_ms_isolated: the same launch with the GPU to itself (median of 5), "
                                "frac_isolated against the burst peak" % n_str,
                 "peak_note": "bf16 dense, sustained, of %s (MEASURED_PEAKS.json); achieved counts useful flops, "
-                             "issued (null with the filter) the 3 bf16 MMAs of each split-bf16 product" % peak_src}
+                             "issued (null where the filter may run) the 3 bf16 MMAs of each split-bf16 product" % peak_src}
     # the solvers of the two fits (stages 8 and 10), timed the same way
     dual = tp > w.n
     m_sys = w.n if dual else tp
