@@ -78,8 +78,9 @@ Layout plan(const arckv_config& c) {
   L.q_l = take(H * n * 128 * 2);
   L.av = take(H * n * 128 * f);
   L.VT = take(H * 128 * ldT * 2);
-  // with T % 4 != 0 a workspace has always held three bf16 [n][T] arrays here,
-  // and keeps its size
+  // nothing uses this room: three bf16 [n][T] arrays of an earlier form of the
+  // softmax-V product at T % 4 != 0, which the size of a workspace is still held to
+  // (tests/test_abi_host.py)
   L.spare = take((T & 3) ? 3 * H * n * ldT * 2 : 0);
   L.qcat = take(H * n * 512 * 2);
   L.vq3 = take(3 * H * n * 128 * 2);

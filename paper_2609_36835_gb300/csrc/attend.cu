@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kAvThreads, 1)
     // first), four keys per lane
     constexpr int kSteps = kR / 32;
     const int cw = warp - 2, hl = lane >> 4, cl = lane & 15;
-    float zl[kSteps], mu[kSteps];   // shift log2 e and scale (0, 0 past the end: P = 0)
+    float zl[kSteps], mu[kSteps];   // shift and scale (0, 0 past the end: P = 0)
 #pragma unroll
     for (int u = 0; u < kSteps; ++u) {
       const int row = m0 + cw * (kR / 16) + 2 * u + hl;

@@ -23,9 +23,10 @@ __host__ __device__ inline int chunk_budget(int T, int t, int Tc) {
   return (int)(q < 1 ? 1 : (q > Tc ? Tc : q));
 }
 // Row pitch (elements) of an fp32 [n][T] logit matrix: T rounded up to the 16
-// bytes that TMA wants, so that every T is stored and read in tiles (before,
-// T % 4 != 0 went through per-thread stores and a probability triple in memory:
-// 0.55 + 0.41 ms against 0.09 + 0.23 for 8 heads, n = 512, T = 20011).
+// bytes that TMA wants, so that the GEMMs store every T in tiles and the softmax-V
+// product reads it in tiles (before, T % 4 != 0 went through per-thread stores and
+// a probability triple in memory: 0.55 + 0.41 ms against 0.09 + 0.23 for 8 heads,
+// n = 512, T = 20011).  Column profiles and pooling read T % 4 != 0 by element.
 inline int logit_ld(int T) { return (T + 3) & ~3; }
 inline int effective_chunk(int T, int chunk_len) { return (chunk_len > 0 && T > kChunkThreshold) ? chunk_len : 0; }
 inline int realized_anchors(int T, int t, int chunk_len) {
