@@ -114,7 +114,9 @@ constexpr int kJStageBytes = 2 * kJKeys * 128 * (int)sizeof(TC);   // K and V ti
 template <typename TC>
 constexpr int kJSmem = kJWarps * kJStages * kJStageBytes<TC>;
 
-template <typename TC, bool kErr>
+// kOne: kErr with one split, a kernel of its own (its shared rows and their norms
+// in the other one cost a call of 160 us 4 of them).
+template <typename TC, bool kErr, bool kOne = false>
 __global__ void __launch_bounds__(32 * kJWarps, kErr ? 2 : 3) attend_warp_kernel(const JointArgs a) {
   chain_wait();
   extern __shared__ __align__(128) unsigned char smraw[];
@@ -324,7 +326,7 @@ __global__ void __launch_bounds__(32 * kJWarps, kErr ? 2 : 3) attend_warp_kernel
   __syncthreads();
   if (abort_flag) return;
   constexpr int kRing = kJStages * kJStageBytes<TC> / 4;   // floats between two warps' accumulators
-  __shared__ float sOut[kErr ? kJR : 1][2][128], sSum[kJR];   // kErr, one split: the merged rows
+  __shared__ float sOut[kOne ? kJR : 1][2][kOne ? 128 : 1], sSum[kJR];   // kOne: the merged rows
   bool bad = false;
 #pragma unroll
   for (int r = 0; r < kJR; ++r) {
@@ -349,26 +351,26 @@ __global__ void __launch_bounds__(32 * kJWarps, kErr ? 2 : 3) attend_warp_kernel
         o *= 1.0f / l;
         bad |= !isfinite(o);
         a.O[((long long)h * n + r0 + r) * 128 + tid] = o;
-      } else if (kErr && a.nsplit == 1) {
-        sOut[kErr ? r : 0][c][tid] = o;
+      } else if constexpr (kOne) {
+        sOut[r][c][tid] = o;
       } else {
         a.Opart[(row * kA + c) * 128 + tid] = o;
       }
     }
     if (tid == 0) {
-      if (a.nsplit > 1) a.ml[row] = make_float2(M, l);
-      else if (kErr) sSum[r] = l;
+      if constexpr (kOne) sSum[r] = l;
+      else a.ml[row] = make_float2(M, l);
     }
   }
   if (bad) set_status(a.stt, ARCKV_ERR_NONFINITE);
-  if (kErr && a.nsplit == 1) {   // one split: nothing to combine, warp w takes row r0 + w
+  if constexpr (kOne) {   // nothing to combine, warp w takes row r0 + w
     __syncthreads();
     if (r0 + w >= n) return;
     float o[4], os[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      o[e] = sOut[kErr ? w : 0][0][lane * 4 + e];
-      os[e] = sOut[kErr ? w : 0][1][lane * 4 + e];
+      o[e] = sOut[w][0][lane * 4 + e];
+      os[e] = sOut[w][1][lane * 4 + e];
     }
     const float er = row_error(o, os, sSum[w], a.eps);
     if (lane == 0) a.err[(long long)h * n + r0 + w] = er;
@@ -507,8 +509,9 @@ int launch_truncated_error(int H, int n, int T, int t, float scale, float eps, c
   const JointSplit s = trunc_split(H, n, T);
   const JointArgs a{Q, n, nullptr, nullptr, nullptr, 0, K, V, T, inS, scale, s.per_split, s.nsplit, Opart, ml, nullptr,
                     stt, err, eps};
-  set_dyn_smem((const void*)attend_warp_kernel<bf16, true>, kJSmem<bf16>);
-  launch_chained(attend_warp_kernel<bf16, true>, dim3(s.nsplit, cdiv(n, kJR), H), 32 * kJWarps, kJSmem<bf16>, st, a);
+  auto kern = s.nsplit > 1 ? attend_warp_kernel<bf16, true> : attend_warp_kernel<bf16, true, true>;
+  set_dyn_smem((const void*)kern, kJSmem<bf16>);
+  launch_chained(kern, dim3(s.nsplit, cdiv(n, kJR), H), 32 * kJWarps, kJSmem<bf16>, st, a);
   const long long rows = (long long)H * n;
   if (s.nsplit > 1)
     launch_chained(trunc_combine_kernel, (unsigned)cdiv(rows, 4), 128, 0, st, Opart, ml, n, s.nsplit, rows, eps, err);
